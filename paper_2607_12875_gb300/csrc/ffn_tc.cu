@@ -514,8 +514,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             if (rank == 0) drain_wait(&full[s], (inflight_par >> s) & 1u);
             if (CG == 2) drain_wait(&empty[s], (inflight_par >> s) & 1u);
         }
-    } else if (warp == 1 && lane == 0 && rank == 0) {
-        // ------------------------------------------------------ MMA issuer
+    } else if (warp == 1 && rank == 0) {
+        // ------------------------- MMA issuer (the whole warp, one lane issues)
+        const uint64_t da0 = sw128_desc(smem_u32(sA)), db0 = sw128_desc(smem_u32(sB));
         int stage = 0;
         uint32_t phase = 0;
         int acc = 0;
@@ -523,35 +524,35 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         bool ok = true;
         bool issued = false;
         for (int w = unit; w < total && ok; w += n_units) {
-            if (!(CG == 1 ? mbar_wait(&tempty[acc], acc_phase ^ 1, abort_flag, p.err, p.wait_limit_ns)
-                          : mbar_wait_cluster(&tempty[acc], acc_phase ^ 1, abort_flag, p.err, p.wait_limit_ns))) {
-                ok = false;
-                break;
-            }
+            if (!warp_wait<CG == 2>(&tempty[acc], acc_phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                if (RAW && !mbar_wait(&conv[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                if (RAW && !warp_wait(&conv[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 tc_fence_after();
-                const uint64_t da = sw128_desc(smem_u32(sA + stage * A_BYTES));
-                const uint64_t db = sw128_desc(smem_u32(sB + stage * BH));
+                const uint64_t da = da0 + (uint64_t)(stage * A_BYTES >> 4);
+                const uint64_t db = db0 + (uint64_t)(stage * BH >> 4);
+                if (elect_one()) {
 #pragma unroll
-                for (int j = 0; j < BK / 16; ++j)  // +32 bytes along K per slice
-                    mma_bf16<CG>(d_tmem, da + 2 * j, db + 2 * j, (kb | j) != 0 ? 1u : 0u);
+                    for (int j = 0; j < BK / 16; ++j)  // +32 bytes along K per slice
+                        mma_bf16<CG>(d_tmem, da + 2 * j, db + 2 * j, (kb | j) != 0 ? 1u : 0u);
+                    commit_to<CG>(&empty[stage], 0x3);
+                    if (kb == nkb - 1) commit_to<CG>(&tfull[acc], 0x3);
+                }
+                __syncwarp();
                 issued = true;
-                commit_to<CG>(&empty[stage], 0x3);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
             if (!ok) break;
-            commit_to<CG>(&tfull[acc], 0x3);
             if (++acc == 2) { acc = 0; acc_phase ^= 1; }
         }
         if (issued) {
             // every MMA issued has finished before TMEM is released (after a
             // normal run the epilogue has seen them all; after an abort in
             // another role this issuer may have run up to two tiles ahead)
-            commit_to<CG>(drain, 0x1);
+            if (elect_one()) commit_to<CG>(drain, 0x1);
+            __syncwarp();
             drain_wait(drain, 0);
         }
     } else if (warp >= 2 && warp < 6) {

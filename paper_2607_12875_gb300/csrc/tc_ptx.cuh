@@ -63,6 +63,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// one poll that does not suspend the thread
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 __device__ __forceinline__ uint64_t global_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -74,37 +87,29 @@ __device__ __forceinline__ uint64_t global_ns() {
 // or another role of this CTA has already given up. The clock is read after
 // every failed poll, so a wait longer than the limit always gives up.
 template <bool kCluster = false>
-__device__ __forceinline__ bool mbar_wait_inl(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* err,
-                                       uint64_t limit_ns) {
-    if (mbar_try_wait<kCluster>(bar, parity)) return true;
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* err,
+                                          uint64_t limit_ns) {
+    // (try_wait may suspend the thread for a while; a limit of 0 takes no wait at all)
+    if (limit_ns != 0 ? mbar_try_wait<kCluster>(bar, parity) : mbar_test_wait(bar, parity)) return true;
     const uint64_t t0 = global_ns();
     for (;;) {
-        if (mbar_try_wait<kCluster>(bar, parity)) return true;
         if (*abort_flag) return false;
-        if (global_ns() - t0 > limit_ns) {
+        if (global_ns() - t0 >= limit_ns) {
             *abort_flag = 1;
             set_error(err, kErrTimeout);
             return false;
         }
+        if (mbar_try_wait<kCluster>(bar, parity)) return true;
     }
-}
-
-static __device__ __noinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* err,
-                                       uint64_t limit_ns) {
-    return mbar_wait_inl(bar, parity, abort_flag, err, limit_ns);
-}
-
-static __device__ __noinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                    int32_t* err, uint64_t limit_ns) {
-    return mbar_wait_inl<true>(bar, parity, abort_flag, err, limit_ns);
 }
 
 // The same wait by every lane of a warp, with one outcome for the whole warp:
 // if any lane gave up, all of them return false together, so no lane goes on
 // to a warp-synchronous step (__syncwarp, tcgen05.ld) its neighbours skip.
+template <bool kCluster = false>
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* err,
                                           uint64_t limit_ns) {
-    const bool ok = mbar_wait_inl(bar, parity, abort_flag, err, limit_ns);  // inline: no call with live registers
+    const bool ok = mbar_wait<kCluster>(bar, parity, abort_flag, err, limit_ns);
     return __all_sync(0xffffffffu, ok);
 }
 
@@ -160,6 +165,20 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
     return d;
+}
+
+// True in one lane of a converged warp. Issuing MMAs under this predicate from
+// warp-uniform code (every lane runs the role's loop and waits) keeps their
+// descriptors in uniform registers; under `lane == 0` the compiler moves each
+// operand there for every MMA.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
