@@ -70,14 +70,16 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
 
 /* Which expert-FFN kernels run. GBMOE_FFN_TC_FP8 (FP8_E4M3_B128 weights and
  * bf16 activations only) multiplies the stored e4m3 weights on the fp8 tensor
- * cores: each GEMM's input rows (x, then h) are brought to e4m3 with one fp32
- * scale s per row and 128 consecutive k (s = amax / 448) as two codes,
- * q1 = e4m3(x / s) and q2 = e4m3(x / s - q1), so that x = s * (q1 + q2) to
- * within max(2^-8 |x / s|, 2^-10) * s, a bf16-like precision; both codes are
+ * cores: each GEMM's input rows (x, then h) are brought to e4m3 with one
+ * power-of-two scale s per row and 128 consecutive k (the block's largest
+ * |x / s| lies in [128, 256)) as two codes, q1 = e4m3(x / s) and
+ * q2 = e4m3(x / s - q1), so that x = s * (q1 + q2) exactly where
+ * |x / s| >= 2^-2 and within 2^-10 * s below that; both codes are
  * multiplied with the weights and each 128-wide k block's partial sum is
  * scaled by both blocks' scales and accumulated in fp32. AUTO takes it for
- * fp8 weights whenever a tensor-core route applies.
- * AUTO streams weights when the average number
+ * fp8 weights with bf16 activations at every size (with few rows per expert
+ * the weights are the GEMM's M operand, with many the rows are).
+ * Otherwise AUTO streams weights when the average number
  * of rows per expert P/E is at most 16 and otherwise runs the grouped GEMM
  * (tensor cores for bf16 activations, CUDA cores for fp32). On the tensor
  * cores, int4/MXFP4 weights are decoded inside the GEMM when P/E < 256; with

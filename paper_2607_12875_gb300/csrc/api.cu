@@ -77,17 +77,17 @@ bool stream_fits(int act_dtype, int H, int I) { return stream_smem_bytes(act_dty
 int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     int r = c->ffn_route;
     if (r != GBMOE_FFN_AUTO) return r;
+    FfnProblem probe{};
+    probe.act_dtype = c->act_dtype;
+    probe.w_dtype = c->w_dtype;
+    probe.H = c->H;
+    probe.I = I;
+    probe.E = E;
+    // fp8 weights with bf16 activations: the fp8 tensor-core route at every
+    // size (no decode; its two-term activation codes keep bf16's accuracy)
+    if (ffn_tc_fp8_supported(probe)) return GBMOE_FFN_TC_FP8;
     if (n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I)) return GBMOE_FFN_STREAM;
     if (c->act_dtype == GBMOE_BF16) {
-        FfnProblem probe{};
-        probe.act_dtype = c->act_dtype;
-        probe.w_dtype = c->w_dtype;
-        probe.H = c->H;
-        probe.I = I;
-        probe.E = E;
-        // fp8 weights: the fp8 tensor-core route (no decode; its two-term
-        // activation codes keep bf16-level accuracy)
-        if (ffn_tc_fp8_supported(probe)) return GBMOE_FFN_TC_FP8;
         if (ffn_tc_supported(probe)) {
             const bool dequant = quantised_weights(c->w_dtype) && n_rows >= kDequantRowsPerExpert * E;
             // CTA pairs (256-row tiles) once experts are deep enough that the
@@ -260,7 +260,10 @@ int run_ffn(const gbmoe_config* c, FfnProblem& p, int route, cudaStream_t stream
     switch (route) {
         case GBMOE_FFN_STREAM: err = launch_ffn_stream(p, stream); break;
         case GBMOE_FFN_SIMT: err = launch_ffn_simt(p, stream); break;
-        case GBMOE_FFN_TC_FP8: err = launch_ffn_tc_fp8(p, stream); break;
+        case GBMOE_FFN_TC_FP8:
+            err = ffn_fm_supported(p) && p.n_rows <= kFmRowsPerExpert * p.E ? launch_ffn_fm(p, stream)
+                                                                            : launch_ffn_tc_fp8(p, stream);
+            break;
         default:  // GBMOE_FFN_TC, _TC_DEQUANT, _TC_PAIR, _TC_PAIR_DEQUANT
             p.cta_pair = pair_route(route) ? 1 : 0;
             err = launch_ffn_tc(p, stream);

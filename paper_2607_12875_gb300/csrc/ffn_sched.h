@@ -7,7 +7,7 @@
 namespace gbmoe {
 
 constexpr int kSchedHeader = 8;  // [0] active experts, [1] tiles, rest reserved
-constexpr int kSchedMinBM = 32;  // smallest tile height any FFN route uses
+constexpr int kSchedMinBM = 16;  // smallest tile height any FFN route uses
 
 inline int64_t sched_max_tiles(int E, int64_t n_rows, int BM) { return (n_rows + BM - 1) / BM + E; }
 

@@ -13,7 +13,7 @@
 namespace gbmoe {
 
 constexpr int kBM = 32, kBN = 32, kBK = 32;
-static_assert(kBM == kSchedMinBM, "tile list is built for the SIMT tile height");
+static_assert(kBM >= kSchedMinBM, "the tile list has room for the SIMT tile height");
 
 template <typename TA, int WQ>
 __global__ void __launch_bounds__(256)

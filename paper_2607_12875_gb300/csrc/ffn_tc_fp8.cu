@@ -4,11 +4,8 @@
 // (e4m3, one fp32 scale per 128x128 block, the format of Section 6.2): the
 // weight tiles go from HBM to shared memory to tcgen05.mma kind::f8f6f4
 // unchanged, with no decode step. The activations entering each GEMM (x,
-// then h) are brought to e4m3 per row and 128 consecutive k: with
-// s = amax / 448 and v = x / s, a first code q1 = e4m3(v) and a second code
-// q2 = e4m3(v - q1) for what the first leaves out, so that x = s * (q1 + q2)
-// with an error of at most max(2^-8 |v|, 2^-10) * s (a single e4m3 code would
-// leave up to 2^-4 |v|: about 4% of a row's largest output). Each 128-wide k
+// then h) are brought to two e4m3 codes q1, q2 per value and one scale s per
+// row and 128 consecutive k (quant_act.cu). Each 128-wide k
 // block takes two MMA passes, q1 x W and q2 x W, into the same partial sum
 // in tensor memory; the epilogue warps promote it,
 // acc += P * s * w_scale[n-block][k-block], into fp32 accumulators held in
@@ -36,10 +33,6 @@
 // up rows of the same output columns; a promoting thread holds 64 gate and the
 // matching 64 up columns of its row, so SwiGLU needs no exchange.
 // Every mbarrier wait is bounded as in the bf16 GEMM (tc_ptx.cuh).
-#include <cuda_fp8.h>
-
-#include <cstdlib>
-
 #include "common.cuh"
 #include "ffn_sched.h"
 #include "kernels.h"
@@ -120,73 +113,6 @@ template <bool SWIGLU>
 __device__ __forceinline__ void b_rows(const Params& p, const Work& wk, int& b0, int& b1) {
     b0 = wk.e * p.b_rows_per_expert + (SWIGLU ? wk.nt * (BN / 2) : wk.nt * BN);
     b1 = SWIGLU ? b0 : b0 + BN / 2;
-}
-
-// ---------------------------------------------- activation quantisation
-
-// e4m3 codes of (a, b), a in the low byte: round to nearest even, saturating
-// at +-448 (the hardware conversion)
-__device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
-    return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3);
-}
-
-// Rows of a bf16 matrix [*, K] -> two e4m3 code planes q1, q2 [n_rows, K]
-// and fp32 scales s [n_rows, K/128]: for every row and 128-wide block,
-// amax = max |x|, s = amax / 448 (1 when amax = 0), v = x / s,
-// q1 = e4m3(v), q2 = e4m3(v - q1) (v - q1 is exact in fp32); both roundings
-// to nearest even, saturating. Row r reads
-// source row sorted_pair[r] / pair_div (r itself without sorted_pair; a
-// negative entry gives a zero row). One warp per row; lane l takes elements
-// 4l .. 4l+3 of every block.
-__global__ void __launch_bounds__(256)
-quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ sorted_pair, int pair_div,
-                  int64_t n_rows, int K, uint8_t* __restrict__ q1, uint8_t* __restrict__ q2,
-                  float* __restrict__ s) {
-    pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int nblk = K / QB;
-    for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_rows; r += warps) {
-        int64_t srow = r;
-        if (sorted_pair) {
-            const int32_t pr = sorted_pair[r];
-            srow = pr >= 0 ? pr / pair_div : -1;
-        }
-        constexpr int U = 8;  // blocks whose loads are in flight together
-        for (int b0 = 0; b0 < nblk; b0 += U) {
-            uint2 raw[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                raw[u] = make_uint2(0, 0);
-                if (srow >= 0 && b0 + u < nblk)
-                    raw[u] = *reinterpret_cast<const uint2*>(src + srow * K + (b0 + u) * QB + 4 * lane);
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int b = b0 + u;
-                if (b >= nblk) break;
-                const float v[4] = {bf16lo(raw[u].x), bf16hi(raw[u].x), bf16lo(raw[u].y), bf16hi(raw[u].y)};
-                float amax = fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3])));
-#pragma unroll
-                for (int d = 16; d >= 1; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
-                const float sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
-                float t[4], rr[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) t[i] = __fdiv_rn(v[i], sc);
-                const uint32_t a = e4m3x2(t[0], t[1]) | (e4m3x2(t[2], t[3]) << 16);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const __half_raw h =
-                        __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)((a >> (8 * i)) & 0xffu), __NV_E4M3);
-                    rr[i] = __fsub_rn(t[i], __half2float(__half(h)));
-                }
-                const uint32_t a2 = e4m3x2(rr[0], rr[1]) | (e4m3x2(rr[2], rr[3]) << 16);
-                *reinterpret_cast<uint32_t*>(q1 + r * K + b * QB + 4 * lane) = a;
-                *reinterpret_cast<uint32_t*>(q2 + r * K + b * QB + 4 * lane) = a2;
-                if (lane == 0) s[r * nblk + b] = sc;
-            }
-        }
-    }
 }
 
 // -------------------------------------------------------------- the GEMM
@@ -272,8 +198,9 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
         }
         for (int s = 0; s < STAGES; ++s)
             if ((inflight >> s) & 1u) drain_wait(&full[s], (inflight_par >> s) & 1u);
-    } else if (warp == 1 && lane == 0) {
-        // ------------------------------------------------------ MMA issuer
+    } else if (warp == 1) {
+        // ------------------------- MMA issuer (the whole warp, one lane issues)
+        const uint64_t da0 = sw128_desc(smem_u32(sA1)), db0 = sw128_desc(smem_u32(sB));
         int stage = 0;
         uint32_t phase = 0;
         uint32_t kbg = 0;  // k blocks issued so far: partial buffer kbg & 1, its use (kbg >> 1)
@@ -282,27 +209,31 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
         for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
             for (int kb = 0; kb < nkb; ++kb, ++kbg) {
                 const uint32_t pb = kbg & 1u, pph = (kbg >> 1) & 1u;
-                if (!mbar_wait(&pempty[pb], pph ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                if (!mbar_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                if (!warp_wait(&pempty[pb], pph ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 tc_fence_after();
-                const uint64_t da1 = sw128_desc(smem_u32(sA1 + stage * A_BYTES));
-                const uint64_t da2 = sw128_desc(smem_u32(sA2 + stage * A_BYTES));
-                const uint64_t db = sw128_desc(smem_u32(sB + stage * B_BYTES));
+                const uint64_t da1 = da0 + (uint64_t)(stage * A_BYTES >> 4);
+                const uint64_t da2 = da1 + (uint64_t)(STAGES * A_BYTES >> 4);
+                const uint64_t db = db0 + (uint64_t)(stage * B_BYTES >> 4);
                 const uint32_t d_tmem = tmem_base + pb * BN;
+                if (elect_one()) {
 #pragma unroll
-                for (int j = 0; j < BK / 32; ++j)  // +32 bytes along K per instruction
-                    mma_fp8(d_tmem, da1 + 2 * j, db + 2 * j, j != 0 ? 1u : 0u);
+                    for (int j = 0; j < BK / 32; ++j)  // +32 bytes along K per instruction
+                        mma_fp8(d_tmem, da1 + 2 * j, db + 2 * j, j != 0 ? 1u : 0u);
 #pragma unroll
-                for (int j = 0; j < BK / 32; ++j)  // the residual codes into the same partial sum
-                    mma_fp8(d_tmem, da2 + 2 * j, db + 2 * j, 1u);
+                    for (int j = 0; j < BK / 32; ++j)  // the residual codes into the same partial sum
+                        mma_fp8(d_tmem, da2 + 2 * j, db + 2 * j, 1u);
+                    mma_commit(&empty[stage]);
+                    mma_commit(&pfull[pb]);
+                }
+                __syncwarp();
                 issued = true;
-                mma_commit(&empty[stage]);
-                mma_commit(&pfull[pb]);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }
         if (issued) {  // every MMA issued has finished before TMEM is released
-            mma_commit(drain);
+            if (elect_one()) mma_commit(drain);
+            __syncwarp();
             drain_wait(drain, 0);
         }
     } else if (warp >= 2) {
@@ -414,19 +345,6 @@ static bool map_e4m3(CUtensorMap* m, const void* base, int64_t rows, int64_t K, 
     return make_map(m, base, rows, K, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, BK, CU_TENSOR_MAP_SWIZZLE_128B, box_rows);
 }
 
-// q holds the two code planes [2, n_rows, K]
-static cudaError_t launch_quant(const void* src, const int32_t* sorted_pair, int pair_div, int64_t n_rows, int K,
-                                void* q, float* s, cudaStream_t stream) {
-    const int blocks = (int)min64((n_rows + 7) / 8, (int64_t)sm_count() * 16);
-    if (blocks <= 0) return cudaSuccess;
-    if (const cudaError_t le = launch_k(quant_rows_kernel, dim3(blocks), dim3(256), 0, stream,
-            static_cast<const __nv_bfloat16*>(src), sorted_pair, pair_div, n_rows, K, static_cast<uint8_t*>(q),
-            static_cast<uint8_t*>(q) + n_rows * K, s);
-        le != cudaSuccess)
-        return le;
-    return cudaGetLastError();
-}
-
 template <bool SWIGLU>
 static cudaError_t launch_gemm(const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& b0,
                                const CUtensorMap& b1, const Params& prm, int64_t max_work, cudaStream_t stream) {
@@ -458,7 +376,7 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     cudaError_t err = launch_ffn_schedule(p.counts, p.E, p.n_rows, BM, p.sched, stream);
     if (err != cudaSuccess) return err;
     // x rows in sorted order (x itself for the shared expert), quantised per 1x128
-    if ((err = launch_quant(p.x, p.sorted_pair, p.pair_div, p.n_rows, p.H, p.a_q, p.a_s, stream)) != cudaSuccess)
+    if ((err = launch_quant_rows(p.x, p.sorted_pair, p.pair_div, p.n_rows, p.H, p.a_q, p.a_s, stream)) != cudaSuccess)
         return err;
     const int64_t max_m = sched_max_tiles(p.E, p.n_rows, BM);
     const uint8_t* aq = static_cast<const uint8_t*>(p.a_q);
@@ -479,7 +397,7 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     g.wait_limit_ns = tc_wait_limit_ns();
     if ((err = launch_gemm<true>(ma1, ma2, mg, mu, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
     // h quantised per 1x128 for the down GEMM
-    if ((err = launch_quant(p.h, nullptr, 1, p.n_rows, p.I, p.h_q, p.h_s, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.h, nullptr, 1, p.n_rows, p.I, p.h_q, p.h_s, stream)) != cudaSuccess) return err;
     Params d = g;
     d.K = p.I; d.n_tiles = p.H / BN; d.out_cols = p.H; d.b_rows_per_expert = p.H;
     d.out = static_cast<__nv_bfloat16*>(p.y);

@@ -94,6 +94,17 @@ bool ffn_tc_supported(const FfnProblem& p);
 bool ffn_tc_pair_supported(const FfnProblem& p);
 cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream);
 bool ffn_tc_fp8_supported(const FfnProblem& p);
+// The feature-major GEMM runs up to this many rows per expert; beyond, its
+// promotion (every row's partial sums, per 128 k) costs more than the 128-row
+// MMAs of the row-major GEMMs. fp8 layer, 256 experts, H 7168, I 2048, both
+// ways: 1.93 against 2.33 ms at 8 rows per expert, 2.30 against 2.50 at 32,
+// 2.67 against 2.66 at 47, 3.40 against 2.79 at 64.
+constexpr int64_t kFmRowsPerExpert = 40;
+// rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales
+cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
+                              float* s, cudaStream_t stream);
+cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream);
+bool ffn_fm_supported(const FfnProblem& p);
 
 cudaError_t launch_combine(const void* y_pairs, const float* topk_w, const int32_t* pair_pos, const void* y_shared,
                            void* out, int T, int k, int H, int act_dtype, cudaStream_t stream);

@@ -1,0 +1,76 @@
+"""The feature-major GEMM (quantised weights as the M operand of tcgen05.mma),
+which AUTO takes for few rows per expert, against the oracle at the edges of
+its row tiles, and with activations that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2607_12875_gb300 as gb
+import synth
+from gpu_helpers import act_np, assert_close, config, to_device, tol_for, wbundle, workspace
+
+pytestmark = pytest.mark.gpu
+
+BASE = synth.WORKLOADS[1].replace(act="bf16")
+
+
+def forward(wl, dev):
+    cfg = config(wl)
+    ws = workspace(cfg)
+    out = torch.empty((wl.T, wl.H), dtype=torch.bfloat16, device="cuda")
+    gb.moe_forward(cfg, dev["x"], dev["w_router"], dev["logit_bias"], dev["select_bias"], wbundle(dev["experts"]),
+                   wbundle(dev["shared"]), out, ws)
+    torch.cuda.synchronize()
+    assert gb.moe_device_status(ws) == gb.OK
+    return out
+
+
+# rows per expert: 1, groups of 8 and one more, whole 16-row tiles, the last
+# size with short tiles (4 rows per expert on average) and the first without,
+# the last before the row-major GEMM takes over; one k block and ragged rings
+@pytest.mark.parametrize("wq", ["fp8_b128"])
+@pytest.mark.parametrize("T,E,k,H,I", [(1, 8, 2, 256, 128), (8, 4, 1, 512, 128), (9, 1, 1, 256, 256),
+                                       (4, 1, 1, 768, 384), (32, 16, 2, 1024, 128), (33, 16, 2, 256, 640),
+                                       (40, 1, 1, 512, 256), (63, 4, 2, 1280, 256)])
+def test_row_tiles(T, E, k, H, I, wq):
+    wl = BASE.replace(T=T, E=E, top_k=k, H=H, I=I, wq=wq, seed=T + 7 * E)
+    inp = synth.make_inputs(wl)
+    out = forward(wl, to_device(wl, inp))
+    assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol_for(wl))
+
+
+@pytest.mark.parametrize("wq", ["fp8_b128"])
+@pytest.mark.parametrize("T", [16, 17, 80, 81, 200])
+def test_all_rows_on_one_expert(T, wq):
+    """A hot expert's rows fill whole row tiles and spill into the next."""
+    wl = BASE.replace(T=T, E=16, top_k=2, H=512, I=256, wq=wq, seed=T)
+    inp = synth.make_inputs(wl)
+    bias = np.zeros(wl.E, np.float32)
+    bias[3] = 1000.0
+    inp["logit_bias"] = bias
+    ref = oracle.forward(wl, inp)
+    assert ref["counts"][3] == T
+    assert_close(act_np(forward(wl, to_device(wl, inp))), ref["out"], tol_for(wl))
+
+
+@pytest.mark.parametrize("wq", ["fp8_b128"])
+def test_not_finite_rows_stay_in_their_token(wq):
+    """An infinity or NaN in one token's activations leaves every other token's
+    output bit for bit as it was; its own output is not finite. Values whose
+    squares or quotients would leave fp32's range are scaled exactly."""
+    wl = BASE.replace(T=24, E=8, top_k=2, H=512, I=256, wq=wq, seed=5)
+    inp = synth.make_inputs(wl)
+    dev = to_device(wl, inp)
+    # the experts are fixed by a bias, so that the routing does not depend on the rows changed below
+    dev["logit_bias"] = torch.arange(wl.E, device="cuda", dtype=torch.float32) * 1e6
+    a = forward(wl, dev)
+    for t, v in ((3, float("inf")), (4, float("nan")), (5, float("-inf"))):
+        dev["x"][t, 130] = v
+    dev["x"][6] = 0
+    dev["x"][7] *= 1e-38
+    b = forward(wl, dev)
+    same = [t for t in range(wl.T) if t not in (3, 4, 5, 6, 7)]
+    assert torch.equal(a[same].view(torch.int16), b[same].view(torch.int16))
+    assert all(not torch.isfinite(b[t].float()).all() for t in (3, 4, 5))
+    assert torch.isfinite(b[6:8].float()).all() and float(b[6].float().abs().max()) == 0.0
