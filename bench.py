@@ -265,7 +265,9 @@ def launches_per_step(wl, route: str, shared_route) -> int:
     itself, + 3 weight-decode passes on the decode-once routes), and the
     combine."""
     def ffn(r, routed):
-        if r == "tc_fp8":  # schedule, x quantisation, gate/up GEMM, h quantisation, down GEMM
+        rows, experts = (wl.P, wl.E) if routed else (wl.T, 1)
+        few = wl.act == "bf16" and wl.wq in ("int4_g128", "mxfp4") and rows <= 40 * experts
+        if r == "tc_fp8" or (r == "tc" and few):  # schedule, x codes, gate/up GEMM, h codes, down GEMM
             return 5
         # the one-CTA bf16 GEMM gathers its own rows; decoding GEMMs and pairs use the gather kernel
         gather = r in ("tc_pair", "tc_pair_dequant") or (r == "tc" and wl.wq != "bf16")

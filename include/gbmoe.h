@@ -79,10 +79,15 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * scaled by both blocks' scales and accumulated in fp32. AUTO takes it for
  * fp8 weights with bf16 activations at every size (with few rows per expert
  * the weights are the GEMM's M operand, with many the rows are).
- * Otherwise AUTO streams weights when the average number
- * of rows per expert P/E is at most 16 and otherwise runs the grouped GEMM
- * (tensor cores for bf16 activations, CUDA cores for fp32). On the tensor
- * cores, int4/MXFP4 weights are decoded inside the GEMM when P/E < 256; with
+ * int4/MXFP4 weights with bf16 activations and at most 40 rows per expert
+ * (P/E) multiply the same activation codes on the fp8 tensor cores under AUTO
+ * (every int4 value and FP4 value is an e4m3 value; group scales are applied
+ * in fp32, and the E8M0 scales of a row's 128 consecutive k relative to the
+ * largest of the four, exactly down to 2^-14 of it); this too is reported as
+ * GBMOE_FFN_TC.
+ * Otherwise AUTO streams weights when P/E is at most 16 and otherwise runs the
+ * grouped GEMM (tensor cores for bf16 activations, CUDA cores for fp32). On
+ * the tensor cores, int4/MXFP4 weights are decoded inside the GEMM when P/E < 256; with
  * more rows per expert (several M tiles reuse each weight tile) AUTO takes
  * GBMOE_FFN_TC_DEQUANT: one pass decodes the active experts' weights to a
  * bf16 copy in the workspace (the same bf16 values the in-GEMM decode makes),

@@ -86,6 +86,10 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     // fp8 weights with bf16 activations: the fp8 tensor-core route at every
     // size (no decode; its two-term activation codes keep bf16's accuracy)
     if (ffn_tc_fp8_supported(probe)) return GBMOE_FFN_TC_FP8;
+    // int4 and MXFP4 weights with bf16 activations and few rows per expert: the
+    // feature-major GEMM (use_fm), reported as TC
+    const bool four_bit = c->w_dtype == GBMOE_INT4_G128 || c->w_dtype == GBMOE_MXFP4;
+    if (four_bit && n_rows <= kFmRowsPerExpert * E && ffn_fm_supported(probe)) return GBMOE_FFN_TC;
     if (n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I)) return GBMOE_FFN_STREAM;
     if (c->act_dtype == GBMOE_BF16) {
         if (ffn_tc_supported(probe)) {
@@ -101,6 +105,20 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     return GBMOE_FFN_SIMT;
 }
 
+// Whether that problem runs on the feature-major GEMM (ffn_fm.cu): fp8 weights
+// on the fp8 route, forced or not; int4 and MXFP4 when AUTO chose (a forced
+// TC is the row-major GEMM).
+bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
+    FfnProblem probe{};
+    probe.act_dtype = c->act_dtype;
+    probe.w_dtype = c->w_dtype;
+    probe.H = c->H;
+    probe.I = I;
+    if (n_rows > kFmRowsPerExpert * E || !ffn_fm_supported(probe)) return false;
+    return c->w_dtype == GBMOE_FP8_E4M3_B128 ? pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8
+                                             : c->ffn_route == GBMOE_FFN_AUTO;
+}
+
 // Bytes of the bf16 weight copy the TC_DEQUANT route decodes into (0 when
 // the route of that problem does not use one).
 size_t dequant_bytes(const gbmoe_config* c, int64_t n_rows, int E, int I) {
@@ -114,6 +132,7 @@ size_t dequant_bytes(const gbmoe_config* c, int64_t n_rows, int E, int I) {
 size_t sorted_x_bytes(const gbmoe_config* c) {
     const int64_t P = (int64_t)c->T * c->top_k;
     const int r = pick_route(c, P, c->E, c->I);
+    if (use_fm(c, P, c->E, c->I)) return 0;
     const bool reads_copy = pair_route(r) || (r == GBMOE_FFN_TC && quantised_weights(c->w_dtype));
     return reads_copy ? (size_t)P * c->H * act_bytes(c->act_dtype) : 0;
 }
@@ -123,10 +142,13 @@ struct Layout {
         wdq_sh, aq, as, hq, hs, total;
 };
 
-// true when the routed or the shared FFN problem of c runs on the fp8 route
-bool uses_fp8_route(const gbmoe_config* c) {
-    if (pick_route(c, (int64_t)c->T * c->top_k, c->E, c->I) == GBMOE_FFN_TC_FP8) return true;
-    return c->has_shared && pick_route(c, c->T, 1, c->I_shared) == GBMOE_FFN_TC_FP8;
+// true when the routed or the shared FFN problem of c multiplies e4m3 codes of
+// its activations (the fp8 route, the feature-major GEMM)
+bool uses_act_codes(const gbmoe_config* c) {
+    auto codes = [&](int64_t n_rows, int E, int I) {
+        return use_fm(c, n_rows, E, I) || pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8;
+    };
+    return codes((int64_t)c->T * c->top_k, c->E, c->I) || (c->has_shared && codes(c->T, 1, c->I_shared));
 }
 
 Layout layout(const gbmoe_config* c) {
@@ -158,11 +180,12 @@ Layout layout(const gbmoe_config* c) {
     L.xout = take((size_t)T * H * ab);
     L.wdq = take(dequant_bytes(c, P, (int)E, c->I));
     L.wdq_sh = take(c->has_shared ? dequant_bytes(c, T, 1, c->I_shared) : 0);
-    const bool f8 = uses_fp8_route(c);  // e4m3 copies of the GEMM inputs and their 1x128 scales
-    L.aq = take(f8 ? (size_t)2 * rows_max * H : 0);  // two e4m3 code planes
-    L.as = take(f8 ? (size_t)rows_max * (H / 128) * 4 : 0);
-    L.hq = take(f8 ? (size_t)2 * rows_max * I_max : 0);
-    L.hs = take(f8 ? (size_t)rows_max * (I_max / 128) * 4 : 0);
+    const bool codes = uses_act_codes(c);  // e4m3 copies of the GEMM inputs, their 1x128 scales (and sums: int4)
+    const size_t per_block = c->w_dtype == GBMOE_INT4_G128 ? 8 : 4;
+    L.aq = take(codes ? (size_t)2 * rows_max * H : 0);  // two e4m3 code planes
+    L.as = take(codes ? (size_t)rows_max * (H / 128) * per_block : 0);
+    L.hq = take(codes ? (size_t)2 * rows_max * I_max : 0);
+    L.hs = take(codes ? (size_t)rows_max * (I_max / 128) * per_block : 0);
     L.total = o;
     return L;
 }
@@ -257,13 +280,11 @@ int route_launchable(const gbmoe_config* c, int route, int I) {
 int run_ffn(const gbmoe_config* c, FfnProblem& p, int route, cudaStream_t stream) {
     if (int s = route_launchable(c, route, p.I)) return s;
     cudaError_t err;
+    if (use_fm(c, p.n_rows, p.E, p.I)) return cuda_status(launch_ffn_fm(p, stream));
     switch (route) {
         case GBMOE_FFN_STREAM: err = launch_ffn_stream(p, stream); break;
         case GBMOE_FFN_SIMT: err = launch_ffn_simt(p, stream); break;
-        case GBMOE_FFN_TC_FP8:
-            err = ffn_fm_supported(p) && p.n_rows <= kFmRowsPerExpert * p.E ? launch_ffn_fm(p, stream)
-                                                                            : launch_ffn_tc_fp8(p, stream);
-            break;
+        case GBMOE_FFN_TC_FP8: err = launch_ffn_tc_fp8(p, stream); break;
         default:  // GBMOE_FFN_TC, _TC_DEQUANT, _TC_PAIR, _TC_PAIR_DEQUANT
             p.cta_pair = pair_route(route) ? 1 : 0;
             err = launch_ffn_tc(p, stream);
@@ -272,9 +293,9 @@ int run_ffn(const gbmoe_config* c, FfnProblem& p, int route, cudaStream_t stream
     return cuda_status(err);
 }
 
-// the fp8 route's scratch (the routed and the shared problem run one after
-// the other, so they share it)
-void set_fp8_buffers(FfnProblem& p, const Layout& L, void* ws) {
+// the activation codes' scratch (the routed and the shared problem run one
+// after the other, so they share it)
+void set_code_buffers(FfnProblem& p, const Layout& L, void* ws) {
     p.a_q = at<char>(ws, L.aq);
     p.a_s = at<float>(ws, L.as);
     p.h_q = at<char>(ws, L.hq);
@@ -295,7 +316,7 @@ FfnProblem routed_problem(const gbmoe_config* c, const void* x, const int32_t* c
     p.x_sorted = sorted_x_bytes(c) ? at<char>(ws, L.xs) : nullptr;
     p.err = at<int32_t>(ws, L.err);
     p.w_dq = dequant_bytes(c, p.n_rows, p.E, p.I) ? at<char>(ws, L.wdq) : nullptr;
-    set_fp8_buffers(p, L, ws);
+    set_code_buffers(p, L, ws);
     return p;
 }
 
@@ -311,7 +332,7 @@ FfnProblem shared_problem(const gbmoe_config* c, const void* x, const gbmoe_expe
     p.h = at<char>(ws, L.h); p.x_sorted = nullptr; p.sched = at<int32_t>(ws, L.sched);  // rows in order
     p.err = at<int32_t>(ws, L.err);
     p.w_dq = dequant_bytes(c, p.n_rows, p.E, p.I) ? at<char>(ws, L.wdq_sh) : nullptr;
-    set_fp8_buffers(p, L, ws);
+    set_code_buffers(p, L, ws);
     return p;
 }
 
@@ -500,8 +521,8 @@ int moe_forward(const gbmoe_config* cfg, const void* x, const void* w_router, co
         if ((s = run_ffn(cfg, ps, r_shared, st))) return s;
     }
     FfnProblem pr = routed_problem(cfg, x, counts, offsets, sorted, experts, y, ws);
-    const bool fused = cfg->combine_route == GBMOE_COMBINE_FUSED &&
-                       bf16_gemm_route(r_routed);
+    const bool fused = cfg->combine_route == GBMOE_COMBINE_FUSED && bf16_gemm_route(r_routed) &&
+                       !use_fm(cfg, P, cfg->E, cfg->I);
     if (fused) {  // Weight Sum in the down GEMM's epilogue
         if ((s = cuda_status(cudaMemsetAsync(at<int32_t>(ws, L.arrive), 0, (size_t)cfg->T * (cfg->H / 256) * 4, st))))
             return s;

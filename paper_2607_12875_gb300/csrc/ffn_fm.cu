@@ -24,13 +24,14 @@
 // One persistent CTA per SM walks (row tile, 256 weight rows) items. Warps:
 //   0       TMA of the weight tile of each k block (2 x 128 rows x 128 k),
 //           128-byte swizzled, into a ring of stages;
-//   1       TMEM (three partial sums) and the MMAs: per k block and 128-row
-//           half, q1 and q2 side by side (N = 2 * rows);
+//   1       TMEM (three or four slots of partial sums) and the MMAs: per k
+//           block and 128-row half, q1 and q2 side by side (N = 2 * rows);
 //   2-3     gather the row codes with cp.async (the token's row of x, so no
 //           sorted copy exists) and their scales;
-//   4-11    promotion and the output: warp w reads TMEM lanes 32 * (w % 4)..
-//           (weight rows); the rows' groups of 8 alternate between the two sets of
-//           four warps.
+//   4-7 or 4-11  promotion and the output: warp w reads TMEM lanes
+//           32 * (w % 4).. (weight rows); tall tiles' groups of 8 rows
+//           alternate between the two sets of four warps;
+//   the last 4 or 8  int4 and MXFP4: decode the tile to e4m3 codes.
 // A gate/up item holds 128 gate rows and the 128 up rows of the same columns,
 // so one thread ends up with gate and up of its column and SwiGLU needs no
 // exchange. Every mbarrier wait is bounded (tc_ptx.cuh).
@@ -40,6 +41,13 @@
 // us against the streaming kernels, 7.5 TB/s; the layer 3121 -> 1347 us. What
 // held it back on the way, per 128-wide k block: waits as calls (2400 -> 1750
 // cycles once inlined) and MMAs issued under `lane == 0` (1750 -> 1500).
+// int4, 17 tokens, top 6 of 64 experts, H 4096, I 2816: layer 1397 -> 255 us;
+// MXFP4, 16 tokens of the fp8 layer: 2896 -> 956 us. These two are bound by the
+// decode warps' instructions (1700 cycles per k block for MXFP4, where HBM
+// would allow 735): eight of them instead of four took the gate/up kernel from
+// 681 to 504 us, both partial sums in one handshake included.
+#include <cuda_fp8.h>
+
 #include "common.cuh"
 #include "ffn_sched.h"
 #include "kernels.h"
@@ -53,36 +61,52 @@ using namespace tc;
 constexpr int MB = 128;                 // weight rows per MMA
 constexpr int BK = 128;                 // k per block: one swizzle row, one activation scale
 constexpr int A_BYTES = 2 * MB * BK;    // the two 128-row halves of an item's weight tile
-constexpr int MAX_ROWS = 80;            // most rows of a row tile
-constexpr int SLOTS = 3;                // partial sums in TMEM
-constexpr int SLOT_COLS = 2 * MAX_ROWS;
-constexpr int TMEM_COLS = 512;          // (an allocation is a power of two)
-constexpr int MAX_STAGES = 6;
-// Scale blocks, used in turn (stages + 2 of them): a block's k block k is
-// written once the MMAs of k - stages are done, which were issued once the
-// partial sums of k - stages - 2 had been promoted (TMEM holds fewer than two
-// k blocks), so the block's last contents have been read by then.
-constexpr int RING = MAX_STAGES + 2;
-constexpr int SETS = 2;                 // of four promotion warps
-constexpr int PROMOTE_WARPS = 4 * SETS;
-constexpr int GROUPS = (MAX_ROWS / 8 + SETS - 1) / SETS;  // most groups of 8 rows of a promotion warp
+constexpr int TMEM_COLS = 512;
 constexpr int GATHER_WARPS = 2;
-constexpr int THREADS = 32 * (2 + GATHER_WARPS + PROMOTE_WARPS);
-constexpr int NUM_BARS = 3 * MAX_STAGES + 2 * SLOTS + RING + 1;
-constexpr int FIXED_BYTES = 1024 + RING * MAX_ROWS * 4 + NUM_BARS * 8 + 16;
+constexpr int LUT_ENTRIES = 256;
 constexpr int SMEM_BUDGET = 232448;
 
-constexpr int stage_bytes(int tile_rows) { return A_BYTES + 2 * tile_rows * BK; }
-constexpr int stages_for(int tile_rows) {
-    const int n = (SMEM_BUDGET - FIXED_BYTES) / stage_bytes(tile_rows);
-    return n < MAX_STAGES ? n : MAX_STAGES;
-}
-static_assert(stages_for(MAX_ROWS) >= 3 && SLOTS <= 4 && SLOTS * SLOT_COLS <= TMEM_COLS, "ring depth");
+// Per weight format and height of a row tile.
+template <int WQ, int ROWS>
+struct Cfg {
+    // int4, MXFP4: bytes of the tile as stored, which the decode warps turn into e4m3
+    static constexpr int RAW = WQ == GBMOE_FP8_E4M3_B128 ? 0 : A_BYTES / 2;
+    // Short tiles: a k block's two partial sums share a slot of TMEM, which
+    // halves the handshakes that then dominate; tall tiles fill it with one.
+    static constexpr bool JOINT = ROWS <= 16;
+    static constexpr int SLOTS = JOINT ? 4 : 3;
+    static constexpr int SLOT_COLS = JOINT ? 4 * ROWS : 2 * ROWS;
+    static constexpr int SETS = JOINT ? 1 : 2;  // of four promotion warps
+    static constexpr int PROMOTE_WARPS = 4 * SETS;
+    static constexpr int GROUPS = (ROWS / 8 + SETS - 1) / SETS;  // most groups of 8 rows of a promotion warp
+    static constexpr int DECODE_WARPS = RAW ? (JOINT ? 8 : 4) : 0;
+    static constexpr int THREADS = 32 * (2 + GATHER_WARPS + PROMOTE_WARPS + DECODE_WARPS);
+    static constexpr int STAGE_BYTES = A_BYTES + RAW + 2 * ROWS * BK;
+    // floats of a scale block: the rows' scales and negated sums of codes, then
+    // (formats that are decoded) the weight rows' scales
+    static constexpr int RING_FLOATS = 2 * ROWS + (RAW ? 2 * MB : 0);
+    static constexpr int LUT_BYTES = WQ == GBMOE_MXFP4 ? LUT_ENTRIES * 8 : 0;
+    static constexpr int MAX_STAGES = 6;
+    static constexpr int MAX_RING = MAX_STAGES + 4;
+    static constexpr int NUM_BARS = 3 * MAX_STAGES + 2 * SLOTS + MAX_RING + 1;
+    static constexpr int FIXED_BYTES = 1024 + MAX_RING * RING_FLOATS * 4 + LUT_BYTES + NUM_BARS * 8 + 16;
+    static constexpr int FIT = (SMEM_BUDGET - FIXED_BYTES) / STAGE_BYTES;
+    static constexpr int STAGES = FIT < MAX_STAGES ? FIT : MAX_STAGES;
+    // Scale blocks, used in turn: k block k's is written once the MMAs of
+    // k - STAGES are done, which were issued once the partial sums of
+    // k - STAGES - AHEAD had been promoted (TMEM holds at most AHEAD k blocks),
+    // so what the block held before, k - RING's scales, has been read by then.
+    static constexpr int AHEAD = JOINT ? SLOTS : 2;
+    static constexpr int RING = STAGES + AHEAD;
+    static constexpr int SMEM_BYTES = FIXED_BYTES + STAGES * STAGE_BYTES;
+    static_assert(STAGES >= 3 && AHEAD <= 4 && SLOTS * SLOT_COLS <= TMEM_COLS, "ring depth");
+    static_assert(ROWS % 8 == 0 && ROWS <= 128, "two rows' scales per gather thread");
+};
 
 struct Params {
     int K, n_tiles, out_cols;
     int w_rows_per_expert;  // rows of the weight tensor per expert
-    int tile_rows;          // rows of a row tile of the work list (a multiple of 16, at most MAX_ROWS)
+    int tile_rows;          // rows of a row tile of the work list
     const int32_t* counts;
     const int32_t* offsets;
     const int32_t* sched;
@@ -95,8 +119,10 @@ struct Params {
     const float* a_scale;    // [plane_rows][K/128]
     const int32_t* gather;   // row r of the sorted order is plane row gather[r] / gather_div; null: r itself
     int gather_div;
-    const float* w_scale0;   // fp8: [E, w_rows_per_expert/128, K/128], first / second half of the item
-    const float* w_scale1;
+    const float* a_sum;      // int4: [plane_rows][K/128] sums of codes
+    const void* w_scale0;    // first / second half of the item: fp8 fp32 [E, w_rows_per_expert/128, K/128],
+    const void* w_scale1;    // int4 bf16 [E, w_rows_per_expert, K/128], MXFP4 E8M0 bytes [E, w_rows_per_expert, K/32]
+    int scale_words;         // MXFP4: the E8M0 bytes are 4-byte aligned (they need only be 2-byte aligned)
     uint64_t wait_limit_ns;
 };
 
@@ -205,55 +231,111 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&a)[8], uint32_t (&b)[8], ui
 }
 
 // acc += (a + b) * (sc * w) over 8 rows: a, b the q1 and q2 partial sums, sc
-// the rows' scales in shared memory, w the weight scale in both halves
+// the rows' scales in shared memory, w the weight scale in both halves. int4
+// (see the decode warps): acc += (a + b - sum) * (sc * w), the rows' negated
+// sums ROWS behind their scales.
+template <int WQ, int ROWS>
 __device__ __forceinline__ void promote8(const uint32_t (&a)[8], const uint32_t (&b)[8], const float* sc, uint64_t w,
                                          uint64_t* acc) {
     const float4 f0 = *reinterpret_cast<const float4*>(sc), f1 = *reinterpret_cast<const float4*>(sc + 4);
     const uint64_t f[4] = {pack2(f0.x, f0.y), pack2(f0.z, f0.w), pack2(f1.x, f1.y), pack2(f1.z, f1.w)};
+    uint64_t v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-        acc[i] = fma2(add2(pack2u(a[2 * i], a[2 * i + 1]), pack2u(b[2 * i], b[2 * i + 1])), mul2(f[i], w), acc[i]);
+    for (int i = 0; i < 4; ++i) v[i] = add2(pack2u(a[2 * i], a[2 * i + 1]), pack2u(b[2 * i], b[2 * i + 1]));
+    if constexpr (WQ == GBMOE_INT4_G128) {
+        const float4 c0 = *reinterpret_cast<const float4*>(sc + ROWS), c1 = *reinterpret_cast<const float4*>(sc + ROWS + 4);
+        v[0] = add2(v[0], pack2(c0.x, c0.y)); v[1] = add2(v[1], pack2(c0.z, c0.w));
+        v[2] = add2(v[2], pack2(c1.x, c1.y)); v[3] = add2(v[3], pack2(c1.z, c1.w));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = fma2(v[i], mul2(f[i], w), acc[i]);
 }
+
+// 16 bytes of int4 weights -> 32 e4m3 codes, the even values of each 8 before
+// the odd ones. A two's complement nibble n with its top bit flipped is
+// u = n + 8, 0 <= u <= 15, and the byte u read as e4m3 is u * 2^-9 (bits 0-2
+// are the mantissa, bit 3 the lowest exponent bit: the subnormals run on into
+// the first normal binade), so a shift and a mask decode 8 values; the 8 is
+// taken back out per block in the promotion (sum of u * q - 8 * sum of q).
+__device__ __forceinline__ void decode_int4_32(const uint4 raw, uint4& o0, uint4& o1) {
+    auto even = [](uint32_t w) { return (w & 0x0f0f0f0fu) ^ 0x08080808u; };
+    o0 = make_uint4(even(raw.x), even(raw.x >> 4), even(raw.y), even(raw.y >> 4));
+    o1 = make_uint4(even(raw.z), even(raw.z >> 4), even(raw.w), even(raw.w >> 4));
+}
+
+// 16 bytes of MXFP4 weights -> 32 e4m3 codes in order: PRMT picks the
+// magnitudes of four nibbles at a time out of the block's 8-entry table, and
+// the sign from its sign-replicating mode (0x80 gives 0x80 or 0xff).
+__device__ __forceinline__ void decode_mxfp4_32(const uint4 raw, uint2 lut, uint4& o0, uint4& o1) {
+    auto four = [&](uint32_t w) {
+        uint32_t sign;  // (__byte_perm has no sign-replicating mode)
+        asm("prmt.b32 %0, %1, %1, %2;" : "=r"(sign) : "r"(0x80808080u), "r"(w));
+        sign <<= 7;
+        return __byte_perm(lut.x, lut.y, w & 0x7777u) | (sign & 0x80808080u);
+    };
+    o0 = make_uint4(four(raw.x), four(raw.x >> 16), four(raw.y), four(raw.y >> 16));
+    o1 = make_uint4(four(raw.z), four(raw.z >> 16), four(raw.w), four(raw.w >> 16));
+}
+
+// 16-byte chunk c (0..3) of row r of a 64-byte-swizzled tile
+__device__ __forceinline__ uint32_t sw64_off(int r, int c) { return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)); }
 
 // -------------------------------------------------------------- the GEMM
 
-template <bool SWIGLU>
-__global__ void __launch_bounds__(THREADS, 1)
-fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant__ CUtensorMap tm_w1, const Params p,
-               const int stages) {
+template <int WQ, int ROWS, bool SWIGLU>
+__global__ void __launch_bounds__(Cfg<WQ, ROWS>::THREADS, 1)
+fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant__ CUtensorMap tm_w1, const Params p) {
     pdl_enter();
+    using C = Cfg<WQ, ROWS>;
+    constexpr int RAW = C::RAW, STAGES = C::STAGES, SLOTS = C::SLOTS, RING = C::RING;
+    constexpr int B_BYTES = 2 * ROWS * BK;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int b_bytes = 2 * p.tile_rows * BK;
     uint8_t* sA = smem;
-    uint8_t* sB = smem + stages * A_BYTES;
-    float* sS = reinterpret_cast<float*>(sB + stages * b_bytes);  // [RING][MAX_ROWS]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sS + RING * MAX_ROWS);
-    uint64_t* wfull = bars;                   // weights of a k block landed
-    uint64_t* bfull = bars + MAX_STAGES;      // its row codes landed
-    uint64_t* empty = bars + 2 * MAX_STAGES;  // MMAs reading the stage finished
-    uint64_t* pfull = bars + 3 * MAX_STAGES;  // partial sum ready
-    uint64_t* pempty = pfull + SLOTS;         // partial sum read by every promoting warp
-    uint64_t* sfull = pempty + SLOTS;         // scale block written
+    uint8_t* sR = smem + STAGES * A_BYTES;        // int4, MXFP4: tiles as stored
+    uint8_t* sB = sR + STAGES * RAW;
+    float* sS = reinterpret_cast<float*>(sB + STAGES * B_BYTES);  // [RING] scale blocks
+    uint2* sLut = reinterpret_cast<uint2*>(sS + RING * C::RING_FLOATS);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(sLut) + C::LUT_BYTES);
+    uint64_t* full = bars;              // weights (decoded) and row codes of a k block are in place
+    uint64_t* rfull = full + STAGES;    // int4, MXFP4: weights landed as stored
+    uint64_t* empty = rfull + STAGES;   // MMAs reading the stage finished
+    uint64_t* pfull = empty + STAGES;   // partial sums ready
+    uint64_t* pempty = pfull + SLOTS;   // partial sums read by every promoting warp
+    uint64_t* sfull = pempty + SLOTS;   // scale block written
     uint64_t* drain = sfull + RING;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < MAX_STAGES; ++s) {
-            mbar_init(&wfull[s], 1);
-            mbar_init(&bfull[s], GATHER_WARPS * 32);
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 32 * GATHER_WARPS + (RAW ? C::DECODE_WARPS : 1));
+            mbar_init(&rfull[s], 1);
             mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < SLOTS; ++b) {
             mbar_init(&pfull[b], 1);
-            mbar_init(&pempty[b], PROMOTE_WARPS);
+            mbar_init(&pempty[b], C::PROMOTE_WARPS);
         }
-        for (int b = 0; b < RING; ++b) mbar_init(&sfull[b], GATHER_WARPS);
+        for (int b = 0; b < RING; ++b) mbar_init(&sfull[b], GATHER_WARPS + C::DECODE_WARPS);
         mbar_init(drain, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (WQ == GBMOE_MXFP4) {
+        // entry d: the magnitudes 0, .5, 1, 1.5, 2, 3, 4, 6 times 2^(6 - d) as
+        // e4m3 (exact for d <= 14, nothing left from d = 20)
+        for (int d = threadIdx.x; d < LUT_ENTRIES; d += C::THREADS) {
+            const float mag[8] = {0.0f, 0.5f, 1.0f, 1.5f, 2.0f, 3.0f, 4.0f, 6.0f};
+            const float f = d < 32 ? __uint_as_float((uint32_t)(127 + 6 - d) << 23) : 0.0f;
+            uint32_t v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                v[i] = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(mag[2 * i] * f, mag[2 * i + 1] * f),
+                                                          __NV_SATFINITE, __NV_E4M3);
+            sLut[d] = make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
+        }
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -269,6 +351,11 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
     const int total = p.sched[1] * p.n_tiles;
     const int nkb = p.K / BK;
 
+    // tall tiles: 16 warps start with 128 registers a thread; the promotion takes 168
+    // (128 threads x (104 + 168 + 168 + 72) = 65536, what the block was launched with)
+    if constexpr (RAW && !C::JOINT) {
+        if (warp < 4) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+    }
     if (warp == 0 && lane == 0) {
         // ------------------------------------------------ weight producer
         int stage = 0;
@@ -282,17 +369,22 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 inflight &= ~(1u << stage);
-                mbar_expect_tx(&wfull[stage], A_BYTES);
-                tma_load_2d(sA + stage * A_BYTES, &tm_w0, kb * BK, a0, &wfull[stage]);
-                tma_load_2d(sA + stage * A_BYTES + A_BYTES / 2, &tm_w1, kb * BK, a1, &wfull[stage]);
+                constexpr int BYTES = RAW ? RAW : A_BYTES;  // (int4: 64 bytes of a row are 128 weights)
+                uint8_t* dst = RAW ? sR + stage * RAW : sA + stage * A_BYTES;
+                const int x = kb * (RAW ? BK / 2 : BK);
+                uint64_t* bar = RAW ? &rfull[stage] : &full[stage];
+                mbar_expect_tx(bar, BYTES);
+                tma_load_2d(dst, &tm_w0, x, a0, bar);
+                tma_load_2d(dst + BYTES / 2, &tm_w1, x, a1, bar);
                 inflight |= 1u << stage;
                 inflight_par = (inflight_par & ~(1u << stage)) | (phase << stage);
-                if (++stage == stages) { stage = 0; phase ^= 1; }
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }
-        // every copy issued lands before the CTA leaves
-        for (int s = 0; s < stages; ++s)
-            if ((inflight >> s) & 1u) drain_wait(&wfull[s], (inflight_par >> s) & 1u);
+        // every copy issued lands before the CTA leaves (after an abort the
+        // phase may lack other arrivals: the copies get the drain limit's time)
+        for (int s = 0; s < STAGES; ++s)
+            if ((inflight >> s) & 1u) drain_wait(RAW ? &rfull[s] : &full[s], (inflight_par >> s) & 1u);
     } else if (warp == 1) {
         // ------------------------- MMA issuer (the whole warp, one lane issues)
         int stage = 0;
@@ -305,33 +397,33 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             const int rp = __shfl_sync(0xffffffffu, rows_pad(wk.rows), 0);  // warp-uniform
             const uint32_t idesc = idesc_f8(2 * rp);
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!warp_wait(&bfull[stage], phase, abort_flag, p.err, p.wait_limit_ns) ||
-                    !warp_wait(&wfull[stage], phase, abort_flag, p.err, p.wait_limit_ns)) {
-                    ok = false;
-                    break;
-                }
+                if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 // the row codes were written through the generic proxy (cp.async)
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                const uint64_t db = db0 + (uint64_t)(stage * b_bytes >> 4);
+                const uint64_t db = db0 + (uint64_t)(stage * B_BYTES >> 4);
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
-                    if (!warp_wait(&pempty[slot], sphase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t d = tmem_base + slot * SLOT_COLS;
+                    if (half == 0 || !C::JOINT) {
+                        if (!warp_wait(&pempty[slot], sphase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                        tc_fence_after();
+                    }
+                    const uint32_t d = tmem_base + slot * C::SLOT_COLS + (C::JOINT ? half * 2 * ROWS : 0);
                     const uint64_t dh = da0 + (uint64_t)((stage * A_BYTES + half * (MB * BK)) >> 4);
                     if (elect_one()) {
 #pragma unroll
                         for (int j = 0; j < BK / 32; ++j)  // +32 bytes along K per instruction
                             mma_f8(d, dh + 2 * j, db + 2 * j, idesc, j != 0 ? 1u : 0u);
-                        mma_commit(&pfull[slot]);
+                        if (half == 1 || !C::JOINT) mma_commit(&pfull[slot]);
                         if (half == 1) mma_commit(&empty[stage]);
                     }
                     __syncwarp();
                     issued = true;
-                    if (++slot == SLOTS) { slot = 0; sphase ^= 1; }
+                    if (half == 1 || !C::JOINT) {
+                        if (++slot == SLOTS) { slot = 0; sphase ^= 1; }
+                    }
                 }
                 if (!ok) break;
-                if (++stage == stages) { stage = 0; phase ^= 1; }
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }
         if (issued) {  // every MMA issued has finished before TMEM is released
@@ -360,37 +452,48 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 const int32_t g = p.gather[r];
                 return g >= 0 ? g / p.gather_div : 0;
             };
-            const uint8_t* src[MAX_ROWS / 8];
+            const uint8_t* src[ROWS / 8];
 #pragma unroll
-            for (int i = 0; i < MAX_ROWS / 8; ++i) src[i] = p.q + (8 * i < rp ? src_row(r0 + 8 * i) : 0) * p.K + 16 * chunk;
-            const float* s0 = p.a_scale + (t < rp ? src_row(t) : 0) * nkb;  // (MAX_ROWS <= 128: two per thread)
+            for (int i = 0; i < ROWS / 8; ++i) src[i] = p.q + (8 * i < rp ? src_row(r0 + 8 * i) : 0) * p.K + 16 * chunk;
+            const float* s0 = p.a_scale + (t < rp ? src_row(t) : 0) * nkb;
             const float* s1 = p.a_scale + (t + 64 < rp ? src_row(t + 64) : 0) * nkb;
             float n0 = s0[0], n1 = s1[0];
+            constexpr bool SUMS = WQ == GBMOE_INT4_G128;
+            const int64_t sum_off = SUMS ? p.a_sum - p.a_scale : 0;
+            float m0 = 0.0f, m1 = 0.0f;  // int4: sums of codes
+            if (SUMS) { m0 = s0[sum_off]; m1 = s1[sum_off]; }
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                uint8_t* dst = sB + stage * b_bytes;
+                uint8_t* dst = sB + stage * B_BYTES;
 #pragma unroll
-                for (int i = 0; i < MAX_ROWS / 8; ++i) {
+                for (int i = 0; i < ROWS / 8; ++i) {
                     if (8 * i >= rp) break;
                     const uint32_t off = sw128_off(r0 + 8 * i, chunk);
                     cp_async_16(dst + off, src[i] + kb * BK);
                     cp_async_16(dst + rp * BK + off, src[i] + plane + kb * BK);
                 }
                 // one arrival of this thread once its copies above have landed
-                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&bfull[stage])) : "memory");
-                float* sc = sS + ring * MAX_ROWS;
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[stage])) : "memory");
+                float* sc = sS + ring * C::RING_FLOATS;
                 if (t < rp) sc[t] = n0;
                 if (t + 64 < rp) sc[t + 64] = n1;
-                if (kb + 1 < nkb) { n0 = s0[kb + 1]; n1 = s1[kb + 1]; }
+                if (SUMS && t < rp) sc[ROWS + t] = -m0;
+                if (SUMS && t + 64 < rp) sc[ROWS + t + 64] = -m1;
+                if (kb + 1 < nkb) {
+                    n0 = s0[kb + 1]; n1 = s1[kb + 1];
+                    if (SUMS) { m0 = s0[sum_off + kb + 1]; m1 = s1[sum_off + kb + 1]; }
+                }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sfull[ring]);
-                if (++ring == stages + 2) ring = 0;
-                if (++stage == stages) { stage = 0; phase ^= 1; }
+                if (++ring == RING) ring = 0;
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");  // (after an abort too) copies land before the CTA leaves
-    } else if (warp >= 4) {
+    } else if (warp >= 4 && warp < 4 + C::PROMOTE_WARPS) {
         // ------------------------------------------ promotion and output
+        if constexpr (RAW && !C::JOINT) asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+        constexpr int SETS = C::SETS, GROUPS = C::GROUPS;
         const int q = warp & 3;            // TMEM lane quarter
         const int set = (warp - 4) >> 2;  // this warp's groups of 8 rows: set, set + SETS, ..
         const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
@@ -402,25 +505,29 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             const int rp = rows_pad(wk.rows);
             const int groups = (rp / 8 + SETS - 1 - set) / SETS;  // groups of 8 rows this warp promotes
             // fp8 weight scales: one per 128 x 128 block, so one per half and k block
-            const int nb_per_e = p.w_rows_per_expert / MB;
-            const int nb = wk.e * nb_per_e + (SWIGLU ? wk.nt : 2 * wk.nt);
-            const float* ws0 = p.w_scale0 + (int64_t)nb * nkb;
-            const float* ws1 = SWIGLU ? p.w_scale1 + (int64_t)nb * nkb : ws0 + nkb;
+            const int64_t nb = (int64_t)wk.e * (p.w_rows_per_expert / MB) + (SWIGLU ? wk.nt : 2 * wk.nt);
+            const float* ws0 = static_cast<const float*>(p.w_scale0) + nb * nkb;
+            const float* ws1 = static_cast<const float*>(p.w_scale1) + (SWIGLU ? nb : nb + 1) * nkb;
             uint64_t acc[2][4 * GROUPS];  // [half of the item][row pair]
 #pragma unroll
             for (int i = 0; i < 4 * GROUPS; ++i) acc[0][i] = acc[1][i] = 0;
-            float wn0 = ws0[0], wn1 = ws1[0];
+            float wn0 = 0.0f, wn1 = 0.0f;
+            if (!RAW) { wn0 = ws0[0]; wn1 = ws1[0]; }
             bool ok = true;
             for (int kb = 0; kb < nkb; ++kb) {
-                const uint64_t wsc[2] = {pack2(wn0, wn0), pack2(wn1, wn1)};
-                if (kb + 1 < nkb) { wn0 = ws0[kb + 1]; wn1 = ws1[kb + 1]; }
-                const float* sc = sS + ring * MAX_ROWS;
+                float wsc[2] = {wn0, wn1};
+                if (!RAW && kb + 1 < nkb) { wn0 = ws0[kb + 1]; wn1 = ws1[kb + 1]; }
+                const float* sc = sS + ring * C::RING_FLOATS;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    if (!warp_wait(&pfull[slot], sphase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                     if (h == 0 && !warp_wait(&sfull[ring], rphase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t t1 = t_lane + slot * SLOT_COLS + 8 * set, t2 = t1 + rp;
+                    if (h == 0 || !C::JOINT) {
+                        if (!warp_wait(&pfull[slot], sphase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                        tc_fence_after();
+                    }
+                    if (RAW) wsc[h] = sc[2 * ROWS + h * MB + q * 32 + lane];  // decoded formats: one per row
+                    const uint64_t w2 = pack2(wsc[h], wsc[h]);
+                    const uint32_t t1 = t_lane + slot * C::SLOT_COLS + (C::JOINT ? h * 2 * ROWS : 0) + 8 * set, t2 = t1 + rp;
                     const float* f = sc + 8 * set;
                     constexpr int D = 8 * SETS;  // from one of this warp's groups to the next
 #pragma unroll
@@ -434,22 +541,24 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                             tmem_ld8(t1 + D * (g + 1), a1);
                             tmem_ld8(t2 + D * (g + 1), b1);
                             tmem_wait(a0, b0, a1, b1);
-                            promote8(a0, b0, f + D * g, wsc[h], &acc[h][4 * g]);
-                            if (g + 1 < GROUPS) promote8(a1, b1, f + D * (g + 1), wsc[h], &acc[h][4 * g + 4]);
+                            promote8<WQ, ROWS>(a0, b0, f + D * g, w2, &acc[h][4 * g]);
+                            if (g + 1 < GROUPS) promote8<WQ, ROWS>(a1, b1, f + D * (g + 1), w2, &acc[h][4 * g + 4]);
                         } else {
                             tmem_ld8(t1 + D * g, a0);
                             tmem_ld8(t2 + D * g, b0);
                             tmem_wait(a0, b0);
-                            promote8(a0, b0, f + D * g, wsc[h], &acc[h][4 * g]);
+                            promote8<WQ, ROWS>(a0, b0, f + D * g, w2, &acc[h][4 * g]);
                         }
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&pempty[slot]);
-                    if (++slot == SLOTS) { slot = 0; sphase ^= 1; }
+                    if (h == 1 || !C::JOINT) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&pempty[slot]);
+                        if (++slot == SLOTS) { slot = 0; sphase ^= 1; }
+                    }
                 }
                 if (!ok) break;
-                if (++ring == stages + 2) { ring = 0; rphase ^= 1; }
+                if (++ring == RING) { ring = 0; rphase ^= 1; }
             }
             if (!ok) break;
             // this thread's weight row is an output column; a warp writes 64 consecutive bytes per row
@@ -474,6 +583,86 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             }
         }
     }
+    if constexpr (RAW) {
+        if (warp >= 4 + C::PROMOTE_WARPS) {
+            // ------------------------------- weight decode, weight rows' scales
+            // A thread owns row r of one half (eight decode warps) or of both:
+            // it decodes the row's 128 values of a k block and writes their
+            // scale to the scale block. MXFP4: the block's four E8M0 scales
+            // (one per 32) differ by small powers of two, which go into the
+            // codes relative to the largest of the four.
+            if constexpr (!C::JOINT) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+            constexpr int HALVES = C::DECODE_WARPS == 8 ? 1 : 2;
+            const int t = threadIdx.x - 32 * (4 + C::PROMOTE_WARPS);
+            const int r = t & (MB - 1), h0 = t >> 7;
+            int stage = 0, ring = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+                const Work wk = decode_work(p, w);
+                int a0, a1;
+                w_rows<SWIGLU>(p, wk, a0, a1);
+                // raw bits of the scale of k block kb of this thread's row in its half i
+                auto scale_bits = [&](int i, int kb) -> uint32_t {
+                    const int h = h0 + i;
+                    const int64_t at = (int64_t)((h ? a1 : a0) + r) * nkb + kb;
+                    const void* base = h ? p.w_scale1 : p.w_scale0;
+                    if constexpr (WQ == GBMOE_INT4_G128) return static_cast<const uint16_t*>(base)[at];
+                    if (p.scale_words) return static_cast<const uint32_t*>(base)[at];
+                    const uint16_t* b = static_cast<const uint16_t*>(base) + 2 * at;
+                    return b[0] | (uint32_t)b[1] << 16;
+                };
+                uint32_t next[HALVES];
+#pragma unroll
+                for (int i = 0; i < HALVES; ++i) next[i] = scale_bits(i, 0);
+                for (int kb = 0; kb < nkb; ++kb) {
+                    uint32_t bits[HALVES];
+#pragma unroll
+                    for (int i = 0; i < HALVES; ++i) {
+                        bits[i] = next[i];
+                        if (kb + 1 < nkb) next[i] = scale_bits(i, kb + 1);
+                    }
+                    if (!warp_wait(&rfull[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                    float* sc = sS + ring * C::RING_FLOATS + 2 * ROWS;
+#pragma unroll
+                    for (int i = 0; i < HALVES; ++i) {
+                        const int h = h0 + i;
+                        const uint8_t* raw = sR + stage * RAW + h * (RAW / 2);
+                        uint8_t* dst = sA + stage * A_BYTES + h * (A_BYTES / 2);
+                        uint32_t below = 0;  // MXFP4: log2 of the largest scale over each block's, a byte each
+                        if constexpr (WQ == GBMOE_INT4_G128) {
+                            sc[h * MB + r] = __uint_as_float(bits[i] << 16) * 512.0f;  // bf16; the codes are u * 2^-9
+                        } else {
+                            const uint32_t b = bits[i];
+                            const uint32_t top = max(max(b & 0xffu, (b >> 8) & 0xffu), max((b >> 16) & 0xffu, b >> 24));
+                            below = top * 0x01010101u - b;
+                            // 2^(top - 127) * 2^-6 (the table's factor); 255 is NaN
+                            float f = __uint_as_float((top - 6u) << 23);
+                            if (top - 7u >= 248u) f = e8m0_to_f32(top) * 0.015625f;
+                            sc[h * MB + r] = f;
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const uint4 v = *reinterpret_cast<const uint4*>(raw + sw64_off(r, c));
+                            uint4 o0, o1;
+                            if constexpr (WQ == GBMOE_INT4_G128) decode_int4_32(v, o0, o1);
+                            else decode_mxfp4_32(v, sLut[(below >> (8 * c)) & 0xffu], o0, o1);
+                            *reinterpret_cast<uint4*>(dst + sw128_off(r, 2 * c)) = o0;
+                            *reinterpret_cast<uint4*>(dst + sw128_off(r, 2 * c + 1)) = o1;
+                        }
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(&sfull[ring]);
+                        mbar_arrive(&full[stage]);
+                    }
+                    if (++ring == RING) ring = 0;
+                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
+                }
+            }
+        }
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -485,67 +674,90 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
 
 // ------------------------------------------------------------------- host
 
-template <bool SWIGLU>
+template <int WQ, int ROWS, bool SWIGLU>
 static cudaError_t launch_gemm(const CUtensorMap& w0, const CUtensorMap& w1, const Params& prm, int64_t max_work,
                                cudaStream_t stream) {
+    using C = Cfg<WQ, ROWS>;
     static DeviceOnce smem_set;
     const cudaError_t e = smem_set.run([] {
-        return cudaFuncSetAttribute(fm_gemm_kernel<SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET);
+        return cudaFuncSetAttribute(fm_gemm_kernel<WQ, ROWS, SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    C::SMEM_BYTES);
     });
     if (e != cudaSuccess) return e;
     const int grid = (int)min64(sm_count(), max_work);
     if (grid <= 0) return cudaSuccess;
-    const int stages = stages_for(prm.tile_rows);
-    return launch_k(fm_gemm_kernel<SWIGLU>, dim3(grid), dim3(THREADS),
-                    (size_t)FIXED_BYTES + stages * stage_bytes(prm.tile_rows), stream, w0, w1, prm, stages);
+    return launch_k(fm_gemm_kernel<WQ, ROWS, SWIGLU>, dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, stream, w0, w1, prm);
 }
 
-static bool map_e4m3(CUtensorMap* m, const void* base, int64_t rows, int64_t K) {
+// [rows, K] weights in boxes of 128 rows x 128 k as stored
+static bool map_weights(CUtensorMap* m, int wq, const void* base, int64_t rows, int64_t K) {
+    if (wq != GBMOE_FP8_E4M3_B128)
+        return make_map(m, base, rows, K / 2, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, BK / 2, CU_TENSOR_MAP_SWIZZLE_64B, MB);
     return make_map(m, base, rows, K, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, BK, CU_TENSOR_MAP_SWIZZLE_128B, MB);
 }
 
-}  // namespace fm
-
-bool ffn_fm_supported(const FfnProblem& p) {
-    return p.act_dtype == GBMOE_BF16 && p.w_dtype == GBMOE_FP8_E4M3_B128 && p.H % 256 == 0 && p.I % 128 == 0 &&
-           tc::encode_fn() != nullptr;
-}
-
-// Rows of a row tile: short tiles leave room for a deeper ring of weight
-// stages (6 stages at 16 rows, 4 at 80)
-static int fm_tile_rows(int64_t n_rows, int E) { return n_rows <= 4 * (int64_t)E ? 16 : fm::MAX_ROWS; }
-
-cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream) {
-    using namespace fm;
-    if (p.n_rows == 0) return cudaSuccess;
-    const int tile = fm_tile_rows(p.n_rows, p.E);
+template <int WQ, int ROWS>
+static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
+    const int tile = ROWS;
     cudaError_t err = launch_ffn_schedule(p.counts, p.E, p.n_rows, tile, p.sched, stream);
     if (err != cudaSuccess) return err;
     // every row of x once (the shared expert's rows are x's own; a routed row is a token's)
     const int64_t x_rows = p.n_rows / p.pair_div;
-    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, stream)) != cudaSuccess) return err;
+    constexpr bool kSums = WQ == GBMOE_INT4_G128;
+    float* a_sum = kSums ? p.a_s + x_rows * (p.H / BK) : nullptr;
+    float* h_sum = kSums ? p.h_s + p.n_rows * (p.I / BK) : nullptr;
+    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, a_sum, stream)) != cudaSuccess) return err;
     const int64_t max_m = sched_max_tiles(p.E, p.n_rows, tile);
     CUtensorMap mg, mu, md;
-    if (!map_e4m3(&mg, p.w_gate, (int64_t)p.E * p.I, p.H) || !map_e4m3(&mu, p.w_up, (int64_t)p.E * p.I, p.H) ||
-        !map_e4m3(&md, p.w_down, (int64_t)p.E * p.H, p.I))
+    if (!map_weights(&mg, WQ, p.w_gate, (int64_t)p.E * p.I, p.H) ||
+        !map_weights(&mu, WQ, p.w_up, (int64_t)p.E * p.I, p.H) ||
+        !map_weights(&md, WQ, p.w_down, (int64_t)p.E * p.H, p.I))
         return cudaErrorInvalidValue;
     Params g{};
     g.K = p.H; g.n_tiles = p.I / MB; g.out_cols = p.I; g.w_rows_per_expert = p.I; g.tile_rows = tile;
     g.counts = p.counts; g.offsets = p.offsets; g.sched = p.sched; g.E = p.E; g.n_rows = p.n_rows;
     g.out = static_cast<__nv_bfloat16*>(p.h); g.err = p.err;
-    g.q = static_cast<const uint8_t*>(p.a_q); g.plane_rows = x_rows; g.a_scale = p.a_s;
+    g.q = static_cast<const uint8_t*>(p.a_q); g.plane_rows = x_rows; g.a_scale = p.a_s; g.a_sum = a_sum;
     g.gather = p.sorted_pair; g.gather_div = p.pair_div;
-    g.w_scale0 = static_cast<const float*>(p.s_gate); g.w_scale1 = static_cast<const float*>(p.s_up);
+    g.w_scale0 = p.s_gate; g.w_scale1 = p.s_up;
+    auto words = [](const void* s) { return reinterpret_cast<uintptr_t>(s) % 4 == 0; };
+    g.scale_words = words(p.s_gate) && words(p.s_up);
     g.wait_limit_ns = tc_wait_limit_ns();
-    if ((err = launch_gemm<true>(mg, mu, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
-    if ((err = launch_quant_rows(p.h, nullptr, 1, p.n_rows, p.I, p.h_q, p.h_s, stream)) != cudaSuccess) return err;
+    if ((err = launch_gemm<WQ, ROWS, true>(mg, mu, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.h, nullptr, 1, p.n_rows, p.I, p.h_q, p.h_s, h_sum, stream)) != cudaSuccess) return err;
     Params d = g;
     d.K = p.I; d.n_tiles = p.H / (2 * MB); d.out_cols = p.H; d.w_rows_per_expert = p.H;
     d.out = static_cast<__nv_bfloat16*>(p.y);
-    d.q = static_cast<const uint8_t*>(p.h_q); d.plane_rows = p.n_rows; d.a_scale = p.h_s;
+    d.q = static_cast<const uint8_t*>(p.h_q); d.plane_rows = p.n_rows; d.a_scale = p.h_s; d.a_sum = h_sum;
     d.gather = nullptr; d.gather_div = 1;
-    d.w_scale0 = d.w_scale1 = static_cast<const float*>(p.s_down);
-    return launch_gemm<false>(md, md, d, max_m * d.n_tiles, stream);
+    d.w_scale0 = d.w_scale1 = p.s_down;
+    d.scale_words = words(p.s_down);
+    return launch_gemm<WQ, ROWS, false>(md, md, d, max_m * d.n_tiles, stream);
+}
+
+// Rows of a row tile: short ones leave shared memory for more weight stages
+// (fp8: 6 at 16 rows, 4 at 80) and pass both partial sums of a k block at once;
+// an expert with more rows takes several tiles, whose weights come from L2.
+template <int WQ>
+static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
+    return p.n_rows <= 4 * (int64_t)p.E ? launch_ffn<WQ, 16>(p, stream) : launch_ffn<WQ, 80>(p, stream);
+}
+
+}  // namespace fm
+
+bool ffn_fm_supported(const FfnProblem& p) {
+    const bool wq_ok = p.w_dtype == GBMOE_FP8_E4M3_B128 || p.w_dtype == GBMOE_INT4_G128 || p.w_dtype == GBMOE_MXFP4;
+    return p.act_dtype == GBMOE_BF16 && wq_ok && p.H % 256 == 0 && p.I % 128 == 0 && tc::encode_fn() != nullptr;
+}
+
+cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream) {
+    if (p.n_rows == 0) return cudaSuccess;
+    switch (p.w_dtype) {
+        case GBMOE_FP8_E4M3_B128: return fm::launch_ffn<GBMOE_FP8_E4M3_B128>(p, stream);
+        case GBMOE_INT4_G128: return fm::launch_ffn<GBMOE_INT4_G128>(p, stream);
+        case GBMOE_MXFP4: return fm::launch_ffn<GBMOE_MXFP4>(p, stream);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace gbmoe

@@ -61,9 +61,10 @@ struct FfnProblem {
                                 // CTA-pair GEMMs read (null on routes that do not use one)
     void* w_dq;                 // bf16 [E, I, H] gate, [E, I, H] up, [E, H, I] down, or null:
                                 // quantised weights are then decoded once into it (TC_DEQUANT)
-    void* a_q;                  // fp8 route (TC_FP8): x rows in sorted order as two e4m3 code planes
-                                //   [2, n_rows, H] (value and residual)
-    float* a_s;                 //   and their 1x128 scales [n_rows, H/128]
+    void* a_q;                  // routes that multiply e4m3 codes: x as two e4m3 code planes (value and
+                                //   residual), [2, rows, H] in sorted order (row-major fp8 GEMM) or
+                                //   token order (feature-major GEMM)
+    float* a_s;                 //   and their 1x128 scales [rows, H/128] (int4: then the sums of codes, the same)
     void* h_q;                  //   h the same way, [2, n_rows, I]
     float* h_s;                 //   and its 1x128 scales [n_rows, I/128]
     int cta_pair;               // tensor-core routes: 1 = CTA pairs (cta_group::2, 256-row M tiles)
@@ -98,11 +99,14 @@ bool ffn_tc_fp8_supported(const FfnProblem& p);
 // promotion (every row's partial sums, per 128 k) costs more than the 128-row
 // MMAs of the row-major GEMMs. fp8 layer, 256 experts, H 7168, I 2048, both
 // ways: 1.93 against 2.33 ms at 8 rows per expert, 2.30 against 2.50 at 32,
-// 2.67 against 2.66 at 47, 3.40 against 2.79 at 64.
+// 2.67 against 2.66 at 47, 3.40 against 2.79 at 64. MXFP4, the same layer: 2.91
+// against 22.9 ms (streaming) at 8, 3.34 against 3.43 (decode in the GEMM) at
+// 32; int4, 64 experts, H 4096, I 2816: 0.64 against 0.78 ms at 24.
 constexpr int64_t kFmRowsPerExpert = 40;
-// rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales
+// rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales;
+// with int4_sums in the order int4 weights take, with the blocks' sums of codes there
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, cudaStream_t stream);
+                              float* s, float* int4_sums, cudaStream_t stream);
 cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream);
 bool ffn_fm_supported(const FfnProblem& p);
 

@@ -24,15 +24,21 @@ __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
     return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3);
 }
 
+// kInt4: the order and the sums that int4 weights are multiplied in (ffn_fm.cu):
+// within 8 consecutive values the even ones come before the odd ones, and
+// sums[n_rows][K/128] receive the blocks' sum of codes, sum(q1 + q2) / 64.
+//
 // Rows of src [*, K] -> code planes q [2][n_rows][K] and scales s
 // [n_rows][K/128]. Row r reads source row gather[r] / gather_div (r itself
 // without gather; a negative entry gives a zero row). Lane l takes elements
 // 4l .. 4l+3 of a block. A block that holds an infinity gets the codes +-1
 // there, 0 elsewhere and an infinite scale, so its sums are infinite as they
 // should be; a NaN makes the scale NaN.
+template <bool kInt4>
 __global__ void __launch_bounds__(QWARPS * 32)
 quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ gather, int gather_div,
-                  int64_t n_rows, int K, uint8_t* __restrict__ q, float* __restrict__ s) {
+                  int64_t n_rows, int K, uint8_t* __restrict__ q, float* __restrict__ s,
+                  float* __restrict__ sums) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int nblk = K / QB, parts = (nblk + QU - 1) / QU;
@@ -77,27 +83,39 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
                 for (int i = 0; i < 4; ++i) t[i] = isinf(v[i]) ? copysignf(1.0f, v[i]) : 0.0f;
             }
             const uint32_t a = e4m3x2(t[0], t[1]) | (e4m3x2(t[2], t[3]) << 16);
-            float rr[4];
-            {
-                const float2 lo = e4m3x2_to_f32x2(a & 0xffffu), hi = e4m3x2_to_f32x2(a >> 16);
-                rr[0] = t[0] - lo.x; rr[1] = t[1] - lo.y; rr[2] = t[2] - hi.x; rr[3] = t[3] - hi.y;
-            }
+            const float2 lo = e4m3x2_to_f32x2(a & 0xffffu), hi = e4m3x2_to_f32x2(a >> 16);
+            const float rr[4] = {t[0] - lo.x, t[1] - lo.y, t[2] - hi.x, t[3] - hi.y};
             const uint32_t a2 = e4m3x2(rr[0], rr[1]) | (e4m3x2(rr[2], rr[3]) << 16);
-            const int64_t at = r * K + b * QB + 4 * lane;
-            *reinterpret_cast<uint32_t*>(q + at) = a;
-            *reinterpret_cast<uint32_t*>(q2 + at) = a2;
+            if constexpr (kInt4) {
+                const float2 lo2 = e4m3x2_to_f32x2(a2 & 0xffffu), hi2 = e4m3x2_to_f32x2(a2 >> 16);
+                float sum = (lo.x + lo.y + hi.x + hi.y) + (lo2.x + lo2.y + hi2.x + hi2.y);
+#pragma unroll
+                for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+                if (lane == 0) sums[r * nblk + b] = sum * 0.015625f;
+                // this lane's values are 0..3 (even lane) or 4..7 of 8: the even two, then the odd two
+                const int64_t at = r * K + b * QB + 8 * (lane >> 1) + 2 * (lane & 1);
+                *reinterpret_cast<uint16_t*>(q + at) = (uint16_t)__byte_perm(a, 0, 0x4420);
+                *reinterpret_cast<uint16_t*>(q + at + 4) = (uint16_t)__byte_perm(a, 0, 0x4431);
+                *reinterpret_cast<uint16_t*>(q2 + at) = (uint16_t)__byte_perm(a2, 0, 0x4420);
+                *reinterpret_cast<uint16_t*>(q2 + at + 4) = (uint16_t)__byte_perm(a2, 0, 0x4431);
+            } else {
+                const int64_t at = r * K + b * QB + 4 * lane;
+                *reinterpret_cast<uint32_t*>(q + at) = a;
+                *reinterpret_cast<uint32_t*>(q2 + at) = a2;
+            }
             if (lane == 0) s[r * nblk + b] = sc;
         }
     }
 }
 
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, cudaStream_t stream) {
+                              float* s, float* int4_sums, cudaStream_t stream) {
     const int64_t units = n_rows * ((K / QB + QU - 1) / QU);
     const int blocks = (int)min64((units + QWARPS - 1) / QWARPS, (int64_t)sm_count() * 16);
     if (blocks <= 0) return cudaSuccess;
-    return launch_k(quant_rows_kernel, dim3(blocks), dim3(QWARPS * 32), 0, stream,
-                    static_cast<const __nv_bfloat16*>(src), gather, gather_div, n_rows, K, static_cast<uint8_t*>(q), s);
+    return launch_k(int4_sums ? quant_rows_kernel<true> : quant_rows_kernel<false>, dim3(blocks), dim3(QWARPS * 32), 0,
+                    stream, static_cast<const __nv_bfloat16*>(src), gather, gather_div, n_rows, K,
+                    static_cast<uint8_t*>(q), s, int4_sums);
 }
 
 }  // namespace gbmoe

@@ -29,7 +29,7 @@ def forward(wl, dev):
 # rows per expert: 1, groups of 8 and one more, whole 16-row tiles, the last
 # size with short tiles (4 rows per expert on average) and the first without,
 # the last before the row-major GEMM takes over; one k block and ragged rings
-@pytest.mark.parametrize("wq", ["fp8_b128"])
+@pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T,E,k,H,I", [(1, 8, 2, 256, 128), (8, 4, 1, 512, 128), (9, 1, 1, 256, 256),
                                        (4, 1, 1, 768, 384), (32, 16, 2, 1024, 128), (33, 16, 2, 256, 640),
                                        (40, 1, 1, 512, 256), (63, 4, 2, 1280, 256)])
@@ -40,7 +40,7 @@ def test_row_tiles(T, E, k, H, I, wq):
     assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol_for(wl))
 
 
-@pytest.mark.parametrize("wq", ["fp8_b128"])
+@pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T", [16, 17, 80, 81, 200])
 def test_all_rows_on_one_expert(T, wq):
     """A hot expert's rows fill whole row tiles and spill into the next."""
@@ -54,7 +54,7 @@ def test_all_rows_on_one_expert(T, wq):
     assert_close(act_np(forward(wl, to_device(wl, inp))), ref["out"], tol_for(wl))
 
 
-@pytest.mark.parametrize("wq", ["fp8_b128"])
+@pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
 def test_not_finite_rows_stay_in_their_token(wq):
     """An infinity or NaN in one token's activations leaves every other token's
     output bit for bit as it was; its own output is not finite. Values whose
@@ -74,3 +74,28 @@ def test_not_finite_rows_stay_in_their_token(wq):
     assert torch.equal(a[same].view(torch.int16), b[same].view(torch.int16))
     assert all(not torch.isfinite(b[t].float()).all() for t in (3, 4, 5))
     assert torch.isfinite(b[6:8].float()).all() and float(b[6].float().abs().max()) == 0.0
+
+
+def test_mxfp4_scales_at_two_byte_alignment():
+    """E8M0 scale tensors need only 2-byte alignment."""
+    wl = BASE.replace(T=20, E=8, top_k=2, H=512, I=256, wq="mxfp4", seed=9)
+    inp = synth.make_inputs(wl)
+    dev = to_device(wl, inp)
+    for k in ("s_gate", "s_up", "s_down"):
+        v = dev["experts"][k]
+        dev["experts"][k] = torch.cat([v.new_zeros(2), v.flatten()])[2:].view(v.shape)
+        assert dev["experts"][k].data_ptr() % 4 == 2
+    assert_close(act_np(forward(wl, dev)), oracle.forward(wl, inp)["out"], tol_for(wl))
+
+
+def test_mxfp4_block_scales_far_apart():
+    """Scales of one row's four 32-blocks that differ by up to 2^12 stay exact
+    in the codes; a block 2^30 below its neighbours only vanishes next to them."""
+    wl = BASE.replace(T=20, E=4, top_k=2, H=512, I=256, wq="mxfp4", seed=10)
+    inp = synth.make_inputs(wl)
+    rng = np.random.default_rng(0)
+    for k in ("s_gate", "s_up", "s_down"):
+        s = inp["experts"][k]
+        inp["experts"][k] = (s.astype(np.int32) - rng.integers(0, 13, s.shape)).astype(np.uint8)
+        inp["experts"][k][..., ::8, 1] -= 18
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
