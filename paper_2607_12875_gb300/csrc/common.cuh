@@ -171,6 +171,26 @@ struct Vec8<float> {
     }
 };
 
+// Eight consecutive activation elements as loaded, widened when used (several
+// loads in flight cost half the registers of Vec8's).
+template <typename TA>
+struct Raw8 {
+    uint4 v[sizeof(TA) / 2];
+    __device__ __forceinline__ void load(const TA* p) {
+#pragma unroll
+        for (int i = 0; i < (int)sizeof(TA) / 2; ++i) v[i] = reinterpret_cast<const uint4*>(p)[i];
+    }
+    __device__ __forceinline__ float at(int i) const {
+        if constexpr (sizeof(TA) == 4) {
+            const uint32_t w[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
+            return __uint_as_float(w[i]);
+        } else {
+            const uint32_t w[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+            return i & 1 ? bf16hi(w[i >> 1]) : bf16lo(w[i >> 1]);
+        }
+    }
+};
+
 template <typename T>
 __device__ __forceinline__ float to_f32(T v);
 template <>

@@ -165,7 +165,8 @@ perm_small_kernel(const int32_t* __restrict__ ids, int64_t P, int E, int32_t* __
     const uint32_t peers = __match_any_sync(0xffffffffu, e);
     const int rank = __popc(peers & ((1u << lane) - 1u));
     int pos = 0;
-    for (int w = 0; w < kPermBlock / 32; ++w) {
+    const int warps = (int)((P + 31) / 32);  // that hold pairs: each turn costs a block barrier
+    for (int w = 0; w < warps; ++w) {
         if (warp == w && valid) {
             pos = s_run[e] + rank;
             __syncwarp(peers);

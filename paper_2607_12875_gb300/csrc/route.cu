@@ -4,7 +4,7 @@
 // fp32 in the fixed order the layer's definition uses (32 partial sums over
 // interleaved 8-element chunks, one fused multiply-add per element, then a
 // butterfly of pairwise sums), so the expert choice is bit-identical to the
-// oracle's. A warp owns TB tokens x 8 experts; lane l holds the partial sums
+// oracle's. A warp owns TB tokens x EB experts; lane l holds the partial sums
 // of chunks l, l+32, ... for all of them, which is exactly the fixed order.
 // select_experts then runs one warp per token over the logits. Large batches
 // use a shared-memory-staged variant with the same order (below).
@@ -16,60 +16,58 @@
 namespace gbmoe {
 
 constexpr int kGateWarps = 8;
-constexpr int kGateExpertsPerWarp = 8;
 
-template <typename TA, int TB>
+// A small batch is bound by the latency of a warp's H / 256 dependent steps:
+// the loads of U steps are in flight together, and small warp tiles spread the
+// work over more SMs (their repeated reads come from L2).
+template <typename TA, int TB, int EB, int U>
 __global__ void __launch_bounds__(kGateWarps * 32)
 gate_logits_kernel(const TA* __restrict__ x, const TA* __restrict__ wg, const float* __restrict__ bias,
                    float* __restrict__ logits, int T, int H, int E) {
     pdl_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t0 = blockIdx.x * TB;
-    const int e0 = (blockIdx.y * kGateWarps + warp) * kGateExpertsPerWarp;
+    const int e0 = (blockIdx.y * kGateWarps + warp) * EB;
     if (e0 >= E) return;
-    float acc[TB][kGateExpertsPerWarp];
+    float acc[TB][EB];
+    const TA* xp[TB];  // rows past the end repeat the last one and are not stored
+    const TA* wp[EB];
+#pragma unroll
+    for (int a = 0; a < TB; ++a) xp[a] = x + (size_t)min(t0 + a, T - 1) * H + 8 * lane;
+#pragma unroll
+    for (int b = 0; b < EB; ++b) wp[b] = wg + (size_t)min(e0 + b, E - 1) * H + 8 * lane;
 #pragma unroll
     for (int a = 0; a < TB; ++a)
 #pragma unroll
-        for (int b = 0; b < kGateExpertsPerWarp; ++b) acc[a][b] = 0.0f;
+        for (int b = 0; b < EB; ++b) acc[a][b] = 0.0f;
 
-    const int nchunk = H / 8;  // H % 256 == 0: every lane gets H/256 chunks
-    // two steps per iteration: their loads are in flight together (each
-    // accumulator still takes its chunks in increasing order)
-#pragma unroll 2
-    for (int c = lane; c < nchunk; c += 32) {
-        float xv[TB][8];
+    const int steps = H / 256;  // H % 256 == 0: a lane's chunks are lane, lane + 32, ..
+    for (int s0 = 0; s0 < steps; s0 += U) {
+        Raw8<TA> xr[U][TB], wr[U][EB];
 #pragma unroll
-        for (int a = 0; a < TB; ++a) {
-            int t = t0 + a;
-            if (t < T) {
-                Vec8<TA>::load(x + (size_t)t * H + 8 * c, xv[a]);
-            } else {
+        for (int u = 0; u < U; ++u) {
+            if (s0 + u >= steps) break;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) xv[a][i] = 0.0f;
-            }
+            for (int a = 0; a < TB; ++a) xr[u][a].load(xp[a] + 256 * (s0 + u));
+#pragma unroll
+            for (int b = 0; b < EB; ++b) wr[u][b].load(wp[b] + 256 * (s0 + u));
         }
 #pragma unroll
-        for (int b = 0; b < kGateExpertsPerWarp; ++b) {
-            int e = e0 + b;
-            float wv[8];
-            if (e < E) {
-                Vec8<TA>::load(wg + (size_t)e * H + 8 * c, wv);
-            } else {
+        for (int u = 0; u < U; ++u) {
+            if (s0 + u >= steps) break;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) wv[i] = 0.0f;
-            }
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int a = 0; a < TB; ++a)
+                for (int a = 0; a < TB; ++a)
 #pragma unroll
-                for (int i = 0; i < 8; ++i) acc[a][b] = __fmaf_rn(xv[a][i], wv[i], acc[a][b]);
+                    for (int b = 0; b < EB; ++b) acc[a][b] = __fmaf_rn(xr[u][a].at(i), wr[u][b].at(i), acc[a][b]);
         }
     }
     // butterfly: s[p] <- s[p] + s[p ^ d], d = 16 .. 1 (one commutative add: all lanes end equal)
 #pragma unroll
     for (int a = 0; a < TB; ++a)
 #pragma unroll
-        for (int b = 0; b < kGateExpertsPerWarp; ++b) {
+        for (int b = 0; b < EB; ++b) {
             float v = acc[a][b];
 #pragma unroll
             for (int d = 16; d >= 1; d >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, d));
@@ -78,14 +76,33 @@ gate_logits_kernel(const TA* __restrict__ x, const TA* __restrict__ wg, const fl
 #pragma unroll
     for (int a = 0; a < TB; ++a)
 #pragma unroll
-        for (int b = 0; b < kGateExpertsPerWarp; ++b) {
-            int t = t0 + a, e = e0 + b;
-            if (lane == ((a * kGateExpertsPerWarp + b) & 31) && t < T && e < E) {
+        for (int b = 0; b < EB; ++b) {
+            const int t = t0 + a, e = e0 + b;
+            if (lane == a * EB + b && t < T && e < E) {
                 float l = acc[a][b];
                 if (bias) l = __fadd_rn(l, bias[e]);
                 logits[(size_t)t * E + e] = l;
             }
         }
+}
+
+template <typename TA, int TB, int EB, int U>
+static cudaError_t launch_gate_logits(const TA* x, const TA* wg, const float* bias, float* logits, int T, int H, int E,
+                                      cudaStream_t stream) {
+    const dim3 grid((unsigned)((T + TB - 1) / TB), (unsigned)((E + kGateWarps * EB - 1) / (kGateWarps * EB)));
+    return launch_k(gate_logits_kernel<TA, TB, EB, U>, grid, dim3(kGateWarps * 32), 0, stream, x, wg, bias, logits, T, H,
+                    E);
+}
+
+// Warp tiles by batch: few tokens leave most SMs idle unless a warp takes few
+// experts; more tokens make the rows' repeated L2 reads the cost.
+template <typename TA>
+static cudaError_t launch_gate_logits(const TA* x, const TA* wg, const float* bias, float* logits, int T, int H, int E,
+                                      cudaStream_t stream) {
+    constexpr int U = 8 / sizeof(TA);  // 4 steps of bf16, 2 of fp32
+    if (T <= 4) return launch_gate_logits<TA, 1, 2, 2 * U>(x, wg, bias, logits, T, H, E, stream);
+    if (T <= 64) return launch_gate_logits<TA, 2, 4, U>(x, wg, bias, logits, T, H, E, stream);
+    return launch_gate_logits<TA, 4, 4, U / 2>(x, wg, bias, logits, T, H, E, stream);
 }
 
 // Large batches: the same fixed order, as a CUDA-core GEMM. A CTA owns 32
@@ -241,29 +258,32 @@ __device__ __forceinline__ float pinned_sigmoid(float l) {
     return __fdiv_rn(1.0f, __fadd_rn(1.0f, pinned_exp(-l)));
 }
 
-// (key, index) with "larger key, then smaller index" as the better candidate.
-// Keys are never NaN here (choice_key), so this is a strict total order, and
-// a real candidate (index < kNone) beats an empty one even at key -inf.
-constexpr int kNone = 0x7fffffff;
-__device__ __forceinline__ bool better(float ka, int ia, float kb, int ib) {
-    return ka > kb || (ka == kb && ia < ib);
-}
+constexpr int kNone = 0x7fffffff;  // the index of no candidate
 
 // Key a score takes in the expert choice: a NaN counts as -infinity, so
 // non-finite logits still give valid, deterministic ids (ties to the lower index).
 __device__ __forceinline__ float choice_key(float v) { return v != v ? -INFINITY : v; }
 
-__device__ __forceinline__ void warp_best(float& k, int& i) {
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        float ko = __shfl_xor_sync(0xffffffffu, k, d);
-        int io = __shfl_xor_sync(0xffffffffu, i, d);
-        if (better(ko, io, k, i)) { k = ko; i = io; }
-    }
+// A key as an unsigned integer of the same order (both zeros alike), above 0
+// for every real candidate, so that the warp's best is one redux each for the
+// key and the index.
+__device__ __forceinline__ uint32_t key_bits(float k) {
+    const uint32_t u = __float_as_uint(k == 0.0f ? 0.0f : k);
+    return u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float key_value(uint32_t b) {
+    return __uint_as_float(b ^ ((b >> 31) ? 0x80000000u : 0xffffffffu));
+}
+
+// the best (largest key, then smallest index) of the lanes' candidates; a lane
+// without one has key bits 0 and index kNone
+__device__ __forceinline__ void warp_best(uint32_t& kb, int& i) {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, kb);
+    i = __reduce_min_sync(0xffffffffu, kb == m ? i : kNone);
+    kb = m;
 }
 
 constexpr int kSelWarps = 4;
-constexpr int kMaxE = 512;
 
 // Audit of router logits computed on the tensor cores (their fp32 sums run in
 // the hardware's own order, not the fixed order of the definition). Those
@@ -279,105 +299,125 @@ struct GateAudit {
     int32_t* n_flagged;       // their count
 };
 
-// One warp per token (every token, or those of `list` in grid-stride order).
-// Expert e lives in lane e % 32, slot e / 32.
-__global__ void __launch_bounds__(kSelWarps * 32)
-select_experts_kernel(const float* __restrict__ logits, const float* __restrict__ select_bias,
-                      int32_t* __restrict__ topk_ids, float* __restrict__ topk_w, RouteParams rp, GateAudit au,
-                      const int32_t* __restrict__ list, const int32_t* __restrict__ n_list) {
-    pdl_enter();
-    __shared__ float s_key[kSelWarps][kMaxE];
-    __shared__ float s_sig[kSelWarps][kMaxE];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n_tok = list ? *n_list : rp.T;
-    for (int i = blockIdx.x * kSelWarps + warp; i < n_tok; i += gridDim.x * kSelWarps) {
-    const int t = list ? list[i] : i;
+// Chooses token t's experts and weights, by one warp: lane j < k returns slot
+// j's expert in sel_id and weight in w. Expert e lives in lane e % 32, register
+// e / 32 (E <= 32 * SLOTS); key and val are this warp's shared arrays of E
+// floats (choice keys; logits or sigmoids).
+template <int SLOTS>
+__device__ __forceinline__ void select_token(const float* __restrict__ l, const float* __restrict__ select_bias,
+                                             const RouteParams& rp, const GateAudit& au, int t, float* key, float* val,
+                                             int& sel_id, float& w) {
+    const int lane = threadIdx.x & 31;
     const int E = rp.E, k = rp.top_k;
-    const float* l = logits + (size_t)t * E;
-    float* key = s_key[warp];
-    float* sig = s_sig[warp];
     const bool sigmoid = rp.score == GBMOE_SIGMOID;
     const int G = sigmoid ? rp.n_group : 1;
     const int gs = E / G;
-    int sel_id = 0;
-    float top_key = 0.0f;
-    {
-        for (int e = lane; e < E; e += 32) {
-            float v = l[e];
+    float raw[SLOTS];
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) raw[s] = lane + 32 * s < E ? l[lane + 32 * s] : 0.0f;
+    uint32_t kb[SLOTS];  // candidates: 0 once chosen, or not allowed
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+        const int e = lane + 32 * s;
+        kb[s] = 0;
+        if (e < E) {
+            float v = raw[s];
             if (sigmoid) {
-                float s = pinned_sigmoid(v);
-                sig[e] = s;
-                v = select_bias ? __fadd_rn(s, select_bias[e]) : s;
+                v = pinned_sigmoid(v);
+                val[e] = v;
+                if (select_bias) v = __fadd_rn(v, select_bias[e]);
+            } else {
+                val[e] = v;
             }
-            key[e] = choice_key(v);
+            v = choice_key(v);
+            kb[s] = key_bits(v);
+            if (G > 1) key[e] = v;
         }
-        __syncwarp();
+    }
+    __syncwarp();
 
-        // groups kept (bit g set); all experts allowed without group limiting.
-        // margin_g: gap between the last kept and the best dropped group score
-        uint32_t kept = 0xffffffffu;
-        float margin_g = INFINITY;
-        if (G > 1) {
-            float gscore = -INFINITY;
-            if (lane < G) {
-                float a = -INFINITY, b = -INFINITY;  // two largest q of group `lane`
-                for (int e = lane * gs; e < (lane + 1) * gs; ++e) {
-                    float v = key[e];
-                    if (v > a) { b = a; a = v; } else if (v > b) { b = v; }
-                }
-                gscore = choice_key(__fadd_rn(a, b));  // inf + -inf is NaN
+    // groups kept (bit g set); all experts allowed without group limiting.
+    // margin_g: gap between the last kept and the best dropped group score
+    float margin_g = INFINITY;
+    if (G > 1) {
+        // the two largest q of each group: 32 / G lanes share a group's
+        // experts when G divides the warp, else one lane takes them all
+        const int L = 32 % G == 0 ? 32 / G : 1;
+        const int g = lane / L;
+        float a = -INFINITY, b = -INFINITY;
+        if (g < G)
+            for (int e = g * gs + lane % L; e < (g + 1) * gs; e += L) {
+                const float v = key[e];
+                if (v > a) { b = a; a = v; } else if (v > b) { b = v; }
             }
-            kept = 0u;
-            bool taken = false;
-            float last = 0.0f;
-            for (int r = 0; r <= rp.topk_group && r < G; ++r) {
-                float kk = (lane < G && !taken) ? gscore : -INFINITY;
-                int ii = (lane < G && !taken) ? lane : kNone;
-                warp_best(kk, ii);
-                if (r == rp.topk_group) {  // the best dropped group
-                    margin_g = last - kk;
-                    break;
-                }
-                if (ii < 32) kept |= 1u << ii;  // always: topk_group <= G groups hold candidates
-                if (lane == ii) taken = true;
-                last = kk;
-            }
+        for (int d = 1; d < L; d <<= 1) {
+            const float ao = __shfl_xor_sync(0xffffffffu, a, d), bo = __shfl_xor_sync(0xffffffffu, b, d);
+            b = fmaxf(fminf(a, ao), fmaxf(b, bo));
+            a = fmaxf(a, ao);
         }
-
-        // top-k over allowed experts, descending key, ties to the lower index;
-        // margin_k: smallest gap between consecutive keys of the k chosen and
-        // the best one left out
-        uint32_t used = 0u;  // bit s: expert lane + 32 s already chosen
-        float prev = 0.0f, margin_k = INFINITY;
-        for (int j = 0; j <= k; ++j) {
-            float kk = -INFINITY;
-            int ii = kNone;
-            for (int s = 0, e = lane; e < E; ++s, e += 32) {
-                if ((used >> s) & 1u) continue;
-                if (!((kept >> (e / gs)) & 1u)) continue;
-                float v = key[e];
-                if (ii == kNone || better(v, e, kk, ii)) { kk = v; ii = e; }
+        const float gscore = choice_key(__fadd_rn(a, b));  // inf + -inf is NaN
+        // one candidate per group, in the group's first lane
+        uint32_t gb = g < G && lane % L == 0 ? key_bits(gscore) : 0u;
+        uint32_t kept = 0u;
+        float last = 0.0f;
+        for (int r = 0; r <= rp.topk_group && r < G; ++r) {
+            uint32_t m = gb;
+            int ii = gb ? g : kNone;
+            warp_best(m, ii);
+            if (r == rp.topk_group) {  // the best dropped group
+                margin_g = last - key_value(m);
+                break;
             }
-            warp_best(kk, ii);
-            if (j > 0 && ii < E) margin_k = fminf(margin_k, prev - kk);
-            if (j == k) break;  // only the margin to the best expert left out
-            // ii < E always (check_config keeps top_k within the kept groups' experts)
-            if (ii < E && (ii & 31) == lane) used |= 1u << (ii >> 5);
-            if (j == 0) top_key = kk;
-            if (lane == j) sel_id = ii < E ? ii : 0;
-            prev = kk;
+            kept |= 1u << (ii & 31);  // topk_group <= G groups hold candidates
+            if (g == ii) gb = 0u;
+            last = key_value(m);
         }
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+            if (!((kept >> (((lane + 32 * s) / gs) & 31)) & 1u)) kb[s] = 0u;
+    }
 
-        if (au.x) {
+    // top-k over allowed experts, descending key, ties to the lower index;
+    // margin_k: smallest gap between consecutive keys of the k chosen and
+    // the best one left out
+    sel_id = 0;
+    float top_key = 0.0f, prev = 0.0f, margin_k = INFINITY;
+    for (int j = 0; j <= k; ++j) {
+        uint32_t m = 0u;
+        int ii = kNone;
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+            if (kb[s] > m) { m = kb[s]; ii = lane + 32 * s; }
+        warp_best(m, ii);
+        const bool found = ii < E;
+        const float kk = found ? key_value(m) : -INFINITY;
+        if (j > 0 && found) margin_k = fminf(margin_k, prev - kk);
+        if (j == k) break;  // only the margin to the best expert left out
+        // found always (check_config keeps top_k within the kept groups' experts)
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+            if (ii == lane + 32 * s) kb[s] = 0u;
+        if (j == 0) top_key = kk;
+        if (lane == j) sel_id = found ? ii : 0;
+        prev = kk;
+    }
+
+    if (au.x) {
         // bound on the logit error, and on the key error it causes (sigmoid:
         // slope <= 1/4, plus a few units in the last place of the fp32 key)
         float xx = 0.0f;
         const __nv_bfloat16* xt = au.x + (size_t)t * rp.H;
-        for (int c = lane; c < rp.H / 8; c += 32) {
-            float xv[8];
-            Vec8<__nv_bfloat16>::load(xt + 8 * c, xv);
+        for (int c0 = lane; c0 < rp.H / 8; c0 += 4 * 32) {
+            Raw8<__nv_bfloat16> xv[4];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) xx = fmaf(xv[i], xv[i], xx);
+            for (int u = 0; u < 4; ++u)
+                if (c0 + 32 * u < rp.H / 8) xv[u].load(xt + 8 * (c0 + 32 * u));
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c0 + 32 * u < rp.H / 8) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) xx = fmaf(xv[u].at(i), xv[u].at(i), xx);
+                }
         }
 #pragma unroll
         for (int d = 16; d >= 1; d >>= 1) xx += __shfl_xor_sync(0xffffffffu, xx, d);
@@ -386,21 +426,24 @@ select_experts_kernel(const float* __restrict__ logits, const float* __restrict_
         const float bk = sigmoid ? 0.25f * bl + 1e-6f : bl;
         const bool close = !(margin_k > 2.0f * bk) || !(margin_g > 4.0f * bk);
         if (close && lane == 0) au.flagged[atomicAdd(au.n_flagged, 1)] = t;
-        }
     }
 
     // routing weights (lane j < k holds slot j)
-    float w = 0.0f;
+    w = 0.0f;
     if (!sigmoid) {
-        float lj = (lane < k) ? l[sel_id] : 0.0f;
+        float lj = (lane < k) ? val[sel_id] : 0.0f;
         float m = top_key, z = 0.0f;
         if (!rp.renormalize) {
             float mm = -INFINITY;
-            for (int e = lane; e < E; e += 32) mm = fmaxf(mm, l[e]);
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s)
+                if (lane + 32 * s < E) mm = fmaxf(mm, raw[s]);
 #pragma unroll
             for (int d = 16; d >= 1; d >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, d));
             m = mm;
-            for (int e = lane; e < E; e += 32) z += expf(l[e] - m);
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s)
+                if (lane + 32 * s < E) z += expf(raw[s] - m);
         } else {
             z = (lane < k) ? expf(lj - m) : 0.0f;
         }
@@ -408,18 +451,44 @@ select_experts_kernel(const float* __restrict__ logits, const float* __restrict_
         for (int d = 16; d >= 1; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
         w = (lane < k) ? expf(lj - m) / z * rp.routed_scale : 0.0f;
     } else {
-        float sj = (lane < k) ? sig[sel_id] : 0.0f;
+        float sj = (lane < k) ? val[sel_id] : 0.0f;
         float z = sj;
 #pragma unroll
         for (int d = 16; d >= 1; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
         w = (rp.renormalize ? sj / z : sj) * rp.routed_scale;
     }
-    if (lane < k) {
-        topk_ids[(size_t)t * k + lane] = sel_id;
-        topk_w[(size_t)t * k + lane] = w;
-    }
     __syncwarp();
+}
+
+// One warp per token (every token, or those of `list` in grid-stride order).
+template <int SLOTS>
+__global__ void __launch_bounds__(kSelWarps * 32)
+select_experts_kernel(const float* __restrict__ logits, const float* __restrict__ select_bias,
+                      int32_t* __restrict__ topk_ids, float* __restrict__ topk_w, RouteParams rp, GateAudit au,
+                      const int32_t* __restrict__ list, const int32_t* __restrict__ n_list) {
+    pdl_enter();
+    __shared__ float s_key[kSelWarps][32 * SLOTS];
+    __shared__ float s_val[kSelWarps][32 * SLOTS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_tok = list ? *n_list : rp.T;
+    for (int i = blockIdx.x * kSelWarps + warp; i < n_tok; i += gridDim.x * kSelWarps) {
+        const int t = list ? list[i] : i;
+        int id;
+        float w;
+        select_token<SLOTS>(logits + (size_t)t * rp.E, select_bias, rp, au, t, s_key[warp], s_val[warp], id, w);
+        if (lane < rp.top_k) {
+            topk_ids[(size_t)t * rp.top_k + lane] = id;
+            topk_w[(size_t)t * rp.top_k + lane] = w;
+        }
     }
+}
+
+static cudaError_t launch_select(const float* logits, const float* select_bias, int32_t* topk_ids, float* topk_w,
+                                 const RouteParams& rp, const GateAudit& au, const int32_t* list, const int32_t* n_list,
+                                 int blocks, cudaStream_t stream) {
+    auto kernel = rp.E <= 128 ? select_experts_kernel<4> : rp.E <= 256 ? select_experts_kernel<8> : select_experts_kernel<16>;
+    return launch_k(kernel, dim3(blocks), dim3(kSelWarps * 32), 0, stream, logits, select_bias, topk_ids, topk_w, rp, au,
+                    list, n_list);
 }
 
 // max over experts of ||wg[e]||_2 (fp32) into *out (zeroed beforehand): a
@@ -522,8 +591,6 @@ cudaError_t launch_route(const RouteParams& rp, const void* x, const void* wg, c
                          const float* select_bias, float* logits, int32_t* topk_ids, float* topk_w,
                          const RouteScratch& rs, cudaStream_t stream) {
     if (rp.T == 0) return cudaSuccess;
-    const int ey = (rp.E + kGateWarps * kGateExpertsPerWarp - 1) / (kGateWarps * kGateExpertsPerWarp);
-    dim3 block(kGateWarps * 32);
     GateAudit au{};
     if (rp.gate_tc) {
         // tensor-core logits, then the audited choice
@@ -549,27 +616,20 @@ cudaError_t launch_route(const RouteParams& rp, const void* x, const void* wg, c
                     stream, xp, wp, logit_bias, logits, rp.T, rp.H, rp.E, static_cast<const int32_t*>(nullptr),
                     static_cast<const int32_t*>(nullptr)); le != cudaSuccess)
                 return le;
-        } else {
-            dim3 grid((rp.T + 1) / 2, ey);
-            if (const cudaError_t le = launch_k(gate_logits_kernel<__nv_bfloat16, 2>, dim3(grid), dim3(block), 0,
-                    stream, xp, wp, logit_bias, logits, rp.T, rp.H, rp.E); le != cudaSuccess)
-                return le;
+        } else if (const cudaError_t le = launch_gate_logits(xp, wp, logit_bias, logits, rp.T, rp.H, rp.E, stream);
+                   le != cudaSuccess) {
+            return le;
         }
     } else {
-        auto xp = static_cast<const float*>(x);
-        auto wp = static_cast<const float*>(wg);
-        dim3 grid((rp.T + 1) / 2, ey);
-        if (const cudaError_t le = launch_k(gate_logits_kernel<float, 2>, dim3(grid), dim3(block), 0, stream, xp,
-                wp, logit_bias, logits, rp.T, rp.H, rp.E); le != cudaSuccess)
+        if (const cudaError_t le = launch_gate_logits(static_cast<const float*>(x), static_cast<const float*>(wg),
+                logit_bias, logits, rp.T, rp.H, rp.E, stream); le != cudaSuccess)
             return le;
     }
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    if (const cudaError_t le = launch_k(select_experts_kernel, dim3((rp.T + kSelWarps - 1) / kSelWarps),
-            dim3(kSelWarps * 32), 0, stream, logits, select_bias, topk_ids, topk_w, rp, au,
-            static_cast<const int32_t*>(nullptr), static_cast<const int32_t*>(nullptr)); le != cudaSuccess)
-        return le;
-    if ((err = cudaGetLastError()) != cudaSuccess || !rp.gate_tc) return err;
+    if ((err = launch_select(logits, select_bias, topk_ids, topk_w, rp, au, nullptr, nullptr,
+                             (rp.T + kSelWarps - 1) / kSelWarps, stream)) != cudaSuccess || !rp.gate_tc)
+        return err;
     // flagged tokens: fixed-order logits, then their choice again (no audit)
     const int32_t* n_flag = reinterpret_cast<const int32_t*>(rs.audit + 1);
     if ((err = gate_tiled_smem()) != cudaSuccess) return err;
@@ -579,13 +639,9 @@ cudaError_t launch_route(const RouteParams& rp, const void* x, const void* wg, c
             rp.H, rp.E, static_cast<const int32_t*>(rs.flagged), n_flag); le != cudaSuccess)
         return le;
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    const int blocks = sm_count() * 4;
-    GateAudit none{};
-    if (const cudaError_t le = launch_k(select_experts_kernel, dim3(blocks), dim3(kSelWarps * 32), 0, stream, logits,
-            select_bias, topk_ids, topk_w, rp, none, static_cast<const int32_t*>(rs.flagged), n_flag);
-        le != cudaSuccess)
-        return le;
-    return cudaGetLastError();
+    const GateAudit none{};
+    return launch_select(logits, select_bias, topk_ids, topk_w, rp, none, static_cast<const int32_t*>(rs.flagged), n_flag,
+                         sm_count() * 4, stream);
 }
 
 }  // namespace gbmoe
