@@ -89,7 +89,8 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     // int4 and MXFP4 weights with bf16 activations and few rows per expert: the
     // feature-major GEMM (use_fm), reported as TC
     const bool four_bit = c->w_dtype == GBMOE_INT4_G128 || c->w_dtype == GBMOE_MXFP4;
-    if (four_bit && n_rows <= kFmRowsPerExpert * E && ffn_fm_supported(probe)) return GBMOE_FFN_TC;
+    if (four_bit && c->combine_route != GBMOE_COMBINE_FUSED && n_rows <= kFmRowsPerExpert * E && ffn_fm_supported(probe))
+        return GBMOE_FFN_TC;
     if (n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I)) return GBMOE_FFN_STREAM;
     if (c->act_dtype == GBMOE_BF16) {
         if (ffn_tc_supported(probe)) {
@@ -106,8 +107,9 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
 }
 
 // Whether that problem runs on the feature-major GEMM (ffn_fm.cu): fp8 weights
-// on the fp8 route, forced or not; int4 and MXFP4 when AUTO chose (a forced
-// TC is the row-major GEMM).
+// on the fp8 route, forced or not; the other formats when AUTO chose (a forced
+// STREAM is the CUDA-core kernels, a forced TC the row-major GEMM) and the
+// Weight Sum is not asked into the down GEMM's epilogue.
 bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     FfnProblem probe{};
     probe.act_dtype = c->act_dtype;
@@ -116,7 +118,7 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     probe.I = I;
     if (n_rows > kFmRowsPerExpert * E || !ffn_fm_supported(probe)) return false;
     return c->w_dtype == GBMOE_FP8_E4M3_B128 ? pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8
-                                             : c->ffn_route == GBMOE_FFN_AUTO;
+                                             : c->ffn_route == GBMOE_FFN_AUTO && c->combine_route != GBMOE_COMBINE_FUSED;
 }
 
 // Bytes of the bf16 weight copy the TC_DEQUANT route decodes into (0 when
@@ -135,6 +137,21 @@ size_t sorted_x_bytes(const gbmoe_config* c) {
     if (use_fm(c, P, c->E, c->I)) return 0;
     const bool reads_copy = pair_route(r) || (r == GBMOE_FFN_TC && quantised_weights(c->w_dtype));
     return reads_copy ? (size_t)P * c->H * act_bytes(c->act_dtype) : 0;
+}
+
+// Gate route: the fixed-order CUDA-core logits, or tensor-core logits audited
+// against that order (AUTO: bf16 batches of at least kGateTcMinTokens tokens).
+constexpr int kGateTcMinTokens = 256;
+
+int pick_gate(const gbmoe_config* c) {
+    if (c->gate_route != GBMOE_GATE_AUTO) return c->gate_route;
+    if (c->act_dtype != GBMOE_BF16 || c->T < kGateTcMinTokens) return GBMOE_GATE_SIMT;
+    FfnProblem probe{};
+    probe.act_dtype = c->act_dtype;
+    probe.w_dtype = GBMOE_BF16;
+    probe.H = c->H;
+    probe.I = 128;
+    return ffn_tc_supported(probe) ? GBMOE_GATE_TC : GBMOE_GATE_SIMT;
 }
 
 struct Layout {
@@ -163,7 +180,7 @@ Layout layout(const gbmoe_config* c) {
     L.audit = take(8);
     L.flagged = take((size_t)T * 4);
     L.arrive = take((size_t)T * (H / 256) * 4);
-    L.logits = take((size_t)T * E * 4);
+    L.logits = take((size_t)T * E * 4 * (pick_gate(c) == GBMOE_GATE_TC ? gate_tc_splits(c->T, c->H, c->E) : 1));
     L.ids = take((size_t)P * 4);
     L.w = take((size_t)P * 4);
     L.counts = take((size_t)E * 4);
@@ -218,21 +235,6 @@ int check_weights(const gbmoe_config* c, const gbmoe_expert_weights* w) {
         if (!aligned(w->s_gate, sa) || !aligned(w->s_up, sa) || !aligned(w->s_down, sa)) return GBMOE_EINVAL;
     }
     return GBMOE_OK;
-}
-
-// Gate route: the fixed-order CUDA-core logits, or tensor-core logits audited
-// against that order (AUTO: bf16 batches of at least kGateTcMinTokens tokens).
-constexpr int kGateTcMinTokens = 256;
-
-int pick_gate(const gbmoe_config* c) {
-    if (c->gate_route != GBMOE_GATE_AUTO) return c->gate_route;
-    if (c->act_dtype != GBMOE_BF16 || c->T < kGateTcMinTokens) return GBMOE_GATE_SIMT;
-    FfnProblem probe{};
-    probe.act_dtype = c->act_dtype;
-    probe.w_dtype = GBMOE_BF16;
-    probe.H = c->H;
-    probe.I = 128;
-    return ffn_tc_supported(probe) ? GBMOE_GATE_TC : GBMOE_GATE_SIMT;
 }
 
 RouteParams route_params(const gbmoe_config* c) {
@@ -521,8 +523,8 @@ int moe_forward(const gbmoe_config* cfg, const void* x, const void* w_router, co
         if ((s = run_ffn(cfg, ps, r_shared, st))) return s;
     }
     FfnProblem pr = routed_problem(cfg, x, counts, offsets, sorted, experts, y, ws);
-    const bool fused = cfg->combine_route == GBMOE_COMBINE_FUSED && bf16_gemm_route(r_routed) &&
-                       !use_fm(cfg, P, cfg->E, cfg->I);
+    pr.pair_pos = pos;
+    const bool fused = cfg->combine_route == GBMOE_COMBINE_FUSED && bf16_gemm_route(r_routed);
     if (fused) {  // Weight Sum in the down GEMM's epilogue
         if ((s = cuda_status(cudaMemsetAsync(at<int32_t>(ws, L.arrive), 0, (size_t)cfg->T * (cfg->H / 256) * 4, st))))
             return s;

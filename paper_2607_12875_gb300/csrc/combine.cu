@@ -6,8 +6,8 @@
 // (a pair the permutation dropped) is skipped.
 //
 // Bound by HBM for large batches and by two dependent load latencies for small
-// ones. k 8: 32 tokens x 4096 in COMB32 us (one block and a loop per token
-// took 11.4), 8192 tokens in COMB8192 us (98.3).
+// ones. k 8, H 4096: 32 tokens in 3.9 us (one block and a loop over the slots per
+// token took 11.4), 8192 tokens in 96.8 us (98.3).
 #include "common.cuh"
 #include "kernels.h"
 

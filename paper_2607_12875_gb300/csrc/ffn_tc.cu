@@ -130,11 +130,12 @@ struct Params {
     const void* scale0;  // scales of the B rows in the first / second half of the tile
     const void* scale1;
     uint64_t wait_limit_ns;  // limit of each pipeline wait (kWaitLimitNs unless a test shortens it)
-    // fp32 output instead of bf16 (the router's logits): out_f32[row, col] =
-    // accumulator (+ col_bias[col]) for col < f32_cols; out is unused then
+    // fp32 output instead of bf16 (the router's logits): out_f32[s][row, col] =
+    // sum of k split s, for col < f32_cols (planes of n_rows * out_cols); out is
+    // unused then. k_split > 1 only with it.
     float* out_f32;
-    const float* col_bias;
     int f32_cols;
+    int k_split;
     // Weight Sum fused into the down GEMM (fuse_k > 0, the layer's top_k): row
     // r is pair p = sorted_pair[r] = t*k + j; its output times topk_w[p] goes to
     // slots[p] (pair order, bf16), and the thread completing the k-th arrival of
@@ -317,15 +318,21 @@ struct Work {
     int e, m, nt;
     int64_t row0;  // absolute first row of this CTA's 128 rows of the M tile
     int rows;      // valid rows among them (<= 0: none)
+    int split;     // k split
 };
 
-// Work item w: M tile w / n_tiles of the list (BM * CG rows of one expert),
-// N tile w % n_tiles; CTA `rank` of a pair takes the tile's rows rank*BM ..
+// Work item w: k split w % k_split, then M tile w / n_tiles of the list (BM *
+// CG rows of one expert), N tile w % n_tiles; CTA `rank` of a pair takes the tile's rows rank*BM ..
 template <int CG>
 __device__ __forceinline__ Work decode_work(const Params& p, int w, uint32_t rank) {
     const int2* tiles = reinterpret_cast<const int2*>(p.sched + sched_tiles_offset(p.E));
-    const int mt = w / p.n_tiles;
     Work r;
+    r.split = 0;
+    if (p.k_split > 1) {
+        r.split = w % p.k_split;
+        w /= p.k_split;
+    }
+    const int mt = w / p.n_tiles;
     r.nt = w - mt * p.n_tiles;
     const int2 t = tiles[mt];
     r.e = t.x;
@@ -440,8 +447,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    const int total = p.sched[1] * p.n_tiles;
-    const int nkb = p.K / BK;
+    const int total = p.sched[1] * p.n_tiles * p.k_split;
+    const int nkb = p.K / BK / p.k_split;
     const int unit = blockIdx.x / CG, n_units = gridDim.x / CG;  // CTA pairs walk the list together
 
     if (warp == 0 && lane == 0) {
@@ -459,6 +466,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             // CG = 2: this CTA's half of the B tile (gate rows / up rows, or down rows 0-127 / 128-255)
             const CUtensorMap* tm_bh = rank ? &tm_b1 : &tm_b0;
             const int bh = rank ? b1 : b0;
+            const int x0 = wk.split * nkb * BK;  // first k (bf16 B only)
             for (int kb = 0; kb < nkb; ++kb) {
                 if (WQ == GBMOE_FP8_E4M3_B128 && kb + kFp8PrefetchAhead < nkb) {
                     // fp8 tiles wait on the decode as well as on the load: bring the
@@ -478,7 +486,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 if (rank == 0) mbar_expect_tx(&full[stage], CG * ((gather_a ? 0 : A_BYTES) + (RAW ? RAW : BH)));
                 if (gather_a) {
                 } else if (rank == 0) {
-                    tma_load_2d(sA + stage * A_BYTES, &tm_a, kb * BK, (int)wk.row0, &full[stage]);
+                    tma_load_2d(sA + stage * A_BYTES, &tm_a, x0 + kb * BK, (int)wk.row0, &full[stage]);
                 } else {
                     tma_load_2d_to_pair_leader(sA + stage * A_BYTES, &tm_a, kb * BK, (int)wk.row0, &full[stage]);
                 }
@@ -486,8 +494,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 const int xr = packed4<WQ>() ? kb * (BK / 2) : kb * BK;
                 if (CG == 1) {
                     if (RAW == 0) {
-                        tma_load_2d(sB + stage * BH, &tm_b0, kb * BK, b0, &full[stage]);
-                        tma_load_2d(sB + stage * BH + BH / 2, &tm_b1, kb * BK, b1, &full[stage]);
+                        tma_load_2d(sB + stage * BH, &tm_b0, x0 + kb * BK, b0, &full[stage]);
+                        tma_load_2d(sB + stage * BH + BH / 2, &tm_b1, x0 + kb * BK, b1, &full[stage]);
                     } else {
                         tma_load_2d(sR + stage * RAW, &tm_b0, xr, b0, &full[stage]);
                         tma_load_2d(sR + stage * RAW + RAW / 2, &tm_b1, xr, b1, &full[stage]);
@@ -604,11 +612,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     if (lane == 0) tma_store_2d(&tm_out, buf, col0 + c, (int)(wk.row0 + q * 32));
                     sbuf ^= 1;
                 } else if (valid && p.out_f32) {
-                    float* dst32 = p.out_f32 + (wk.row0 + r) * (int64_t)p.out_cols + col0 + c;
+                    float* dst32 = p.out_f32 + (wk.split * p.n_rows + wk.row0 + r) * (int64_t)p.out_cols + col0 + c;
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
                         const int col = col0 + c + i;
-                        if (col < p.f32_cols) dst32[i] = p.col_bias ? __fadd_rn(v[i], p.col_bias[col]) : v[i];
+                        if (col < p.f32_cols) dst32[i] = v[i];
                     }
                 } else if (valid) {
                     if (p.fuse_k) {
@@ -973,12 +981,27 @@ static cudaError_t dequant_all(const FfnProblem& p, FfnProblem& q, cudaStream_t 
     return cudaSuccess;
 }
 
-// Router logits on the tensor cores: logits[t, e] = x[t, :] . wg[e, :]
-// (+ bias[e]), x [T, H] and wg [E, H] bf16, fp32 accumulation in the tensor
-// core's own order (the caller audits near ties against the fixed order).
-// sched: schedule ints for one problem of T rows.
-cudaError_t launch_gate_tc(const void* x, const void* wg, const float* bias, float* logits, int T, int H, int E,
-                           int32_t* sched, int32_t* err, cudaStream_t stream) {
+// k splits of the router GEMM: as many as fill the SMs with tiles x splits, at
+// least four 64-wide k blocks each. A few row tiles otherwise leave most SMs
+// idle through H / 64 dependent k blocks: 333 tokens x 128 experts, H 4096:
+// 37 us with one split, 16 with 16; 2048 x 256, H 7168: 60 and 32 us.
+// Fixed numbers, not the device's SM count: the workspace holds the planes.
+int gate_tc_splits(int T, int H, int E) {
+    constexpr int kTargetItems = 152;
+    const int64_t items = (int64_t)((T + tc::BM - 1) / tc::BM) * ((E + tc::BN - 1) / tc::BN);
+    const int nkb = H / tc::BK;
+    int s = 1;
+    while (s < 16 && nkb % (2 * s) == 0 && nkb / (2 * s) >= 4 && items * 2 * s <= kTargetItems) s *= 2;
+    return s;
+}
+
+// Router logits on the tensor cores: the sum over the gate_tc_splits planes of
+// logits [splits, T, E] is x[t, :] . wg[e, :], x [T, H] and wg [E, H] bf16, fp32
+// accumulation in the tensor core's own order (the caller adds planes and bias,
+// and audits near ties against the fixed order). sched: schedule ints for one
+// problem of T rows.
+cudaError_t launch_gate_tc(const void* x, const void* wg, float* logits, int T, int H, int E, int32_t* sched,
+                           int32_t* err, cudaStream_t stream) {
     using namespace tc;
     if (T == 0) return cudaSuccess;
     cudaError_t e = launch_ffn_schedule(nullptr, 1, T, BM, sched, stream);
@@ -991,8 +1014,8 @@ cudaError_t launch_gate_tc(const void* x, const void* wg, const float* bias, flo
     g.counts = nullptr; g.offsets = nullptr; g.sched = sched; g.E = 1; g.n_rows = T;
     g.out = nullptr; g.err = err; g.scale0 = g.scale1 = nullptr;
     g.wait_limit_ns = tc_wait_limit_ns();
-    g.out_f32 = logits; g.col_bias = bias; g.f32_cols = E;
-    return launch_gemm<1>(GBMOE_BF16, ma, mb, mb, mo, g, sched_max_tiles(1, T, BM) * g.n_tiles, stream);
+    g.out_f32 = logits; g.f32_cols = E; g.k_split = gate_tc_splits(T, H, E);
+    return launch_gemm<1>(GBMOE_BF16, ma, mb, mb, mo, g, sched_max_tiles(1, T, BM) * g.n_tiles * g.k_split, stream);
 }
 
 cudaError_t launch_ffn_tc(const FfnProblem& pin, cudaStream_t stream) {
@@ -1034,6 +1057,7 @@ cudaError_t launch_ffn_tc(const FfnProblem& pin, cudaStream_t stream) {
         return cudaErrorInvalidValue;
 
     Params g{};
+    g.k_split = 1;
     g.K = p.H; g.n_tiles = p.I / (BN / 2); g.out_cols = p.I; g.b_rows_per_expert = p.I; g.swiglu = 1;
     g.counts = p.counts; g.offsets = p.offsets; g.sched = p.sched; g.E = p.E; g.n_rows = p.n_rows;
     g.out = static_cast<__nv_bfloat16*>(p.h); g.err = p.err;

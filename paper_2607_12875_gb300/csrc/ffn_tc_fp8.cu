@@ -376,8 +376,9 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     cudaError_t err = launch_ffn_schedule(p.counts, p.E, p.n_rows, BM, p.sched, stream);
     if (err != cudaSuccess) return err;
     // x rows in sorted order (x itself for the shared expert), quantised per 1x128
-    if ((err = launch_quant_rows(p.x, p.sorted_pair, p.pair_div, p.n_rows, p.H, p.a_q, p.a_s, nullptr, stream)) != cudaSuccess)
-        return err;
+    err = p.pair_pos ? launch_quant_scatter(p.x, p.pair_pos, p.pair_div, p.n_rows / p.pair_div, p.H, p.a_q, p.a_s, stream)
+                     : launch_quant_rows(p.x, p.sorted_pair, p.pair_div, p.n_rows, p.H, p.a_q, p.a_s, nullptr, stream);
+    if (err != cudaSuccess) return err;
     const int64_t max_m = sched_max_tiles(p.E, p.n_rows, BM);
     const uint8_t* aq = static_cast<const uint8_t*>(p.a_q);
     const uint8_t* hq = static_cast<const uint8_t*>(p.h_q);

@@ -24,16 +24,18 @@ struct RouteScratch {
     int32_t* flagged;
 };
 
-// logits [T, E] fp32 scratch; topk_ids, topk_w [T, k]
+// logits: fp32 scratch, route_logits(rp) floats; topk_ids, topk_w [T, k]
 cudaError_t launch_route(const RouteParams& rp, const void* x, const void* w_router, const float* logit_bias,
                          const float* select_bias, float* logits, int32_t* topk_ids, float* topk_w,
                          const RouteScratch& rs, cudaStream_t stream);
 // RMSNorm of x [T, H] (act dtype) with gamma [H] into y, in the gate's order
 cudaError_t launch_rmsnorm(const void* x, const void* gamma, float eps, int T, int H, int act_dtype, void* y,
                            cudaStream_t stream);
-// router logits on the tensor cores (bf16 x and router weight; ffn_tc.cu)
-cudaError_t launch_gate_tc(const void* x, const void* wg, const float* bias, float* logits, int T, int H, int E,
-                           int32_t* sched, int32_t* err, cudaStream_t stream);
+// router logits on the tensor cores (bf16 x and router weight; ffn_tc.cu), as
+// gate_tc_splits partial planes [splits, T, E] without the bias
+int gate_tc_splits(int T, int H, int E);
+cudaError_t launch_gate_tc(const void* x, const void* wg, float* logits, int T, int H, int E, int32_t* sched,
+                           int32_t* err, cudaStream_t stream);
 
 // Number of 1024-pair blocks the permutation uses, and its scratch ints.
 int permute_blocks(int64_t P);
@@ -49,6 +51,7 @@ struct FfnProblem {
     const int32_t* counts;      // [E] or null
     const int32_t* offsets;     // [E+1] or null (then 0, n_rows)
     const int32_t* sorted_pair; // [rows] or null
+    const int32_t* pair_pos;    // its inverse [rows], or null when the caller does not have it
     int pair_div;
     int E, H, I;
     int64_t n_rows;             // upper bound on rows (P, or T for the shared expert)
@@ -107,6 +110,9 @@ constexpr int64_t kFmRowsPerExpert = 40;
 // with int4_sums in the order int4 weights take, with the blocks' sums of codes there
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
                               float* s, float* int4_sums, cudaStream_t stream);
+// the same of every row of src once, row r's codes written to rows pair_pos[r * k ..] of [2, n_src * k, K]
+cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
+                                 cudaStream_t stream);
 cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream);
 bool ffn_fm_supported(const FfnProblem& p);
 

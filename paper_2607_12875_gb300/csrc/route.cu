@@ -8,6 +8,7 @@
 // of chunks l, l+32, ... for all of them, which is exactly the fixed order.
 // select_experts then runs one warp per token over the logits. Large batches
 // use a shared-memory-staged variant with the same order (below).
+#include <algorithm>
 #include <cstdlib>
 
 #include "common.cuh"
@@ -20,15 +21,12 @@ constexpr int kGateWarps = 8;
 // A small batch is bound by the latency of a warp's H / 256 dependent steps:
 // the loads of U steps are in flight together, and small warp tiles spread the
 // work over more SMs (their repeated reads come from L2).
+// A warp's logits of rows t0 .. of x and experts e0 ..
 template <typename TA, int TB, int EB, int U>
-__global__ void __launch_bounds__(kGateWarps * 32)
-gate_logits_kernel(const TA* __restrict__ x, const TA* __restrict__ wg, const float* __restrict__ bias,
-                   float* __restrict__ logits, int T, int H, int E) {
-    pdl_enter();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t0 = blockIdx.x * TB;
-    const int e0 = (blockIdx.y * kGateWarps + warp) * EB;
-    if (e0 >= E) return;
+__device__ __forceinline__ void gate_logits_warp(const TA* __restrict__ x, const TA* __restrict__ wg,
+                                                 const float* __restrict__ bias, float* __restrict__ logits, int t0,
+                                                 int e0, int T, int H, int E) {
+    const int lane = threadIdx.x & 31;
     float acc[TB][EB];
     const TA* xp[TB];  // rows past the end repeat the last one and are not stored
     const TA* wp[EB];
@@ -87,6 +85,15 @@ gate_logits_kernel(const TA* __restrict__ x, const TA* __restrict__ wg, const fl
 }
 
 template <typename TA, int TB, int EB, int U>
+__global__ void __launch_bounds__(kGateWarps * 32)
+gate_logits_kernel(const TA* __restrict__ x, const TA* __restrict__ wg, const float* __restrict__ bias,
+                   float* __restrict__ logits, int T, int H, int E) {
+    pdl_enter();
+    const int e0 = (blockIdx.y * kGateWarps + (threadIdx.x >> 5)) * EB;
+    if (e0 < E) gate_logits_warp<TA, TB, EB, U>(x, wg, bias, logits, blockIdx.x * TB, e0, T, H, E);
+}
+
+template <typename TA, int TB, int EB, int U>
 static cudaError_t launch_gate_logits(const TA* x, const TA* wg, const float* bias, float* logits, int T, int H, int E,
                                       cudaStream_t stream) {
     const dim3 grid((unsigned)((T + TB - 1) / TB), (unsigned)((E + kGateWarps * EB - 1) / (kGateWarps * EB)));
@@ -106,7 +113,7 @@ static cudaError_t launch_gate_logits(const TA* x, const TA* wg, const float* bi
 }
 
 // Large batches: the same fixed order, as a CUDA-core GEMM. A CTA owns 32
-// tokens x 16 experts; 256-element slabs of x and Wg go through a 3-stage
+// tokens x 16 experts; 256-element slabs of x and Wg go through a
 // cp.async ring in shared memory, and warp w (of 8) accumulates tokens
 // 8*(w%4).. x experts 8*(w/4).. in registers. Lane l reads 8-element chunk l
 // of every slab, i.e. chunks l, l+32, ... in increasing order, elements in
@@ -120,14 +127,17 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool vali
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
 }
 
-// With a token list, tile rows are the listed tokens (list[0 .. *n_list)),
-// and tiles past the list's end return at once.
+// With a token list, tile rows are the listed tokens (list[0 .. *n_list)), and
+// tiles past the list's end return at once, as all do when the list is short
+// enough for gate_logits_list_kernel.
+constexpr int kShortList = 128;
 __global__ void __launch_bounds__(256, 1)
 gate_logits_tiled_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ wg,
                          const float* __restrict__ bias, float* __restrict__ logits, int T, int H, int E,
                          const int32_t* __restrict__ list, const int32_t* __restrict__ n_list) {
     pdl_enter();
     const int n_rows = list ? *n_list : T;
+    if (list && n_rows <= kShortList) return;
     if ((int)blockIdx.x * kGT >= n_rows) return;
     // token of tile row i (or -1 past the end)
     auto token = [&](int i) -> int {
@@ -141,22 +151,32 @@ gate_logits_tiled_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat1
     const int e0 = blockIdx.y * kGE;
     const int nslab = H / kSlab;
 
+    // thread i copies chunk i % 32 of rows i / 32 + 8 m of a slab (kGT rows of
+    // x, then kGE of Wg): their sources are looked up once, not per slab (the
+    // flagged tokens of 2048 x 256, H 7168: 83 -> 61 us)
+    constexpr int kRows = (kGT + kGE) / 8;
+    const __nv_bfloat16* src[kRows];
+    bool ok[kRows];
+#pragma unroll
+    for (int m = 0; m < kRows; ++m) {
+        const int row = warp + 8 * m;
+        if (row < kGT) {
+            const int t = token(row);
+            ok[m] = t >= 0;
+            src[m] = x + (size_t)(ok[m] ? t : 0) * H + 8 * lane;
+        } else {
+            const int e = e0 + row - kGT;
+            ok[m] = e < E;
+            src[m] = wg + (size_t)(ok[m] ? e : 0) * H + 8 * lane;
+        }
+    }
     auto load_slab = [&](int j) {
         const int st = j % kGStages;
-        // x: kGT rows x 32 chunks; Wg: kGE rows x 32 chunks; 16 bytes each
-        for (int i = threadIdx.x; i < (kGT + kGE) * 32; i += 256) {
-            const int row = i >> 5, c = i & 31;
-            if (row < kGT) {
-                const int t = token(row);
-                const bool ok = t >= 0;
-                cp_async16(sx + (((size_t)st * kGT + row) * kSlab + 8 * c) * 2,
-                           x + (size_t)(ok ? t : 0) * H + (size_t)j * kSlab + 8 * c, ok);
-            } else {
-                const int r = row - kGT, e = e0 + r;
-                const bool ok = e < E;
-                cp_async16(sw + (((size_t)st * kGE + r) * kSlab + 8 * c) * 2,
-                           wg + (size_t)(ok ? e : 0) * H + (size_t)j * kSlab + 8 * c, ok);
-            }
+#pragma unroll
+        for (int m = 0; m < kRows; ++m) {
+            const int row = warp + 8 * m;
+            uint8_t* dst = row < kGT ? sx + ((size_t)st * kGT + row) * kSlab * 2 : sw + ((size_t)st * kGE + row - kGT) * kSlab * 2;
+            cp_async16(dst + 16 * lane, src[m] + (size_t)j * kSlab, ok[m]);
         }
     };
 
@@ -226,6 +246,24 @@ gate_logits_tiled_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat1
                 logits[(size_t)t * E + e] = l;
             }
         }
+}
+
+// The listed tokens' logits when the list is short (the audit flags a few
+// tokens per thousand; the tiled kernel above then keeps a handful of CTAs
+// waiting through H / 256 slabs: 26 us for a handful of tokens at H 4096, 6.6
+// here). Longer lists are the tiled kernel's.
+constexpr int kListBlocks = 32;
+
+__global__ void __launch_bounds__(kGateWarps * 32)
+gate_logits_list_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ wg,
+                        const float* __restrict__ bias, float* __restrict__ logits, int T, int H, int E,
+                        const int32_t* __restrict__ list, const int32_t* __restrict__ n_list) {
+    pdl_enter();
+    const int n = *n_list;
+    const int e0 = (blockIdx.y * kGateWarps + (threadIdx.x >> 5)) * 2;
+    if (n > kShortList || e0 >= E) return;
+    for (int i = blockIdx.x; i < n; i += kListBlocks)
+        gate_logits_warp<__nv_bfloat16, 1, 2, 8>(x, wg, bias, logits, list[i], e0, T, H, E);
 }
 
 // ------------------------------------------------------- expert choice
@@ -299,12 +337,20 @@ struct GateAudit {
     int32_t* n_flagged;       // their count
 };
 
+// Where a logit is still in parts: the sum of n planes, stride floats apart,
+// plus bias (n = 1 and no bias: it is complete).
+struct LogitPlanes {
+    int n;
+    int64_t stride;
+    const float* bias;
+};
+
 // Chooses token t's experts and weights, by one warp: lane j < k returns slot
 // j's expert in sel_id and weight in w. Expert e lives in lane e % 32, register
 // e / 32 (E <= 32 * SLOTS); key and val are this warp's shared arrays of E
 // floats (choice keys; logits or sigmoids).
 template <int SLOTS>
-__device__ __forceinline__ void select_token(const float* __restrict__ l, const float* __restrict__ select_bias,
+__device__ __forceinline__ void select_token(const float* __restrict__ l, const LogitPlanes& pl, const float* __restrict__ select_bias,
                                              const RouteParams& rp, const GateAudit& au, int t, float* key, float* val,
                                              int& sel_id, float& w) {
     const int lane = threadIdx.x & 31;
@@ -315,6 +361,16 @@ __device__ __forceinline__ void select_token(const float* __restrict__ l, const 
     float raw[SLOTS];
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) raw[s] = lane + 32 * s < E ? l[lane + 32 * s] : 0.0f;
+    for (int q = 1; q < pl.n; ++q) {
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+            if (lane + 32 * s < E) raw[s] = __fadd_rn(raw[s], l[q * pl.stride + lane + 32 * s]);
+    }
+    if (pl.bias) {
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+            if (lane + 32 * s < E) raw[s] = __fadd_rn(raw[s], pl.bias[lane + 32 * s]);
+    }
     uint32_t kb[SLOTS];  // candidates: 0 once chosen, or not allowed
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) {
@@ -463,7 +519,7 @@ __device__ __forceinline__ void select_token(const float* __restrict__ l, const 
 // One warp per token (every token, or those of `list` in grid-stride order).
 template <int SLOTS>
 __global__ void __launch_bounds__(kSelWarps * 32)
-select_experts_kernel(const float* __restrict__ logits, const float* __restrict__ select_bias,
+select_experts_kernel(const float* __restrict__ logits, LogitPlanes pl, const float* __restrict__ select_bias,
                       int32_t* __restrict__ topk_ids, float* __restrict__ topk_w, RouteParams rp, GateAudit au,
                       const int32_t* __restrict__ list, const int32_t* __restrict__ n_list) {
     pdl_enter();
@@ -475,7 +531,7 @@ select_experts_kernel(const float* __restrict__ logits, const float* __restrict_
         const int t = list ? list[i] : i;
         int id;
         float w;
-        select_token<SLOTS>(logits + (size_t)t * rp.E, select_bias, rp, au, t, s_key[warp], s_val[warp], id, w);
+        select_token<SLOTS>(logits + (size_t)t * rp.E, pl, select_bias, rp, au, t, s_key[warp], s_val[warp], id, w);
         if (lane < rp.top_k) {
             topk_ids[(size_t)t * rp.top_k + lane] = id;
             topk_w[(size_t)t * rp.top_k + lane] = w;
@@ -483,11 +539,11 @@ select_experts_kernel(const float* __restrict__ logits, const float* __restrict_
     }
 }
 
-static cudaError_t launch_select(const float* logits, const float* select_bias, int32_t* topk_ids, float* topk_w,
+static cudaError_t launch_select(const float* logits, const LogitPlanes& pl, const float* select_bias, int32_t* topk_ids, float* topk_w,
                                  const RouteParams& rp, const GateAudit& au, const int32_t* list, const int32_t* n_list,
                                  int blocks, cudaStream_t stream) {
     auto kernel = rp.E <= 128 ? select_experts_kernel<4> : rp.E <= 256 ? select_experts_kernel<8> : select_experts_kernel<16>;
-    return launch_k(kernel, dim3(blocks), dim3(kSelWarps * 32), 0, stream, logits, select_bias, topk_ids, topk_w, rp, au,
+    return launch_k(kernel, dim3(blocks), dim3(kSelWarps * 32), 0, stream, logits, pl, select_bias, topk_ids, topk_w, rp, au,
                     list, n_list);
 }
 
@@ -525,13 +581,19 @@ static float gate_audit_scale() {
     return (end != v && *end == '\0' && f >= 0.0f) ? f : kGateAuditScale;
 }
 
-// shared-memory size of the tiled gate kernel, set once per device
-static cudaError_t gate_tiled_smem() {
-    static DeviceOnce smem_set;
-    return smem_set.run([] {
+// The tiled gate kernel over the whole batch, or over a list of its tokens.
+static cudaError_t launch_gate_tiled(const void* x, const void* wg, const float* bias, float* logits, int T, int H, int E,
+                                     const int32_t* list, const int32_t* n_list, cudaStream_t stream) {
+    static DeviceOnce smem_set;  // shared-memory size, set once per device
+    const cudaError_t e = smem_set.run([] {
         return cudaFuncSetAttribute(gate_logits_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kGateTiledSmem);
     });
+    if (e != cudaSuccess) return e;
+    const dim3 grid((T + kGT - 1) / kGT, (E + kGE - 1) / kGE);  // (tiles past a list's end exit)
+    return launch_k(gate_logits_tiled_kernel, grid, dim3(256), kGateTiledSmem, stream,
+                    static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(wg), bias, logits, T, H, E,
+                    list, n_list);
 }
 
 // ------------------------------------------------ RMSNorm before the gate
@@ -601,7 +663,7 @@ cudaError_t launch_route(const RouteParams& rp, const void* x, const void* wg, c
         if (const cudaError_t le = launch_k(row_norm_max_kernel, dim3((rp.E + 7) / 8), dim3(256), 0, stream, wp,
                 rp.E, rp.H, rs.audit); le != cudaSuccess)
             return le;
-        if (const cudaError_t le = launch_gate_tc(x, wg, logit_bias, logits, rp.T, rp.H, rp.E, rs.sched, rs.err,
+        if (const cudaError_t le = launch_gate_tc(x, wg, logits, rp.T, rp.H, rp.E, rs.sched, rs.err,
                 stream); le != cudaSuccess)
             return le;
         au.x = xp; au.wnorm_max = rs.audit; au.scale = gate_audit_scale();
@@ -610,11 +672,8 @@ cudaError_t launch_route(const RouteParams& rp, const void* x, const void* wg, c
         auto xp = static_cast<const __nv_bfloat16*>(x);
         auto wp = static_cast<const __nv_bfloat16*>(wg);
         if (rp.T >= 1024) {
-            if (const cudaError_t e = gate_tiled_smem(); e != cudaSuccess) return e;
-            dim3 grid((rp.T + kGT - 1) / kGT, (rp.E + kGE - 1) / kGE);
-            if (const cudaError_t le = launch_k(gate_logits_tiled_kernel, dim3(grid), dim3(256), kGateTiledSmem,
-                    stream, xp, wp, logit_bias, logits, rp.T, rp.H, rp.E, static_cast<const int32_t*>(nullptr),
-                    static_cast<const int32_t*>(nullptr)); le != cudaSuccess)
+            if (const cudaError_t le = launch_gate_tiled(x, wg, logit_bias, logits, rp.T, rp.H, rp.E, nullptr,
+                    nullptr, stream); le != cudaSuccess)
                 return le;
         } else if (const cudaError_t le = launch_gate_logits(xp, wp, logit_bias, logits, rp.T, rp.H, rp.E, stream);
                    le != cudaSuccess) {
@@ -627,21 +686,25 @@ cudaError_t launch_route(const RouteParams& rp, const void* x, const void* wg, c
     }
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    if ((err = launch_select(logits, select_bias, topk_ids, topk_w, rp, au, nullptr, nullptr,
+    const LogitPlanes whole{1, 0, nullptr};
+    const LogitPlanes parts{rp.gate_tc ? gate_tc_splits(rp.T, rp.H, rp.E) : 1, (int64_t)rp.T * rp.E, logit_bias};
+    if ((err = launch_select(logits, rp.gate_tc ? parts : whole, select_bias, topk_ids, topk_w, rp, au, nullptr, nullptr,
                              (rp.T + kSelWarps - 1) / kSelWarps, stream)) != cudaSuccess || !rp.gate_tc)
         return err;
     // flagged tokens: fixed-order logits, then their choice again (no audit)
     const int32_t* n_flag = reinterpret_cast<const int32_t*>(rs.audit + 1);
-    if ((err = gate_tiled_smem()) != cudaSuccess) return err;
-    const dim3 lgrid((rp.T + kGT - 1) / kGT, (rp.E + kGE - 1) / kGE);  // tiles past the flagged count exit
-    if (const cudaError_t le = launch_k(gate_logits_tiled_kernel, lgrid, dim3(256), kGateTiledSmem, stream,
-            static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(wg), logit_bias, logits, rp.T,
-            rp.H, rp.E, static_cast<const int32_t*>(rs.flagged), n_flag); le != cudaSuccess)
-        return le;
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    const int32_t* flagged = rs.flagged;
+    if ((err = launch_k(gate_logits_list_kernel,
+                        dim3(std::min(rp.T, kListBlocks), (rp.E + 2 * kGateWarps - 1) / (2 * kGateWarps)),
+                        dim3(kGateWarps * 32), 0, stream, static_cast<const __nv_bfloat16*>(x),
+                        static_cast<const __nv_bfloat16*>(wg), logit_bias, logits, rp.T, rp.H, rp.E, flagged,
+                        n_flag)) != cudaSuccess)
+        return err;
+    if ((err = launch_gate_tiled(x, wg, logit_bias, logits, rp.T, rp.H, rp.E, flagged, n_flag, stream)) !=
+        cudaSuccess)
+        return err;
     const GateAudit none{};
-    return launch_select(logits, select_bias, topk_ids, topk_w, rp, none, static_cast<const int32_t*>(rs.flagged), n_flag,
-                         sm_count() * 4, stream);
+    return launch_select(logits, whole, select_bias, topk_ids, topk_w, rp, none, flagged, n_flag, sm_count() * 4, stream);
 }
 
 }  // namespace gbmoe
