@@ -86,8 +86,10 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * largest of the four, exactly down to 2^-14 of it); this too is reported as
  * GBMOE_FFN_TC.
  * Otherwise AUTO streams weights when P/E is at most 16 and otherwise runs the
- * grouped GEMM (tensor cores for bf16 activations, CUDA cores for fp32). On
- * the tensor cores, int4/MXFP4 weights are decoded inside the GEMM when P/E < 256; with
+ * grouped GEMM (tensor cores for bf16 activations, CUDA cores for fp32). (With
+ * bf16 weights and activations AUTO's STREAM and TC run the feature-major
+ * tensor-core GEMM from one row per expert to 40.) On the tensor cores,
+ * int4/MXFP4 weights are decoded inside the GEMM when P/E < 256; with
  * more rows per expert (several M tiles reuse each weight tile) AUTO takes
  * GBMOE_FFN_TC_DEQUANT: one pass decodes the active experts' weights to a
  * bf16 copy in the workspace (the same bf16 values the in-GEMM decode makes),

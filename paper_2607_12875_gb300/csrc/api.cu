@@ -117,6 +117,7 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     probe.H = c->H;
     probe.I = I;
     if (n_rows > kFmRowsPerExpert * E || !ffn_fm_supported(probe)) return false;
+    if (c->w_dtype == GBMOE_BF16 && n_rows < kFmBf16MinRowsPerExpert * E) return false;
     return c->w_dtype == GBMOE_FP8_E4M3_B128 ? pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8
                                              : c->ffn_route == GBMOE_FFN_AUTO && c->combine_route != GBMOE_COMBINE_FUSED;
 }
@@ -163,7 +164,7 @@ struct Layout {
 // its activations (the fp8 route, the feature-major GEMM)
 bool uses_act_codes(const gbmoe_config* c) {
     auto codes = [&](int64_t n_rows, int E, int I) {
-        return use_fm(c, n_rows, E, I) || pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8;
+        return (c->w_dtype != GBMOE_BF16 && use_fm(c, n_rows, E, I)) || pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8;
     };
     return codes((int64_t)c->T * c->top_k, c->E, c->I) || (c->has_shared && codes(c->T, 1, c->I_shared));
 }

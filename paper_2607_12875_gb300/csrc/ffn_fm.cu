@@ -230,6 +230,12 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&a)[8], uint32_t (&b)[8], ui
                  : "memory");
 }
 
+// after the wait for the load: the registers pass through here, so that no use
+// of them moves above the wait (volatile statements keep their order)
+__device__ __forceinline__ void tmem_pin(uint32_t (&a)[8]) {
+    asm volatile("" : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]));
+}
+
 // acc += (a + b) * (sc * w) over 8 rows: a, b the q1 and q2 partial sums, sc
 // the rows' scales in shared memory, w the weight scale in both halves. int4
 // (see the decode warps): acc += (a + b - sum) * (sc * w), the rows' negated
@@ -672,6 +678,245 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
     }
 }
 
+// ------------------------------------------------------------ bf16 weights
+//
+// The same item and the same way of the weights for bf16: 64 k per block, the
+// rows' bf16 values as they are (one plane, gathered from x), kind::f16, and
+// the sums of an item stay in tensor memory over all of K, so nothing is
+// promoted: four warps read a finished slot, apply SwiGLU and store while the
+// next item's MMAs fill another. 32 tokens, top 8 of 128 experts, H 4096, I
+// 1536: gate/up 435 -> 405 us, down 237 -> 213 us against the streaming kernels
+// (6.3 -> 6.8 TB/s).
+
+template <int ROWS>
+struct CfgBf16 {
+    static constexpr int B_BYTES = ROWS * BK;  // (a block's 64 bf16 are BK bytes)
+    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int SLOTS = 4;
+    static constexpr int SLOT_COLS = 2 * ROWS;  // both halves of an item
+    static constexpr int THREADS = 32 * (2 + GATHER_WARPS + 4);
+    static constexpr int MAX_STAGES = 6;
+    static constexpr int FIXED_BYTES = 1024 + (2 * MAX_STAGES + 2 * SLOTS + 1) * 8 + 16;
+    static constexpr int FIT = (SMEM_BUDGET - FIXED_BYTES) / STAGE_BYTES;
+    static constexpr int STAGES = FIT < MAX_STAGES ? FIT : MAX_STAGES;
+    static constexpr int SMEM_BYTES = FIXED_BYTES + STAGES * STAGE_BYTES;
+    static_assert(SLOTS * SLOT_COLS <= TMEM_COLS && ROWS % 16 == 0, "tile");
+};
+
+// kind::f16, fp32 accumulator, bf16 x bf16, K-major, M = 128
+__device__ __forceinline__ uint32_t idesc_bf16(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(MB >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+template <int ROWS, bool SWIGLU>
+__global__ void __launch_bounds__(CfgBf16<ROWS>::THREADS, 1)
+fm_bf16_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant__ CUtensorMap tm_w1, const Params p) {
+    pdl_enter();
+    using C = CfgBf16<ROWS>;
+    constexpr int STAGES = C::STAGES, SLOTS = C::SLOTS;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* sA = smem;
+    uint8_t* sB = smem + STAGES * A_BYTES;
+    uint64_t* full = reinterpret_cast<uint64_t*>(sB + STAGES * C::B_BYTES);  // weights and rows of a k block landed
+    uint64_t* empty = full + STAGES;                                         // MMAs reading the stage finished
+    uint64_t* pfull = empty + STAGES;                                        // an item's sums are complete
+    uint64_t* pempty = pfull + SLOTS;                                        // and read by every epilogue warp
+    uint64_t* drain = pempty + SLOTS;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 32 * GATHER_WARPS + 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < SLOTS; ++b) {
+            mbar_init(&pfull[b], 1);
+            mbar_init(&pempty[b], 4);
+        }
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    const int total = p.sched[1] * p.n_tiles;
+    const int nkb = p.K / (BK / 2);
+    auto pad16 = [](int rows) { return (rows + 15) & ~15; };
+
+    if (warp == 0 && lane == 0) {
+        // ------------------------------------------------ weight producer
+        int stage = 0;
+        uint32_t phase = 0;
+        uint32_t inflight = 0, inflight_par = 0;  // stages loaded but not seen consumed
+        bool ok = true;
+        for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+            const Work wk = decode_work(p, w);
+            int a0, a1;
+            w_rows<SWIGLU>(p, wk, a0, a1);
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                inflight &= ~(1u << stage);
+                uint8_t* dst = sA + stage * A_BYTES;
+                mbar_expect_tx(&full[stage], A_BYTES);
+                tma_load_2d(dst, &tm_w0, kb * (BK / 2), a0, &full[stage]);
+                tma_load_2d(dst + A_BYTES / 2, &tm_w1, kb * (BK / 2), a1, &full[stage]);
+                inflight |= 1u << stage;
+                inflight_par = (inflight_par & ~(1u << stage)) | (phase << stage);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+        }
+        // every copy issued lands before the CTA leaves (after an abort the
+        // phase may lack other arrivals: the copies get the drain limit's time)
+        for (int s = 0; s < STAGES; ++s)
+            if ((inflight >> s) & 1u) drain_wait(&full[s], (inflight_par >> s) & 1u);
+    } else if (warp == 1) {
+        // ------------------------- MMA issuer (the whole warp, one lane issues)
+        int stage = 0;
+        uint32_t phase = 0;
+        uint32_t slot = 0, sphase = 0;
+        bool ok = true, issued = false;
+        const uint64_t da0 = sw128_desc(smem_u32(sA)), db0 = sw128_desc(smem_u32(sB));
+        for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+            const Work wk = decode_work(p, w);
+            const uint32_t idesc = idesc_bf16(__shfl_sync(0xffffffffu, pad16(wk.rows), 0));  // warp-uniform
+            if (!warp_wait(&pempty[slot], sphase ^ 1, abort_flag, p.err, p.wait_limit_ns)) break;
+            tc_fence_after();
+            const uint32_t d = tmem_base + slot * C::SLOT_COLS;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                // the rows were written through the generic proxy (cp.async)
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                const uint64_t db = db0 + (uint64_t)(stage * C::B_BYTES >> 4);
+                const uint64_t da = da0 + (uint64_t)(stage * A_BYTES >> 4);
+                if (elect_one()) {
+#pragma unroll
+                    for (int half = 0; half < 2; ++half)
+#pragma unroll
+                        for (int j = 0; j < BK / 32; ++j)  // 16 k, +32 bytes, per instruction
+                            mma_bf16(d + half * ROWS, da + (uint64_t)(half * (MB * BK) >> 4) + 2 * j, db + 2 * j, idesc,
+                                     (kb | j) != 0 ? 1u : 0u);
+                    mma_commit(&empty[stage]);
+                    if (kb == nkb - 1) mma_commit(&pfull[slot]);
+                }
+                __syncwarp();
+                issued = true;
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+            if (!ok) break;
+            if (++slot == SLOTS) { slot = 0; sphase ^= 1; }
+        }
+        if (issued) {  // every MMA issued has finished before TMEM is released
+            if (elect_one()) mma_commit(drain);
+            __syncwarp();
+            drain_wait(drain, 0);
+        }
+    } else if (warp >= 2 && warp < 2 + GATHER_WARPS) {
+        // --------------------------------------------------- row gather
+        // thread t copies 16-byte chunk t % 8 of rows t / 8 + 8 i
+        const int t = threadIdx.x - 64;
+        const int chunk = t & 7, r0 = t >> 3;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+            const Work wk = decode_work(p, w);
+            const int rp = pad16(wk.rows);
+            const uint8_t* src[ROWS / 8];
+#pragma unroll
+            for (int i = 0; i < ROWS / 8; ++i) {  // (rows past the tile's end: any valid row, never stored)
+                const int j = r0 + 8 * i;
+                int64_t row = 0;
+                if (j < wk.rows) {
+                    row = wk.row0 + j;
+                    if (p.gather) {
+                        const int32_t g = p.gather[row];
+                        row = g >= 0 ? g / p.gather_div : 0;
+                    }
+                }
+                src[i] = p.q + row * p.K * 2 + 16 * chunk;
+            }
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                uint8_t* dst = sB + stage * C::B_BYTES;
+#pragma unroll
+                for (int i = 0; i < ROWS / 8; ++i) {
+                    if (8 * i >= rp) break;
+                    cp_async_16(dst + sw128_off(r0 + 8 * i, chunk), src[i] + kb * BK);
+                }
+                // one arrival of this thread once its copies above have landed
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[stage])) : "memory");
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");  // (after an abort too) copies land before the CTA leaves
+    } else if (warp >= 4) {
+        // -------------------------------------------------------- epilogue
+        const int q = warp & 3;  // TMEM lane quarter
+        const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
+        uint32_t slot = 0, sphase = 0;
+        for (int w = blockIdx.x; w < total; w += gridDim.x) {
+            const Work wk = decode_work(p, w);
+            if (!warp_wait(&pfull[slot], sphase, abort_flag, p.err, p.wait_limit_ns)) break;
+            tc_fence_after();
+            // this thread's weight row is an output column; a warp writes 64 consecutive bytes per row
+            __nv_bfloat16* dst = p.out + wk.row0 * p.out_cols + wk.nt * (SWIGLU ? MB : 2 * MB) + q * 32 + lane;
+            const uint32_t t1 = t_lane + slot * C::SLOT_COLS;
+            for (int j0 = 0; j0 < wk.rows; j0 += 8) {
+                uint32_t a[8], b[8];
+                tmem_ld8(t1 + j0, a);
+                tmem_ld8(t1 + ROWS + j0, b);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tmem_pin(a);
+                tmem_pin(b);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (j0 + i >= wk.rows) break;
+                    __nv_bfloat16* o = dst + (int64_t)(j0 + i) * p.out_cols;
+                    const float v0 = __uint_as_float(a[i]), v1 = __uint_as_float(b[i]);
+                    if constexpr (SWIGLU) {
+                        o[0] = __float2bfloat16_rn(silu_mul(v0, v1));
+                    } else {
+                        o[0] = __float2bfloat16_rn(v0);
+                        o[MB] = __float2bfloat16_rn(v1);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&pempty[slot]);
+            if (++slot == SLOTS) { slot = 0; sphase ^= 1; }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
+                     : "memory");
+    }
+}
+
 // ------------------------------------------------------------------- host
 
 template <int WQ, int ROWS, bool SWIGLU>
@@ -743,16 +988,60 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     return p.n_rows <= 4 * (int64_t)p.E ? launch_ffn<WQ, 16>(p, stream) : launch_ffn<WQ, 80>(p, stream);
 }
 
+template <int ROWS, bool SWIGLU>
+static cudaError_t launch_gemm_bf16(const CUtensorMap& w0, const CUtensorMap& w1, const Params& prm, int64_t max_work,
+                                    cudaStream_t stream) {
+    using C = CfgBf16<ROWS>;
+    static DeviceOnce smem_set;
+    const cudaError_t e = smem_set.run([] {
+        return cudaFuncSetAttribute(fm_bf16_kernel<ROWS, SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    });
+    if (e != cudaSuccess) return e;
+    const int grid = (int)min64(sm_count(), max_work);
+    if (grid <= 0) return cudaSuccess;
+    return launch_k(fm_bf16_kernel<ROWS, SWIGLU>, dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, stream, w0, w1, prm);
+}
+
+template <int ROWS>
+static cudaError_t launch_ffn_bf16(const FfnProblem& p, cudaStream_t stream) {
+    cudaError_t err = launch_ffn_schedule(p.counts, p.E, p.n_rows, ROWS, p.sched, stream);
+    if (err != cudaSuccess) return err;
+    const int64_t max_m = sched_max_tiles(p.E, p.n_rows, ROWS);
+    auto map = [](CUtensorMap* m, const void* base, int64_t rows, int64_t K) {
+        return make_map(m, base, rows, K * 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, BK / 2, CU_TENSOR_MAP_SWIZZLE_128B, MB);
+    };
+    CUtensorMap mg, mu, md;
+    if (!map(&mg, p.w_gate, (int64_t)p.E * p.I, p.H) || !map(&mu, p.w_up, (int64_t)p.E * p.I, p.H) ||
+        !map(&md, p.w_down, (int64_t)p.E * p.H, p.I))
+        return cudaErrorInvalidValue;
+    Params g{};
+    g.K = p.H; g.n_tiles = p.I / MB; g.out_cols = p.I; g.w_rows_per_expert = p.I; g.tile_rows = ROWS;
+    g.counts = p.counts; g.offsets = p.offsets; g.sched = p.sched; g.E = p.E; g.n_rows = p.n_rows;
+    g.out = static_cast<__nv_bfloat16*>(p.h); g.err = p.err;
+    g.q = static_cast<const uint8_t*>(p.x);
+    g.gather = p.sorted_pair; g.gather_div = p.pair_div;
+    g.wait_limit_ns = tc_wait_limit_ns();
+    if ((err = launch_gemm_bf16<ROWS, true>(mg, mu, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
+    Params d = g;
+    d.K = p.I; d.n_tiles = p.H / (2 * MB); d.out_cols = p.H; d.w_rows_per_expert = p.H;
+    d.out = static_cast<__nv_bfloat16*>(p.y);
+    d.q = static_cast<const uint8_t*>(p.h);
+    d.gather = nullptr; d.gather_div = 1;
+    return launch_gemm_bf16<ROWS, false>(md, md, d, max_m * d.n_tiles, stream);
+}
+
 }  // namespace fm
 
 bool ffn_fm_supported(const FfnProblem& p) {
-    const bool wq_ok = p.w_dtype == GBMOE_FP8_E4M3_B128 || p.w_dtype == GBMOE_INT4_G128 || p.w_dtype == GBMOE_MXFP4;
+    const bool wq_ok = p.w_dtype == GBMOE_BF16 || p.w_dtype == GBMOE_FP8_E4M3_B128 || p.w_dtype == GBMOE_INT4_G128 || p.w_dtype == GBMOE_MXFP4;
     return p.act_dtype == GBMOE_BF16 && wq_ok && p.H % 256 == 0 && p.I % 128 == 0 && tc::encode_fn() != nullptr;
 }
 
 cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream) {
     if (p.n_rows == 0) return cudaSuccess;
     switch (p.w_dtype) {
+        case GBMOE_BF16:
+            return p.n_rows <= 4 * (int64_t)p.E ? fm::launch_ffn_bf16<16>(p, stream) : fm::launch_ffn_bf16<64>(p, stream);
         case GBMOE_FP8_E4M3_B128: return fm::launch_ffn<GBMOE_FP8_E4M3_B128>(p, stream);
         case GBMOE_INT4_G128: return fm::launch_ffn<GBMOE_INT4_G128>(p, stream);
         case GBMOE_MXFP4: return fm::launch_ffn<GBMOE_MXFP4>(p, stream);

@@ -87,6 +87,12 @@ struct FfnProblem {
 size_t ffn_sched_ints(int E, int64_t n_rows);
 constexpr int64_t kDequantRowsPerExpert = 256;  // AUTO: TC_DEQUANT from this many rows per expert
 constexpr int64_t kPairRowsPerExpert = 1024;    // AUTO: CTA pairs from this many rows per expert
+// bf16 weights stream on the CUDA cores below this many rows per expert: a
+// weight then meets one row or two, and the streaming CTAs split a few experts'
+// weights finer than the feature-major items (the same layer at 0.06 rows per
+// expert: 71 us streaming against 73, 0.13: 111 against 120, 0.5: 299 against
+// 306).
+constexpr int64_t kFmBf16MinRowsPerExpert = 1;
 cudaError_t launch_ffn_stream(const FfnProblem& p, cudaStream_t stream);
 size_t stream_smem_bytes(int act_dtype, int H, int I);  // per CTA, streaming route
 // dynamic shared memory a CTA may use on sm_103a (227 KB); a streaming problem
@@ -105,6 +111,8 @@ bool ffn_tc_fp8_supported(const FfnProblem& p);
 // 2.67 against 2.66 at 47, 3.40 against 2.79 at 64. MXFP4, the same layer: 2.91
 // against 22.9 ms (streaming) at 8, 3.34 against 3.43 (decode in the GEMM) at
 // 32; int4, 64 experts, H 4096, I 2816: 0.64 against 0.78 ms at 24.
+// bf16 layer, 128 experts, H 4096, I 1536: 0.775 against 0.800 ms (row-major) at
+// 21 rows per expert, 0.62 against 0.70 (streaming) at 2.
 constexpr int64_t kFmRowsPerExpert = 40;
 // rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales;
 // with int4_sums in the order int4 weights take, with the blocks' sums of codes there

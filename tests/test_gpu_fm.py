@@ -29,7 +29,7 @@ def forward(wl, dev):
 # rows per expert: 1, groups of 8 and one more, whole 16-row tiles, the last
 # size with short tiles (4 rows per expert on average) and the first without,
 # the last before the row-major GEMM takes over; one k block and ragged rings
-@pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
+@pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T,E,k,H,I", [(1, 8, 2, 256, 128), (8, 4, 1, 512, 128), (9, 1, 1, 256, 256),
                                        (4, 1, 1, 768, 384), (32, 16, 2, 1024, 128), (33, 16, 2, 256, 640),
                                        (40, 1, 1, 512, 256), (63, 4, 2, 1280, 256)])
@@ -40,7 +40,7 @@ def test_row_tiles(T, E, k, H, I, wq):
     assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol_for(wl))
 
 
-@pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
+@pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T", [16, 17, 80, 81, 200])
 def test_all_rows_on_one_expert(T, wq):
     """A hot expert's rows fill whole row tiles and spill into the next."""
@@ -54,7 +54,7 @@ def test_all_rows_on_one_expert(T, wq):
     assert_close(act_np(forward(wl, to_device(wl, inp))), ref["out"], tol_for(wl))
 
 
-@pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
+@pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
 def test_not_finite_rows_stay_in_their_token(wq):
     """An infinity or NaN in one token's activations leaves every other token's
     output bit for bit as it was; its own output is not finite. Values whose
