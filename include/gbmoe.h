@@ -89,7 +89,7 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * grouped GEMM (tensor cores for bf16 activations, CUDA cores for fp32). (With
  * bf16 weights and activations AUTO's STREAM and TC run the feature-major
  * tensor-core GEMM from one row per expert to 40.) On the tensor cores,
- * int4/MXFP4 weights are decoded inside the GEMM when P/E < 256; with
+ * int4/MXFP4 weights are decoded inside the GEMM when P/E < 400; with
  * more rows per expert (several M tiles reuse each weight tile) AUTO takes
  * GBMOE_FFN_TC_DEQUANT: one pass decodes the active experts' weights to a
  * bf16 copy in the workspace (the same bf16 values the in-GEMM decode makes),
@@ -97,7 +97,8 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * pairs (tcgen05 cta_group::2): one MMA of 256 rows per pair, each CTA
  * holding 128 rows of A and half of the bf16 weight tile, which halves the
  * weight bytes each SM reads per MMA; an expert's rows are then covered in
- * 256-row tiles, so AUTO takes them only from P/E >= 1024 (little padding).
+ * 256-row tiles, so AUTO takes them only from P/E >= 1024 (little padding; from
+ * 400 after a decode-once pass).
  * Their outputs equal the one-CTA routes' bit for bit. TC_PAIR needs bf16
  * weights; quantised weights take TC_PAIR_DEQUANT. */
 enum {

@@ -98,7 +98,8 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
             // CTA pairs (256-row tiles) once experts are deep enough that the
             // padding of their last tile stays small; they multiply bf16 tiles
             if (dequant) probe.w_dq = &probe;
-            const bool pairs = n_rows >= kPairRowsPerExpert * E && ffn_tc_pair_supported(probe);
+            const int64_t from = dequant ? kPairDequantRowsPerExpert : kPairRowsPerExpert;
+            const bool pairs = n_rows >= from * E && ffn_tc_pair_supported(probe);
             if (dequant) return pairs ? GBMOE_FFN_TC_PAIR_DEQUANT : GBMOE_FFN_TC_DEQUANT;
             return pairs && c->w_dtype == GBMOE_BF16 ? GBMOE_FFN_TC_PAIR : GBMOE_FFN_TC;
         }

@@ -85,8 +85,16 @@ struct FfnProblem {
 };
 
 size_t ffn_sched_ints(int E, int64_t n_rows);
-constexpr int64_t kDequantRowsPerExpert = 256;  // AUTO: TC_DEQUANT from this many rows per expert
-constexpr int64_t kPairRowsPerExpert = 1024;    // AUTO: CTA pairs from this many rows per expert
+// AUTO: 4-bit weights are decoded once (TC_DEQUANT) from this many rows per
+// expert on; below, inside the GEMM. int4, 64 experts, H 4096, I 2816: 1.32
+// against 1.85 ms at 192 rows per expert, 2.28 against 2.30 at 384.
+constexpr int64_t kDequantRowsPerExpert = 400;
+// AUTO: CTA pairs from this many rows per expert on. bf16, 128 experts, H 4096,
+// I 1536, pairs against single CTAs: 2.245 and 2.252 ms at 512 rows per expert,
+// 3.93 and 3.99 at 1024; after a decode-once pass 2.30 and 2.35 at 384 (int4
+// as above).
+constexpr int64_t kPairRowsPerExpert = 1024;
+constexpr int64_t kPairDequantRowsPerExpert = 400;
 // bf16 weights stream on the CUDA cores below this many rows per expert: a
 // weight then meets one row or two, and the streaming CTAs split a few experts'
 // weights finer than the feature-major items (the same layer at 0.06 rows per
