@@ -11,13 +11,20 @@ size_t ffn_sched_ints(int E, int64_t n_rows) {
     return (size_t)kSchedHeader + E + (E + 1) + 2 * (size_t)sched_max_tiles(E, n_rows, kSchedMinBM) + 64;
 }
 
-__global__ void __launch_bounds__(512)
-ffn_schedule_kernel(const int32_t* __restrict__ counts, int E, int64_t n_rows, int BM, int32_t* __restrict__ sched) {
+constexpr int kSchedThreads = 544;  // one per expert: up to 512 routed and a shared one
+
+__global__ void __launch_bounds__(kSchedThreads)
+ffn_schedule_kernel(const int32_t* __restrict__ counts, int E, int64_t n_rows, int BM, int64_t n_shared,
+                    int32_t* __restrict__ sched) {
     pdl_enter();
-    __shared__ int32_t s_warp_t[16], s_warp_a[16];
+    __shared__ int32_t s_warp_t[kSchedThreads / 32], s_warp_a[kSchedThreads / 32];
     const int e = threadIdx.x, lane = e & 31, warp = e >> 5;
     int cnt = 0;
     if (e < E) cnt = counts ? counts[e] : (int)n_rows;
+    if (n_shared) {
+        if (e == E) cnt = (int)n_shared;
+        ++E;
+    }
     const int nt = (cnt + BM - 1) / BM;
     const int act = cnt > 0 ? 1 : 0;
     int it = nt, ia = act;
@@ -55,9 +62,9 @@ ffn_schedule_kernel(const int32_t* __restrict__ counts, int E, int64_t n_rows, i
 }
 
 cudaError_t launch_ffn_schedule(const int32_t* counts, int E, int64_t n_rows, int BM, int32_t* sched,
-                                cudaStream_t stream) {
-    if (const cudaError_t le = launch_k(ffn_schedule_kernel, dim3(1), dim3(512), 0, stream, counts, E, n_rows, BM,
-            sched); le != cudaSuccess)
+                                cudaStream_t stream, int64_t n_shared) {
+    if (const cudaError_t le = launch_k(ffn_schedule_kernel, dim3(1), dim3(kSchedThreads), 0, stream, counts, E, n_rows,
+            BM, n_shared, sched); le != cudaSuccess)
         return le;
     return cudaGetLastError();
 }

@@ -17,7 +17,8 @@ __host__ __device__ inline size_t sched_tiles_offset(int E) {
     return (o + 1) & ~(size_t)1;
 }
 
+// n_shared > 0: one more expert (index E) with that many rows after the routed ones; the lists are then those of E + 1
 cudaError_t launch_ffn_schedule(const int32_t* counts, int E, int64_t n_rows, int BM, int32_t* sched,
-                                cudaStream_t stream);
+                                cudaStream_t stream, int64_t n_shared = 0);
 
 }  // namespace gbmoe

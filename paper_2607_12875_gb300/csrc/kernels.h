@@ -70,6 +70,11 @@ struct FfnProblem {
     float* a_s;                 //   and their 1x128 scales [rows, H/128] (int4: then the sums of codes, the same)
     void* h_q;                  //   h the same way, [2, n_rows, I]
     float* h_s;                 //   and its 1x128 scales [n_rows, I/128]
+    // Feature-major GEMM: the shared expert (same I and weight format) as one more
+    // expert of the problem, its n_shared rows (token order) after the routed
+    // ones in h, y and h's codes; 0: none
+    int64_t n_shared;
+    const void *sw_gate, *sw_up, *sw_down, *ss_gate, *ss_up, *ss_down;
     int cta_pair;               // tensor-core routes: 1 = CTA pairs (cta_group::2, 256-row M tiles)
     int32_t* sched;             // schedule ints, ffn_sched_ints(E, n_rows)
     int32_t* err;               // device error word
@@ -112,15 +117,15 @@ bool ffn_tc_supported(const FfnProblem& p);
 bool ffn_tc_pair_supported(const FfnProblem& p);
 cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream);
 bool ffn_tc_fp8_supported(const FfnProblem& p);
-// The feature-major GEMM runs up to this many rows per expert; beyond, its
-// promotion (every row's partial sums, per 128 k) costs more than the 128-row
-// MMAs of the row-major GEMMs. fp8 layer, 256 experts, H 7168, I 2048, both
-// ways: 1.93 against 2.33 ms at 8 rows per expert, 2.30 against 2.50 at 32,
-// 2.67 against 2.66 at 47, 3.40 against 2.79 at 64. MXFP4, the same layer: 2.91
-// against 22.9 ms (streaming) at 8, 3.34 against 3.43 (decode in the GEMM) at
-// 32; int4, 64 experts, H 4096, I 2816: 0.64 against 0.78 ms at 24.
-// bf16 layer, 128 experts, H 4096, I 1536: 0.775 against 0.800 ms (row-major) at
-// 21 rows per expert, 0.62 against 0.70 (streaming) at 2.
+// The feature-major GEMM runs up to this many rows per expert; beyond, the
+// 128-row MMAs of the row-major GEMMs waste less than its second pass over the
+// weights' operand costs. Feature-major against row-major, 256 experts, H 7168,
+// I 2048: fp8 2.14 against 2.48 ms at 32 rows per expert, 2.37 against 2.52 at
+// 47, 2.83 against 2.66 at 64; MXFP4 3.08 against 3.43 (decode in the GEMM) at
+// 32, 3.37 against 3.38 at 47; int4, 64 experts, H 4096, I 2816: 0.59 against
+// 0.78 at 24, 0.78 against 0.78 at 48; bf16, 128 experts, H 4096, I 1536: 0.775
+// against 0.800 at 21, 0.62 against 0.70 (streaming) at 2.
+constexpr int64_t kFmFp8RowsPerExpert = 52;
 constexpr int64_t kFmRowsPerExpert = 40;
 // rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales;
 // with int4_sums in the order int4 weights take, with the blocks' sums of codes there

@@ -27,12 +27,14 @@ def forward(wl, dev):
 
 
 # rows per expert: 1, groups of 8 and one more, whole 16-row tiles, the last
-# size with short tiles (4 rows per expert on average) and the first without,
+# size with the shortest tiles (4 rows per expert on average), 16 and 17 (the next
+# tile height) and the first without,
 # the last before the row-major GEMM takes over; one k block and ragged rings
 @pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T,E,k,H,I", [(1, 8, 2, 256, 128), (8, 4, 1, 512, 128), (9, 1, 1, 256, 256),
                                        (4, 1, 1, 768, 384), (32, 16, 2, 1024, 128), (33, 16, 2, 256, 640),
-                                       (40, 1, 1, 512, 256), (63, 4, 2, 1280, 256)])
+                                       (40, 1, 1, 512, 256), (63, 4, 2, 1280, 256),
+                                       (16, 1, 1, 512, 128), (17, 1, 1, 512, 128), (52, 1, 1, 256, 384), (53, 1, 1, 256, 128)])
 def test_row_tiles(T, E, k, H, I, wq):
     wl = BASE.replace(T=T, E=E, top_k=k, H=H, I=I, wq=wq, seed=T + 7 * E)
     inp = synth.make_inputs(wl)
@@ -41,7 +43,7 @@ def test_row_tiles(T, E, k, H, I, wq):
 
 
 @pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
-@pytest.mark.parametrize("T", [16, 17, 80, 81, 200])
+@pytest.mark.parametrize("T", [16, 17, 32, 33, 80, 81, 200])
 def test_all_rows_on_one_expert(T, wq):
     """A hot expert's rows fill whole row tiles and spill into the next."""
     wl = BASE.replace(T=T, E=16, top_k=2, H=512, I=256, wq=wq, seed=T)
@@ -98,4 +100,22 @@ def test_mxfp4_block_scales_far_apart():
         s = inp["experts"][k]
         inp["experts"][k] = (s.astype(np.int32) - rng.integers(0, 13, s.shape)).astype(np.uint8)
         inp["experts"][k][..., ::8, 1] -= 18
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+
+
+@pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
+@pytest.mark.parametrize("T,I_shared", [(5, 256), (60, 256), (150, 256), (60, 384)])
+def test_shared_expert_with_the_routed_ones(T, I_shared, wq):
+    """The shared expert runs as one more expert of the same launches when its
+    intermediate size is the routed ones', else by itself; 128 routed experts and
+    the shared one fill the schedule's warps unevenly."""
+    wl = BASE.replace(T=T, E=128, top_k=3, H=512, I=256, wq=wq, seed=T, score="sigmoid", routed_scale=2.5, n_group=4,
+                      topk_group=2, has_shared=True, I_shared=I_shared, select_bias_sigma=0.01)
+    inp = synth.make_inputs(wl)
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+
+
+def test_shared_expert_after_512_routed_ones():
+    wl = BASE.replace(T=40, E=512, top_k=4, H=256, I=128, wq="fp8_b128", seed=3, has_shared=True, I_shared=128)
+    inp = synth.make_inputs(wl)
     assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
