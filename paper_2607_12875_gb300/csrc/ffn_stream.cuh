@@ -84,17 +84,31 @@ __device__ __forceinline__ void dot4(const uint8_t* const (&wrow)[4], const void
     }
 }
 
+// Sums of the 4 * NT partial sums over the warp, each the same tree as a
+// butterfly over d = 16 .. 1, but halving the values a lane carries at each step
+// (31 shuffles for 32 values, not 160): lane l returns the sum of value
+// l >> (5 - log2(4 * NT)), value q * NT + r being acc[q][r].
 template <int NT>
-__device__ __forceinline__ void warp_sum(float (&acc)[4][NT]) {
+__device__ __forceinline__ float warp_sums(const float (&acc)[4][NT]) {
+    constexpr int V = 4 * NT;
+    const int lane = threadIdx.x & 31;
+    float v[V];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int i = 0; i < V; ++i) v[i] = acc[i / NT][i % NT];
 #pragma unroll
-        for (int r = 0; r < NT; ++r) {
-            float v = acc[q][r];
+    for (int n = V / 2, d = 16; d >= 1; d >>= 1, n >>= 1) {
+        if (n >= 1) {
+            const bool upper = lane & d;
 #pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-            acc[q][r] = v;
+            for (int i = 0; i < n; ++i) {
+                const float keep = upper ? v[i + n] : v[i], give = upper ? v[i] : v[i + n];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, give, d);
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
         }
+    }
+    return v[0];
 }
 
 // Copies nt activation rows into shared memory: row r is source row
@@ -187,19 +201,16 @@ __device__ __forceinline__ void stream_ffn_cta(const FfnProblem& p, int gpc) {
 #pragma unroll
                     for (int r = 0; r < NT; ++r) acc[q][r] = 0.0f;
                 dot4<TA, WQ, NT>(wrow, srow, xs, K, acc);
-                warp_sum<NT>(acc);
-#pragma unroll
-                for (int r = 0; r < NT; ++r)
-                    if (r == lane && r < nt) {
-                        TA* dst = out + (row0 + p0 + r) * out_cols + col0;
-                        if (STAGE == 1) {
-                            dst[0] = from_f32<TA>(silu_mul(acc[0][r], acc[2][r]));
-                            dst[1] = from_f32<TA>(silu_mul(acc[1][r], acc[3][r]));
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) dst[q] = from_f32<TA>(acc[q][r]);
-                        }
-                    }
+                const float sum = warp_sums<NT>(acc);
+                constexpr int COPIES = 8 / NT;  // lanes that hold the same sum
+                const int value = lane / COPIES, q = value / NT, r = value % NT;
+                TA* dst = out + (row0 + p0 + r) * out_cols + col0;
+                if (STAGE == 1) {  // q 0, 1: gate; the up sums are 16 lanes on
+                    const float up = __shfl_xor_sync(0xffffffffu, sum, 16);
+                    if (q < 2 && r < nt && lane % COPIES == 0) dst[q] = from_f32<TA>(silu_mul(sum, up));
+                } else if (r < nt && lane % COPIES == 0) {
+                    dst[q] = from_f32<TA>(sum);
+                }
             }
         });
     }
