@@ -3,7 +3,7 @@
 // With ~2 rows per expert the layer is bound by reading each active expert's
 // weights once from HBM. Each CTA takes one active expert and a slice of
 // output columns; its warps stream weight rows with 16-byte non-allocating
-// loads (kUnroll chunks of each of its 4 rows in flight per lane: 8 KB per
+// loads (four 16-byte chunks of each of its 4 rows in flight per lane: 8 KB per
 // warp) and dot them against the expert's activation rows, which sit in
 // shared memory. Lane l takes the 16-byte chunks l, l+32, ... of a row, so a
 // warp reads 512 contiguous bytes per row and step. The inner loop reloads
@@ -27,15 +27,20 @@ namespace gbmoe {
 
 constexpr int kStreamWarps = 8;
 constexpr int kNT = 8;      // activation rows per weight pass
-constexpr int kUnroll = 4;  // chunks per row loaded before use
 constexpr int kMaxGroupsPerCta = 4;
 constexpr int kMinWaves = 8;
 
-// CTAs per SM the register budget is set for: two for bf16 weights (the
-// decode path); fp32 and quantised weights hold or decode more per element
-// and get the whole register file
+// CTAs per SM the register budget is set for: two for plain weights; quantised
+// ones decode more per element and get the whole register file
 template <int WQ>
-constexpr int stream_min_blocks() { return WQ == GBMOE_BF16 ? 2 : 1; }
+constexpr int stream_min_blocks() { return WQ == GBMOE_BF16 || WQ == GBMOE_F32 ? 2 : 1; }
+
+// 8-element (or 16-byte) chunks of a row loaded before use. fp32: two of 32 bytes
+// fit 128 registers, so two CTAs share an SM; with four one CTA took it alone
+// (tiny fp32 layer: gate/up 17.2 -> 12.0 us, the passes apart as well, see
+// passes_apart; 4 tokens of 16 experts, H 1024, I 768: layer 56 -> 42 us).
+template <int WQ>
+constexpr int kUnroll = WQ == GBMOE_F32 ? 2 : 4;
 
 // acc[q][r] += W_q . xs[r] for 4 weight rows q (byte pointers wrow, scale rows
 // srow) and NT activation rows r in shared memory (row stride K).
@@ -46,10 +51,11 @@ __device__ __forceinline__ void dot4(const uint8_t* const (&wrow)[4], const void
     const int lane = threadIdx.x & 31;
     const int nchunk = K / F::CE;
     constexpr int CB = F::NV * 16;  // bytes per chunk
-    for (int c0 = lane; c0 < nchunk; c0 += 32 * kUnroll) {
-        uint4 raw[kUnroll][4][F::NV];
+    constexpr int U = kUnroll<WQ>;
+    for (int c0 = lane; c0 < nchunk; c0 += 32 * U) {
+        uint4 raw[U][4][F::NV];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int c = c0 + 32 * u;
 #pragma unroll
             for (int q = 0; q < 4; ++q)
@@ -58,7 +64,7 @@ __device__ __forceinline__ void dot4(const uint8_t* const (&wrow)[4], const void
                     raw[u][q][v] = c < nchunk ? ld_stream16(wrow[q] + (size_t)c * CB + 16 * v) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int c = c0 + 32 * u;
             if (c >= nchunk) break;
             float sc[4];
@@ -181,7 +187,7 @@ __device__ __forceinline__ void stream_ffn_cta(const FfnProblem& p, int gpc) {
     const int K = STAGE == 1 ? p.H : p.I;
     TA* out = static_cast<TA*>(STAGE == 1 ? p.h : p.y);
     const int out_cols = STAGE == 1 ? p.I : p.H;
-    for (int64_t p0 = 0; p0 < cnt; p0 += kNT) {
+    for (int64_t p0 = (int64_t)blockIdx.z * kNT; p0 < cnt; p0 += (int64_t)gridDim.z * kNT) {
         const int nt = (int)min64(kNT, cnt - p0);
         __syncthreads();
         if (STAGE == 1) stage_rows<TA>(xs, static_cast<const TA*>(p.x), K, p.sorted_pair, p.pair_div, row0 + p0, nt);
@@ -240,6 +246,16 @@ inline int groups_per_cta(int max_active, int groups) {
     return gpc;
 }
 
+// Passes of kNT rows that run side by side, in CTAs of their own: as many as an
+// expert has on average, while the grid does not fill the SMs (the weights of
+// such a grid stay in L2, so reading them again costs less than waiting).
+inline int passes_apart(int64_t n_rows, int max_active, int ctas) {
+    const int64_t avg = (n_rows + (int64_t)max_active * kNT - 1) / ((int64_t)max_active * kNT);
+    int z = 1;
+    while (2 * z <= avg && (int64_t)ctas * z < (int64_t)sm_count() * 2) z *= 2;
+    return z;
+}
+
 template <typename TA, int WQ>
 static cudaError_t launch_stream_t(const FfnProblem& p, cudaStream_t stream) {
     const int max_active = (int)min64(p.E, p.n_rows);
@@ -260,11 +276,13 @@ static cudaError_t launch_stream_t(const FfnProblem& p, cudaStream_t stream) {
     const int groups1 = p.I / (2 * kStreamWarps), groups2 = p.H / (4 * kStreamWarps);
     const int gpc1 = groups_per_cta(max_active, groups1), gpc2 = groups_per_cta(max_active, groups2);
     dim3 g1(max_active, groups1 / gpc1);
+    g1.z = passes_apart(p.n_rows, max_active, g1.x * g1.y);
     if (const cudaError_t le = launch_k(stream_gateup_kernel<TA, WQ>, dim3(g1), dim3(kStreamWarps * 32), smem1,
             stream, p, gpc1); le != cudaSuccess)
         return le;
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     dim3 g2(max_active, groups2 / gpc2);
+    g2.z = passes_apart(p.n_rows, max_active, g2.x * g2.y);
     if (const cudaError_t le = launch_k(stream_down_kernel<TA, WQ>, dim3(g2), dim3(kStreamWarps * 32), smem2,
             stream, p, gpc2); le != cudaSuccess)
         return le;
