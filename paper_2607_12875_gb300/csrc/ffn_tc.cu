@@ -95,7 +95,6 @@ struct Cfg {
     // thread per row; 10 warps keep a thread's 168 registers)
     static constexpr bool GATHER = WQ == GBMOE_BF16 && CG == 1;
     static constexpr int GATHER_WARPS = GATHER ? BM / 32 : 0;
-    static constexpr int GATHER_AHEAD = 2;  // k blocks a gather warp keeps in flight before signalling
     static constexpr int THREADS = 192 + CONVERT_WARPS * 32 + GATHER_WARPS * 32;
     static constexpr int STAGES = CG == 1 ? (WQ == GBMOE_FP8_E4M3_B128 ? 3 : 4) : (RAW ? 5 : 6);
 };
@@ -428,7 +427,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (threadIdx.x == 0) {
         const bool gathering = C::GATHER && p.a_gather != nullptr;
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], gathering ? 1 + C::GATHER_WARPS : 1);  // + one arrival per gather warp
+            mbar_init(&full[s], gathering ? 1 + 32 * C::GATHER_WARPS : 1);  // + one arrival per gather thread
             mbar_init(&empty[s], 1);
             mbar_init(&conv[s], C::CONVERT_WARPS ? C::CONVERT_WARPS : 1);
         }
@@ -538,6 +537,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 if (RAW && !warp_wait(&conv[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                // gathered rows were written through the generic proxy (cp.async)
+                if (C::GATHER && p.a_gather != nullptr) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 tc_fence_after();
                 const uint64_t da = da0 + (uint64_t)(stage * A_BYTES >> 4);
                 const uint64_t db = db0 + (uint64_t)(stage * BH >> 4);
@@ -718,15 +719,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         // warp g copies A rows 32g .. 32g+31 of each k block (64 bf16 = 128
         // bytes a row) from their x rows into the 128-byte-swizzled slot, four
         // whole rows per instruction (lane l: row 4i + l/8, 16-byte chunk l%8);
-        // a warp signals a slot once its copies of it landed (GATHER_AHEAD k
-        // blocks later), after a proxy fence that makes them visible to the MMAs
-        constexpr int D = C::GATHER_AHEAD;
-        static_assert(!C::GATHER || D < STAGES, "a gather warp must signal a slot before it needs that slot again");
+        // each thread's arrival follows when its copies have landed, so the
+        // warp goes on to the next free slot at once (waiting for the copies
+        // here held a slot's signal back by two k blocks)
         const int row_base = (warp - 6 - C::CONVERT_WARPS) * 32 + (lane >> 3);
         const int chunk = lane & 7;
         int stage = 0;
         uint32_t phase = 0;
-        int64_t issued = 0;
         bool ok = true;
         for (int w = unit; w < total && ok; w += n_units) {
             const Work wk = decode_work<CG>(p, w, rank);
@@ -746,23 +745,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 uint8_t* dst = sA + stage * A_BYTES;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) cp_async_16(dst + sw128_off(row_base + 4 * i, chunk), src[i] + kb * BK);
-                asm volatile("cp.async.commit_group;" ::: "memory");
-                if (++issued > D) {  // the k block D back has landed: signal its slot
-                    asm volatile("cp.async.wait_group %0;" ::"n"(D) : "memory");
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&full[(stage + STAGES - D) % STAGES]);
-                }
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[stage])) : "memory");
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }
-        // the last k blocks' copies land before the CTA leaves; after a normal
-        // run their slots are signalled too
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (ok && lane == 0)
-            for (int64_t i = issued > D ? issued - D : 0; i < issued; ++i) mbar_arrive(&full[i % STAGES]);
+        asm volatile("cp.async.wait_all;" ::: "memory");  // (after an abort too) copies land before the CTA leaves
     }
     tc_fence_before();
     __syncthreads();
