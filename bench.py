@@ -266,7 +266,7 @@ def launches_per_step(wl, route: str, shared_route) -> int:
     combine."""
     def ffn(r, routed):
         rows, experts = (wl.P, wl.E) if routed else (wl.T, 1)
-        few = wl.act == "bf16" and wl.wq in ("int4_g128", "mxfp4") and rows <= 40 * experts
+        few = wl.act == "bf16" and rows <= {"int4_g128": 40, "mxfp4": 60}.get(wl.wq, 0) * experts
         if r == "tc_fp8" or (r == "tc" and few):  # schedule, x codes, gate/up GEMM, h codes, down GEMM
             return 5
         # the one-CTA bf16 GEMM gathers its own rows; decoding GEMMs and pairs use the gather kernel

@@ -79,12 +79,11 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * scaled by both blocks' scales and accumulated in fp32. AUTO takes it for
  * fp8 weights with bf16 activations at every size (with few rows per expert
  * the weights are the GEMM's M operand, with many the rows are).
- * int4/MXFP4 weights with bf16 activations and at most 40 rows per expert
- * (P/E) multiply the same activation codes on the fp8 tensor cores under AUTO
- * (every int4 value and FP4 value is an e4m3 value; group scales are applied
- * in fp32, and the E8M0 scales of a row's 128 consecutive k relative to the
- * largest of the four, exactly down to 2^-14 of it); this too is reported as
- * GBMOE_FFN_TC.
+ * int4 (MXFP4) weights with bf16 activations and at most 40 (60) rows per
+ * expert (P/E) multiply the same activation codes on the fp8 tensor cores under
+ * AUTO: every int4 and FP4 value is an e4m3 value; int4's group scales are
+ * applied in fp32 per 128 k, the E8M0 scales by the MMAs (kind::mxf8f6f4).
+ * This too is reported as GBMOE_FFN_TC.
  * Otherwise AUTO streams weights when P/E is at most 16 and otherwise runs the
  * grouped GEMM (tensor cores for bf16 activations, CUDA cores for fp32). (With
  * bf16 weights and activations AUTO's STREAM and TC run the feature-major

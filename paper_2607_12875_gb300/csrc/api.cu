@@ -73,6 +73,13 @@ int check_cfg(const gbmoe_config* c) {
 
 bool stream_fits(int act_dtype, int H, int I) { return stream_smem_bytes(act_dtype, H, I) <= stream_smem_budget(); }
 
+// most rows per expert of the feature-major GEMM
+int64_t fm_rows_per_expert(int w_dtype) {
+    return w_dtype == GBMOE_FP8_E4M3_B128 ? kFmFp8RowsPerExpert
+           : w_dtype == GBMOE_MXFP4       ? kFmMxfp4RowsPerExpert
+                                          : kFmRowsPerExpert;
+}
+
 // Kernel route for an FFN problem with n_rows rows over E experts.
 int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     int r = c->ffn_route;
@@ -89,7 +96,7 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     // int4 and MXFP4 weights with bf16 activations and few rows per expert: the
     // feature-major GEMM (use_fm), reported as TC
     const bool four_bit = c->w_dtype == GBMOE_INT4_G128 || c->w_dtype == GBMOE_MXFP4;
-    if (four_bit && c->combine_route != GBMOE_COMBINE_FUSED && n_rows <= kFmRowsPerExpert * E && ffn_fm_supported(probe))
+    if (four_bit && c->combine_route != GBMOE_COMBINE_FUSED && n_rows <= fm_rows_per_expert(c->w_dtype) * E && ffn_fm_supported(probe))
         return GBMOE_FFN_TC;
     if (n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I)) return GBMOE_FFN_STREAM;
     if (c->act_dtype == GBMOE_BF16) {
@@ -117,8 +124,7 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     probe.w_dtype = c->w_dtype;
     probe.H = c->H;
     probe.I = I;
-    const int64_t most = c->w_dtype == GBMOE_FP8_E4M3_B128 ? kFmFp8RowsPerExpert : kFmRowsPerExpert;
-    if (n_rows > most * E || !ffn_fm_supported(probe)) return false;
+    if (n_rows > fm_rows_per_expert(c->w_dtype) * E || !ffn_fm_supported(probe)) return false;
     if (c->w_dtype == GBMOE_BF16 && n_rows < kFmBf16MinRowsPerExpert * E) return false;
     return c->w_dtype == GBMOE_FP8_E4M3_B128 ? pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8
                                              : c->ffn_route == GBMOE_FFN_AUTO && c->combine_route != GBMOE_COMBINE_FUSED;
@@ -129,7 +135,8 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
 // the same intermediate size and few tokens (its own launches leave most SMs
 // idle; many rows are cheaper on the row-major GEMM). 256 experts, H 7168, I
 // 2048, joined against apart: fp8 1.30 against 1.35 ms at 48 tokens, 2.20
-// against 2.15 at 1024; MXFP4 0.82 against 0.87 at 16, 3.34 against 3.08 at 1024.
+// against 2.15 at 1024 (MXFP4, before its MMAs scaled by themselves: 0.82
+// against 0.87 at 16, 3.34 against 3.08 at 1024).
 constexpr int kJoinTokens = 512;
 bool shared_joins(const gbmoe_config* c) {
     return c->has_shared && c->I_shared == c->I && c->w_dtype != GBMOE_BF16 && c->T <= kJoinTokens &&

@@ -42,13 +42,12 @@
 // us against the streaming kernels, 7.5 TB/s; the layer 3121 -> 1347 us. What
 // held it back on the way, per 128-wide k block: waits as calls (2400 -> 1750
 // cycles once inlined) and MMAs issued under `lane == 0` (1750 -> 1500).
-// int4, 17 tokens, top 6 of 64 experts, H 4096, I 2816: layer 1397 -> 255 us;
-// MXFP4, 16 tokens of the fp8 layer: 2896 -> 956 us. These two are bound by the
-// decode warps' instructions (1700 cycles per k block for MXFP4, where HBM
-// would allow 735): eight of them instead of four took the gate/up kernel from
-// 681 to 504 us, both partial sums in one handshake included.
-#include <cuda_fp8.h>
-
+// int4, 17 tokens, top 6 of 64 experts, H 4096, I 2816: layer 1397 -> 220 us.
+// MXFP4, 16 tokens of the fp8 layer: 2896 -> 635 us. Its E8M0 scales go to the
+// MMAs (kind::mxf8f6f4), so the decode is shifts and masks; scaling the codes in
+// the decode warps, relative to the largest scale of a row's 128 k, cost twice
+// the instructions and bound the kernel (819 us, and 3.08 against 2.61 ms at
+// 1024 tokens).
 #include "common.cuh"
 #include "ffn_sched.h"
 #include "kernels.h"
@@ -64,7 +63,6 @@ constexpr int BK = 128;                 // k per block: one swizzle row, one act
 constexpr int A_BYTES = 2 * MB * BK;    // the two 128-row halves of an item's weight tile
 constexpr int TMEM_COLS = 512;
 constexpr int GATHER_WARPS = 2;
-constexpr int LUT_ENTRIES = 256;
 constexpr int SMEM_BUDGET = 232448;
 
 // Per weight format and height of a row tile.
@@ -78,24 +76,29 @@ struct Cfg {
     // half of the item has two slots and a set of warps of its own, and the sets
     // meet once per item (X_COL: where the up half hands its sums over).
     static constexpr bool JOINT = ROWS <= 32;
-    static constexpr int SLOTS = 4;
+    static constexpr int SLOTS = WQ == GBMOE_MXFP4 && ROWS == 32 ? 3 : 4;  // (MXFP4's scales need columns too)
     static constexpr int SLOT_COLS = JOINT ? 4 * ROWS : ROWS;
     static constexpr int X_COL = SLOTS * SLOT_COLS;
+    // MXFP4: the MMAs' scale factors in TMEM. Ones for the rows (8 columns), then
+    // two k blocks' weight scales, 4 columns per 128-row half.
+    static constexpr bool BLOCK_SCALE = WQ == GBMOE_MXFP4;
+    static constexpr int SF_COL = X_COL + (JOINT ? 0 : ROWS);
+    static constexpr int SF_COLS = BLOCK_SCALE ? 8 + 16 : 0;
+    static constexpr int SF_BYTES = BLOCK_SCALE ? 2 * 512 : 0;  // a stage's weight scales in shared memory
     static constexpr int SETS = JOINT ? 1 : 2;  // of four promotion warps
     static constexpr int PROMOTE_WARPS = 4 * SETS;
     static constexpr int GROUPS = ROWS / 8;  // most groups of 8 rows
     static constexpr int HALVES_HELD = JOINT ? 2 : 1;  // halves whose sums a promotion warp holds
     static constexpr int DECODE_WARPS = RAW ? (JOINT ? 8 : 4) : 0;
     static constexpr int THREADS = 32 * (2 + GATHER_WARPS + PROMOTE_WARPS + DECODE_WARPS);
-    static constexpr int STAGE_BYTES = A_BYTES + RAW + 2 * ROWS * BK;
+    static constexpr int STAGE_BYTES = A_BYTES + RAW + SF_BYTES + 2 * ROWS * BK;
     // floats of a scale block: the rows' scales and negated sums of codes, then
-    // (formats that are decoded) the weight rows' scales
-    static constexpr int RING_FLOATS = 2 * ROWS + (RAW ? 2 * MB : 0);
-    static constexpr int LUT_BYTES = WQ == GBMOE_MXFP4 ? LUT_ENTRIES * 8 : 0;
+    // (int4) the weight rows' scales
+    static constexpr int RING_FLOATS = 2 * ROWS + (WQ == GBMOE_INT4_G128 ? 2 * MB : 0);
     static constexpr int MAX_STAGES = 6;
     static constexpr int MAX_RING = MAX_STAGES + 4;
     static constexpr int NUM_BARS = 3 * MAX_STAGES + 2 * SLOTS + MAX_RING + 1 + 8;
-    static constexpr int FIXED_BYTES = 1024 + MAX_RING * RING_FLOATS * 4 + LUT_BYTES + NUM_BARS * 8 + 16;
+    static constexpr int FIXED_BYTES = 1024 + MAX_RING * RING_FLOATS * 4 + NUM_BARS * 8 + 16;
     static constexpr int FIT = (SMEM_BUDGET - FIXED_BYTES) / STAGE_BYTES;
     static constexpr int STAGES = FIT < MAX_STAGES ? FIT : MAX_STAGES;
     // Scale blocks, used in turn: k block k's is written once the MMAs of
@@ -105,7 +108,7 @@ struct Cfg {
     static constexpr int AHEAD = JOINT ? SLOTS : 2;
     static constexpr int RING = STAGES + AHEAD;
     static constexpr int SMEM_BYTES = FIXED_BYTES + STAGES * STAGE_BYTES;
-    static_assert(STAGES >= 3 && AHEAD <= 4 && SLOTS * SLOT_COLS + (JOINT ? 0 : ROWS) <= TMEM_COLS, "ring depth");
+    static_assert(STAGES >= 3 && AHEAD <= 4 && SF_COL + SF_COLS <= TMEM_COLS, "ring depth");
     static_assert(ROWS % 16 == 0 && ROWS <= 128, "two rows' scales per gather thread");
 };
 
@@ -218,6 +221,31 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return r;
 }
 
+// kind::mxf8f6f4: the same with E8M0 scales per 32 k of each operand row (bit
+// 23). A k step's scale is byte j (bits 29-30 for A; B's are all ones) of the
+// row's 32-bit word in TMEM.
+__device__ __forceinline__ uint32_t idesc_mxf8(int n) {
+    return (1u << 23) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(MB >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_mxf8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t sfa, uint32_t sfb,
+                                         uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb)
+        : "memory");
+}
+
+// 128 rows' scale words to 4 TMEM columns: 512 bytes of shared memory, 16 per
+// lane l, words 0..3 of it being rows l, 32 + l, 64 + l, 96 + l; every 32-lane
+// quarter of TMEM receives them.
+__device__ __forceinline__ void tmem_copy_scales(uint32_t taddr, uint32_t saddr) {
+    const uint64_t desc = (uint64_t)((saddr & 0x3FFFFu) >> 4) | (uint64_t)(128 >> 4) << 32 | (uint64_t)1 << 46;
+    asm volatile("tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;" ::"r"(taddr), "l"(desc) : "memory");
+}
+
 // 8 columns of this thread's TMEM lane, not waited for
 __device__ __forceinline__ void tmem_ld8(uint32_t t, uint32_t (&a)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -319,18 +347,15 @@ __device__ __forceinline__ void decode_int4_32(const uint4 raw, uint4& o0, uint4
     o1 = make_uint4(even(raw.z), even(raw.z >> 4), even(raw.w), even(raw.w >> 4));
 }
 
-// 16 bytes of MXFP4 weights -> 32 e4m3 codes in order: PRMT picks the
-// magnitudes of four nibbles at a time out of the block's 8-entry table, and
-// the sign from its sign-replicating mode (0x80 gives 0x80 or 0xff).
-__device__ __forceinline__ void decode_mxfp4_32(const uint4 raw, uint2 lut, uint4& o0, uint4& o1) {
-    auto four = [&](uint32_t w) {
-        uint32_t sign;  // (__byte_perm has no sign-replicating mode)
-        asm("prmt.b32 %0, %1, %1, %2;" : "=r"(sign) : "r"(0x80808080u), "r"(w));
-        sign <<= 7;
-        return __byte_perm(lut.x, lut.y, w & 0x7777u) | (sign & 0x80808080u);
-    };
-    o0 = make_uint4(four(raw.x), four(raw.x >> 16), four(raw.y), four(raw.y >> 16));
-    o1 = make_uint4(four(raw.z), four(raw.z >> 16), four(raw.w), four(raw.w >> 16));
+// 16 bytes of MXFP4 weights -> 32 e4m3 codes in the order of int4's. The
+// exponent and mantissa bits eem of an E2M1 code, put into bits 2-4 of a byte,
+// read as e4m3 as the value times 2^-6 (0.5 as a subnormal too), so shifts and
+// masks decode 8 values with their signs.
+__device__ __forceinline__ void decode_mxfp4_32(const uint4 raw, uint4& o0, uint4& o1) {
+    auto even = [](uint32_t w) { return ((w << 2) & 0x1c1c1c1cu) | ((w << 4) & 0x80808080u); };
+    auto odd = [](uint32_t w) { return ((w >> 2) & 0x1c1c1c1cu) | (w & 0x80808080u); };
+    o0 = make_uint4(even(raw.x), odd(raw.x), even(raw.y), odd(raw.y));
+    o1 = make_uint4(even(raw.z), odd(raw.z), even(raw.w), odd(raw.w));
 }
 
 // 16-byte chunk c (0..3) of row r of a 64-byte-swizzled tile
@@ -351,9 +376,9 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
     uint8_t* sA = smem;
     uint8_t* sR = smem + STAGES * A_BYTES;        // int4, MXFP4: tiles as stored
     uint8_t* sB = sR + STAGES * RAW;
-    float* sS = reinterpret_cast<float*>(sB + STAGES * B_BYTES);  // [RING] scale blocks
-    uint2* sLut = reinterpret_cast<uint2*>(sS + RING * C::RING_FLOATS);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(sLut) + C::LUT_BYTES);
+    uint8_t* sF = sB + STAGES * B_BYTES;          // MXFP4: weight scales
+    float* sS = reinterpret_cast<float*>(sF + STAGES * C::SF_BYTES);  // [RING] scale blocks
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sS + RING * C::RING_FLOATS);
     uint64_t* full = bars;              // weights (decoded) and row codes of a k block are in place
     uint64_t* rfull = full + STAGES;    // int4, MXFP4: weights landed as stored
     uint64_t* empty = rfull + STAGES;   // MMAs reading the stage finished
@@ -386,20 +411,6 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (WQ == GBMOE_MXFP4) {
-        // entry d: the magnitudes 0, .5, 1, 1.5, 2, 3, 4, 6 times 2^(6 - d) as
-        // e4m3 (exact for d <= 14, nothing left from d = 20)
-        for (int d = threadIdx.x; d < LUT_ENTRIES; d += C::THREADS) {
-            const float mag[8] = {0.0f, 0.5f, 1.0f, 1.5f, 2.0f, 3.0f, 4.0f, 6.0f};
-            const float f = d < 32 ? __uint_as_float((uint32_t)(127 + 6 - d) << 23) : 0.0f;
-            uint32_t v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                v[i] = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(mag[2 * i] * f, mag[2 * i + 1] * f),
-                                                          __NV_SATFINITE, __NV_E4M3);
-            sLut[d] = make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
-        }
-    }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(TMEM_COLS)
@@ -410,6 +421,18 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    if constexpr (C::BLOCK_SCALE) {  // the rows' scale factors: ones (E8M0 127)
+        if (warp >= 4 && warp < 8) {
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(
+                             tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + C::SF_COL),
+                         "r"(0x7f7f7f7fu)
+                         : "memory");
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        }
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+    }
 
     const int total = p.sched[1] * p.n_tiles;
     const int nkb = p.K / BK;
@@ -458,7 +481,8 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
         for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
             const Work wk = decode_work(p, w);
             const int rp = __shfl_sync(0xffffffffu, rows_pad<C::JOINT>(wk.rows), 0);  // warp-uniform
-            const uint32_t idesc = idesc_f8(C::JOINT ? 2 * rp : rp);
+            const int n = C::JOINT ? 2 * rp : rp;
+            const uint32_t idesc = C::BLOCK_SCALE ? idesc_mxf8(n) : idesc_f8(n);
             for (int kb = 0; kb < nkb; ++kb, ++kc) {
                 if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 // the row codes were written through the generic proxy (cp.async)
@@ -475,14 +499,20 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                     }
                     const uint32_t d = tmem_base + slot * C::SLOT_COLS + (C::JOINT ? half * 2 * ROWS : 0);
                     const uint64_t dh = da0 + (uint64_t)((stage * A_BYTES + half * (MB * BK)) >> 4);
+                    const uint32_t sfb = tmem_base + C::SF_COL, sfa = sfb + 8 + (kc & 1) * 8 + half * 4;
                     if (elect_one()) {
+                        if constexpr (C::BLOCK_SCALE)  // (copies and MMAs run in the order of their issue)
+                            tmem_copy_scales(sfa, smem_u32(sF + stage * C::SF_BYTES + half * 512));
 #pragma unroll
-                        for (int j = 0; j < BK / 32; ++j)  // +32 bytes along K per instruction
-                            mma_f8(d, dh + 2 * j, db + 2 * j, idesc, j != 0 ? 1u : 0u);
-                        if (!C::JOINT) {
+                        for (int pass = 0; pass < (C::JOINT ? 1 : 2); ++pass)
 #pragma unroll
-                            for (int j = 0; j < BK / 32; ++j) mma_f8(d, dh + 2 * j, db2 + 2 * j, idesc, 1u);
-                        }
+                            for (int j = 0; j < BK / 32; ++j) {  // +32 bytes along K per instruction
+                                const uint32_t accumulate = pass + j != 0 ? 1u : 0u;
+                                const uint64_t bj = (pass ? db2 : db) + 2 * j;
+                                if constexpr (C::BLOCK_SCALE)
+                                    mma_mxf8(d, dh + 2 * j, bj, idesc | (uint32_t)j << 29, sfa, sfb, accumulate);
+                                else mma_f8(d, dh + 2 * j, bj, idesc, accumulate);
+                            }
                         if (half == 1 || !C::JOINT) mma_commit(&pfull[slot]);
                         if (half == 1) mma_commit(&empty[stage]);
                     }
@@ -583,7 +613,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             for (int h = 0; h < C::HALVES_HELD; ++h) {
 #pragma unroll
                 for (int i = 0; i < 4 * GROUPS; ++i) acc[h][i] = 0;
-                wn[h] = RAW ? 0.0f : ws[h][0];
+                wn[h] = RAW ? 64.0f : ws[h][0];  // (MXFP4's codes are the values times 2^-6, the MMAs scale)
             }
             bool ok = true;
             for (int kb = 0; kb < nkb; ++kb, ++kc) {
@@ -604,8 +634,8 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 tc_fence_after();
 #pragma unroll
                 for (int h = 0; h < C::HALVES_HELD; ++h) {
-                    // decoded formats: one weight scale per row
-                    if (RAW) wsc[h] = sc[2 * ROWS + (C::JOINT ? h : set) * MB + q * 32 + lane];
+                    // int4: one weight scale per row
+                    if (WQ == GBMOE_INT4_G128) wsc[h] = sc[2 * ROWS + (C::JOINT ? h : set) * MB + q * 32 + lane];
                     const uint64_t w2 = pack2(wsc[h], wsc[h]);
                     const uint32_t t1 = t_lane + slot * C::SLOT_COLS + h * 2 * ROWS, t2 = t1 + rp;
                     // (straight-line code per number of groups: nothing may come between loads and wait)
@@ -701,9 +731,8 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             // ------------------------------- weight decode, weight rows' scales
             // A thread owns row r of one half (eight decode warps) or of both:
             // it decodes the row's 128 values of a k block and writes their
-            // scale to the scale block. MXFP4: the block's four E8M0 scales
-            // (one per 32) differ by small powers of two, which go into the
-            // codes relative to the largest of the four.
+            // scale to the scale block (int4) or its four E8M0 scales to where
+            // the MMA issuer copies them to TMEM from (MXFP4).
             if constexpr (!C::JOINT) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
             constexpr int HALVES = C::DECODE_WARPS == 8 ? 1 : 2;
             const int t = threadIdx.x - 32 * (4 + C::PROMOTE_WARPS);
@@ -736,30 +765,23 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                         if (kb + 1 < nkb) next[i] = scale_bits(i, kb + 1);
                     }
                     if (!warp_wait(&rfull[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                    float* sc = sS + ring * C::RING_FLOATS + 2 * ROWS;
+                    float* sc = sS + ring * C::RING_FLOATS + 2 * ROWS;  // (int4)
 #pragma unroll
                     for (int i = 0; i < HALVES; ++i) {
                         const int h = h0 + i;
                         const uint8_t* raw = sR + stage * RAW + h * (RAW / 2);
                         uint8_t* dst = sA + stage * A_BYTES + h * (A_BYTES / 2);
-                        uint32_t below = 0;  // MXFP4: log2 of the largest scale over each block's, a byte each
-                        if constexpr (WQ == GBMOE_INT4_G128) {
+                        if constexpr (WQ == GBMOE_INT4_G128)
                             sc[h * MB + r] = __uint_as_float(bits[i] << 16) * 512.0f;  // bf16; the codes are u * 2^-9
-                        } else {
-                            const uint32_t b = bits[i];
-                            const uint32_t top = max(max(b & 0xffu, (b >> 8) & 0xffu), max((b >> 16) & 0xffu, b >> 24));
-                            below = top * 0x01010101u - b;
-                            // 2^(top - 127) * 2^-6 (the table's factor); 255 is NaN
-                            float f = __uint_as_float((top - 6u) << 23);
-                            if (top - 7u >= 248u) f = e8m0_to_f32(top) * 0.015625f;
-                            sc[h * MB + r] = f;
-                        }
+                        else
+                            *reinterpret_cast<uint32_t*>(sF + stage * C::SF_BYTES + h * 512 + 16 * (r & 31) + 4 * (r >> 5)) =
+                                bits[i];
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             const uint4 v = *reinterpret_cast<const uint4*>(raw + sw64_off(r, c));
                             uint4 o0, o1;
                             if constexpr (WQ == GBMOE_INT4_G128) decode_int4_32(v, o0, o1);
-                            else decode_mxfp4_32(v, sLut[(below >> (8 * c)) & 0xffu], o0, o1);
+                            else decode_mxfp4_32(v, o0, o1);
                             *reinterpret_cast<uint4*>(dst + sw128_off(r, 2 * c)) = o0;
                             *reinterpret_cast<uint4*>(dst + sw128_off(r, 2 * c + 1)) = o1;
                         }
@@ -1058,10 +1080,11 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     const int64_t rows = p.n_rows + p.n_shared;
     // every row of x once (the shared expert's rows are x's own; a routed row is a token's)
     const int64_t x_rows = p.n_rows / p.pair_div;
+    constexpr bool kFour = WQ != GBMOE_FP8_E4M3_B128;  // the order 4-bit weights are decoded in
     constexpr bool kSums = WQ == GBMOE_INT4_G128;
     float* a_sum = kSums ? p.a_s + x_rows * (p.H / BK) : nullptr;
     float* h_sum = kSums ? p.h_s + rows * (p.I / BK) : nullptr;
-    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, a_sum, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, kFour, a_sum, stream)) != cudaSuccess) return err;
     const int64_t max_m = sched_max_tiles(experts, rows, tile);
     CUtensorMap mg, mu, md, sg, su, sd;
     if (!map_weights(&mg, WQ, p.w_gate, (int64_t)p.E * p.I, p.H) ||
@@ -1084,7 +1107,7 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     g.scale_words = words(p.s_gate) && words(p.s_up) && words(p.ss_gate) && words(p.ss_up);
     g.wait_limit_ns = tc_wait_limit_ns();
     if ((err = launch_gemm<WQ, ROWS, true>(mg, mu, sg, su, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
-    if ((err = launch_quant_rows(p.h, nullptr, 1, rows, p.I, p.h_q, p.h_s, h_sum, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.h, nullptr, 1, rows, p.I, p.h_q, p.h_s, kFour, h_sum, stream)) != cudaSuccess) return err;
     Params d = g;
     d.K = p.I; d.n_tiles = p.H / (2 * MB); d.out_cols = p.H; d.w_rows_per_expert = p.H;
     d.out = static_cast<__nv_bfloat16*>(p.y);

@@ -24,9 +24,9 @@ __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
     return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3);
 }
 
-// kInt4: the order and the sums that int4 weights are multiplied in (ffn_fm.cu):
-// within 8 consecutive values the even ones come before the odd ones, and
-// sums[n_rows][K/128] receive the blocks' sum of codes, sum(q1 + q2) / 64.
+// kFourBit: the order that 4-bit weights are decoded in (ffn_fm.cu): within 8
+// consecutive values the even ones come before the odd ones; sums[n_rows][K/128]
+// (int4, else null) receive the blocks' sum of codes, sum(q1 + q2) / 64.
 //
 // Rows of src [*, K] -> code planes q [2][n_rows][K] and scales s
 // [n_rows][K/128]. Row r reads source row gather[r] / gather_div (r itself
@@ -36,7 +36,7 @@ __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
 // 4l .. 4l+3 of a block. A block that holds an infinity gets the codes +-1
 // there, 0 elsewhere and an infinite scale, so its sums are infinite as they
 // should be; a NaN makes the scale NaN.
-template <bool kInt4, bool kScatter>
+template <bool kFourBit, bool kScatter>
 __global__ void __launch_bounds__(QWARPS * 32)
 quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ gather, int gather_div,
                   const int32_t* __restrict__ scatter, int n_copies,
@@ -89,12 +89,14 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
             const float2 lo = e4m3x2_to_f32x2(a & 0xffffu), hi = e4m3x2_to_f32x2(a >> 16);
             const float rr[4] = {t[0] - lo.x, t[1] - lo.y, t[2] - hi.x, t[3] - hi.y};
             const uint32_t a2 = e4m3x2(rr[0], rr[1]) | (e4m3x2(rr[2], rr[3]) << 16);
-            if constexpr (kInt4) {
-                const float2 lo2 = e4m3x2_to_f32x2(a2 & 0xffffu), hi2 = e4m3x2_to_f32x2(a2 >> 16);
-                float sum = (lo.x + lo.y + hi.x + hi.y) + (lo2.x + lo2.y + hi2.x + hi2.y);
+            if constexpr (kFourBit) {
+                if (sums) {
+                    const float2 lo2 = e4m3x2_to_f32x2(a2 & 0xffffu), hi2 = e4m3x2_to_f32x2(a2 >> 16);
+                    float sum = (lo.x + lo.y + hi.x + hi.y) + (lo2.x + lo2.y + hi2.x + hi2.y);
 #pragma unroll
-                for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-                if (lane == 0) sums[r * nblk + b] = sum * 0.015625f;
+                    for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+                    if (lane == 0) sums[r * nblk + b] = sum * 0.015625f;
+                }
                 // this lane's values are 0..3 (even lane) or 4..7 of 8: the even two, then the odd two
                 const int64_t at = r * K + b * QB + 8 * (lane >> 1) + 2 * (lane & 1);
                 *reinterpret_cast<uint16_t*>(q + at) = (uint16_t)__byte_perm(a, 0, 0x4420);
@@ -115,34 +117,34 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
                     put(r);
                 }
             }
-            if (kInt4 && lane == 0) s[r * nblk + b] = sc;
+            if (kFourBit && lane == 0) s[r * nblk + b] = sc;
         }
     }
 }
 
 static cudaError_t launch_quant(const void* src, const int32_t* gather, int gather_div, const int32_t* scatter,
-                                int n_copies, int64_t n_rows, int K, void* q, float* s, float* int4_sums,
-                                cudaStream_t stream) {
+                                int n_copies, int64_t n_rows, int K, void* q, float* s, bool four_bit,
+                                float* int4_sums, cudaStream_t stream) {
     const int64_t units = n_rows * ((K / QB + QU - 1) / QU);
     const int blocks = (int)min64((units + QWARPS - 1) / QWARPS, (int64_t)sm_count() * 16);
     if (blocks <= 0) return cudaSuccess;
     auto kernel = scatter     ? quant_rows_kernel<false, true>
-                  : int4_sums ? quant_rows_kernel<true, false>
+                  : four_bit  ? quant_rows_kernel<true, false>
                               : quant_rows_kernel<false, false>;
     return launch_k(kernel, dim3(blocks), dim3(QWARPS * 32), 0, stream, static_cast<const __nv_bfloat16*>(src), gather, gather_div, scatter, n_copies, n_rows, K,
                     static_cast<uint8_t*>(q), s, int4_sums);
 }
 
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, float* int4_sums, cudaStream_t stream) {
-    return launch_quant(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, int4_sums, stream);
+                              float* s, bool four_bit, float* int4_sums, cudaStream_t stream) {
+    return launch_quant(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, four_bit, int4_sums, stream);
 }
 
 // 2048 tokens x 8 copies, H 7168: 45 us, against 86 quantising each of the
 // 16384 gathered rows (every one a full read and all the arithmetic again).
 cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
                                  cudaStream_t stream) {
-    return launch_quant(src, nullptr, 1, pair_pos, k, n_src, K, q, s, nullptr, stream);
+    return launch_quant(src, nullptr, 1, pair_pos, k, n_src, K, q, s, false, nullptr, stream);
 }
 
 }  // namespace gbmoe

@@ -91,8 +91,8 @@ def test_mxfp4_scales_at_two_byte_alignment():
 
 
 def test_mxfp4_block_scales_far_apart():
-    """Scales of one row's four 32-blocks that differ by up to 2^12 stay exact
-    in the codes; a block 2^30 below its neighbours only vanishes next to them."""
+    """Scales of one row's four 32-blocks that differ by up to 2^12, and blocks
+    2^30 below their neighbours."""
     wl = BASE.replace(T=20, E=4, top_k=2, H=512, I=256, wq="mxfp4", seed=10)
     inp = synth.make_inputs(wl)
     rng = np.random.default_rng(0)
