@@ -19,13 +19,13 @@
 // One persistent CTA per SM walks the (M tile, N tile) list built on the
 // device. Warp roles (320 threads):
 //   warp 0    one lane issues TMA loads of q1 and q2 (128 rows x 128 e4m3
-//             each, as two 64-row boxes: the second only when the tile holds
-//             rows there) and B (2 x 128 rows x 128 e4m3), 128-byte
-//             swizzled, into a 3-stage ring;
+//             each, as two 64-row boxes; tiles of up to 64 rows as 16-row boxes
+//             of the two in turn, one 128-row operand) and B (2 x 128 rows x
+//             128 e4m3), 128-byte swizzled, into a 3-stage ring;
 //   warp 1    allocates 512 TMEM columns (two 128 x 256 fp32 partial sums)
 //             and one lane issues tcgen05.mma (M=128, N=256, K=32): four for
-//             q1 and four for q2 per 128-wide k block, alternating between
-//             the two partial sums;
+//             q1 and four for q2 (four for both up to 64 rows) per 128-wide k
+//             block, alternating between the two partial sums;
 //   warps 2-9 promote: warp w reads TMEM lanes 32*(w%4).. (tile rows) and
 //             half (w-2)/4 of the columns, accumulates in registers, and at
 //             the tile's end applies SwiGLU (gate/up) or stores y.
@@ -33,6 +33,11 @@
 // up rows of the same output columns; a promoting thread holds 64 gate and the
 // matching 64 up columns of its row, so SwiGLU needs no exchange.
 // Every mbarrier wait is bounded as in the bf16 GEMM (tc_ptx.cuh).
+//
+// Bound by the MMAs and their operand reads above 64 rows, near HBM below: 2048
+// tokens, top 8 of 256 experts, H 7168, I 2048 (64 rows per expert, about half
+// of the tiles stacked): gate/up 1454 us with waits as calls, 1374 inlined, 1300
+// with tiles of up to 64 rows stacked; down 764, 722, 698.
 #include "common.cuh"
 #include "ffn_sched.h"
 #include "kernels.h"
@@ -120,6 +125,7 @@ __device__ __forceinline__ void b_rows(const Params& p, const Work& wk, int& b0,
 template <bool SWIGLU>  // gate/up GEMM with the SwiGLU epilogue, or the down GEMM
 __global__ void __launch_bounds__(THREADS, 1)
 tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_constant__ CUtensorMap tm_a2,
+                   const __grid_constant__ CUtensorMap tm_s1, const __grid_constant__ CUtensorMap tm_s2,
                    const __grid_constant__ CUtensorMap tm_b0, const __grid_constant__ CUtensorMap tm_b1,
                    const Params p) {
     pdl_enter();
@@ -175,17 +181,26 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
             const Work wk = decode_work(p, w);
             int b0, b1;
             b_rows<SWIGLU>(p, wk, b0, b1);
-            // A in two 64-row boxes; the second only when the tile has rows
-            // there (the MMA's rows past the tile's end read whatever the slot
-            // held, and their accumulators are never stored)
+            // up to 64 rows: both codes stacked in one 128-row operand, 16 rows of
+            // q1 then the same 16 of q2, so that one MMA pass does both; else q1
+            // and q2 in two 64-row boxes each (the MMA's rows past the tile's end
+            // read whatever the slot held, and their accumulators are never stored)
             const bool upper = wk.rows > BM / 2;
+            const int boxes = (wk.rows + 15) / 16;  // up to 64 rows: stacked, in 16-row boxes
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 inflight &= ~(1u << stage);
-                mbar_expect_tx(&full[stage], (upper ? 2 * A_BYTES : A_BYTES) + B_BYTES);
-                tma_load_2d(sA1 + stage * A_BYTES, &tm_a1, kb * BK, (int)wk.row0, &full[stage]);
-                tma_load_2d(sA2 + stage * A_BYTES, &tm_a2, kb * BK, (int)wk.row0, &full[stage]);
-                if (upper) {
+                if (!upper) {
+                    mbar_expect_tx(&full[stage], boxes * 2 * 16 * BK + B_BYTES);
+                    for (int b = 0; b < boxes; ++b) {
+                        uint8_t* dst = sA1 + stage * A_BYTES + b * 32 * BK;
+                        tma_load_2d(dst, &tm_s1, kb * BK, (int)wk.row0 + 16 * b, &full[stage]);
+                        tma_load_2d(dst + 16 * BK, &tm_s2, kb * BK, (int)wk.row0 + 16 * b, &full[stage]);
+                    }
+                } else {
+                    mbar_expect_tx(&full[stage], 2 * A_BYTES + B_BYTES);
+                    tma_load_2d(sA1 + stage * A_BYTES, &tm_a1, kb * BK, (int)wk.row0, &full[stage]);
+                    tma_load_2d(sA2 + stage * A_BYTES, &tm_a2, kb * BK, (int)wk.row0, &full[stage]);
                     tma_load_2d(sA1 + stage * A_BYTES + A_BYTES / 2, &tm_a1, kb * BK, (int)wk.row0 + BM / 2, &full[stage]);
                     tma_load_2d(sA2 + stage * A_BYTES + A_BYTES / 2, &tm_a2, kb * BK, (int)wk.row0 + BM / 2, &full[stage]);
                 }
@@ -207,6 +222,7 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
         bool ok = true;
         bool issued = false;
         for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+            const bool stacked = __shfl_sync(0xffffffffu, decode_work(p, w).rows, 0) <= BM / 2;  // warp-uniform
             for (int kb = 0; kb < nkb; ++kb, ++kbg) {
                 const uint32_t pb = kbg & 1u, pph = (kbg >> 1) & 1u;
                 if (!warp_wait(&pempty[pb], pph ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
@@ -220,9 +236,11 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
 #pragma unroll
                     for (int j = 0; j < BK / 32; ++j)  // +32 bytes along K per instruction
                         mma_fp8(d_tmem, da1 + 2 * j, db + 2 * j, j != 0 ? 1u : 0u);
+                    if (!stacked) {
 #pragma unroll
-                    for (int j = 0; j < BK / 32; ++j)  // the residual codes into the same partial sum
-                        mma_fp8(d_tmem, da2 + 2 * j, db + 2 * j, 1u);
+                        for (int j = 0; j < BK / 32; ++j)  // the residual codes into the same partial sum
+                            mma_fp8(d_tmem, da2 + 2 * j, db + 2 * j, 1u);
+                    }
                     mma_commit(&empty[stage]);
                     mma_commit(&pfull[pb]);
                 }
@@ -240,7 +258,6 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
         // ------------------------------------------ promotion and epilogue
         const int q = warp & 3;            // TMEM lane quarter of this warp
         const int half = (warp - 2) >> 2;  // which half of the tile's columns
-        const int r = q * 32 + lane;       // tile row of this thread
         const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
         const int kq = p.K / QB;
         const int nb_per_e = p.b_rows_per_expert / QB;
@@ -253,9 +270,12 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
             // thread's columns, as element offsets (int: the library refuses
             // fp8 configs whose scale tensors reach 2^31 entries)
             int sa_off, s_off;
+            bool active;  // this warp's lanes hold rows of the tile
             {
                 const Work wk = decode_work(p, w);
-                const int64_t row = wk.row0 + r;
+                const bool stacked = wk.rows <= BM / 2;
+                const int64_t row = wk.row0 + (stacked ? q * 16 + (lane & 15) : q * 32 + lane);
+                active = q * (stacked ? 16 : 32) < wk.rows;
                 sa_off = row < p.n_rows ? (int)(row * kq) : -1;
                 // gate/up: 128 gate rows nt*128.. are n-block nt of the gate scales, up the same;
                 // down: columns 128*half .. are n-block 2*nt + half
@@ -286,6 +306,7 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
                 // 16 columns at a time: next to 128 accumulators, wider loads spill
 #pragma unroll
                 for (int part = 0; part < 8; ++part) {
+                    if (!active) break;
                     float v[16];
                     tmem_ld16(tb + (uint32_t)((part < 4 ? c0 : c1) + 16 * (part & 3)), v);
                     const float f = part < 4 ? f0 : f1;
@@ -298,6 +319,38 @@ tc_fp8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a1, const __grid_const
             }
             if (!ok) break;
             const Work wk = decode_work(p, w);
+            if (wk.rows <= BM / 2) {
+                // stacked: lanes l and l + 16 hold a row's q1 and q2 sums; each stores
+                // half of the columns
+                if (!active) continue;
+                const int r = q * 16 + (lane & 15), upper = lane >> 4;
+#pragma unroll
+                for (int i = 0; i < 128; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+                if (r >= wk.rows) continue;
+                __nv_bfloat16* dst = p.out + (wk.row0 + r) * (int64_t)p.out_cols;
+                if constexpr (SWIGLU) {
+                    dst += wk.nt * (BN / 2) + 64 * half + 32 * upper;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        float h[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            h[i] = silu_mul(upper ? acc[32 + 8 * c + i] : acc[8 * c + i], upper ? acc[96 + 8 * c + i] : acc[64 + 8 * c + i]);
+                        Vec8<__nv_bfloat16>::store(dst + 8 * c, h);
+                    }
+                } else {
+                    dst += wk.nt * BN + 128 * half + 64 * upper;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        float y[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = upper ? acc[64 + 8 * c + i] : acc[8 * c + i];
+                        Vec8<__nv_bfloat16>::store(dst + 8 * c, y);
+                    }
+                }
+                continue;
+            }
+            const int r = q * 32 + lane;  // tile row of this thread
             const int64_t row = wk.row0 + r;
             if (r < wk.rows) {
                 if constexpr (SWIGLU) {
@@ -346,8 +399,8 @@ static bool map_e4m3(CUtensorMap* m, const void* base, int64_t rows, int64_t K, 
 }
 
 template <bool SWIGLU>
-static cudaError_t launch_gemm(const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& b0,
-                               const CUtensorMap& b1, const Params& prm, int64_t max_work, cudaStream_t stream) {
+static cudaError_t launch_gemm(const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& s1,
+                               const CUtensorMap& s2, const CUtensorMap& b0, const CUtensorMap& b1, const Params& prm, int64_t max_work, cudaStream_t stream) {
     static DeviceOnce smem_set;
     cudaError_t e = smem_set.run([] {
         return cudaFuncSetAttribute(tc_fp8_gemm_kernel<SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -357,7 +410,7 @@ static cudaError_t launch_gemm(const CUtensorMap& a1, const CUtensorMap& a2, con
     const int grid = (int)min64(sm_count(), max_work);
     if (grid <= 0) return cudaSuccess;
     if (const cudaError_t le = launch_k(tc_fp8_gemm_kernel<SWIGLU>, dim3(grid), dim3(THREADS), SMEM_BYTES, stream, a1, a2,
-                                        b0, b1, prm);
+                                        s1, s2, b0, b1, prm);
         le != cudaSuccess)
         return le;
     return cudaGetLastError();
@@ -382,8 +435,10 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     const int64_t max_m = sched_max_tiles(p.E, p.n_rows, BM);
     const uint8_t* aq = static_cast<const uint8_t*>(p.a_q);
     const uint8_t* hq = static_cast<const uint8_t*>(p.h_q);
-    CUtensorMap ma1, ma2, mg, mu, mh1, mh2, md;
-    if (!map_e4m3(&ma1, aq, p.n_rows, p.H, BM / 2) || !map_e4m3(&ma2, aq + p.n_rows * p.H, p.n_rows, p.H, BM / 2) ||
+    CUtensorMap ma1, ma2, ms1, ms2, mg, mu, mh1, mh2, mt1, mt2, md;
+    if (!map_e4m3(&ms1, aq, p.n_rows, p.H, 16) || !map_e4m3(&ms2, aq + p.n_rows * p.H, p.n_rows, p.H, 16) ||
+        !map_e4m3(&mt1, hq, p.n_rows, p.I, 16) || !map_e4m3(&mt2, hq + p.n_rows * p.I, p.n_rows, p.I, 16) ||
+        !map_e4m3(&ma1, aq, p.n_rows, p.H, BM / 2) || !map_e4m3(&ma2, aq + p.n_rows * p.H, p.n_rows, p.H, BM / 2) ||
         !map_e4m3(&mg, p.w_gate, (int64_t)p.E * p.I, p.H, BN / 2) ||
         !map_e4m3(&mu, p.w_up, (int64_t)p.E * p.I, p.H, BN / 2) || !map_e4m3(&mh1, hq, p.n_rows, p.I, BM / 2) ||
         !map_e4m3(&mh2, hq + p.n_rows * p.I, p.n_rows, p.I, BM / 2) ||
@@ -396,7 +451,7 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     g.a_scale = p.a_s;
     g.w_scale0 = static_cast<const float*>(p.s_gate); g.w_scale1 = static_cast<const float*>(p.s_up);
     g.wait_limit_ns = tc_wait_limit_ns();
-    if ((err = launch_gemm<true>(ma1, ma2, mg, mu, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
+    if ((err = launch_gemm<true>(ma1, ma2, ms1, ms2, mg, mu, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
     // h quantised per 1x128 for the down GEMM
     if ((err = launch_quant_rows(p.h, nullptr, 1, p.n_rows, p.I, p.h_q, p.h_s, false, nullptr, stream)) != cudaSuccess) return err;
     Params d = g;
@@ -404,7 +459,7 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     d.out = static_cast<__nv_bfloat16*>(p.y);
     d.a_scale = p.h_s;
     d.w_scale0 = static_cast<const float*>(p.s_down); d.w_scale1 = d.w_scale0;
-    return launch_gemm<false>(mh1, mh2, md, md, d, max_m * d.n_tiles, stream);
+    return launch_gemm<false>(mh1, mh2, mt1, mt2, md, md, d, max_m * d.n_tiles, stream);
 }
 
 }  // namespace gbmoe
