@@ -257,24 +257,35 @@ def workload_config(wl):
             "l2": "no flush: the active experts' weights read each step exceed the 126 MB L2"}
 
 
-def launches_per_step(wl, route: str, shared_route) -> int:
+# most rows per expert of the feature-major GEMM by quantised weight format
+# (bf16 activations, AUTO), and most tokens of a shared expert that joins it
+FM_ROWS_PER_EXPERT = {"fp8_b128": 52, "int4_g128": 40, "mxfp4": 60}
+FM_JOIN_TOKENS = 512
+
+
+def launches_per_step(wl, route: str, shared_route, gate: str = "simt") -> int:
     """Kernels this library launches per layer forward: gate logits + expert
-    choice, the permutation (one kernel up to 1024 pairs, else three), per FFN
-    problem a schedule kernel + 2 GEMM/stream kernels (+ a row gather for the
-    routed experts on the CTA-pair routes, whose GEMM does not gather its rows
-    itself, + 3 weight-decode passes on the decode-once routes), and the
-    combine."""
-    def ffn(r, routed):
+    choice (on the tensor cores: router row norms, schedule, GEMM, choice, two
+    recomputing kernels for the flagged tokens and their choice), the
+    permutation (one kernel up to 1024 pairs, else three), per FFN problem a
+    schedule kernel + 2 GEMM/stream kernels (+ two activation quantisations on
+    the routes that multiply codes, + a row gather for the routed experts on the
+    routes whose GEMM does not gather its rows itself, + 3 weight-decode passes
+    on the decode-once routes), and the combine."""
+    def few(routed):  # the feature-major GEMM on coded activations
         rows, experts = (wl.P, wl.E) if routed else (wl.T, 1)
-        few = wl.act == "bf16" and rows <= {"int4_g128": 40, "mxfp4": 60}.get(wl.wq, 0) * experts
-        if r == "tc_fp8" or (r == "tc" and few):  # schedule, x codes, gate/up GEMM, h codes, down GEMM
+        return wl.act == "bf16" and rows <= FM_ROWS_PER_EXPERT.get(wl.wq, 0) * experts
+
+    def ffn(r, routed):
+        if r == "tc_fp8" or (r == "tc" and few(routed)):
             return 5
         # the one-CTA bf16 GEMM gathers its own rows; decoding GEMMs and pairs use the gather kernel
         gather = r in ("tc_pair", "tc_pair_dequant") or (r == "tc" and wl.wq != "bf16")
         return 3 + (1 if routed and gather else 0) + (3 if r in ("tc_dequant", "tc_pair_dequant") else 0)
 
-    n = 2 + (1 if wl.P <= 1024 else 3) + ffn(route, True) + 1
-    if shared_route is not None:
+    n = (7 if gate == "tc" else 2) + (1 if wl.P <= 1024 else 3) + ffn(route, True) + 1
+    joins = wl.has_shared and wl.I_shared == wl.I and wl.T <= FM_JOIN_TOKENS and few(True)
+    if shared_route is not None and not joins:
         n += ffn(shared_route, False)
     return n
 
@@ -440,7 +451,8 @@ def measure(args, wid: int, overrides, dist, world: int, rank: int, local: int, 
     e2e = {"value": replica_throughput(wl.T, args.steps, world, e2e_s), "unit": "tokens/s",
            "h2d_bytes_per_step": io_bytes, "d2h_bytes_per_step": io_bytes}
 
-    per_step = launches_per_step(wl, route, gb.ffn_route(cfg, shared=True) if wl.has_shared else None)
+    per_step = launches_per_step(wl, route, gb.ffn_route(cfg, shared=True) if wl.has_shared else None,
+                                 gb.gate_route(cfg))
     cpu = cpu_baseline_entry(wl, inp) if with_cpu else None
     del x, wr, lb, sb, experts, shared, keep1, keep2, ws, out, x_host, out_host
     torch.cuda.empty_cache()
