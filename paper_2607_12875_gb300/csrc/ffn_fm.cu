@@ -469,8 +469,9 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
         }
         // every copy issued lands before the CTA leaves (after an abort the
         // phase may lack other arrivals: the copies get the drain limit's time)
+        const uint64_t t0 = global_ns();
         for (int s = 0; s < STAGES; ++s)
-            if ((inflight >> s) & 1u) drain_wait(RAW ? &rfull[s] : &full[s], (inflight_par >> s) & 1u);
+            if ((inflight >> s) & 1u) drain_wait(RAW ? &rfull[s] : &full[s], (inflight_par >> s) & 1u, t0);
     } else if (warp == 1) {
         // ------------------------- MMA issuer (the whole warp, one lane issues)
         int stage = 0;
@@ -917,8 +918,9 @@ fm_bf16_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
         }
         // every copy issued lands before the CTA leaves (after an abort the
         // phase may lack other arrivals: the copies get the drain limit's time)
+        const uint64_t t0 = global_ns();
         for (int s = 0; s < STAGES; ++s)
-            if ((inflight >> s) & 1u) drain_wait(&full[s], (inflight_par >> s) & 1u);
+            if ((inflight >> s) & 1u) drain_wait(&full[s], (inflight_par >> s) & 1u, t0);
     } else if (warp == 1) {
         // ------------------------- MMA issuer (the whole warp, one lane issues)
         int stage = 0;

@@ -516,10 +516,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         // for the release of those slots instead (the MMAs that read them
         // finished), which also keeps the even CTA's last arrivals on this
         // CTA's barriers before it leaves.
+        const uint64_t t0 = global_ns();
         for (int s = 0; s < STAGES; ++s) {
             if (!((inflight >> s) & 1u)) continue;
-            if (rank == 0) drain_wait(&full[s], (inflight_par >> s) & 1u);
-            if (CG == 2) drain_wait(&empty[s], (inflight_par >> s) & 1u);
+            if (rank == 0) drain_wait(&full[s], (inflight_par >> s) & 1u, t0);
+            if (CG == 2) drain_wait(&empty[s], (inflight_par >> s) & 1u, t0);
         }
     } else if (warp == 1 && rank == 0) {
         // ------------------------- MMA issuer (the whole warp, one lane issues)

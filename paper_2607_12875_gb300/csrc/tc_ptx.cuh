@@ -113,11 +113,11 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     return __all_sync(0xffffffffu, ok);
 }
 
-// Waits (at most kWaitLimitNs) for a phase that work this thread issued will
-// complete; used at exit so that no copy or MMA is still in flight when the
-// CTA releases its shared memory and TMEM.
-__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
-    const uint64_t t0 = global_ns();
+// Waits (at most kWaitLimitNs from t0 on) for a phase that work this thread
+// issued will complete; used at exit so that no copy or MMA is still in flight
+// when the CTA releases its shared memory and TMEM. Several drains in a row
+// share a t0: after an abort a phase may lack other roles' arrivals for good.
+__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity, uint64_t t0 = global_ns()) {
     while (!mbar_try_wait(bar, parity) && global_ns() - t0 < kWaitLimitNs) {
     }
 }

@@ -119,3 +119,24 @@ def test_shared_expert_after_512_routed_ones():
     wl = BASE.replace(T=40, E=512, top_k=4, H=256, I=128, wq="fp8_b128", seed=3, has_shared=True, I_shared=128)
     inp = synth.make_inputs(wl)
     assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+
+
+@pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
+@pytest.mark.parametrize("T", [24, 120])
+def test_bounded_waits_give_up_and_the_next_call_is_clean(T, wq, monkeypatch):
+    """With the wait limit lowered to 0 ns every role of the kernel stops, drains
+    what it issued and reports; the next call with the normal limit is clean."""
+    wl = BASE.replace(T=T, E=8, top_k=2, H=1024, I=256, wq=wq, seed=77)
+    inp = synth.make_inputs(wl)
+    dev = to_device(wl, inp)
+    cfg = config(wl)
+    ws = workspace(cfg)
+    out = torch.empty((wl.T, wl.H), dtype=torch.bfloat16, device="cuda")
+    args = (cfg, dev["x"], dev["w_router"], None, None, wbundle(dev["experts"]), None, out, ws)
+    monkeypatch.setenv("GBMOE_TC_WAIT_LIMIT_NS", "0")
+    gb.moe_forward(*args)
+    assert gb.moe_device_status(ws) == gb.EDEVICE_TIMEOUT
+    monkeypatch.delenv("GBMOE_TC_WAIT_LIMIT_NS")
+    gb.moe_forward(*args)
+    assert gb.moe_device_status(ws) == gb.OK
+    assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol_for(wl))
