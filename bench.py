@@ -259,7 +259,7 @@ def workload_config(wl):
 
 # most rows per expert of the feature-major GEMM by quantised weight format
 # (bf16 activations, AUTO), and most tokens of a shared expert that joins it
-FM_ROWS_PER_EXPERT = {"fp8_b128": 52, "int4_g128": 40, "mxfp4": 60}
+FM_ROWS_PER_EXPERT = {"fp8_b128": 52, "int4_g128": 40, "mxfp4": 64}
 FM_JOIN_TOKENS = 512
 
 

@@ -32,7 +32,9 @@
 //   4-7 or 4-11  promotion and the output: warp w reads TMEM lanes
 //           32 * (w % 4).. (weight rows); in tall tiles each half of the item
 //           has four warps of its own;
-//   the last 4 or 8  int4 and MXFP4: decode the tile to e4m3 codes.
+//   the last 4 or 8  int4: decode the tile to e4m3 codes; MXFP4: bring the weight
+//           rows' scales (TMA unpacks the tile), or decode like int4 when a
+//           weight pointer is not 32-byte aligned, as the unpacking TMA wants.
 // A gate/up item holds 128 gate rows and the 128 up rows of the same columns, so
 // gate and up of a column end up in one thread (short tiles) or in the same TMEM
 // lane of two warps, which meet there once per item. Every mbarrier wait is bounded (tc_ptx.cuh).
@@ -43,11 +45,11 @@
 // held it back on the way, per 128-wide k block: waits as calls (2400 -> 1750
 // cycles once inlined) and MMAs issued under `lane == 0` (1750 -> 1500).
 // int4, 17 tokens, top 6 of 64 experts, H 4096, I 2816: layer 1397 -> 220 us.
-// MXFP4, 16 tokens of the fp8 layer: 2896 -> 635 us. Its E8M0 scales go to the
-// MMAs (kind::mxf8f6f4), so the decode is shifts and masks; scaling the codes in
-// the decode warps, relative to the largest scale of a row's 128 k, cost twice
-// the instructions and bound the kernel (819 us, and 3.08 against 2.61 ms at
-// 1024 tokens).
+// MXFP4, 16 tokens of the fp8 layer: 2896 -> 495 us. Its E8M0 scales go to the
+// MMAs (kind::mxf8f6f4) and its codes are an operand as TMA unpacks them, so no
+// warp touches a weight. Decoding them to e4m3 with shifts and masks was bound by
+// the decode (635 us; 2.15 ms in place of 1.35 at 256 tokens), and scaling the
+// codes there too, relative to the largest scale of a row's 128 k, more so (819).
 #include "common.cuh"
 #include "ffn_sched.h"
 #include "kernels.h"
@@ -64,24 +66,29 @@ constexpr int A_BYTES = 2 * MB * BK;    // the two 128-row halves of an item's w
 constexpr int TMEM_COLS = 512;
 constexpr int GATHER_WARPS = 2;
 constexpr int SMEM_BUDGET = 232448;
+// MXFP4 whose tiles TMA unpacks: 16 E2M1 codes of 8 bytes become 8 bytes and 8
+// bytes of padding in shared memory, which kind::mxf8f6f4 reads as they are
+// (an e2m1 operand takes as much shared memory as an e4m3 one).
+constexpr int kMxfp4Unpacked = 256 + GBMOE_MXFP4;
 
 // Per weight format and height of a row tile.
 template <int WQ, int ROWS>
 struct Cfg {
     // int4, MXFP4: bytes of the tile as stored, which the decode warps turn into e4m3
-    static constexpr int RAW = WQ == GBMOE_FP8_E4M3_B128 ? 0 : A_BYTES / 2;
+    static constexpr bool UNPACKED = WQ == kMxfp4Unpacked;
+    static constexpr int RAW = WQ == GBMOE_FP8_E4M3_B128 || UNPACKED ? 0 : A_BYTES / 2;
+    static constexpr bool BLOCK_SCALE = WQ == GBMOE_MXFP4 || UNPACKED;
     // Short tiles: a k block's two partial sums, q1 and q2 side by side, share a
     // slot of TMEM, which halves the handshakes that then dominate, and the same
     // warps promote both. Tall tiles: q1 and q2 add up in the same columns, each
     // half of the item has two slots and a set of warps of its own, and the sets
     // meet once per item (X_COL: where the up half hands its sums over).
     static constexpr bool JOINT = ROWS <= 32;
-    static constexpr int SLOTS = WQ == GBMOE_MXFP4 && ROWS == 32 ? 3 : 4;  // (MXFP4's scales need columns too)
+    static constexpr int SLOTS = BLOCK_SCALE && ROWS == 32 ? 3 : 4;  // (MXFP4's scales need columns too)
     static constexpr int SLOT_COLS = JOINT ? 4 * ROWS : ROWS;
     static constexpr int X_COL = SLOTS * SLOT_COLS;
     // MXFP4: the MMAs' scale factors in TMEM. Ones for the rows (8 columns), then
     // two k blocks' weight scales, 4 columns per 128-row half.
-    static constexpr bool BLOCK_SCALE = WQ == GBMOE_MXFP4;
     static constexpr int SF_COL = X_COL + (JOINT ? 0 : ROWS);
     static constexpr int SF_COLS = BLOCK_SCALE ? 8 + 16 : 0;
     static constexpr int SF_BYTES = BLOCK_SCALE ? 2 * 512 : 0;  // a stage's weight scales in shared memory
@@ -90,12 +97,19 @@ struct Cfg {
     static constexpr int GROUPS = ROWS / 8;  // most groups of 8 rows
     static constexpr int HALVES_HELD = JOINT ? 2 : 1;  // halves whose sums a promotion warp holds
     static constexpr int DECODE_WARPS = RAW ? (JOINT ? 8 : 4) : 0;
-    static constexpr int THREADS = 32 * (2 + GATHER_WARPS + PROMOTE_WARPS + DECODE_WARPS);
+    static constexpr int SCALE_WARPS = UNPACKED ? 4 : 0;
+    static constexpr int THREADS = 32 * (2 + GATHER_WARPS + PROMOTE_WARPS + DECODE_WARPS + SCALE_WARPS);
+    static constexpr bool SPLIT_REGS = !JOINT && DECODE_WARPS + SCALE_WARPS == 4;  // 16 warps, see setmaxnreg
     static constexpr int STAGE_BYTES = A_BYTES + RAW + SF_BYTES + 2 * ROWS * BK;
     // floats of a scale block: the rows' scales and negated sums of codes, then
     // (int4) the weight rows' scales
     static constexpr int RING_FLOATS = 2 * ROWS + (WQ == GBMOE_INT4_G128 ? 2 * MB : 0);
-    static constexpr int MAX_STAGES = 6;
+    // UNPACKED: the ring leaves the L1 cache 60 KB. A k block reads 4 bytes of
+    // scales in each of 256 lines, and eight k blocks share a sector, so the lines
+    // (32 KB) have to outlive a k block: with all 228 KB as shared memory they
+    // were refetched each time (16-row tiles 597 us with 6 stages, 495 with 5 or
+    // 4; 32-row tiles at 8 rows per expert 1631 with 5, 1351 with 4, 1434 with 3).
+    static constexpr int MAX_STAGES = !UNPACKED ? 6 : ROWS == 16 ? 5 : ROWS == 32 ? 4 : 3;
     static constexpr int MAX_RING = MAX_STAGES + 4;
     static constexpr int NUM_BARS = 3 * MAX_STAGES + 2 * SLOTS + MAX_RING + 1 + 8;
     static constexpr int FIXED_BYTES = 1024 + MAX_RING * RING_FLOATS * 4 + NUM_BARS * 8 + 16;
@@ -188,6 +202,10 @@ __device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
+__device__ __forceinline__ void cp_async_4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
 // ------------------------------- pairs of fp32 (one instruction for two)
 
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
@@ -224,8 +242,9 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 // kind::mxf8f6f4: the same with E8M0 scales per 32 k of each operand row (bit
 // 23). A k step's scale is byte j (bits 29-30 for A; B's are all ones) of the
 // row's 32-bit word in TMEM.
+template <bool A_E2M1>
 __device__ __forceinline__ uint32_t idesc_mxf8(int n) {
-    return (1u << 23) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(MB >> 4) << 24);
+    return (A_E2M1 ? 5u << 7 : 0u) | (1u << 23) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(MB >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_mxf8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t sfa, uint32_t sfb,
@@ -394,7 +413,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 32 * GATHER_WARPS + (RAW ? C::DECODE_WARPS : 1));
+            mbar_init(&full[s], 32 * (GATHER_WARPS + C::SCALE_WARPS) + (RAW ? C::DECODE_WARPS : 1));
             mbar_init(&rfull[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -439,7 +458,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
 
     // tall tiles: 16 warps start with 128 registers a thread; the promotion takes 168
     // (128 threads x (104 + 168 + 168 + 72) = 65536, what the block was launched with)
-    if constexpr (RAW && !C::JOINT) {
+    if constexpr (C::SPLIT_REGS) {
         if (warp < 4) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
     }
     if (warp == 0 && lane == 0) {
@@ -459,7 +478,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 uint8_t* dst = RAW ? sR + stage * RAW : sA + stage * A_BYTES;
                 const int x = kb * (RAW ? BK / 2 : BK);
                 uint64_t* bar = RAW ? &rfull[stage] : &full[stage];
-                mbar_expect_tx(bar, BYTES);
+                mbar_expect_tx(bar, C::UNPACKED ? BYTES / 2 : BYTES);  // (padding does not count)
                 tma_load_2d(dst, wk.shared ? &tm_s0 : &tm_w0, x, a0, bar);
                 tma_load_2d(dst + BYTES / 2, wk.shared ? &tm_s1 : &tm_w1, x, a1, bar);
                 inflight |= 1u << stage;
@@ -483,7 +502,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             const Work wk = decode_work(p, w);
             const int rp = __shfl_sync(0xffffffffu, rows_pad<C::JOINT>(wk.rows), 0);  // warp-uniform
             const int n = C::JOINT ? 2 * rp : rp;
-            const uint32_t idesc = C::BLOCK_SCALE ? idesc_mxf8(n) : idesc_f8(n);
+            const uint32_t idesc = C::BLOCK_SCALE ? idesc_mxf8<C::UNPACKED>(n) : idesc_f8(n);
             for (int kb = 0; kb < nkb; ++kb, ++kc) {
                 if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 // the row codes were written through the generic proxy (cp.async)
@@ -591,7 +610,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
         asm volatile("cp.async.wait_all;" ::: "memory");  // (after an abort too) copies land before the CTA leaves
     } else if (warp >= 4 && warp < 4 + C::PROMOTE_WARPS) {
         // ------------------------------------------ promotion and output
-        if constexpr (RAW && !C::JOINT) asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+        if constexpr (C::SPLIT_REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
         constexpr int GROUPS = C::GROUPS;
         const int q = warp & 3;            // TMEM lane quarter
         const int set = (warp - 4) >> 2;   // tall tiles: the half of the item this warp promotes
@@ -614,7 +633,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             for (int h = 0; h < C::HALVES_HELD; ++h) {
 #pragma unroll
                 for (int i = 0; i < 4 * GROUPS; ++i) acc[h][i] = 0;
-                wn[h] = RAW ? 64.0f : ws[h][0];  // (MXFP4's codes are the values times 2^-6, the MMAs scale)
+                wn[h] = C::UNPACKED ? 1.0f : RAW ? 64.0f : ws[h][0];  // (MXFP4's decoded codes are the values times 2^-6, the MMAs scale)
             }
             bool ok = true;
             for (int kb = 0; kb < nkb; ++kb, ++kc) {
@@ -622,7 +641,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
 #pragma unroll
                 for (int h = 0; h < C::HALVES_HELD; ++h) {
                     wsc[h] = wn[h];
-                    if (!RAW && kb + 1 < nkb) wn[h] = ws[h][kb + 1];
+                    if (!RAW && !C::UNPACKED && kb + 1 < nkb) wn[h] = ws[h][kb + 1];
                 }
                 const float* sc = sS + ring * C::RING_FLOATS;
                 const uint32_t slot = C::JOINT ? kc % SLOTS : 2 * set + (kc & 1);
@@ -727,6 +746,42 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             }
         }
     }
+    if constexpr (C::UNPACKED) {
+        if (warp >= 4 + C::PROMOTE_WARPS) {
+            // ------------------------------------- weight rows' E8M0 scales
+            // Thread r brings the four scales of a k block of row r of each half
+            // to where the MMA issuer copies them to TMEM from.
+            if constexpr (C::SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+            const int r = threadIdx.x - 32 * (4 + C::PROMOTE_WARPS);
+            int stage = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+                const Work wk = decode_work(p, w);
+                int a0, a1;
+                w_rows<SWIGLU>(p, wk, a0, a1);
+                const uint8_t* s0 = static_cast<const uint8_t*>(wk.shared ? p.s_scale0 : p.w_scale0) + (int64_t)(a0 + r) * nkb * 4;
+                const uint8_t* s1 = static_cast<const uint8_t*>(wk.shared ? p.s_scale1 : p.w_scale1) + (int64_t)(a1 + r) * nkb * 4;
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                    uint8_t* dst = sF + stage * C::SF_BYTES + 16 * (r & 31) + 4 * (r >> 5);
+                    if (p.scale_words) {
+                        cp_async_4(dst, s0 + 4 * kb);
+                        cp_async_4(dst + 512, s1 + 4 * kb);
+                        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[stage])) : "memory");
+                    } else {
+                        const uint16_t* b0 = reinterpret_cast<const uint16_t*>(s0 + 4 * kb);
+                        const uint16_t* b1 = reinterpret_cast<const uint16_t*>(s1 + 4 * kb);
+                        *reinterpret_cast<uint32_t*>(dst) = b0[0] | (uint32_t)b0[1] << 16;
+                        *reinterpret_cast<uint32_t*>(dst + 512) = b1[0] | (uint32_t)b1[1] << 16;
+                        mbar_arrive(&full[stage]);  // (the MMA issuer has the proxy fence)
+                    }
+                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
+                }
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");  // (after an abort too) copies land before the CTA leaves
+        }
+    }
     if constexpr (RAW) {
         if (warp >= 4 + C::PROMOTE_WARPS) {
             // ------------------------------- weight decode, weight rows' scales
@@ -734,7 +789,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             // it decodes the row's 128 values of a k block and writes their
             // scale to the scale block (int4) or its four E8M0 scales to where
             // the MMA issuer copies them to TMEM from (MXFP4).
-            if constexpr (!C::JOINT) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+            if constexpr (C::SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
             constexpr int HALVES = C::DECODE_WARPS == 8 ? 1 : 2;
             const int t = threadIdx.x - 32 * (4 + C::PROMOTE_WARPS);
             const int r = t & (MB - 1), h0 = t >> 7;
@@ -1068,6 +1123,17 @@ static cudaError_t launch_gemm(const CUtensorMap& w0, const CUtensorMap& w1, con
 
 // [rows, K] weights in boxes of 128 rows x 128 k as stored
 static bool map_weights(CUtensorMap* m, int wq, const void* base, int64_t rows, int64_t K) {
+    if (wq == kMxfp4Unpacked) {
+        // wants a 32-byte aligned base, strides that are multiples of 32 bytes,
+        // extents of multiples of 128 codes and boxes of 128 codes
+        const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
+        const cuuint64_t strides[1] = {(cuuint64_t)K / 2};
+        const cuuint32_t box[2] = {BK, MB};
+        const cuuint32_t estr[2] = {1, 1};
+        return encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_16U4_ALIGN16B, 2, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    }
     if (wq != GBMOE_FP8_E4M3_B128)
         return make_map(m, base, rows, K / 2, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, BK / 2, CU_TENSOR_MAP_SWIZZLE_64B, MB);
     return make_map(m, base, rows, K, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, BK, CU_TENSOR_MAP_SWIZZLE_128B, MB);
@@ -1082,7 +1148,7 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     const int64_t rows = p.n_rows + p.n_shared;
     // every row of x once (the shared expert's rows are x's own; a routed row is a token's)
     const int64_t x_rows = p.n_rows / p.pair_div;
-    constexpr bool kFour = WQ != GBMOE_FP8_E4M3_B128;  // the order 4-bit weights are decoded in
+    constexpr bool kFour = Cfg<WQ, ROWS>::RAW != 0;  // the order 4-bit weights are decoded in
     constexpr bool kSums = WQ == GBMOE_INT4_G128;
     float* a_sum = kSums ? p.a_s + x_rows * (p.H / BK) : nullptr;
     float* h_sum = kSums ? p.h_s + rows * (p.I / BK) : nullptr;
@@ -1190,7 +1256,12 @@ cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream) {
             return p.n_rows <= 4 * (int64_t)p.E ? fm::launch_ffn_bf16<16>(p, stream) : fm::launch_ffn_bf16<64>(p, stream);
         case GBMOE_FP8_E4M3_B128: return fm::launch_ffn<GBMOE_FP8_E4M3_B128>(p, stream);
         case GBMOE_INT4_G128: return fm::launch_ffn<GBMOE_INT4_G128>(p, stream);
-        case GBMOE_MXFP4: return fm::launch_ffn<GBMOE_MXFP4>(p, stream);
+        case GBMOE_MXFP4: {
+            auto aligned = [](const void* w) { return reinterpret_cast<uintptr_t>(w) % 32 == 0; };  // (or null: no shared expert)
+            const bool unpacked = aligned(p.w_gate) && aligned(p.w_up) && aligned(p.w_down) && aligned(p.sw_gate) &&
+                                  aligned(p.sw_up) && aligned(p.sw_down);
+            return unpacked ? fm::launch_ffn<fm::kMxfp4Unpacked>(p, stream) : fm::launch_ffn<GBMOE_MXFP4>(p, stream);
+        }
         default: return cudaErrorInvalidValue;
     }
 }

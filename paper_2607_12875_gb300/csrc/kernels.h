@@ -121,12 +121,13 @@ bool ffn_tc_fp8_supported(const FfnProblem& p);
 // 128-row MMAs of the row-major GEMMs waste less than its second pass over the
 // weights' operand costs. Feature-major against row-major, 256 experts, H 7168,
 // I 2048: fp8 2.14 against 2.48 ms at 32 rows per expert, 2.37 against 2.52 at
-// 47, 2.83 against 2.66 at 64; MXFP4 2.61 against 3.43 (decode in the GEMM) at
-// 32, 2.87 against 3.39 at 47, 3.46 against 3.47 at 64; int4, 64 experts, H 4096, I 2816: 0.59 against
+// 47, 2.83 against 2.66 at 64; MXFP4 2.56 against 3.43 (decode in the GEMM) at
+// 32, 2.81 against 3.39 at 47, 3.23 against 3.47 at 64, 3.65 against 3.55 at 72 (with decode warps, at
+// unaligned weights, 3.46 at 64); int4, 64 experts, H 4096, I 2816: 0.59 against
 // 0.78 at 24, 0.78 against 0.78 at 48, 0.96 against 0.85 at 72; bf16, 128 experts, H 4096, I 1536: 0.775
 // against 0.800 at 21, 0.62 against 0.70 (streaming) at 2.
 constexpr int64_t kFmFp8RowsPerExpert = 52;
-constexpr int64_t kFmMxfp4RowsPerExpert = 60;
+constexpr int64_t kFmMxfp4RowsPerExpert = 64;
 constexpr int64_t kFmRowsPerExpert = 40;
 // rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales;
 // four_bit: in the order 4-bit weights are decoded in, with the blocks' sums of codes in int4_sums if not null

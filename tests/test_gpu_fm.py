@@ -90,6 +90,25 @@ def test_mxfp4_scales_at_two_byte_alignment():
     assert_close(act_np(forward(wl, dev)), oracle.forward(wl, inp)["out"], tol_for(wl))
 
 
+@pytest.mark.parametrize("T", [8, 40, 120])
+def test_mxfp4_weights_at_16_byte_alignment(T):
+    """Weights that TMA cannot unpack (it wants 32-byte aligned ones) are decoded
+    by the kernel: the same products and scales, so nearly the same output."""
+    wl = BASE.replace(T=T, E=4, top_k=2, H=512, I=256, wq="mxfp4", seed=11)
+    inp = synth.make_inputs(wl)
+    dev = to_device(wl, inp)
+    aligned = act_np(forward(wl, dev))
+    for k in ("w_gate", "w_up", "w_down"):
+        v = dev["experts"][k]
+        assert v.data_ptr() % 32 == 0
+        dev["experts"][k] = torch.cat([v.flatten()[:16], v.flatten()])[16:].view(v.shape)
+        assert dev["experts"][k].data_ptr() % 32 == 16
+    got = act_np(forward(wl, dev))
+    want = oracle.forward(wl, inp)["out"]
+    assert_close(got, want, tol_for(wl))
+    assert_close(aligned, want, tol_for(wl))
+
+
 def test_mxfp4_block_scales_far_apart():
     """Scales of one row's four 32-blocks that differ by up to 2^12, and blocks
     2^30 below their neighbours."""
