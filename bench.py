@@ -428,6 +428,9 @@ def measure(args, wid: int, overrides, dist, world: int, rank: int, local: int, 
     if route == "tc" and wl.wq != "bf16":  # decoding GEMMs read a gathered copy of x
         kernel = ("moe_grouped_ffn, tcgen05 route (row gather + gate/up GEMM decoding its weight tiles, with "
                   "SwiGLU + down GEMM)")
+    if wl.act == "bf16" and wl.P <= FM_ROWS_PER_EXPERT.get(wl.wq, 0) * wl.E:
+        kernel = ("moe_grouped_ffn, feature-major tcgen05 GEMM (quantisation of the rows + gate/up GEMM with SwiGLU + "
+                  "quantisation of h + down GEMM)")
     tpe = TRAFFIC_PER_ACTIVE_EXPERT.get((wl.name, route))
     extra = {"traffic": None if tpe is None else tpe * active, "kernel": kernel, "active_experts": active,
              "route": route, "gate": gb.gate_route(cfg)}
