@@ -88,9 +88,12 @@ struct Cfg {
     static constexpr int SLOT_COLS = JOINT ? 4 * ROWS : ROWS;
     static constexpr int X_COL = SLOTS * SLOT_COLS;
     // MXFP4: the MMAs' scale factors in TMEM. Ones for the rows (8 columns), then
-    // two k blocks' weight scales, 4 columns per 128-row half.
+    // weight scales, 4 columns per 128-row half, as many k blocks' as can have
+    // MMAs in flight: the wait for a slot of partial sums then covers its scales,
+    // which the MMAs that filled the slot before were the last to read.
     static constexpr int SF_COL = X_COL + (JOINT ? 0 : ROWS);
-    static constexpr int SF_COLS = BLOCK_SCALE ? 8 + 16 : 0;
+    static constexpr int SF_BLOCKS = JOINT ? SLOTS : 2;
+    static constexpr int SF_COLS = BLOCK_SCALE ? 8 + 8 * SF_BLOCKS : 0;
     static constexpr int SF_BYTES = BLOCK_SCALE ? 2 * 512 : 0;  // a stage's weight scales in shared memory
     static constexpr int SETS = JOINT ? 1 : 2;  // of four promotion warps
     static constexpr int PROMOTE_WARPS = 4 * SETS;
@@ -519,9 +522,9 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                     }
                     const uint32_t d = tmem_base + slot * C::SLOT_COLS + (C::JOINT ? half * 2 * ROWS : 0);
                     const uint64_t dh = da0 + (uint64_t)((stage * A_BYTES + half * (MB * BK)) >> 4);
-                    const uint32_t sfb = tmem_base + C::SF_COL, sfa = sfb + 8 + (kc & 1) * 8 + half * 4;
+                    const uint32_t sfb = tmem_base + C::SF_COL, sfa = sfb + 8 + kc % C::SF_BLOCKS * 8 + half * 4;
                     if (elect_one()) {
-                        if constexpr (C::BLOCK_SCALE)  // (copies and MMAs run in the order of their issue)
+                        if constexpr (C::BLOCK_SCALE)  // (a copy runs before the MMAs issued after it)
                             tmem_copy_scales(sfa, smem_u32(sF + stage * C::SF_BYTES + half * 512));
 #pragma unroll
                         for (int pass = 0; pass < (C::JOINT ? 1 : 2); ++pass)

@@ -122,6 +122,21 @@ def test_mxfp4_block_scales_far_apart():
     assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
 
 
+@pytest.mark.parametrize("T", [6, 24, 60])
+def test_mxfp4_scales_of_each_k_block_are_its_own(T):
+    """Scales that step by 2^-3, 2^0 and 2^3 from one 128-wide k block to the
+    next, over many k blocks: a block multiplied with the scales of one of the
+    blocks whose MMAs are in flight beside it (16-, 32- and 80-row tiles) would
+    be off by at least 2^3."""
+    wl = BASE.replace(T=T, E=4, top_k=2, H=4096, I=1024, wq="mxfp4", seed=T)
+    inp = synth.make_inputs(wl)
+    for k in ("s_gate", "s_up", "s_down"):
+        s = inp["experts"][k].astype(np.int32)
+        step = np.repeat(3 * (np.arange(s.shape[-1] // 4) % 3 - 1), 4)
+        inp["experts"][k] = (s + step).astype(np.uint8)
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+
+
 @pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T,I_shared", [(5, 256), (60, 256), (150, 256), (60, 384)])
 def test_shared_expert_with_the_routed_ones(T, I_shared, wq):
