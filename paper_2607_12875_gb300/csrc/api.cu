@@ -220,12 +220,11 @@ Layout layout(const gbmoe_config* c) {
     L.xout = take((size_t)T * H * ab);
     L.wdq = take(dequant_bytes(c, P, (int)E, c->I));
     L.wdq_sh = take(c->has_shared ? dequant_bytes(c, T, 1, c->I_shared) : 0);
-    const bool codes = uses_act_codes(c);  // e4m3 copies of the GEMM inputs, their 1x128 scales (and sums: int4)
-    const size_t per_block = c->w_dtype == GBMOE_INT4_G128 ? 8 : 4;
+    const bool codes = uses_act_codes(c);  // e4m3 copies of the GEMM inputs and their 1x128 scales
     L.aq = take(codes ? (size_t)2 * rows_max * H : 0);  // two e4m3 code planes
-    L.as = take(codes ? (size_t)rows_max * (H / 128) * per_block : 0);
+    L.as = take(codes ? (size_t)rows_max * (H / 128) * 4 : 0);
     L.hq = take(codes ? (size_t)2 * rows_max * I_max : 0);
-    L.hs = take(codes ? (size_t)rows_max * (I_max / 128) * per_block : 0);
+    L.hs = take(codes ? (size_t)rows_max * (I_max / 128) * 4 : 0);
     L.total = o;
     return L;
 }

@@ -104,9 +104,8 @@ struct Cfg {
     static constexpr int THREADS = 32 * (2 + GATHER_WARPS + PROMOTE_WARPS + DECODE_WARPS + SCALE_WARPS);
     static constexpr bool SPLIT_REGS = !JOINT && DECODE_WARPS + SCALE_WARPS == 4;  // 16 warps, see setmaxnreg
     static constexpr int STAGE_BYTES = A_BYTES + RAW + SF_BYTES + 2 * ROWS * BK;
-    // floats of a scale block: the rows' scales and negated sums of codes, then
-    // (int4) the weight rows' scales
-    static constexpr int RING_FLOATS = 2 * ROWS + (WQ == GBMOE_INT4_G128 ? 2 * MB : 0);
+    // floats of a scale block: the rows' scales, then (int4) the weight rows'
+    static constexpr int RING_FLOATS = ROWS + (WQ == GBMOE_INT4_G128 ? 2 * MB : 0);
     // UNPACKED: the ring leaves the L1 cache 60 KB. A k block reads 4 bytes of
     // scales in each of 256 lines, and eight k blocks share a sector, so the lines
     // (32 KB) have to outlive a k block: with all 228 KB as shared memory they
@@ -146,7 +145,6 @@ struct Params {
     const float* a_scale;    // [plane_rows][K/128]
     const int32_t* gather;   // row r of the sorted order is plane row gather[r] / gather_div; null: r itself
     int gather_div;
-    const float* a_sum;      // int4: [plane_rows][K/128] sums of codes
     const void* w_scale0;    // first / second half of the item: fp8 fp32 [E, w_rows_per_expert/128, K/128],
     const void* w_scale1;    // int4 bf16 [E, w_rows_per_expert, K/128], MXFP4 E8M0 bytes [E, w_rows_per_expert, K/32]
     const void* s_scale0;    // the shared expert's
@@ -300,24 +298,16 @@ __device__ __forceinline__ void tmem_pin(uint32_t (&a)[8]) {
 }
 
 // acc += v * (sc * w) over 8 rows: v their partial sums, sc the rows' scales in
-// shared memory, w the weight scale in both halves. int4 (see the decode
-// warps): acc += (v - sum) * (sc * w), the rows' negated sums ROWS behind their
-// scales.
-template <int WQ, int ROWS>
-__device__ __forceinline__ void promote8(uint64_t (&v)[4], const float* sc, uint64_t w, uint64_t* acc) {
+// shared memory, w the weight scale in both halves.
+__device__ __forceinline__ void promote8(const uint64_t (&v)[4], const float* sc, uint64_t w, uint64_t* acc) {
     const float4 f0 = *reinterpret_cast<const float4*>(sc), f1 = *reinterpret_cast<const float4*>(sc + 4);
     const uint64_t f[4] = {pack2(f0.x, f0.y), pack2(f0.z, f0.w), pack2(f1.x, f1.y), pack2(f1.z, f1.w)};
-    if constexpr (WQ == GBMOE_INT4_G128) {
-        const float4 c0 = *reinterpret_cast<const float4*>(sc + ROWS), c1 = *reinterpret_cast<const float4*>(sc + ROWS + 4);
-        v[0] = add2(v[0], pack2(c0.x, c0.y)); v[1] = add2(v[1], pack2(c0.z, c0.w));
-        v[2] = add2(v[2], pack2(c1.x, c1.y)); v[3] = add2(v[3], pack2(c1.z, c1.w));
-    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i] = fma2(v[i], mul2(f[i], w), acc[i]);
 }
 
 // Promotes N groups of 8 rows: all their loads in flight, one wait. SIDE: the q2 sums are at t2, and added.
-template <int WQ, int ROWS, int N, bool SIDE>
+template <int N, bool SIDE>
 __device__ __forceinline__ void promote(uint32_t t1, uint32_t t2, const float* sc, uint64_t w, uint64_t* acc) {
     uint32_t a[N][8], b[SIDE ? N : 1][8];
 #pragma unroll
@@ -339,7 +329,7 @@ __device__ __forceinline__ void promote(uint32_t t1, uint32_t t2, const float* s
             v[i] = pack2u(a[g][2 * i], a[g][2 * i + 1]);
             if constexpr (SIDE) v[i] = add2(v[i], pack2u(b[g][2 * i], b[g][2 * i + 1]));
         }
-        promote8<WQ, ROWS>(v, sc + 8 * g, w, acc + 4 * g);
+        promote8(v, sc + 8 * g, w, acc + 4 * g);
     }
 }
 
@@ -358,15 +348,24 @@ __device__ __forceinline__ void tmem_st8(uint32_t t, const uint64_t* v) {
 }
 
 // 16 bytes of int4 weights -> 32 e4m3 codes, the even values of each 8 before
-// the odd ones. A two's complement nibble n with its top bit flipped is
-// u = n + 8, 0 <= u <= 15, and the byte u read as e4m3 is u * 2^-9 (bits 0-2
-// are the mantissa, bit 3 the lowest exponent bit: the subnormals run on into
-// the first normal binade), so a shift and a mask decode 8 values; the 8 is
-// taken back out per block in the promotion (sum of u * q - 8 * sum of q).
+// the odd ones. The byte m <= 8 read as e4m3 is m * 2^-9 (bits 0-2 are the
+// mantissa, bit 3 the lowest exponent bit: the subnormals run on into the first
+// normal binade), so the code of a nibble n is |n| with n's sign in bit 7. In
+// the bytes of negative n (all ones in neg, from their sign in bit 7 of signs)
+// n ^ neg is 0xf0 + |n| - 1, and 0x80 + |n| is 0x6f less. (One instruction
+// decodes n + 8 for four values, but then 8 times the sum of the row's codes has
+// to be taken back out in fp32, with the largest of them in it: 17 tokens of the
+// layer above 219 us like that, 233 like this; 170 tokens 496 and 475.)
 __device__ __forceinline__ void decode_int4_32(const uint4 raw, uint4& o0, uint4& o1) {
-    auto even = [](uint32_t w) { return (w & 0x0f0f0f0fu) ^ 0x08080808u; };
-    o0 = make_uint4(even(raw.x), even(raw.x >> 4), even(raw.y), even(raw.y >> 4));
-    o1 = make_uint4(even(raw.z), even(raw.z >> 4), even(raw.w), even(raw.w >> 4));
+    auto codes = [](uint32_t signs, uint32_t w) {
+        uint32_t neg;
+        asm("prmt.b32 %0, %1, %1, 0xba98;" : "=r"(neg) : "r"(signs));
+        return ((w & 0x0f0f0f0fu) ^ neg) - (neg & 0x6f6f6f6fu);
+    };
+    auto even = [&](uint32_t w) { return codes(w << 4, w); };
+    auto odd = [&](uint32_t w) { return codes(w, w >> 4); };
+    o0 = make_uint4(even(raw.x), odd(raw.x), even(raw.y), odd(raw.y));
+    o1 = make_uint4(even(raw.z), odd(raw.z), even(raw.w), odd(raw.w));
 }
 
 // 16 bytes of MXFP4 weights -> 32 e4m3 codes in the order of int4's. The
@@ -579,10 +578,6 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             const float* s0 = p.a_scale + (t < rp ? src_row(t) : 0) * nkb;
             const float* s1 = p.a_scale + (t + 64 < rp ? src_row(t + 64) : 0) * nkb;
             float n0 = s0[0], n1 = s1[0];
-            constexpr bool SUMS = WQ == GBMOE_INT4_G128;
-            const int64_t sum_off = SUMS ? p.a_sum - p.a_scale : 0;
-            float m0 = 0.0f, m1 = 0.0f;  // int4: sums of codes
-            if (SUMS) { m0 = s0[sum_off]; m1 = s1[sum_off]; }
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 uint8_t* dst = sB + stage * B_BYTES;
@@ -598,12 +593,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 float* sc = sS + ring * C::RING_FLOATS;
                 if (t < rp) sc[t] = n0;
                 if (t + 64 < rp) sc[t + 64] = n1;
-                if (SUMS && t < rp) sc[ROWS + t] = -m0;
-                if (SUMS && t + 64 < rp) sc[ROWS + t + 64] = -m1;
-                if (kb + 1 < nkb) {
-                    n0 = s0[kb + 1]; n1 = s1[kb + 1];
-                    if (SUMS) { m0 = s0[sum_off + kb + 1]; m1 = s1[sum_off + kb + 1]; }
-                }
+                if (kb + 1 < nkb) { n0 = s0[kb + 1]; n1 = s1[kb + 1]; }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sfull[ring]);
                 if (++ring == RING) ring = 0;
@@ -658,23 +648,23 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
 #pragma unroll
                 for (int h = 0; h < C::HALVES_HELD; ++h) {
                     // int4: one weight scale per row
-                    if (WQ == GBMOE_INT4_G128) wsc[h] = sc[2 * ROWS + (C::JOINT ? h : set) * MB + q * 32 + lane];
+                    if (WQ == GBMOE_INT4_G128) wsc[h] = sc[ROWS + (C::JOINT ? h : set) * MB + q * 32 + lane];
                     const uint64_t w2 = pack2(wsc[h], wsc[h]);
                     const uint32_t t1 = t_lane + slot * C::SLOT_COLS + h * 2 * ROWS, t2 = t1 + rp;
                     // (straight-line code per number of groups: nothing may come between loads and wait)
                     if constexpr (C::JOINT) {
 #pragma unroll
                         for (int g = 0; g < GROUPS; g += 2) {
-                            if (g + 1 < groups) promote<WQ, ROWS, 2, true>(t1 + 8 * g, t2 + 8 * g, sc + 8 * g, w2, &acc[h][4 * g]);
-                            else if (g < groups) promote<WQ, ROWS, 1, true>(t1 + 8 * g, t2 + 8 * g, sc + 8 * g, w2, &acc[h][4 * g]);
+                            if (g + 1 < groups) promote<2, true>(t1 + 8 * g, t2 + 8 * g, sc + 8 * g, w2, &acc[h][4 * g]);
+                            else if (g < groups) promote<1, true>(t1 + 8 * g, t2 + 8 * g, sc + 8 * g, w2, &acc[h][4 * g]);
                         }
                     } else {  // groups is even
                         static_assert(C::JOINT || GROUPS == 10);
-                        if (groups >= 6) promote<WQ, ROWS, 6, false>(t1, 0, sc, w2, acc[h]);
-                        else if (groups == 4) promote<WQ, ROWS, 4, false>(t1, 0, sc, w2, acc[h]);
-                        else promote<WQ, ROWS, 2, false>(t1, 0, sc, w2, acc[h]);
-                        if (groups == 8) promote<WQ, ROWS, 2, false>(t1 + 48, 0, sc + 48, w2, &acc[h][24]);
-                        else if (groups == 10) promote<WQ, ROWS, 4, false>(t1 + 48, 0, sc + 48, w2, &acc[h][24]);
+                        if (groups >= 6) promote<6, false>(t1, 0, sc, w2, acc[h]);
+                        else if (groups == 4) promote<4, false>(t1, 0, sc, w2, acc[h]);
+                        else promote<2, false>(t1, 0, sc, w2, acc[h]);
+                        if (groups == 8) promote<2, false>(t1 + 48, 0, sc + 48, w2, &acc[h][24]);
+                        else if (groups == 10) promote<4, false>(t1 + 48, 0, sc + 48, w2, &acc[h][24]);
                     }
                 }
                 tc_fence_before();
@@ -824,14 +814,14 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                         if (kb + 1 < nkb) next[i] = scale_bits(i, kb + 1);
                     }
                     if (!warp_wait(&rfull[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                    float* sc = sS + ring * C::RING_FLOATS + 2 * ROWS;  // (int4)
+                    float* sc = sS + ring * C::RING_FLOATS + ROWS;  // (int4)
 #pragma unroll
                     for (int i = 0; i < HALVES; ++i) {
                         const int h = h0 + i;
                         const uint8_t* raw = sR + stage * RAW + h * (RAW / 2);
                         uint8_t* dst = sA + stage * A_BYTES + h * (A_BYTES / 2);
                         if constexpr (WQ == GBMOE_INT4_G128)
-                            sc[h * MB + r] = __uint_as_float(bits[i] << 16) * 512.0f;  // bf16; the codes are u * 2^-9
+                            sc[h * MB + r] = __uint_as_float(bits[i] << 16) * 512.0f;  // bf16; the codes are n * 2^-9
                         else
                             *reinterpret_cast<uint32_t*>(sF + stage * C::SF_BYTES + h * 512 + 16 * (r & 31) + 4 * (r >> 5)) =
                                 bits[i];
@@ -1152,10 +1142,7 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     // every row of x once (the shared expert's rows are x's own; a routed row is a token's)
     const int64_t x_rows = p.n_rows / p.pair_div;
     constexpr bool kFour = Cfg<WQ, ROWS>::RAW != 0;  // the order 4-bit weights are decoded in
-    constexpr bool kSums = WQ == GBMOE_INT4_G128;
-    float* a_sum = kSums ? p.a_s + x_rows * (p.H / BK) : nullptr;
-    float* h_sum = kSums ? p.h_s + rows * (p.I / BK) : nullptr;
-    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, kFour, a_sum, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, kFour, stream)) != cudaSuccess) return err;
     const int64_t max_m = sched_max_tiles(experts, rows, tile);
     CUtensorMap mg, mu, md, sg, su, sd;
     if (!map_weights(&mg, WQ, p.w_gate, (int64_t)p.E * p.I, p.H) ||
@@ -1171,18 +1158,18 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     g.counts = p.counts; g.offsets = p.offsets; g.sched = p.sched; g.E = experts; g.n_rows = p.n_rows;
     g.n_shared = p.n_shared;
     g.out = static_cast<__nv_bfloat16*>(p.h); g.err = p.err;
-    g.q = static_cast<const uint8_t*>(p.a_q); g.plane_rows = x_rows; g.a_scale = p.a_s; g.a_sum = a_sum;
+    g.q = static_cast<const uint8_t*>(p.a_q); g.plane_rows = x_rows; g.a_scale = p.a_s;
     g.gather = p.sorted_pair; g.gather_div = p.pair_div;
     g.w_scale0 = p.s_gate; g.w_scale1 = p.s_up; g.s_scale0 = p.ss_gate; g.s_scale1 = p.ss_up;
     auto words = [](const void* s) { return reinterpret_cast<uintptr_t>(s) % 4 == 0; };
     g.scale_words = words(p.s_gate) && words(p.s_up) && words(p.ss_gate) && words(p.ss_up);
     g.wait_limit_ns = tc_wait_limit_ns();
     if ((err = launch_gemm<WQ, ROWS, true>(mg, mu, sg, su, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
-    if ((err = launch_quant_rows(p.h, nullptr, 1, rows, p.I, p.h_q, p.h_s, kFour, h_sum, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.h, nullptr, 1, rows, p.I, p.h_q, p.h_s, kFour, stream)) != cudaSuccess) return err;
     Params d = g;
     d.K = p.I; d.n_tiles = p.H / (2 * MB); d.out_cols = p.H; d.w_rows_per_expert = p.H;
     d.out = static_cast<__nv_bfloat16*>(p.y);
-    d.q = static_cast<const uint8_t*>(p.h_q); d.plane_rows = rows; d.a_scale = p.h_s; d.a_sum = h_sum;
+    d.q = static_cast<const uint8_t*>(p.h_q); d.plane_rows = rows; d.a_scale = p.h_s;
     d.gather = nullptr; d.gather_div = 1;
     d.w_scale0 = d.w_scale1 = p.s_down; d.s_scale0 = d.s_scale1 = p.ss_down;
     d.scale_words = words(p.s_down) && words(p.ss_down);

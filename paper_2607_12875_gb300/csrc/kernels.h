@@ -67,7 +67,7 @@ struct FfnProblem {
     void* a_q;                  // routes that multiply e4m3 codes: x as two e4m3 code planes (value and
                                 //   residual), [2, rows, H] in sorted order (row-major fp8 GEMM) or
                                 //   token order (feature-major GEMM)
-    float* a_s;                 //   and their 1x128 scales [rows, H/128] (int4: then the sums of codes, the same)
+    float* a_s;                 //   and their 1x128 scales [rows, H/128]
     void* h_q;                  //   h the same way, [2, n_rows, I]
     float* h_s;                 //   and its 1x128 scales [n_rows, I/128]
     // Feature-major GEMM: the shared expert (same I and weight format) as one more
@@ -130,9 +130,9 @@ constexpr int64_t kFmFp8RowsPerExpert = 52;
 constexpr int64_t kFmMxfp4RowsPerExpert = 64;
 constexpr int64_t kFmRowsPerExpert = 40;
 // rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales;
-// four_bit: in the order 4-bit weights are decoded in, with the blocks' sums of codes in int4_sums if not null
+// four_bit: in the order 4-bit weights are decoded in
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, bool four_bit, float* int4_sums, cudaStream_t stream);
+                              float* s, bool four_bit, cudaStream_t stream);
 // the same of every row of src once, row r's codes written to rows pair_pos[r * k ..] of [2, n_src * k, K]
 cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
                                  cudaStream_t stream);

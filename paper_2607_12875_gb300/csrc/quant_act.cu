@@ -25,8 +25,7 @@ __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
 }
 
 // kFourBit: the order that 4-bit weights are decoded in (ffn_fm.cu): within 8
-// consecutive values the even ones come before the odd ones; sums[n_rows][K/128]
-// (int4, else null) receive the blocks' sum of codes, sum(q1 + q2) / 64.
+// consecutive values the even ones come before the odd ones.
 //
 // Rows of src [*, K] -> code planes q [2][n_rows][K] and scales s
 // [n_rows][K/128]. Row r reads source row gather[r] / gather_div (r itself
@@ -40,8 +39,7 @@ template <bool kFourBit, bool kScatter>
 __global__ void __launch_bounds__(QWARPS * 32)
 quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ gather, int gather_div,
                   const int32_t* __restrict__ scatter, int n_copies,
-                  int64_t n_rows, int K, uint8_t* __restrict__ q, float* __restrict__ s,
-                  float* __restrict__ sums) {
+                  int64_t n_rows, int K, uint8_t* __restrict__ q, float* __restrict__ s) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int nblk = K / QB, parts = (nblk + QU - 1) / QU;
@@ -90,13 +88,6 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
             const float rr[4] = {t[0] - lo.x, t[1] - lo.y, t[2] - hi.x, t[3] - hi.y};
             const uint32_t a2 = e4m3x2(rr[0], rr[1]) | (e4m3x2(rr[2], rr[3]) << 16);
             if constexpr (kFourBit) {
-                if (sums) {
-                    const float2 lo2 = e4m3x2_to_f32x2(a2 & 0xffffu), hi2 = e4m3x2_to_f32x2(a2 >> 16);
-                    float sum = (lo.x + lo.y + hi.x + hi.y) + (lo2.x + lo2.y + hi2.x + hi2.y);
-#pragma unroll
-                    for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-                    if (lane == 0) sums[r * nblk + b] = sum * 0.015625f;
-                }
                 // this lane's values are 0..3 (even lane) or 4..7 of 8: the even two, then the odd two
                 const int64_t at = r * K + b * QB + 8 * (lane >> 1) + 2 * (lane & 1);
                 *reinterpret_cast<uint16_t*>(q + at) = (uint16_t)__byte_perm(a, 0, 0x4420);
@@ -124,7 +115,7 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
 
 static cudaError_t launch_quant(const void* src, const int32_t* gather, int gather_div, const int32_t* scatter,
                                 int n_copies, int64_t n_rows, int K, void* q, float* s, bool four_bit,
-                                float* int4_sums, cudaStream_t stream) {
+                                cudaStream_t stream) {
     const int64_t units = n_rows * ((K / QB + QU - 1) / QU);
     const int blocks = (int)min64((units + QWARPS - 1) / QWARPS, (int64_t)sm_count() * 16);
     if (blocks <= 0) return cudaSuccess;
@@ -132,19 +123,19 @@ static cudaError_t launch_quant(const void* src, const int32_t* gather, int gath
                   : four_bit  ? quant_rows_kernel<true, false>
                               : quant_rows_kernel<false, false>;
     return launch_k(kernel, dim3(blocks), dim3(QWARPS * 32), 0, stream, static_cast<const __nv_bfloat16*>(src), gather, gather_div, scatter, n_copies, n_rows, K,
-                    static_cast<uint8_t*>(q), s, int4_sums);
+                    static_cast<uint8_t*>(q), s);
 }
 
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, bool four_bit, float* int4_sums, cudaStream_t stream) {
-    return launch_quant(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, four_bit, int4_sums, stream);
+                              float* s, bool four_bit, cudaStream_t stream) {
+    return launch_quant(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, four_bit, stream);
 }
 
 // 2048 tokens x 8 copies, H 7168: 45 us, against 86 quantising each of the
 // 16384 gathered rows (every one a full read and all the arithmetic again).
 cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
                                  cudaStream_t stream) {
-    return launch_quant(src, nullptr, 1, pair_pos, k, n_src, K, q, s, false, nullptr, stream);
+    return launch_quant(src, nullptr, 1, pair_pos, k, n_src, K, q, s, false, stream);
 }
 
 }  // namespace gbmoe

@@ -78,6 +78,56 @@ def test_not_finite_rows_stay_in_their_token(wq):
     assert torch.isfinite(b[6:8].float()).all() and float(b[6].float().abs().max()) == 0.0
 
 
+CODED = ["fp8_b128", "int4_g128", "mxfp4"]
+
+
+def one_hot(wq, rows, K):
+    """[1, rows, K] weights in the format wq, row n being 1.0 at k = n where there is such a k."""
+    n = np.arange(min(rows, K))
+    if wq == "fp8_b128":
+        w = np.zeros((1, rows, K), np.uint8)
+        w[0, n, n] = 0x38
+        return w, np.ones((1, rows // 128, K // 128), np.float32)
+    w = np.zeros((1, rows, K // 2), np.uint8)
+    w[0, n, n // 2] = (2 if wq == "mxfp4" else 1) << (4 * (n % 2)).astype(np.uint8)
+    if wq == "mxfp4":
+        return w, np.full((1, rows, K // 32), 127, np.uint8)
+    return w, np.full((1, rows, K // 128), 0x3F80, np.uint16)
+
+
+# 16-, 32- and 80-row tiles; fp8: the row-major GEMM with both codes stacked and with a pass each
+@pytest.mark.parametrize("wq,T", [(wq, T) for wq in CODED for T in (4, 16, 40)] + [("fp8_b128", 64), ("fp8_b128", 200)])
+def test_activation_codes_keep_every_value(wq, T):
+    """Every element of x, and every element of h, on its own way through the
+    two-code activations: gate rows pick a constant, up and down rows one element
+    each, so out[t, n] = bf16(silu(g) * x[t, n]). All values are positive and
+    most of them large, so that a block's sum is 2^15 times its smallest value, and
+    lie within 2^9, so that the two codes hold them exactly: each comes out within
+    bf16 rounding."""
+    H, I = 512, 256
+    rng = np.random.default_rng(T)
+    x = rng.uniform(1, 2, (T, H)) * 2.0 ** np.where(rng.random((T, H)) < 0.8, -1, rng.integers(-9, 0, (T, H)))
+    g = 8.0
+    x[:, H - 1] = g  # (in a block of its own: up rows pick the first I)
+    xd = torch.from_numpy(x).float().cuda().bfloat16()
+    w_up, s = one_hot(wq, I, H)
+    w_gate = np.zeros_like(w_up)
+    w_gate[..., -1] = 0x38 if wq == "fp8_b128" else (2 if wq == "mxfp4" else 1) << 4
+    w_down, s_down = one_hot(wq, H, I)
+    dev = lambda a: torch.from_numpy(a.view(np.int16) if a.dtype == np.uint16 else a).cuda()
+    d = {k: dev(v) for k, v in dict(w_gate=w_gate, w_up=w_up, w_down=w_down, s_gate=s, s_up=s, s_down=s_down).items()}
+    cfg = gb.make_config(T, H, I, 1, 1, act="bf16", w=wq)
+    ws, out = workspace(cfg), torch.empty((T, H), dtype=torch.bfloat16, device="cuda")
+    gb.moe_forward(cfg, xd, torch.zeros((1, H), dtype=torch.bfloat16, device="cuda"), None, None, wbundle(d), None, out, ws)
+    torch.cuda.synchronize()
+    assert gb.moe_device_status(ws) == gb.OK
+    got, xs = act_np(out), act_np(xd)[:, :I]
+    h = g / (1 + np.exp(-g)) * xs
+    worst = np.max(np.abs(got[:, :I] - h) / (2.0**-8 * np.abs(h)))
+    assert worst <= 1.0, worst
+    assert np.all(got[:, I:] == 0)
+
+
 def test_mxfp4_scales_at_two_byte_alignment():
     """E8M0 scale tensors need only 2-byte alignment."""
     wl = BASE.replace(T=20, E=8, top_k=2, H=512, I=256, wq="mxfp4", seed=9)
