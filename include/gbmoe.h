@@ -71,14 +71,18 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
 /* Which expert-FFN kernels run. GBMOE_FFN_TC_FP8 (FP8_E4M3_B128 weights and
  * bf16 activations only) multiplies the stored e4m3 weights on the fp8 tensor
  * cores: each GEMM's input rows (x, then h) are brought to e4m3 with one
- * power-of-two scale s per row and 128 consecutive k (the block's largest
- * |x / s| lies in [128, 256)) as two codes, q1 = e4m3(x / s) and
- * q2 = e4m3(x / s - q1), so that x = s * (q1 + q2) exactly where
- * |x / s| >= 2^-2 and within 2^-10 * s below that; both codes are
- * multiplied with the weights and each 128-wide k block's partial sum is
- * scaled by both blocks' scales and accumulated in fp32. AUTO takes it for
- * fp8 weights with bf16 activations at every size (with few rows per expert
- * the weights are the GEMM's M operand, with many the rows are).
+ * power-of-two scale s per row and 128 consecutive k as two codes, q1 =
+ * e4m3(x / s) and q2 = e4m3((x / s - q1) * 2^j), so that x is about
+ * s * (q1 + 2^-j * q2); both codes are multiplied with the weights and each
+ * 128-wide k block's partial sum is scaled by both blocks' scales and
+ * accumulated in fp32. With few rows per expert (the weights are the GEMM's M
+ * operand) j = 5 and the block's largest |x / s| lies in [128, 256): a bf16 x is
+ * held exactly where |x / s| >= 2^-7 and within 2^-15 * s below, 2^-22 of the
+ * block's largest value. With many (the rows are the M operand) j = 0 and it lies
+ * in [224, 448]: exactly where |x / s| >= 2^-2 and within 2^-10 * s below, 2^-17
+ * of the block's largest value. A block that holds a NaN contributes NaN; one
+ * with infinities contributes infinities or NaN to every output. AUTO takes it
+ * for fp8 weights with bf16 activations at every size.
  * int4 (MXFP4) weights with bf16 activations and at most 40 (60) rows per
  * expert (P/E) multiply the same activation codes on the fp8 tensor cores under
  * AUTO: every int4 and FP4 value is an e4m3 value; int4's group scales are

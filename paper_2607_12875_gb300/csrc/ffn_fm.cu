@@ -10,9 +10,12 @@
 // with the rows and the weights' way from HBM to the tensor core is left as
 // the bound.
 //
-// Activations enter as two e4m3 codes per value with one power-of-two scale
-// per row and 128 consecutive k, bf16's 8 significant bits in full
-// (quant_act.cu).
+// Activations enter as two e4m3 codes per value with one power-of-two scale s
+// per row and 128 consecutive k, x = s * (q1 + 2^-kLowBits * q2): bf16's 8
+// significant bits in full down to 2^-14 of the 128's largest value, and within
+// 2^-22 of that value below (quant_act.cu). q2's factor 2^-kLowBits is applied in
+// the promotion (short tiles) or by the MMAs, as a scale of their N operand (tall
+// ones, kind::mxf8f6f4 for every format).
 // Products of codes accumulate in fp32 in tensor memory over 128 k, then the
 // promotion warps add the partial sum times its scales to fp32 accumulators
 // in registers.
@@ -65,6 +68,7 @@ constexpr int BK = 128;                 // k per block: one swizzle row, one act
 constexpr int A_BYTES = 2 * MB * BK;    // the two 128-row halves of an item's weight tile
 constexpr int TMEM_COLS = 512;
 constexpr int GATHER_WARPS = 2;
+constexpr float kLowScale = 1.0f / (1 << kLowBits);  // of a second code
 constexpr int SMEM_BUDGET = 232448;
 // MXFP4 whose tiles TMA unpacks: 16 E2M1 codes of 8 bytes become 8 bytes and 8
 // bytes of padding in shared memory, which kind::mxf8f6f4 reads as they are
@@ -87,13 +91,17 @@ struct Cfg {
     static constexpr int SLOTS = BLOCK_SCALE && ROWS == 32 ? 3 : 4;  // (MXFP4's scales need columns too)
     static constexpr int SLOT_COLS = JOINT ? 4 * ROWS : ROWS;
     static constexpr int X_COL = SLOTS * SLOT_COLS;
-    // MXFP4: the MMAs' scale factors in TMEM. Ones for the rows (8 columns), then
-    // weight scales, 4 columns per 128-row half, as many k blocks' as can have
-    // MMAs in flight: the wait for a slot of partial sums then covers its scales,
-    // which the MMAs that filled the slot before were the last to read.
+    // The scale factors in TMEM of MMAs that scale. 8 columns of ones, for the
+    // rows' first codes (and weights whose scales are applied in fp32); tall
+    // tiles: 8 of 2^-kLowBits, for the second codes; MXFP4: weight scales, 4
+    // columns per 128-row half, as many k blocks' as can have MMAs in flight: the
+    // wait for a slot of partial sums then covers its scales, which the MMAs that
+    // filled the slot before were the last to read.
+    static constexpr bool MX = BLOCK_SCALE || !JOINT;
     static constexpr int SF_COL = X_COL + (JOINT ? 0 : ROWS);
+    static constexpr int SFA_COL = SF_COL + (JOINT ? 8 : 16);
     static constexpr int SF_BLOCKS = JOINT ? SLOTS : 2;
-    static constexpr int SF_COLS = BLOCK_SCALE ? 8 + 8 * SF_BLOCKS : 0;
+    static constexpr int SF_COLS = MX ? SFA_COL - SF_COL + (BLOCK_SCALE ? 8 * SF_BLOCKS : 0) : 0;
     static constexpr int SF_BYTES = BLOCK_SCALE ? 2 * 512 : 0;  // a stage's weight scales in shared memory
     static constexpr int SETS = JOINT ? 1 : 2;  // of four promotion warps
     static constexpr int PROMOTE_WARPS = 4 * SETS;
@@ -224,11 +232,6 @@ __device__ __forceinline__ float2 unpack2(uint64_t v) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
     return r;
 }
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
     uint64_t r;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -272,25 +275,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t t, uint32_t (&a)[8]) {
                  : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7])
                  : "r"(t));
 }
-// the wait for the loads above; their registers pass through it, so that no
-// use of them moves above it
-__device__ __forceinline__ void tmem_wait(uint32_t (&a)[8], uint32_t (&b)[8]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
-                   "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
-                 :
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_wait(uint32_t (&a)[8], uint32_t (&b)[8], uint32_t (&c)[8], uint32_t (&d)[8]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
-                   "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]),
-                   "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6]), "+r"(c[7]),
-                   "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7])
-                 :
-                 : "memory");
-}
-
 // after the wait for the load: the registers pass through here, so that no use
 // of them moves above the wait (volatile statements keep their order)
 __device__ __forceinline__ void tmem_pin(uint32_t (&a)[8]) {
@@ -306,7 +290,8 @@ __device__ __forceinline__ void promote8(const uint64_t (&v)[4], const float* sc
     for (int i = 0; i < 4; ++i) acc[i] = fma2(v[i], mul2(f[i], w), acc[i]);
 }
 
-// Promotes N groups of 8 rows: all their loads in flight, one wait. SIDE: the q2 sums are at t2, and added.
+// Promotes N groups of 8 rows: all their loads in flight, one wait. SIDE: the q2 sums are at t2, and added
+// times 2^-kLowBits.
 template <int N, bool SIDE>
 __device__ __forceinline__ void promote(uint32_t t1, uint32_t t2, const float* sc, uint64_t w, uint64_t* acc) {
     uint32_t a[N][8], b[SIDE ? N : 1][8];
@@ -327,7 +312,7 @@ __device__ __forceinline__ void promote(uint32_t t1, uint32_t t2, const float* s
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             v[i] = pack2u(a[g][2 * i], a[g][2 * i + 1]);
-            if constexpr (SIDE) v[i] = add2(v[i], pack2u(b[g][2 * i], b[g][2 * i + 1]));
+            if constexpr (SIDE) v[i] = fma2(pack2u(b[g][2 * i], b[g][2 * i + 1]), pack2(kLowScale, kLowScale), v[i]);
         }
         promote8(v, sc + 8 * g, w, acc + 4 * g);
     }
@@ -442,12 +427,15 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    if constexpr (C::BLOCK_SCALE) {  // the rows' scale factors: ones (E8M0 127)
+    if constexpr (C::MX) {  // the rows' scale factors, as E8M0 bytes
         if (warp >= 4 && warp < 8) {
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(
-                             tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + C::SF_COL),
-                         "r"(0x7f7f7f7fu)
-                         : "memory");
+            const uint32_t t = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + C::SF_COL;
+            auto fill = [](uint32_t at, uint32_t v) {
+                asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(at), "r"(v)
+                             : "memory");
+            };
+            fill(t, 127u * 0x01010101u);
+            if constexpr (!C::JOINT) fill(t + 8, (127u - kLowBits) * 0x01010101u);
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         }
         tc_fence_before();
@@ -504,7 +492,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             const Work wk = decode_work(p, w);
             const int rp = __shfl_sync(0xffffffffu, rows_pad<C::JOINT>(wk.rows), 0);  // warp-uniform
             const int n = C::JOINT ? 2 * rp : rp;
-            const uint32_t idesc = C::BLOCK_SCALE ? idesc_mxf8<C::UNPACKED>(n) : idesc_f8(n);
+            const uint32_t idesc = C::MX ? idesc_mxf8<C::UNPACKED>(n) : idesc_f8(n);
             for (int kb = 0; kb < nkb; ++kb, ++kc) {
                 if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 // the row codes were written through the generic proxy (cp.async)
@@ -521,7 +509,8 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                     }
                     const uint32_t d = tmem_base + slot * C::SLOT_COLS + (C::JOINT ? half * 2 * ROWS : 0);
                     const uint64_t dh = da0 + (uint64_t)((stage * A_BYTES + half * (MB * BK)) >> 4);
-                    const uint32_t sfb = tmem_base + C::SF_COL, sfa = sfb + 8 + kc % C::SF_BLOCKS * 8 + half * 4;
+                    const uint32_t sfb = tmem_base + C::SF_COL;
+                    const uint32_t sfa = C::BLOCK_SCALE ? tmem_base + C::SFA_COL + kc % C::SF_BLOCKS * 8 + half * 4 : sfb;
                     if (elect_one()) {
                         if constexpr (C::BLOCK_SCALE)  // (a copy runs before the MMAs issued after it)
                             tmem_copy_scales(sfa, smem_u32(sF + stage * C::SF_BYTES + half * 512));
@@ -531,8 +520,8 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                             for (int j = 0; j < BK / 32; ++j) {  // +32 bytes along K per instruction
                                 const uint32_t accumulate = pass + j != 0 ? 1u : 0u;
                                 const uint64_t bj = (pass ? db2 : db) + 2 * j;
-                                if constexpr (C::BLOCK_SCALE)
-                                    mma_mxf8(d, dh + 2 * j, bj, idesc | (uint32_t)j << 29, sfa, sfb, accumulate);
+                                if constexpr (C::MX)
+                                    mma_mxf8(d, dh + 2 * j, bj, idesc | (uint32_t)j << 29, sfa, sfb + 8 * pass, accumulate);
                                 else mma_f8(d, dh + 2 * j, bj, idesc, accumulate);
                             }
                         if (half == 1 || !C::JOINT) mma_commit(&pfull[slot]);
@@ -1142,7 +1131,7 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     // every row of x once (the shared expert's rows are x's own; a routed row is a token's)
     const int64_t x_rows = p.n_rows / p.pair_div;
     constexpr bool kFour = Cfg<WQ, ROWS>::RAW != 0;  // the order 4-bit weights are decoded in
-    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, kFour, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, kFour, kLowBits, stream)) != cudaSuccess) return err;
     const int64_t max_m = sched_max_tiles(experts, rows, tile);
     CUtensorMap mg, mu, md, sg, su, sd;
     if (!map_weights(&mg, WQ, p.w_gate, (int64_t)p.E * p.I, p.H) ||
@@ -1165,7 +1154,7 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     g.scale_words = words(p.s_gate) && words(p.s_up) && words(p.ss_gate) && words(p.ss_up);
     g.wait_limit_ns = tc_wait_limit_ns();
     if ((err = launch_gemm<WQ, ROWS, true>(mg, mu, sg, su, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
-    if ((err = launch_quant_rows(p.h, nullptr, 1, rows, p.I, p.h_q, p.h_s, kFour, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.h, nullptr, 1, rows, p.I, p.h_q, p.h_s, kFour, kLowBits, stream)) != cudaSuccess) return err;
     Params d = g;
     d.K = p.I; d.n_tiles = p.H / (2 * MB); d.out_cols = p.H; d.w_rows_per_expert = p.H;
     d.out = static_cast<__nv_bfloat16*>(p.y);

@@ -129,11 +129,13 @@ bool ffn_tc_fp8_supported(const FfnProblem& p);
 constexpr int64_t kFmFp8RowsPerExpert = 52;
 constexpr int64_t kFmMxfp4RowsPerExpert = 64;
 constexpr int64_t kFmRowsPerExpert = 40;
-// rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales;
-// four_bit: in the order 4-bit weights are decoded in
+// Factor 2^-kLowBits between the feature-major GEMM's second codes and its first (quant_act.cu).
+constexpr int kLowBits = 5;
+// rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales, the
+// second codes times 2^-low (low: kLowBits, or 0 without four_bit); four_bit: in the order 4-bit weights are decoded in
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, bool four_bit, cudaStream_t stream);
-// the same of every row of src once, row r's codes written to rows pair_pos[r * k ..] of [2, n_src * k, K]
+                              float* s, bool four_bit, int low, cudaStream_t stream);
+// the same (low 0) of every row of src once, row r's codes written to rows pair_pos[r * k ..] of [2, n_src * k, K]
 cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
                                  cudaStream_t stream);
 cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream);

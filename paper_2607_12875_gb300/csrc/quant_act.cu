@@ -1,14 +1,21 @@
 // Activation rows as two e4m3 codes per value, the operand of the fp8 tensor
-// cores: with s the power of two that brings the largest magnitude of a row's
-// 128 consecutive values into [128, 256), v = x / s (exact), q1 = e4m3(v) and
-// q2 = e4m3(v - q1). A bf16 value has 8 significant bits and the two codes
-// hold 4 each, so x = s * (q1 + q2) exactly for every |v| >= 2^-2 and within
-// 2^-10 * s below that (2^-17 of the block's largest value).
+// cores: with one power of two s per row and 128 consecutive values, v = x / s
+// (exact), q1 = e4m3(v) and q2 = e4m3((v - q1) * 2^kLow), so that x is
+// s * (q1 + 2^-kLow * q2). A bf16 value has 8 significant bits and the two codes
+// hold 4 each; what limits them is e4m3's lowest bit, 2^-9.
+//   kLow = 5 (feature-major GEMM, which scales the second codes' sums apart): s
+//     brings the block's largest magnitude into [128, 256), so that q2 just fits;
+//     x is exact for every |v| >= 2^-7 and within 2^-15 * s below that, 2^-22 of
+//     the block's largest value. Beside an outlier 10^4 times the rest of its
+//     block the rest keeps a relative accuracy of 2^-9, bf16's own.
+//   kLow = 0 (row-major fp8 GEMM, which adds both codes' products up in the same
+//     columns): s brings it into [224, 448], as far up as e4m3 goes; x is exact
+//     for every |v| >= 2^-2 and within 2^-10 * s below that.
 //
 // Bound by its writes (two codes per value) once there are rows enough. One
 // warp takes 4 blocks of a row, not a whole row: 48 rows of 7168 quantised in
 // 4.2 us against 22.4 us with a warp per row, and the exact scaling needs no
-// division (16384 gathered rows: see launch_quant_rows).
+// division (16384 gathered rows: see launch_quant_scatter).
 #include <cuda_fp8.h>
 
 #include "common.cuh"
@@ -35,7 +42,7 @@ __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
 // 4l .. 4l+3 of a block. A block that holds an infinity gets the codes +-1
 // there, 0 elsewhere and an infinite scale, so its sums are infinite as they
 // should be; a NaN makes the scale NaN.
-template <bool kFourBit, bool kScatter>
+template <bool kFourBit, bool kScatter, int kLow>
 __global__ void __launch_bounds__(QWARPS * 32)
 quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ gather, int gather_div,
                   const int32_t* __restrict__ scatter, int n_copies,
@@ -70,12 +77,12 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
 #pragma unroll
             for (int i = 0; i < 4; ++i) m = max(m, __float_as_uint(v[i]) & 0x7fffffffu);
             m = __reduce_max_sync(0xffffffffu, m);
-            // s = 2^(exponent of the largest - 7), at least 2^-126
-            const int e = max((int)(m >> 23) - 7, 1);
+            // s = 2^(exponent of the largest - 7), or - 8 where it then is at most 448; at least 2^-126
+            const int e = max((int)(m >> 23) - (kLow == 0 && (m & 0x7fffffu) <= 0x600000u ? 8 : 7), 1);
             float sc = __uint_as_float((uint32_t)e << 23);
             float t[4];
             if (m < 0x7f800000u) {
-                const float inv = __uint_as_float((uint32_t)(254 - e) << 23);  // 1 / s, exact (e >= 1, <= 247)
+                const float inv = __uint_as_float((uint32_t)(254 - e) << 23);  // 1 / s, exact (1 <= e <= 247)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) t[i] = v[i] * inv;
             } else {
@@ -85,7 +92,8 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
             }
             const uint32_t a = e4m3x2(t[0], t[1]) | (e4m3x2(t[2], t[3]) << 16);
             const float2 lo = e4m3x2_to_f32x2(a & 0xffffu), hi = e4m3x2_to_f32x2(a >> 16);
-            const float rr[4] = {t[0] - lo.x, t[1] - lo.y, t[2] - hi.x, t[3] - hi.y};
+            constexpr float kUp = 1 << kLow;
+            const float rr[4] = {(t[0] - lo.x) * kUp, (t[1] - lo.y) * kUp, (t[2] - hi.x) * kUp, (t[3] - hi.y) * kUp};
             const uint32_t a2 = e4m3x2(rr[0], rr[1]) | (e4m3x2(rr[2], rr[3]) << 16);
             if constexpr (kFourBit) {
                 // this lane's values are 0..3 (even lane) or 4..7 of 8: the even two, then the odd two
@@ -114,28 +122,29 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
 }
 
 static cudaError_t launch_quant(const void* src, const int32_t* gather, int gather_div, const int32_t* scatter,
-                                int n_copies, int64_t n_rows, int K, void* q, float* s, bool four_bit,
+                                int n_copies, int64_t n_rows, int K, void* q, float* s, bool four_bit, int low,
                                 cudaStream_t stream) {
     const int64_t units = n_rows * ((K / QB + QU - 1) / QU);
     const int blocks = (int)min64((units + QWARPS - 1) / QWARPS, (int64_t)sm_count() * 16);
     if (blocks <= 0) return cudaSuccess;
-    auto kernel = scatter     ? quant_rows_kernel<false, true>
-                  : four_bit  ? quant_rows_kernel<true, false>
-                              : quant_rows_kernel<false, false>;
+    auto kernel = scatter     ? quant_rows_kernel<false, true, 0>
+                  : four_bit  ? quant_rows_kernel<true, false, kLowBits>
+                  : low       ? quant_rows_kernel<false, false, kLowBits>
+                              : quant_rows_kernel<false, false, 0>;
     return launch_k(kernel, dim3(blocks), dim3(QWARPS * 32), 0, stream, static_cast<const __nv_bfloat16*>(src), gather, gather_div, scatter, n_copies, n_rows, K,
                     static_cast<uint8_t*>(q), s);
 }
 
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, bool four_bit, cudaStream_t stream) {
-    return launch_quant(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, four_bit, stream);
+                              float* s, bool four_bit, int low, cudaStream_t stream) {
+    return launch_quant(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, four_bit, low, stream);
 }
 
 // 2048 tokens x 8 copies, H 7168: 45 us, against 86 quantising each of the
 // 16384 gathered rows (every one a full read and all the arithmetic again).
 cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
                                  cudaStream_t stream) {
-    return launch_quant(src, nullptr, 1, pair_pos, k, n_src, K, q, s, false, stream);
+    return launch_quant(src, nullptr, 1, pair_pos, k, n_src, K, q, s, false, 0, stream);
 }
 
 }  // namespace gbmoe

@@ -96,17 +96,20 @@ def one_hot(wq, rows, K):
 
 
 # 16-, 32- and 80-row tiles; fp8: the row-major GEMM with both codes stacked and with a pass each
+@pytest.mark.parametrize("spread", [9, 24])
 @pytest.mark.parametrize("wq,T", [(wq, T) for wq in CODED for T in (4, 16, 40)] + [("fp8_b128", 64), ("fp8_b128", 200)])
-def test_activation_codes_keep_every_value(wq, T):
+def test_activation_codes_keep_every_value(wq, T, spread):
     """Every element of x, and every element of h, on its own way through the
     two-code activations: gate rows pick a constant, up and down rows one element
     each, so out[t, n] = bf16(silu(g) * x[t, n]). All values are positive and
-    most of them large, so that a block's sum is 2^15 times its smallest value, and
-    lie within 2^9, so that the two codes hold them exactly: each comes out within
-    bf16 rounding."""
+    most of them large, so that a block's sum is 2^15 times its smallest value.
+    Within 2^9 of each other the two codes hold them exactly, and each comes out
+    within bf16 rounding; over 2^24 there is also (for x and for h) half of the
+    second code's lowest bit, 2^-22 of the block's largest value (row-major GEMM:
+    2^-17, the largest being at least 224 and the bit 2^-9)."""
     H, I = 512, 256
     rng = np.random.default_rng(T)
-    x = rng.uniform(1, 2, (T, H)) * 2.0 ** np.where(rng.random((T, H)) < 0.8, -1, rng.integers(-9, 0, (T, H)))
+    x = rng.uniform(1, 2, (T, H)) * 2.0 ** np.where(rng.random((T, H)) < 0.8, -1, rng.integers(-spread, 0, (T, H)))
     g = 8.0
     x[:, H - 1] = g  # (in a block of its own: up rows pick the first I)
     xd = torch.from_numpy(x).float().cuda().bfloat16()
@@ -123,9 +126,36 @@ def test_activation_codes_keep_every_value(wq, T):
     assert gb.moe_device_status(ws) == gb.OK
     got, xs = act_np(out), act_np(xd)[:, :I]
     h = g / (1 + np.exp(-g)) * xs
-    worst = np.max(np.abs(got[:, :I] - h) / (2.0**-8 * np.abs(h)))
+    top = np.abs(h).reshape(T, I // 128, 128).max(-1).repeat(128, axis=1)
+    low = 0.0 if spread == 9 else 2.0 ** (-17 if T >= 64 else -22)
+    worst = np.max(np.abs(got[:, :I] - h) / (2.0**-8 * np.abs(h) + 2 * low * top))
     assert worst <= 1.0, worst
     assert np.all(got[:, I:] == 0)
+
+
+@pytest.mark.parametrize("wq", CODED)
+@pytest.mark.parametrize("T", [8, 24, 60])
+def test_values_beside_an_outlier_keep_their_precision(T, wq):
+    """One channel in 128 of x, and (4-bit formats) of h, is 2^12 or more times the
+    others, and every weight is 0 there, so that the output is made of the others
+    alone: 16-, 32- and 80-row tiles. 1e-2: bf16 rounding of h and y (5e-3 at most
+    over rows of this length), and as much again for codes that end at 2^-22 of
+    the outlier."""
+    wl = BASE.replace(T=T, E=4, top_k=2, H=512, I=384, wq=wq, seed=T)
+    inp = synth.make_inputs(wl)
+    inp["x"].reshape(-1, 128)[:, 5] = 0x4600  # bf16 8192
+    inp["w_router"].reshape(-1, 128)[:, 5] = 0
+    ex = inp["experts"]
+    for k in ("w_gate", "w_up"):
+        if wq == "fp8_b128":
+            ex[k][..., 5::128] = 0
+        else:
+            ex[k][..., 2::64] &= 0x0F  # (the high nibble of byte 2 is channel 5)
+    if wq != "fp8_b128":
+        for k in ("s_gate", "s_up"):  # rows 9, 137, .. times 2^7: h there about 2^14 times the rest
+            ex[k][:, 9::128] += 7 if wq == "mxfp4" else 7 << 7
+        ex["w_down"][..., 4::64] &= 0x0F
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], 1e-2)
 
 
 def test_mxfp4_scales_at_two_byte_alignment():
