@@ -83,15 +83,16 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * of the block's largest value. A block that holds a NaN contributes NaN; one
  * with infinities contributes infinities or NaN to every output. AUTO takes it
  * for fp8 weights with bf16 activations at every size.
- * int4 (MXFP4) weights with bf16 activations and at most 40 (60) rows per
+ * int4 (MXFP4) weights with bf16 activations and at most 40 (64) rows per
  * expert (P/E) multiply the same activation codes on the fp8 tensor cores under
- * AUTO: every int4 and FP4 value is an e4m3 value; int4's group scales are
- * applied in fp32 per 128 k, the E8M0 scales by the MMAs (kind::mxf8f6f4).
- * This too is reported as GBMOE_FFN_TC.
+ * AUTO (as GBMOE_FFN_TC): every int4 and FP4 value is an e4m3 value; int4's group
+ * scales are applied in fp32 per 128 k, the E8M0 scales by the MMAs
+ * (kind::mxf8f6f4).
  * Otherwise AUTO streams weights when P/E is at most 16 and otherwise runs the
- * grouped GEMM (tensor cores for bf16 activations, CUDA cores for fp32). (With
- * bf16 weights and activations AUTO's STREAM and TC run the feature-major
- * tensor-core GEMM from one row per expert to 40.) On the tensor cores,
+ * grouped GEMM (tensor cores for bf16 activations, CUDA cores for fp32). With
+ * bf16 weights and activations AUTO runs the feature-major tensor-core GEMM from
+ * one row per expert to 40, as whichever of STREAM and TC P/E calls for;
+ * gbmoe_ffn_kernel says which kernels run. On the tensor cores,
  * int4/MXFP4 weights are decoded inside the GEMM when P/E < 400; with
  * more rows per expert (several M tiles reuse each weight tile) AUTO takes
  * GBMOE_FFN_TC_DEQUANT: one pass decodes the active experts' weights to a
@@ -116,6 +117,12 @@ enum {
                                  (each CTA holds half the weight tile); bf16
                                  weights only (quantised: TC_PAIR_DEQUANT)          */
     GBMOE_FFN_TC_PAIR_DEQUANT = 7 /* as TC_DEQUANT, the bf16 GEMM on CTA pairs      */
+};
+
+/* What gbmoe_ffn_kernel reports besides these routes (no values of ffn_route). */
+enum {
+    GBMOE_FFN_FM = 16,     /* feature-major tcgen05 GEMM: the weights are its M operand */
+    GBMOE_FFN_JOINED = 17  /* shared expert: one more expert of the routed launches     */
 };
 
 /* How the MoE Gate computes the router logits. SIMT: CUDA cores in the fixed
@@ -206,10 +213,17 @@ int gbmoe_check_config(const gbmoe_config* cfg);
  * other calls need no more). 0 if the config is invalid. */
 size_t gbmoe_workspace_size(const gbmoe_config* cfg);
 
-/* The FFN route (one of GBMOE_FFN_STREAM .. _TC_PAIR_DEQUANT) that moe_forward runs for
- * cfg: for the routed experts (shared = 0) or the shared expert (shared = 1).
- * Negative status if the config is invalid. */
+/* The FFN route (one of GBMOE_FFN_STREAM .. _TC_PAIR_DEQUANT) of cfg: what was
+ * asked for, or AUTO's choice, for the routed experts (shared = 0) or the shared
+ * expert on its own (shared = 1). Negative status if the config is invalid. */
 int gbmoe_ffn_route(const gbmoe_config* cfg, int shared);
+
+/* The FFN kernels that moe_forward launches for cfg, for the routed experts
+ * (shared = 0) or the shared expert (shared = 1): GBMOE_FFN_FM where a route's
+ * problem runs on the feature-major GEMM, GBMOE_FFN_JOINED for a shared expert
+ * that runs in the routed experts' launches (moe_shared_ffn, called by itself,
+ * runs its own route), else the route. Negative status if the config is invalid. */
+int gbmoe_ffn_kernel(const gbmoe_config* cfg, int shared);
 
 /* The gate route (GBMOE_GATE_SIMT or _TC) that moe_route and moe_forward run
  * for cfg. Negative status if the config is invalid. */
@@ -328,10 +342,12 @@ int moe_forward_hostio(const gbmoe_config* cfg, const void* x_host, const void* 
  * Reads (and clears) the device error word that bounded device-side waits
  * set in `workspace`, after synchronising `stream`. *status receives GBMOE_OK
  * or GBMOE_EDEVICE_TIMEOUT. This is the only call that synchronises.
- * The waits are those of the tensor-core FFN kernels (the GBMOE_FFN_TC*
- * routes): each gives up after 2 s, stops issuing work, lets the copies
+ * The waits are those of the tensor-core kernels (the GBMOE_FFN_TC* routes, the
+ * feature-major GEMM that AUTO's STREAM may run as, see gbmoe_ffn_kernel, and the
+ * tensor-core gate): each gives up after 2 s, stops issuing work, lets the copies
  * and MMAs it issued finish, and sets the word; the call's outputs are then
- * incomplete. For tests of this path the environment variable
+ * incomplete. moe_forward clears the word at its start; the other calls only add
+ * to what the workspace held. For tests of this path the environment variable
  * GBMOE_TC_WAIT_LIMIT_NS (read at every call) lowers the limit, in ns.
  */
 int moe_device_status(void* workspace, void* stream, int32_t* status);

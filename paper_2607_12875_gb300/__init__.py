@@ -28,11 +28,11 @@ GATES = {"auto": GATE_AUTO, "simt": GATE_SIMT, "tc": GATE_TC}
 COMBINES = {"auto": COMBINE_AUTO, "separate": COMBINE_SEPARATE, "fused": COMBINE_FUSED}
 ROUTES = {"auto": FFN_AUTO, "stream": FFN_STREAM, "simt": FFN_SIMT, "tc": FFN_TC, "tc_dequant": FFN_TC_DEQUANT,
           "tc_fp8": FFN_TC_FP8, "tc_pair": FFN_TC_PAIR, "tc_pair_dequant": FFN_TC_PAIR_DEQUANT}
+KERNELS = {**ROUTES, "fm": 16, "joined": 17}  # what ffn_kernel reports
 
 # every function include/gbmoe.h declares
 EXPORTS = ("gbmoe_status_string", "gbmoe_check_config", "gbmoe_workspace_size", "gbmoe_ffn_route",
-           "gbmoe_gate_route", "moe_route",
-           "moe_permute",
+           "gbmoe_ffn_kernel", "gbmoe_gate_route", "moe_route", "moe_permute",
            "moe_grouped_ffn", "moe_shared_ffn", "moe_combine", "moe_forward", "moe_forward_hostio",
            "moe_device_status", "moe_permute_noalloc", "gbmoe_last_cuda_error", "moe_rmsnorm")
 
@@ -82,6 +82,7 @@ def lib() -> ctypes.CDLL:
         L.gbmoe_workspace_size.argtypes = [cfgp]
         L.gbmoe_workspace_size.restype = sz
         L.gbmoe_ffn_route.argtypes = [cfgp, ctypes.c_int]
+        L.gbmoe_ffn_kernel.argtypes = [cfgp, ctypes.c_int]
         L.gbmoe_gate_route.argtypes = [cfgp]
         L.moe_route.argtypes = [cfgp, vp, vp, fp, fp, vp, vp, vp, sz, vp]
         L.moe_rmsnorm.argtypes = [cfgp, vp, vp, ctypes.c_float, vp, vp]
@@ -150,11 +151,20 @@ def workspace_size(cfg: Config) -> int:
 
 
 def ffn_route(cfg: Config, shared: bool = False) -> str:
-    """Name of the FFN route moe_forward runs for cfg ("stream", "simt", "tc", "tc_dequant", "tc_fp8")."""
+    """Name of cfg's FFN route, asked for or AUTO's choice (a key of ROUTES other than "auto")."""
     r = lib().gbmoe_ffn_route(ctypes.byref(cfg), int(bool(shared)))
     if r < 0:
         raise GbmoeError(r, "gbmoe_ffn_route")
     return {v: k for k, v in ROUTES.items()}[r]
+
+
+def ffn_kernel(cfg: Config, shared: bool = False) -> str:
+    """Name of the FFN kernels moe_forward launches for cfg: "fm" (feature-major GEMM), "joined" (a shared
+    expert in the routed launches) or the route."""
+    r = lib().gbmoe_ffn_kernel(ctypes.byref(cfg), int(bool(shared)))
+    if r < 0:
+        raise GbmoeError(r, "gbmoe_ffn_kernel")
+    return {v: k for k, v in KERNELS.items()}[r]
 
 
 def moe_rmsnorm(cfg, x, gamma, eps, y, stream=None):

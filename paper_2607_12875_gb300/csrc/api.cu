@@ -423,6 +423,15 @@ int gbmoe_ffn_route(const gbmoe_config* cfg, int shared) {
     return pick_route(cfg, (int64_t)cfg->T * cfg->top_k, cfg->E, cfg->I);
 }
 
+int gbmoe_ffn_kernel(const gbmoe_config* cfg, int shared) {
+    const int route = gbmoe_ffn_route(cfg, shared);
+    if (route < 0) return route;
+    if (shared && shared_joins(cfg)) return GBMOE_FFN_JOINED;
+    const bool fm = shared ? use_fm(cfg, cfg->T, 1, cfg->I_shared)
+                           : use_fm(cfg, (int64_t)cfg->T * cfg->top_k, cfg->E, cfg->I);
+    return fm ? GBMOE_FFN_FM : route;
+}
+
 int gbmoe_gate_route(const gbmoe_config* cfg) {
     int s = check_cfg(cfg);
     return s ? s : pick_gate(cfg);

@@ -15,8 +15,15 @@ pytestmark = pytest.mark.gpu
 BASE = synth.WORKLOADS[1].replace(act="bf16")
 
 
+# what runs beyond the feature-major GEMM's last row per expert, and that row
+BEYOND = {"bf16": (40, "tc"), "fp8_b128": (52, "tc_fp8"), "int4_g128": (40, "tc"), "mxfp4": (64, "tc")}
+
+
 def forward(wl, dev):
     cfg = config(wl)
+    most, other = BEYOND[wl.wq]
+    few = wl.wq == "bf16" and wl.P < wl.E
+    assert gb.ffn_kernel(cfg) == ("fm" if wl.P <= most * wl.E and not few else "stream" if few else other)
     ws = workspace(cfg)
     out = torch.empty((wl.T, wl.H), dtype=torch.bfloat16, device="cuda")
     gb.moe_forward(cfg, dev["x"], dev["w_router"], dev["logit_bias"], dev["select_bias"], wbundle(dev["experts"]),
@@ -24,6 +31,30 @@ def forward(wl, dev):
     torch.cuda.synchronize()
     assert gb.moe_device_status(ws) == gb.OK
     return out
+
+
+@pytest.mark.parametrize("wq", list(BEYOND))
+def test_which_kernels_run(wq):
+    """The route is AUTO's choice by rows per expert; the kernels reported are
+    those launched, on both sides of each limit, for forced routes and for a
+    shared expert in the routed launches or by itself."""
+    most, other = BEYOND[wq]
+    cfg = lambda T, **kw: gb.make_config(T, 4096, 4096, 4, 1, act="bf16", w=wq, **kw)
+    assert gb.ffn_kernel(cfg(4 * most)) == "fm"
+    assert gb.ffn_kernel(cfg(4 * most + 1)) == other == gb.ffn_route(cfg(4 * most + 1))
+    assert gb.ffn_kernel(cfg(40, ffn_route="simt")) == "simt"
+    assert gb.ffn_kernel(cfg(40, ffn_route="tc")) == "tc"
+    if wq == "bf16":
+        assert gb.ffn_kernel(cfg(3)) == "stream" and gb.ffn_kernel(cfg(4)) == "fm"
+        assert gb.ffn_route(cfg(4)) == "stream" and gb.ffn_route(cfg(65)) == "tc"
+    else:
+        assert gb.ffn_route(cfg(40)) == ("tc_fp8" if wq == "fp8_b128" else "tc")
+    same = dict(has_shared=True, I_shared=4096)
+    assert gb.ffn_kernel(cfg(40, **same), shared=True) == ("fm" if wq == "bf16" else "joined")
+    assert gb.ffn_kernel(cfg(40, has_shared=True, I_shared=2048), shared=True) == "fm"
+    assert gb.ffn_kernel(cfg(40, ffn_route="tc", **same), shared=True) == "tc"
+    wide = gb.make_config(513, 4096, 4096, 64, 1, act="bf16", w=wq, **same)  # more tokens than join
+    assert gb.ffn_kernel(wide) == "fm" and gb.ffn_kernel(wide, shared=True) == gb.ffn_route(wide, shared=True)
 
 
 # rows per expert: 1, groups of 8 and one more, whole 16-row tiles, the last
