@@ -81,9 +81,11 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * block's largest value. With many (the rows are the M operand) j = 0 and it lies
  * in [224, 448]: exactly where |x / s| >= 2^-2 and within 2^-10 * s below, 2^-17
  * of the block's largest value. A block that holds a NaN contributes NaN; one
- * with infinities contributes infinities or NaN to every output. AUTO takes it
- * for fp8 weights with bf16 activations at every size.
- * int4 (MXFP4) weights with bf16 activations and at most 40 (64) rows per
+ * with infinities contributes infinities or NaN to every output.
+ * AUTO: with bf16 activations and so few rows that P - 1 <= c * (1/H + 1/I) (c:
+ * 12000 for bf16 weights, 5000 fp8, 4800 int4, 1600 MXFP4) and P/E at most 16,
+ * the weights are streamed. Else fp8 weights take GBMOE_FFN_TC_FP8, and
+ * int4 (MXFP4) weights with at most 40 (64) rows per
  * expert (P/E) multiply the same activation codes on the fp8 tensor cores under
  * AUTO (as GBMOE_FFN_TC): every int4 and FP4 value is an e4m3 value; int4's group
  * scales are applied in fp32 per 128 k, the E8M0 scales by the MMAs

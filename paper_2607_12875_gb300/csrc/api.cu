@@ -80,6 +80,13 @@ int64_t fm_rows_per_expert(int w_dtype) {
                                           : kFmRowsPerExpert;
 }
 
+// Whether a problem has so few rows that AUTO streams its weights whatever their
+// format (few_rows in kernels.h).
+bool streams_few_rows(const gbmoe_config* c, int64_t n_rows, int E, int I) {
+    return c->act_dtype == GBMOE_BF16 && n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I) &&
+           (double)(n_rows - 1) <= few_rows(c->w_dtype) * (1.0 / c->H + 1.0 / I);
+}
+
 // Kernel route for an FFN problem with n_rows rows over E experts.
 int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     int r = c->ffn_route;
@@ -90,8 +97,9 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     probe.H = c->H;
     probe.I = I;
     probe.E = E;
-    // fp8 weights with bf16 activations: the fp8 tensor-core route at every
-    // size (no decode; its two-term activation codes keep bf16's accuracy)
+    if (streams_few_rows(c, n_rows, E, I)) return GBMOE_FFN_STREAM;
+    // fp8 weights with bf16 activations: the fp8 tensor-core route from there on
+    // (no decode; its two-term activation codes keep bf16's accuracy)
     if (ffn_tc_fp8_supported(probe)) return GBMOE_FFN_TC_FP8;
     // int4 and MXFP4 weights with bf16 activations and few rows per expert: the
     // feature-major GEMM (use_fm), reported as TC
@@ -126,6 +134,7 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     probe.I = I;
     if (n_rows > fm_rows_per_expert(c->w_dtype) * E || !ffn_fm_supported(probe)) return false;
     if (c->w_dtype == GBMOE_BF16 && n_rows < kFmBf16MinRowsPerExpert * E) return false;
+    if (c->ffn_route == GBMOE_FFN_AUTO && streams_few_rows(c, n_rows, E, I)) return false;
     return c->w_dtype == GBMOE_FP8_E4M3_B128 ? pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8
                                              : c->ffn_route == GBMOE_FFN_AUTO && c->combine_route != GBMOE_COMBINE_FUSED;
 }

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/gbmoe.h"
+
 namespace gbmoe {
 
 struct RouteParams {
@@ -106,6 +108,25 @@ constexpr int64_t kPairDequantRowsPerExpert = 400;
 // expert: 71 us streaming against 73, 0.13: 111 against 120, 0.5: 299 against
 // 306).
 constexpr int64_t kFmBf16MinRowsPerExpert = 1;
+// A layer with few rows in all streams, in any format: up to 1 + few_rows * (1/H +
+// 1/I) rows. Streaming splits an expert's weights over the SMs, and its time grows with
+// rows x H x I; the feature-major GEMM with few items on its list (I / 128 per
+// expert with rows, H / 256 in the down GEMM) takes H / 128 and then I / 128 k
+// blocks one after the other, whatever the rows. Where the two meet was measured
+// on 14 shapes from H 1024, I 768 to H 4096, I 6144 and from 1 expert to 128,
+// 1 to 96 rows: the lines below are within 11 % of the better one everywhere, and on
+// the streaming side where it is close. Streaming against feature-major, one expert, H 4096, I 1536, with
+// the gate: bf16 31 against 51 us at 1 row, 49 against 53 at 6, 57 against 55 at 16;
+// fp8 29 and 46 at 1, 53 and 48 at 6; int4 30 and 56 at 1, 63 and 59 at 6; MXFP4 36
+// and 50 at 1, 53 and 51 at 3. 8 experts, top 2, H 2048, I 512: fp8 26 and 34 at 2
+// rows, 38 and 36 at 16.
+constexpr double few_rows(int w_dtype) {
+    return w_dtype == GBMOE_BF16            ? 12000.0
+           : w_dtype == GBMOE_FP8_E4M3_B128 ? 5000.0
+           : w_dtype == GBMOE_INT4_G128     ? 4800.0
+           : w_dtype == GBMOE_MXFP4         ? 1600.0
+                                            : 0.0;
+}
 cudaError_t launch_ffn_stream(const FfnProblem& p, cudaStream_t stream);
 size_t stream_smem_bytes(int act_dtype, int H, int I);  // per CTA, streaming route
 // dynamic shared memory a CTA may use on sm_103a (227 KB); a streaming problem

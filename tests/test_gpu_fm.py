@@ -15,15 +15,26 @@ pytestmark = pytest.mark.gpu
 BASE = synth.WORKLOADS[1].replace(act="bf16")
 
 
-# what runs beyond the feature-major GEMM's last row per expert, and that row
-BEYOND = {"bf16": (40, "tc"), "fp8_b128": (52, "tc_fp8"), "int4_g128": (40, "tc"), "mxfp4": (64, "tc")}
+# the feature-major GEMM's last row per expert, what runs beyond it, and the rows
+# (less one) times H * I / (H + I) up to which the weights are streamed instead
+LIMITS = {"bf16": (40, "tc", 12000), "fp8_b128": (52, "tc_fp8", 5000), "int4_g128": (40, "tc", 4800),
+          "mxfp4": (64, "tc", 1600)}
 
 
-def forward(wl, dev):
+def few_rows(wq, H, I):
+    return 1 + int(LIMITS[wq][2] * (1 / H + 1 / I))
+
+
+def kernel_of(wl):
+    most, beyond, _ = LIMITS[wl.wq]
+    if wl.P <= min(few_rows(wl.wq, wl.H, wl.I), 16 * wl.E) or (wl.wq == "bf16" and wl.P < wl.E):
+        return "stream"
+    return "fm" if wl.P <= most * wl.E else beyond
+
+
+def forward(wl, dev, kernel="fm"):
     cfg = config(wl)
-    most, other = BEYOND[wl.wq]
-    few = wl.wq == "bf16" and wl.P < wl.E
-    assert gb.ffn_kernel(cfg) == ("fm" if wl.P <= most * wl.E and not few else "stream" if few else other)
+    assert gb.ffn_kernel(cfg) == kernel
     ws = workspace(cfg)
     out = torch.empty((wl.T, wl.H), dtype=torch.bfloat16, device="cuda")
     gb.moe_forward(cfg, dev["x"], dev["w_router"], dev["logit_bias"], dev["select_bias"], wbundle(dev["experts"]),
@@ -33,25 +44,27 @@ def forward(wl, dev):
     return out
 
 
-@pytest.mark.parametrize("wq", list(BEYOND))
+@pytest.mark.parametrize("wq", list(LIMITS))
 def test_which_kernels_run(wq):
     """The route is AUTO's choice by rows per expert; the kernels reported are
     those launched, on both sides of each limit, for forced routes and for a
     shared expert in the routed launches or by itself."""
-    most, other = BEYOND[wq]
+    most, other, _ = LIMITS[wq]
     cfg = lambda T, **kw: gb.make_config(T, 4096, 4096, 4, 1, act="bf16", w=wq, **kw)
     assert gb.ffn_kernel(cfg(4 * most)) == "fm"
     assert gb.ffn_kernel(cfg(4 * most + 1)) == other == gb.ffn_route(cfg(4 * most + 1))
     assert gb.ffn_kernel(cfg(40, ffn_route="simt")) == "simt"
     assert gb.ffn_kernel(cfg(40, ffn_route="tc")) == "tc"
     if wq == "bf16":
-        assert gb.ffn_kernel(cfg(3)) == "stream" and gb.ffn_kernel(cfg(4)) == "fm"
-        assert gb.ffn_route(cfg(4)) == "stream" and gb.ffn_route(cfg(65)) == "tc"
+        deep = lambda T: gb.make_config(T, 4096, 4096, 16, 1, act="bf16", w=wq)
+        assert gb.ffn_kernel(deep(15)) == "stream" and gb.ffn_kernel(deep(16)) == "fm"
+        assert gb.ffn_route(deep(16)) == "stream" and gb.ffn_route(deep(257)) == "tc"
     else:
         assert gb.ffn_route(cfg(40)) == ("tc_fp8" if wq == "fp8_b128" else "tc")
     same = dict(has_shared=True, I_shared=4096)
     assert gb.ffn_kernel(cfg(40, **same), shared=True) == ("fm" if wq == "bf16" else "joined")
     assert gb.ffn_kernel(cfg(40, has_shared=True, I_shared=2048), shared=True) == "fm"
+    assert gb.ffn_kernel(cfg(2, **same), shared=True) == {"mxfp4": "joined"}.get(wq, "stream")
     assert gb.ffn_kernel(cfg(40, ffn_route="tc", **same), shared=True) == "tc"
     wide = gb.make_config(513, 4096, 4096, 64, 1, act="bf16", w=wq, **same)  # more tokens than join
     assert gb.ffn_kernel(wide) == "fm" and gb.ffn_kernel(wide, shared=True) == gb.ffn_route(wide, shared=True)
@@ -61,23 +74,40 @@ def test_which_kernels_run(wq):
 # size with the shortest tiles (4 rows per expert on average), 16 and 17 (the next
 # tile height) and the first without,
 # the last before the row-major GEMM takes over; one k block and ragged rings
+# (few rows of small matrices are streamed: the last six are large enough)
 @pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T,E,k,H,I", [(1, 8, 2, 256, 128), (8, 4, 1, 512, 128), (9, 1, 1, 256, 256),
                                        (4, 1, 1, 768, 384), (32, 16, 2, 1024, 128), (33, 16, 2, 256, 640),
                                        (40, 1, 1, 512, 256), (63, 4, 2, 1280, 256),
-                                       (16, 1, 1, 512, 128), (17, 1, 1, 512, 128), (52, 1, 1, 256, 384), (53, 1, 1, 256, 128)])
+                                       (16, 1, 1, 512, 128), (17, 1, 1, 512, 128), (52, 1, 1, 256, 384), (53, 1, 1, 256, 128),
+                                       (8, 64, 2, 1024, 512), (8, 2, 1, 4096, 4096), (40, 10, 1, 1024, 512),
+                                       (9, 1, 1, 4096, 2560), (16, 1, 1, 2048, 1536), (32, 16, 2, 1024, 256)])
 def test_row_tiles(T, E, k, H, I, wq):
     wl = BASE.replace(T=T, E=E, top_k=k, H=H, I=I, wq=wq, seed=T + 7 * E)
     inp = synth.make_inputs(wl)
-    out = forward(wl, to_device(wl, inp))
+    out = forward(wl, to_device(wl, inp), kernel_of(wl))
     assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol_for(wl))
+
+
+@pytest.mark.parametrize("E,k", [(1, 1), (8, 2)])
+@pytest.mark.parametrize("wq", list(LIMITS))
+def test_few_rows_are_streamed(wq, E, k):
+    """The last size whose weights are streamed and the first that takes the
+    feature-major GEMM, against the oracle and against each other's rows."""
+    wl = BASE.replace(E=E, top_k=k, H=2048, I=1024, wq=wq, seed=E)
+    last = min(few_rows(wq, wl.H, wl.I), 16 * E) // k
+    for T, kernel in ((last, "stream"), (last + 1, "fm")):
+        w = wl.replace(T=T)
+        assert kernel_of(w) == kernel
+        inp = synth.make_inputs(w)
+        assert_close(act_np(forward(w, to_device(w, inp), kernel)), oracle.forward(w, inp)["out"], tol_for(w))
 
 
 @pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
 @pytest.mark.parametrize("T", [16, 17, 32, 33, 80, 81, 200])
 def test_all_rows_on_one_expert(T, wq):
     """A hot expert's rows fill whole row tiles and spill into the next."""
-    wl = BASE.replace(T=T, E=16, top_k=2, H=512, I=256, wq=wq, seed=T)
+    wl = BASE.replace(T=T, E=16, top_k=2, H=2048, I=512, wq=wq, seed=T)
     inp = synth.make_inputs(wl)
     bias = np.zeros(wl.E, np.float32)
     bias[3] = 1000.0
@@ -92,7 +122,7 @@ def test_not_finite_rows_stay_in_their_token(wq):
     """An infinity or NaN in one token's activations leaves every other token's
     output bit for bit as it was; its own output is not finite. Values whose
     squares or quotients would leave fp32's range are scaled exactly."""
-    wl = BASE.replace(T=24, E=8, top_k=2, H=512, I=256, wq=wq, seed=5)
+    wl = BASE.replace(T=24, E=8, top_k=2, H=1024, I=512, wq=wq, seed=5)
     inp = synth.make_inputs(wl)
     dev = to_device(wl, inp)
     # the experts are fixed by a bias, so that the routing does not depend on the rows changed below
@@ -126,9 +156,10 @@ def one_hot(wq, rows, K):
     return w, np.full((1, rows, K // 128), 0x3F80, np.uint16)
 
 
-# 16-, 32- and 80-row tiles; fp8: the row-major GEMM with both codes stacked and with a pass each
+# all rows on one of eight experts: 16-, 32- and 80-row tiles; fp8: the row-major GEMM's 128-row tiles, a pass
+# for each code, and a last one of 64 rows with both codes stacked
 @pytest.mark.parametrize("spread", [9, 24])
-@pytest.mark.parametrize("wq,T", [(wq, T) for wq in CODED for T in (4, 16, 40)] + [("fp8_b128", 64), ("fp8_b128", 200)])
+@pytest.mark.parametrize("wq,T", [(wq, T) for wq in CODED for T in (32, 128, 320)] + [("fp8_b128", 448)])
 def test_activation_codes_keep_every_value(wq, T, spread):
     """Every element of x, and every element of h, on its own way through the
     two-code activations: gate rows pick a constant, up and down rows one element
@@ -138,7 +169,7 @@ def test_activation_codes_keep_every_value(wq, T, spread):
     within bf16 rounding; over 2^24 there is also (for x and for h) half of the
     second code's lowest bit, 2^-22 of the block's largest value (row-major GEMM:
     2^-17, the largest being at least 224 and the bit 2^-9)."""
-    H, I = 512, 256
+    E, H, I = 8, 512, 256
     rng = np.random.default_rng(T)
     x = rng.uniform(1, 2, (T, H)) * 2.0 ** np.where(rng.random((T, H)) < 0.8, -1, rng.integers(-spread, 0, (T, H)))
     g = 8.0
@@ -150,15 +181,17 @@ def test_activation_codes_keep_every_value(wq, T, spread):
     w_down, s_down = one_hot(wq, H, I)
     dev = lambda a: torch.from_numpy(a.view(np.int16) if a.dtype == np.uint16 else a).cuda()
     d = {k: dev(v) for k, v in dict(w_gate=w_gate, w_up=w_up, w_down=w_down, s_gate=s, s_up=s, s_down=s_down).items()}
-    cfg = gb.make_config(T, H, I, 1, 1, act="bf16", w=wq)
+    d = {k: v.expand(E, *v.shape[1:]).contiguous() for k, v in d.items()}
+    cfg = gb.make_config(T, H, I, E, 1, act="bf16", w=wq)
+    assert gb.ffn_kernel(cfg) == ("tc_fp8" if T == 448 else "fm")
     ws, out = workspace(cfg), torch.empty((T, H), dtype=torch.bfloat16, device="cuda")
-    gb.moe_forward(cfg, xd, torch.zeros((1, H), dtype=torch.bfloat16, device="cuda"), None, None, wbundle(d), None, out, ws)
+    gb.moe_forward(cfg, xd, torch.zeros((E, H), dtype=torch.bfloat16, device="cuda"), None, None, wbundle(d), None, out, ws)
     torch.cuda.synchronize()
     assert gb.moe_device_status(ws) == gb.OK
     got, xs = act_np(out), act_np(xd)[:, :I]
     h = g / (1 + np.exp(-g)) * xs
     top = np.abs(h).reshape(T, I // 128, 128).max(-1).repeat(128, axis=1)
-    low = 0.0 if spread == 9 else 2.0 ** (-17 if T >= 64 else -22)
+    low = 0.0 if spread == 9 else 2.0 ** (-17 if T == 448 else -22)
     worst = np.max(np.abs(got[:, :I] - h) / (2.0**-8 * np.abs(h) + 2 * low * top))
     assert worst <= 1.0, worst
     assert np.all(got[:, I:] == 0)
@@ -172,7 +205,7 @@ def test_values_beside_an_outlier_keep_their_precision(T, wq):
     alone: 16-, 32- and 80-row tiles. 1e-2: bf16 rounding of h and y (5e-3 at most
     over rows of this length), and as much again for codes that end at 2^-22 of
     the outlier."""
-    wl = BASE.replace(T=T, E=4, top_k=2, H=512, I=384, wq=wq, seed=T)
+    wl = BASE.replace(T=T, E=4, top_k=2, H=1024, I=768, wq=wq, seed=T)
     inp = synth.make_inputs(wl)
     inp["x"].reshape(-1, 128)[:, 5] = 0x4600  # bf16 8192
     inp["w_router"].reshape(-1, 128)[:, 5] = 0
@@ -249,7 +282,7 @@ def test_mxfp4_scales_of_each_k_block_are_its_own(T):
 
 
 @pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
-@pytest.mark.parametrize("T,I_shared", [(5, 256), (60, 256), (150, 256), (60, 384)])
+@pytest.mark.parametrize("T,I_shared", [(5, 256), (20, 256), (60, 256), (150, 256), (60, 384)])
 def test_shared_expert_with_the_routed_ones(T, I_shared, wq):
     """The shared expert runs as one more expert of the same launches when its
     intermediate size is the routed ones', else by itself; 128 routed experts and
@@ -257,7 +290,9 @@ def test_shared_expert_with_the_routed_ones(T, I_shared, wq):
     wl = BASE.replace(T=T, E=128, top_k=3, H=512, I=256, wq=wq, seed=T, score="sigmoid", routed_scale=2.5, n_group=4,
                       topk_group=2, has_shared=True, I_shared=I_shared, select_bias_sigma=0.01)
     inp = synth.make_inputs(wl)
-    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+    alone = kernel_of(wl) != "fm" or I_shared != wl.I
+    assert gb.ffn_kernel(config(wl), shared=True) == (kernel_of(wl.replace(E=1, top_k=1, I=I_shared)) if alone else "joined")
+    assert_close(act_np(forward(wl, to_device(wl, inp), kernel_of(wl))), oracle.forward(wl, inp)["out"], tol_for(wl))
 
 
 def test_shared_expert_after_512_routed_ones():
@@ -271,7 +306,7 @@ def test_shared_expert_after_512_routed_ones():
 def test_bounded_waits_give_up_and_the_next_call_is_clean(T, wq, monkeypatch):
     """With the wait limit lowered to 0 ns every role of the kernel stops, drains
     what it issued and reports; the next call with the normal limit is clean."""
-    wl = BASE.replace(T=T, E=8, top_k=2, H=1024, I=256, wq=wq, seed=77)
+    wl = BASE.replace(T=T, E=8, top_k=2, H=1024, I=512, wq=wq, seed=77)
     inp = synth.make_inputs(wl)
     dev = to_device(wl, inp)
     cfg = config(wl)
