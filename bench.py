@@ -8,8 +8,8 @@ Weight Sum) over one batch of the workload, through the C ABI (moe_forward)
 on inputs already resident in HBM. The headline workload is the decode-shaped
 bf16 layer: T=32 tokens, hidden 4096, 128 experts, top-8, intermediate 1536;
 the same line carries, under per_config, the same measurements for the
-prefill bf16 (T=8192), DeepSeek-style fp8 (T=2048, 256 + 1 experts) and
-skewed int4 (T=16384) layers. Every workload's active expert weights (1.1 GB
+prefill bf16 (T=8192), DeepSeek-style fp8 and MXFP4 (T=2048, 256 + 1 experts)
+and skewed int4 (T=16384) layers. Every workload's active expert weights (1.1 GB
 and up) exceed the 126 MB L2, so no flush is needed between steps. With N
 GPUs (torchrun) every rank runs its own replica on its own batch (the layer
 has no exchange step here): weak scaling.
@@ -44,7 +44,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # of a reduced case with the same H, I, dtypes and rows per expert as the full
 # workload (the kernels read each active expert's weights and its rows, so the
 # traffic grows with the number of active experts); the bench line reports it
-# times this run's active experts. Keyed by (workload, route); absent (null)
+# times this run's active experts. Keyed by (workload, FFN kernels); absent (null)
 # whenever the kernels changed since the counters were taken. Captures
 # (python bench.py --workload W --set ... --profile 1 under
 # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum):
@@ -55,10 +55,10 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # (the skewed int4 workload's offsets exist for its full size only, so its
 # reduced case differs in I and is not scaled here)
 TRAFFIC_PER_ACTIVE_EXPERT: dict = {
-    ("decode_bf16_T32_H4096_E128_k8_I1536", "stream"): 1.0962e9 / 29,
+    ("decode_bf16_T32_H4096_E128_k8_I1536", "fm"): 1.0962e9 / 29,
     ("prefill_bf16_T8192_H4096_E128_k8_I1536", "tc"): 1.6488e9 / 32,
     ("dsv3_fp8_T2048_H7168_E256s1_k8_I2048", "tc_fp8"): 2.9961e9 / 64,
-    ("dsv4_mxfp4_T2048_H7168_E256s1_k8_I2048", "tc"): 1.6966e9 / 64,
+    ("dsv4_mxfp4_T2048_H7168_E256s1_k8_I2048", "fm"): 1.6966e9 / 64,
 }
 
 
@@ -257,14 +257,35 @@ def workload_config(wl):
             "l2": "no flush: the active experts' weights read each step exceed the 126 MB L2"}
 
 
-# most rows per expert of the feature-major GEMM by quantised weight format
-# (bf16 activations, AUTO), and most tokens of a shared expert that joins it
-FM_ROWS_PER_EXPERT = {"fp8_b128": 52, "int4_g128": 40, "mxfp4": 64}
-FM_JOIN_TOKENS = 512
+# the expert FFN of moe_grouped_ffn by kernels (paper_2607_12875_gb300.ffn_kernel)
+FFN_KERNELS = {
+    "stream": "weight-streaming route (gate/up + down)",
+    "tc": "tcgen05 route (gate/up GEMM gathering its rows, with SwiGLU + down GEMM)",
+    "tc_dequant": "tcgen05 decode-once route (3 weight-decode passes + gate/up GEMM gathering its rows, with SwiGLU + "
+                  "down GEMM)",
+    "tc_fp8": "fp8 tcgen05 route (two-term e4m3 quantisation of the rows + gate/up GEMM with per-k-block promotion and "
+              "SwiGLU + quantisation of h + down GEMM)",
+    "tc_pair": "tcgen05 CTA-pair route (row gather + gate/up GEMM with SwiGLU + down GEMM, cta_group::2 MMAs of 256 rows)",
+    "tc_pair_dequant": "tcgen05 CTA-pair decode-once route (3 weight-decode passes + row gather + gate/up GEMM with SwiGLU "
+                       "+ down GEMM, cta_group::2 MMAs)",
+    "fm": "feature-major tcgen05 GEMM (quantisation of the rows + gate/up GEMM with SwiGLU + quantisation of h + down GEMM)",
+    "simt": "CUDA-core route",
+}
 
 
-def launches_per_step(wl, route: str, shared_route, gate: str = "simt") -> int:
-    """Kernels this library launches per layer forward: gate logits + expert
+def kernel_text(kernel: str, wq: str) -> str:
+    """The bench line's description of the expert FFN's kernels."""
+    text = FFN_KERNELS[kernel]
+    if kernel == "tc" and wq != "bf16":  # decoding GEMMs read a gathered copy of x
+        text = "tcgen05 route (row gather + gate/up GEMM decoding its weight tiles, with SwiGLU + down GEMM)"
+    if kernel == "fm" and wq == "bf16":  # rows as they are
+        text = "feature-major tcgen05 GEMM (gate/up GEMM gathering its rows, with SwiGLU + down GEMM)"
+    return "moe_grouped_ffn, " + text
+
+
+def launches_per_step(wl, kernel: str, shared_kernel, gate: str = "simt") -> int:
+    """Kernels this library launches per layer forward, by what it says runs for
+    the routed experts and the shared one (None: there is none): gate logits + expert
     choice (on the tensor cores: router row norms, schedule, GEMM, choice, two
     recomputing kernels for the flagged tokens and their choice), the
     permutation (one kernel up to 1024 pairs, else three), per FFN problem a
@@ -272,21 +293,16 @@ def launches_per_step(wl, route: str, shared_route, gate: str = "simt") -> int:
     the routes that multiply codes, + a row gather for the routed experts on the
     routes whose GEMM does not gather its rows itself, + 3 weight-decode passes
     on the decode-once routes), and the combine."""
-    def few(routed):  # the feature-major GEMM on coded activations
-        rows, experts = (wl.P, wl.E) if routed else (wl.T, 1)
-        return wl.act == "bf16" and rows <= FM_ROWS_PER_EXPERT.get(wl.wq, 0) * experts
-
     def ffn(r, routed):
-        if r == "tc_fp8" or (r == "tc" and few(routed)):
+        if r == "tc_fp8" or (r == "fm" and wl.wq != "bf16"):
             return 5
         # the one-CTA bf16 GEMM gathers its own rows; decoding GEMMs and pairs use the gather kernel
         gather = r in ("tc_pair", "tc_pair_dequant") or (r == "tc" and wl.wq != "bf16")
         return 3 + (1 if routed and gather else 0) + (3 if r in ("tc_dequant", "tc_pair_dequant") else 0)
 
-    n = (7 if gate == "tc" else 2) + (1 if wl.P <= 1024 else 3) + ffn(route, True) + 1
-    joins = wl.has_shared and wl.I_shared == wl.I and wl.T <= FM_JOIN_TOKENS and few(True)
-    if shared_route is not None and not joins:
-        n += ffn(shared_route, False)
+    n = (7 if gate == "tc" else 2) + (1 if wl.P <= 1024 else 3) + ffn(kernel, True) + 1
+    if shared_kernel not in (None, "joined"):
+        n += ffn(shared_kernel, False)
     return n
 
 
@@ -358,7 +374,7 @@ def measure(args, wid: int, overrides, dist, world: int, rank: int, local: int, 
         for _ in range(args.profile):
             step()
         torch.cuda.synchronize()
-        print(f"profile run: {wl.name} {overrides} route={gb.ffn_route(cfg)} status={gb.moe_device_status(ws)}")
+        print(f"profile run: {wl.name} {overrides} route={gb.ffn_route(cfg)} kernel={gb.ffn_kernel(cfg)} status={gb.moe_device_status(ws)}")
         return None
 
     for _ in range(args.warmup):
@@ -409,31 +425,14 @@ def measure(args, wid: int, overrides, dist, world: int, rank: int, local: int, 
     ffn_ms = fs.elapsed_time(fe) / args.steps
     del y
     pk, pk_kind = peaks()
-    route = gb.ffn_route(cfg)
+    kernel = gb.ffn_kernel(cfg)
     # the expert FFN's roofline: the slower of its algorithmic weight bytes over
     # HBM bandwidth and its FLOPs over the bf16 tensor peak
     routed_bytes = algorithmic_weight_bytes(wl.replace(has_shared=False), active)
     flops = 6.0 * wl.P * wl.H * wl.I
-    kernel = {"stream": "moe_grouped_ffn, weight-streaming route (gate/up + down)",
-              "tc": "moe_grouped_ffn, tcgen05 route (gate/up GEMM gathering its rows, with SwiGLU + down GEMM)",
-              "tc_dequant": "moe_grouped_ffn, tcgen05 decode-once route (3 weight-decode passes + gate/up GEMM "
-                            "gathering its rows, with SwiGLU + down GEMM)",
-              "tc_fp8": "moe_grouped_ffn, fp8 tcgen05 route (two-term e4m3 quantisation of the rows + gate/up "
-                        "GEMM with per-k-block promotion and SwiGLU + quantisation of h + down GEMM)",
-              "tc_pair": "moe_grouped_ffn, tcgen05 CTA-pair route (row gather + gate/up GEMM with SwiGLU + down "
-                         "GEMM, cta_group::2 MMAs of 256 rows)",
-              "tc_pair_dequant": "moe_grouped_ffn, tcgen05 CTA-pair decode-once route (3 weight-decode passes + "
-                                 "row gather + gate/up GEMM with SwiGLU + down GEMM, cta_group::2 MMAs)",
-              "simt": "moe_grouped_ffn, CUDA-core route"}[route]
-    if route == "tc" and wl.wq != "bf16":  # decoding GEMMs read a gathered copy of x
-        kernel = ("moe_grouped_ffn, tcgen05 route (row gather + gate/up GEMM decoding its weight tiles, with "
-                  "SwiGLU + down GEMM)")
-    if wl.act == "bf16" and wl.P <= FM_ROWS_PER_EXPERT.get(wl.wq, 0) * wl.E:
-        kernel = ("moe_grouped_ffn, feature-major tcgen05 GEMM (quantisation of the rows + gate/up GEMM with SwiGLU + "
-                  "quantisation of h + down GEMM)")
-    tpe = TRAFFIC_PER_ACTIVE_EXPERT.get((wl.name, route))
-    extra = {"traffic": None if tpe is None else tpe * active, "kernel": kernel, "active_experts": active,
-             "route": route, "gate": gb.gate_route(cfg)}
+    tpe = TRAFFIC_PER_ACTIVE_EXPERT.get((wl.name, kernel))
+    extra = {"traffic": None if tpe is None else tpe * active, "kernel": kernel_text(kernel, wl.wq),
+             "active_experts": active, "route": gb.ffn_route(cfg), "ffn_kernel": kernel, "gate": gb.gate_route(cfg)}
     roofline = roofline_entry(routed_bytes, flops, ffn_ms, pk, pk_kind, extra)
 
     # end to end through the public host-buffer entry point
@@ -454,7 +453,7 @@ def measure(args, wid: int, overrides, dist, world: int, rank: int, local: int, 
     e2e = {"value": replica_throughput(wl.T, args.steps, world, e2e_s), "unit": "tokens/s",
            "h2d_bytes_per_step": io_bytes, "d2h_bytes_per_step": io_bytes}
 
-    per_step = launches_per_step(wl, route, gb.ffn_route(cfg, shared=True) if wl.has_shared else None,
+    per_step = launches_per_step(wl, kernel, gb.ffn_kernel(cfg, shared=True) if wl.has_shared else None,
                                  gb.gate_route(cfg))
     cpu = cpu_baseline_entry(wl, inp) if with_cpu else None
     del x, wr, lb, sb, experts, shared, keep1, keep2, ws, out, x_host, out_host
@@ -484,7 +483,7 @@ def main():
     ap.add_argument("--ref-tokens", type=int, default=1, help="tokens per oracle step (reference arm)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-per-config", action="store_true",
-                    help="time only the headline workload (by default workloads 3, 4 and 5 are timed too)")
+                    help="time only the headline workload (by default workloads 3 to 6 are timed too)")
     ap.add_argument("--set", action="append", default=[], metavar="KEY=INT",
                     help="override a workload field (reduced cases for profiling), e.g. --set T=2048 --set E=32")
     ap.add_argument("--profile", type=int, default=0, metavar="N",

@@ -53,3 +53,18 @@ def test_fallback_peaks_have_every_key_the_roofline_reads():
 def test_roofline_without_a_sustained_peak():
     r = bench.roofline_entry(5.0e9, 2.5e12, 2.0, {"hbm_gbs": 6780.0, "bf16_tflops": 1908.6}, "measured", {})
     assert r["bound"] == "tensor" and "frac_sustained" not in r
+
+
+def test_launches_and_text_follow_the_kernels_that_run():
+    """A forced route and AUTO's choice on the same workload differ in launches
+    and description; a joined shared expert launches nothing of its own."""
+    wl = synth.WORKLOADS[6]  # MXFP4, one shared expert, more than 1024 pairs
+    around = 7 + 3 + 1  # tensor-core gate, permutation, Weight Sum
+    assert bench.launches_per_step(wl, "fm", "joined", "tc") == around + 5
+    assert bench.launches_per_step(wl, "fm", "fm", "tc") == around + 5 + 5
+    assert bench.launches_per_step(wl, "tc", "tc", "tc") == around + 4 + 3
+    assert bench.launches_per_step(wl, "stream", None) == 2 + 3 + 3 + 1
+    bf16 = synth.WORKLOADS[2]
+    assert bench.launches_per_step(bf16, "fm", None) == bench.launches_per_step(bf16, "stream", None) == 2 + 1 + 3 + 1
+    assert "feature-major" in bench.kernel_text("fm", "bf16") and "quantisation" not in bench.kernel_text("fm", "bf16")
+    assert "decoding" in bench.kernel_text("tc", "mxfp4") and "quantisation" in bench.kernel_text("fm", "mxfp4")
