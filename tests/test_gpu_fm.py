@@ -32,6 +32,14 @@ def kernel_of(wl):
     return "fm" if wl.P <= most * wl.E else beyond
 
 
+def tol(wl, kernel="fm"):
+    """1e-2 for the feature-major GEMM, whose activation codes keep bf16's
+    precision and whose weights are exact: h and y rounded to bf16 give up to 5e-3
+    of a row's largest value (0.004 to 0.005 measured). Without the second codes
+    these rows are 0.04 to 0.06 off. Other kernels: tol_for."""
+    return 1e-2 if kernel == "fm" else tol_for(wl)
+
+
 def forward(wl, dev, kernel="fm"):
     cfg = config(wl)
     assert gb.ffn_kernel(cfg) == kernel
@@ -86,7 +94,7 @@ def test_row_tiles(T, E, k, H, I, wq):
     wl = BASE.replace(T=T, E=E, top_k=k, H=H, I=I, wq=wq, seed=T + 7 * E)
     inp = synth.make_inputs(wl)
     out = forward(wl, to_device(wl, inp), kernel_of(wl))
-    assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol_for(wl))
+    assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol(wl, kernel_of(wl)))
 
 
 @pytest.mark.parametrize("E,k", [(1, 1), (8, 2)])
@@ -100,7 +108,7 @@ def test_few_rows_are_streamed(wq, E, k):
         w = wl.replace(T=T)
         assert kernel_of(w) == kernel
         inp = synth.make_inputs(w)
-        assert_close(act_np(forward(w, to_device(w, inp), kernel)), oracle.forward(w, inp)["out"], tol_for(w))
+        assert_close(act_np(forward(w, to_device(w, inp), kernel)), oracle.forward(w, inp)["out"], tol(w, kernel))
 
 
 @pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
@@ -114,7 +122,28 @@ def test_all_rows_on_one_expert(T, wq):
     inp["logit_bias"] = bias
     ref = oracle.forward(wl, inp)
     assert ref["counts"][3] == T
-    assert_close(act_np(forward(wl, to_device(wl, inp))), ref["out"], tol_for(wl))
+    assert_close(act_np(forward(wl, to_device(wl, inp))), ref["out"], tol(wl))
+
+
+@pytest.fixture(scope="module", params=list(LIMITS))
+def many_items(request):
+    """A layer whose two GEMMs have more items than a GB300 has SMs at every tile
+    height, so that CTAs take two items and more: its inputs and the oracle's
+    outputs, which tokens share only through the weights."""
+    wl = BASE.replace(T=384, E=24, top_k=2, H=2048, I=2048, wq=request.param, seed=21)
+    inp = synth.make_inputs(wl)
+    return wl, to_device(wl, inp), oracle.forward(wl, inp)["out"]
+
+
+@pytest.mark.parametrize("T", [48, 192, 384])
+def test_more_items_than_sms(many_items, T):
+    """16-, 32- and 80-row tiles (bf16: 16 and 64), the same bits from call to call."""
+    wl, dev, ref = many_items
+    wl = wl.replace(T=T)
+    dev = dict(dev, x=dev["x"][:T])
+    out = forward(wl, dev)
+    assert_close(act_np(out), ref[:T], tol(wl))
+    assert torch.equal(out.view(torch.int16), forward(wl, dev).view(torch.int16))
 
 
 @pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
@@ -231,7 +260,7 @@ def test_mxfp4_scales_at_two_byte_alignment():
         v = dev["experts"][k]
         dev["experts"][k] = torch.cat([v.new_zeros(2), v.flatten()])[2:].view(v.shape)
         assert dev["experts"][k].data_ptr() % 4 == 2
-    assert_close(act_np(forward(wl, dev)), oracle.forward(wl, inp)["out"], tol_for(wl))
+    assert_close(act_np(forward(wl, dev)), oracle.forward(wl, inp)["out"], tol(wl))
 
 
 @pytest.mark.parametrize("T", [8, 40, 120])
@@ -249,8 +278,8 @@ def test_mxfp4_weights_at_16_byte_alignment(T):
         assert dev["experts"][k].data_ptr() % 32 == 16
     got = act_np(forward(wl, dev))
     want = oracle.forward(wl, inp)["out"]
-    assert_close(got, want, tol_for(wl))
-    assert_close(aligned, want, tol_for(wl))
+    assert_close(got, want, tol(wl))
+    assert_close(aligned, want, tol(wl))
 
 
 def test_mxfp4_block_scales_far_apart():
@@ -263,7 +292,7 @@ def test_mxfp4_block_scales_far_apart():
         s = inp["experts"][k]
         inp["experts"][k] = (s.astype(np.int32) - rng.integers(0, 13, s.shape)).astype(np.uint8)
         inp["experts"][k][..., ::8, 1] -= 18
-    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol(wl))
 
 
 @pytest.mark.parametrize("T", [6, 24, 60])
@@ -278,7 +307,7 @@ def test_mxfp4_scales_of_each_k_block_are_its_own(T):
         s = inp["experts"][k].astype(np.int32)
         step = np.repeat(3 * (np.arange(s.shape[-1] // 4) % 3 - 1), 4)
         inp["experts"][k] = (s + step).astype(np.uint8)
-    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol(wl))
 
 
 @pytest.mark.parametrize("wq", ["fp8_b128", "int4_g128", "mxfp4"])
@@ -292,13 +321,13 @@ def test_shared_expert_with_the_routed_ones(T, I_shared, wq):
     inp = synth.make_inputs(wl)
     alone = kernel_of(wl) != "fm" or I_shared != wl.I
     assert gb.ffn_kernel(config(wl), shared=True) == (kernel_of(wl.replace(E=1, top_k=1, I=I_shared)) if alone else "joined")
-    assert_close(act_np(forward(wl, to_device(wl, inp), kernel_of(wl))), oracle.forward(wl, inp)["out"], tol_for(wl))
+    assert_close(act_np(forward(wl, to_device(wl, inp), kernel_of(wl))), oracle.forward(wl, inp)["out"], tol(wl, kernel_of(wl)))
 
 
 def test_shared_expert_after_512_routed_ones():
     wl = BASE.replace(T=40, E=512, top_k=4, H=256, I=128, wq="fp8_b128", seed=3, has_shared=True, I_shared=128)
     inp = synth.make_inputs(wl)
-    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol_for(wl))
+    assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], tol(wl))
 
 
 @pytest.mark.parametrize("wq", ["bf16", "fp8_b128", "int4_g128", "mxfp4"])
@@ -319,4 +348,4 @@ def test_bounded_waits_give_up_and_the_next_call_is_clean(T, wq, monkeypatch):
     monkeypatch.delenv("GBMOE_TC_WAIT_LIMIT_NS")
     gb.moe_forward(*args)
     assert gb.moe_device_status(ws) == gb.OK
-    assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol_for(wl))
+    assert_close(act_np(out), oracle.forward(wl, inp)["out"], tol(wl))

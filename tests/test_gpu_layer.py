@@ -20,7 +20,7 @@ pytestmark = pytest.mark.gpu
 
 ROUTES = {1: ["simt", "stream", "auto"], 2: ["stream", "simt", "auto"], 3: ["simt", "auto", "tc", "tc_pair"],
           4: ["simt", "auto", "tc", "tc_dequant"], 5: ["simt", "auto", "tc", "tc_pair_dequant"],
-          6: ["simt", "auto", "tc_dequant", "tc_pair_dequant"]}
+          6: ["simt", "auto", "tc", "tc_dequant", "tc_pair_dequant"]}
 ALL_ROUTES = ["auto", "stream", "simt", "tc", "tc_dequant", "tc_fp8", "tc_pair", "tc_pair_dequant"]
 
 

@@ -150,8 +150,12 @@ def test_bounded_wait_timeout_is_reported_and_the_next_call_is_clean(wq, pair, m
 
 
 # fp8 tensor-core route (kind::f8f6f4): fp8 weights as stored, activations
-# quantised to e4m3 per 1x128 block; against the oracle with exact
-# activations, within the fp8 bound (5e-2) and per row
+# quantised to two e4m3 codes per 1x128 block; against the oracle with exact
+# activations and per row, within twice what bf16 rounding of h and y gives
+# (5e-3): one code alone leaves 0.04 to 0.06
+CODED_TOL = 1e-2
+
+
 @pytest.mark.parametrize("T,E,k,H,I", [(200, 4, 2, 512, 256), (1000, 4, 2, 256, 384), (333, 16, 3, 768, 128),
                                        (64, 8, 8, 1024, 512)])
 def test_tc_fp8_route_small_ragged(T, E, k, H, I):
@@ -161,7 +165,7 @@ def test_tc_fp8_route_small_ragged(T, E, k, H, I):
     out, ids = forward(wl, dev, "tc_fp8")
     ref = oracle.forward(wl, inp)
     assert np.array_equal(ids.cpu().numpy(), ref["topk_ids"])
-    assert_close(act_np(out), ref["out"], tol_for(wl))
+    assert_close(act_np(out), ref["out"], CODED_TOL)
 
 
 def test_tc_fp8_route_with_shared_expert_and_timeout():
@@ -175,7 +179,7 @@ def test_tc_fp8_route_with_shared_expert_and_timeout():
     out, ids = forward(wl, dev, "tc_fp8")
     ref = oracle.forward(wl, inp)
     assert np.array_equal(ids.cpu().numpy(), ref["topk_ids"])
-    assert_close(act_np(out), ref["out"], tol_for(wl))
+    assert_close(act_np(out), ref["out"], CODED_TOL)
     cfg = config(wl, "tc_fp8")
     ws = workspace(cfg)
     os.environ["GBMOE_TC_WAIT_LIMIT_NS"] = "0"
@@ -186,7 +190,7 @@ def test_tc_fp8_route_with_shared_expert_and_timeout():
     finally:
         del os.environ["GBMOE_TC_WAIT_LIMIT_NS"]
     out2, _ = forward(wl, dev, "tc_fp8")
-    assert_close(act_np(out2), ref["out"], tol_for(wl))
+    assert_close(act_np(out2), ref["out"], CODED_TOL)
 
 
 
