@@ -142,13 +142,16 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
 // Whether moe_forward runs the shared expert as one more expert of the routed
 // problem: on the feature-major GEMM with coded activations, when the two have
 // the same intermediate size and few tokens (its own launches leave most SMs
-// idle; many rows are cheaper on the row-major GEMM). 256 experts, H 7168, I
-// 2048, joined against apart: fp8 1.30 against 1.35 ms at 48 tokens, 2.20
-// against 2.15 at 1024 (MXFP4, before its MMAs scaled by themselves: 0.82
-// against 0.87 at 16, 3.34 against 3.08 at 1024).
-constexpr int kJoinTokens = 512;
+// idle; many rows are cheaper on the row-major GEMM). Joined against apart, ms:
+// fp8, 256 experts, H 7168, I 2048: 0.64 and 0.67 at 16 tokens, 1.36 and 1.42 at
+// 48, 1.78 and 1.79 at 256, 1.87 and 1.83 at 512, 2.18 and 2.14 at 1024; MXFP4, the
+// same layer: 0.52 and 0.57 at 16, 1.33 and 1.39 at 256, 1.52 and 1.78 at 512, 2.27
+// and 2.50 at 1024; int4, 64 experts, top 6, H 4096, I 2816: 0.29 and 0.34 at 16,
+// 0.62 and 0.66 at 256, 0.65 and 0.70 at 400 (512 is beyond its feature-major rows).
+constexpr int kJoinTokensFp8 = 256, kJoinTokens4Bit = 512;
 bool shared_joins(const gbmoe_config* c) {
-    return c->has_shared && c->I_shared == c->I && c->w_dtype != GBMOE_BF16 && c->T <= kJoinTokens &&
+    return c->has_shared && c->I_shared == c->I && c->w_dtype != GBMOE_BF16 &&
+           c->T <= (c->w_dtype == GBMOE_FP8_E4M3_B128 ? kJoinTokensFp8 : kJoinTokens4Bit) &&
            use_fm(c, (int64_t)c->T * c->top_k, c->E, c->I);
 }
 

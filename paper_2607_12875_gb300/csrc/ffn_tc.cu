@@ -154,11 +154,6 @@ struct Params {
     const __nv_bfloat16* a_src;  // x [*, K]
 };
 
-// 16-byte global -> shared copy through L2 (cp.async), tracked by commit groups
-__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-
 // Instruction descriptor, kind::f16: fp32 accumulator (bits 4-5 = 1), bf16 A
 // and B (bits 7-9, 10-12 = 1), both K-major, N/8 in bits 17-22, M/16 in 24-28
 // (M = 128 per CTA, 256 for a CTA pair).

@@ -26,7 +26,7 @@ struct RouteScratch {
     int32_t* flagged;
 };
 
-// logits: fp32 scratch, route_logits(rp) floats; topk_ids, topk_w [T, k]
+// logits: fp32 scratch, T * E floats (gate_tc: gate_tc_splits planes of them); topk_ids, topk_w [T, k]
 cudaError_t launch_route(const RouteParams& rp, const void* x, const void* w_router, const float* logit_bias,
                          const float* select_bias, float* logits, int32_t* topk_ids, float* topk_w,
                          const RouteScratch& rs, cudaStream_t stream);

@@ -121,7 +121,7 @@ static cudaError_t launch_gate_logits(const TA* x, const TA* wg, const float* bi
 constexpr int kGT = 32, kGE = 16, kSlab = 256, kGStages = 3;
 constexpr size_t kGateTiledSmem = (size_t)kGStages * (kGT + kGE) * kSlab * 2;
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
+__device__ __forceinline__ void cp_async_16_or_zero(void* dst, const void* src, bool valid) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
     const int n = valid ? 16 : 0;  // 0 bytes read: the 16 bytes are zero-filled
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
@@ -176,7 +176,7 @@ gate_logits_tiled_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat1
         for (int m = 0; m < kRows; ++m) {
             const int row = warp + 8 * m;
             uint8_t* dst = row < kGT ? sx + ((size_t)st * kGT + row) * kSlab * 2 : sw + ((size_t)st * kGE + row - kGT) * kSlab * 2;
-            cp_async16(dst + 16 * lane, src[m] + (size_t)j * kSlab, ok[m]);
+            cp_async_16_or_zero(dst + 16 * lane, src[m] + (size_t)j * kSlab, ok[m]);
         }
     };
 
