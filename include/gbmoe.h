@@ -95,16 +95,17 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * bf16 weights and activations AUTO runs the feature-major tensor-core GEMM from
  * one row per expert to 40, as whichever of STREAM and TC P/E calls for;
  * gbmoe_ffn_kernel says which kernels run. On the tensor cores,
- * int4/MXFP4 weights are decoded inside the GEMM when P/E < 400; with
- * more rows per expert (several M tiles reuse each weight tile) AUTO takes
+ * int4/MXFP4 weights are decoded inside the GEMM when P/E < 256 to 384 (fewer
+ * rows for fewer weights E * H * I); with more rows per expert (several M tiles reuse each weight tile) AUTO takes
  * GBMOE_FFN_TC_DEQUANT: one pass decodes the active experts' weights to a
  * bf16 copy in the workspace (the same bf16 values the in-GEMM decode makes),
  * then the bf16 GEMM runs on it. The _PAIR routes run the same GEMM on CTA
  * pairs (tcgen05 cta_group::2): one MMA of 256 rows per pair, each CTA
  * holding 128 rows of A and half of the bf16 weight tile, which halves the
  * weight bytes each SM reads per MMA; an expert's rows are then covered in
- * 256-row tiles, so AUTO takes them only from P/E >= 1024 (little padding; from
- * 400 after a decode-once pass).
+ * 256-row tiles, so AUTO takes them only from P/E >= 1024 (little padding; after
+ * a decode-once pass from 400 with H and I of 1280 or more and 256 items of 256
+ * rows x 128 columns).
  * Their outputs equal the one-CTA routes' bit for bit. TC_PAIR needs bf16
  * weights; quantised weights take TC_PAIR_DEQUANT. */
 enum {

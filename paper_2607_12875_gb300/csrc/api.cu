@@ -109,11 +109,12 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     if (n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I)) return GBMOE_FFN_STREAM;
     if (c->act_dtype == GBMOE_BF16) {
         if (ffn_tc_supported(probe)) {
-            const bool dequant = quantised_weights(c->w_dtype) && n_rows >= kDequantRowsPerExpert * E;
+            const bool dequant = quantised_weights(c->w_dtype) && n_rows >= dequant_rows_per_expert(E, c->H, I) * E;
             // CTA pairs (256-row tiles) once experts are deep enough that the
             // padding of their last tile stays small; they multiply bf16 tiles
             if (dequant) probe.w_dq = &probe;
-            const int64_t from = dequant ? kPairDequantRowsPerExpert : kPairRowsPerExpert;
+            const bool wide = dequant && std::min(c->H, I) >= kPairDequantMinWidth && n_rows / 256 * (I / 128) >= kPairDequantMinItems;
+            const int64_t from = wide ? kPairDequantRowsPerExpert : kPairRowsPerExpert;
             const bool pairs = n_rows >= from * E && ffn_tc_pair_supported(probe);
             if (dequant) return pairs ? GBMOE_FFN_TC_PAIR_DEQUANT : GBMOE_FFN_TC_DEQUANT;
             return pairs && c->w_dtype == GBMOE_BF16 ? GBMOE_FFN_TC_PAIR : GBMOE_FFN_TC;

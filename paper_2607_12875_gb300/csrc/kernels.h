@@ -93,15 +93,30 @@ struct FfnProblem {
 
 size_t ffn_sched_ints(int E, int64_t n_rows);
 // AUTO: 4-bit weights are decoded once (TC_DEQUANT) from this many rows per
-// expert on; below, inside the GEMM. int4, 64 experts, H 4096, I 2816: 1.32
-// against 1.85 ms at 192 rows per expert, 2.28 against 2.30 at 384.
-constexpr int64_t kDequantRowsPerExpert = 400;
+// expert on; below, inside the GEMM. With few weights in all the decode pass costs
+// little and its bf16 copy stays in L2; with many it is a full round trip through
+// HBM, while the GEMM has work items enough to hide its own decode. In the GEMM
+// against decoded once, us: 24 experts, H 1024, I 512 (13 M weights a matrix) 114
+// and 103 at 256 rows per expert; 24, 2048, 1024 (50 M) 222 and 221 at 260; 48, 3072,
+// 1024 (151 M) 478 and 498 at 260, 534 and 526 at 300; 40, 4096, 1408 (231 M) 724 and
+// 746 at 349, 910 and 842 at 399; 64, 4096, 2816 (738 M) 2018 and 2184 at 349, 2432 and
+// 2428 at 399.
+inline int64_t dequant_rows_per_expert(int E, int H, int I) {
+    const int64_t weights = (int64_t)E * H * I;
+    return weights < 90000000 ? 256 : weights < 200000000 ? 288 : weights < 400000000 ? 352 : 384;
+}
 // AUTO: CTA pairs from this many rows per expert on. bf16, 128 experts, H 4096,
 // I 1536, pairs against single CTAs: 2.245 and 2.252 ms at 512 rows per expert,
-// 3.93 and 3.99 at 1024; after a decode-once pass 2.30 and 2.35 at 384 (int4
-// as above).
+// 3.93 and 3.99 at 1024.
 constexpr int64_t kPairRowsPerExpert = 1024;
+// After a decode-once pass, with wide experts and enough 256-row items, from here
+// on (pairs against single CTAs, us: I 4096, 8 experts, H 4096, 486 and 546 at 400
+// rows per expert; I 2816 2488 and 2627 at 499; I 1280, 16 experts, H 4096, 359 and 352
+// at 400, 440 and 458 at 700; I 512, 40 experts, 560 and 512 at 700; one expert of I
+// 2688, H 1536, 809 rows: layer 106 and 101).
 constexpr int64_t kPairDequantRowsPerExpert = 400;
+constexpr int kPairDequantMinWidth = 1280;  // H and I
+constexpr int64_t kPairDequantMinItems = 256;  // of 256 rows x 128 gate and up rows
 // bf16 weights stream on the CUDA cores below this many rows per expert: a
 // weight then meets one row or two, and the streaming CTAs split a few experts'
 // weights finer than the feature-major items (the same layer at 0.06 rows per

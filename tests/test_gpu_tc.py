@@ -111,7 +111,7 @@ def test_dequant_route_with_shared_expert_and_inactive_experts():
 def test_auto_route_choice():
     """AUTO: streaming for decode; fp8 weights on the fp8 tensor-core route;
     int4/MXFP4 decoded in the GEMM for few rows per expert, decoded once for
-    many; CTA pairs for deep experts (>= 1024 rows each)."""
+    many; CTA pairs for deep experts (the lines between: the next test)."""
     assert gb.ffn_route(config(synth.WORKLOADS[2])) == "stream"
     assert gb.ffn_route(config(synth.WORKLOADS[3])) == "tc"
     assert gb.ffn_route(config(synth.WORKLOADS[4])) == "tc_fp8"
@@ -119,6 +119,19 @@ def test_auto_route_choice():
     assert gb.ffn_route(config(synth.WORKLOADS[5])) == "tc_pair_dequant"  # 1536 rows per expert: CTA pairs
     assert gb.ffn_route(config(synth.WORKLOADS[6])) == "tc"
     assert gb.ffn_route(config(synth.WORKLOADS[6]), shared=True) == "tc_pair_dequant"
+
+
+@pytest.mark.parametrize("E,H,I,first,pairs_from", [(24, 1024, 512, 256, 1024), (48, 3072, 1024, 288, 1024),
+                                                    (40, 4096, 1408, 352, 400), (64, 4096, 2816, 384, 400),
+                                                    (1, 1536, 2688, 256, 1024)])
+def test_decode_once_and_pairs_by_size(E, H, I, first, pairs_from):
+    """AUTO's lines for 4-bit weights: the rows per expert from which they are
+    decoded once (by the number of weights), and from which that takes CTA pairs
+    (wide experts with enough work items, else 1024 rows)."""
+    for wq in ("int4_g128", "mxfp4"):
+        route = lambda rows: gb.ffn_route(gb.make_config(rows * E, H, I, E, 1, act="bf16", w=wq))
+        assert route(first - 1) == "tc" and route(first) == "tc_dequant"
+        assert route(pairs_from - 1) == "tc_dequant" and route(pairs_from) == "tc_pair_dequant"
 
 
 @pytest.mark.parametrize("pair", [False, True])
