@@ -30,28 +30,29 @@ constexpr int kNT = 8;      // activation rows per weight pass
 constexpr int kMaxGroupsPerCta = 4;
 constexpr int kMinWaves = 8;
 
-// CTAs per SM the register budget is set for: two for plain weights; quantised
-// ones decode more per element and get the whole register file
-template <int WQ>
-constexpr int stream_min_blocks() { return WQ == GBMOE_BF16 || WQ == GBMOE_F32 ? 2 : 1; }
+// CTAs per SM the register budget is set for: two for plain weights (fp32: kTwo,
+// see two_ctas); quantised ones decode more per element and get the whole register
+// file
+template <int WQ, bool kTwo>
+constexpr int stream_min_blocks() { return WQ == GBMOE_BF16 || (WQ == GBMOE_F32 && kTwo) ? 2 : 1; }
 
 // 8-element (or 16-byte) chunks of a row loaded before use. fp32: two of 32 bytes
 // fit 128 registers, so two CTAs share an SM; with four one CTA took it alone
 // (tiny fp32 layer: gate/up 17.2 -> 12.0 us, the passes apart as well, see
 // passes_apart; 4 tokens of 16 experts, H 1024, I 768: layer 56 -> 42 us).
-template <int WQ>
-constexpr int kUnroll = WQ == GBMOE_F32 ? 2 : 4;
+template <int WQ, bool kTwo>
+constexpr int kUnroll = WQ == GBMOE_F32 && kTwo ? 2 : 4;
 
 // acc[q][r] += W_q . xs[r] for 4 weight rows q (byte pointers wrow, scale rows
 // srow) and NT activation rows r in shared memory (row stride K).
-template <typename TA, int WQ, int NT>
+template <typename TA, int WQ, int NT, bool kTwo>
 __device__ __forceinline__ void dot4(const uint8_t* const (&wrow)[4], const void* const (&srow)[4], const TA* xs,
                                      int K, float (&acc)[4][NT]) {
     using F = WFmt<WQ>;
     const int lane = threadIdx.x & 31;
     const int nchunk = K / F::CE;
     constexpr int CB = F::NV * 16;  // bytes per chunk
-    constexpr int U = kUnroll<WQ>;
+    constexpr int U = kUnroll<WQ, kTwo>;
     for (int c0 = lane; c0 < nchunk; c0 += 32 * U) {
         uint4 raw[U][4][F::NV];
 #pragma unroll
@@ -174,7 +175,7 @@ __device__ __forceinline__ void group_rows(const FfnProblem& p, int e, int g, in
 // all of the CTA's groups.
 //   stage 1: h[r, i] = silu(x_r . Wgate[i]) * (x_r . Wup[i])
 //   stage 2: y[r, n] = h_r . Wdown[n]
-template <typename TA, int WQ, int STAGE>
+template <typename TA, int WQ, int STAGE, bool kTwo>
 __device__ __forceinline__ void stream_ffn_cta(const FfnProblem& p, int gpc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TA* xs = reinterpret_cast<TA*>(smem_raw);
@@ -206,7 +207,7 @@ __device__ __forceinline__ void stream_ffn_cta(const FfnProblem& p, int gpc) {
                 for (int q = 0; q < 4; ++q)
 #pragma unroll
                     for (int r = 0; r < NT; ++r) acc[q][r] = 0.0f;
-                dot4<TA, WQ, NT>(wrow, srow, xs, K, acc);
+                dot4<TA, WQ, NT, kTwo>(wrow, srow, xs, K, acc);
                 const float sum = warp_sums<NT>(acc);
                 constexpr int COPIES = 8 / NT;  // lanes that hold the same sum
                 const int value = lane / COPIES, q = value / NT, r = value % NT;
@@ -222,18 +223,18 @@ __device__ __forceinline__ void stream_ffn_cta(const FfnProblem& p, int gpc) {
     }
 }
 
-template <typename TA, int WQ>
-__global__ void __launch_bounds__(kStreamWarps * 32, stream_min_blocks<WQ>())
+template <typename TA, int WQ, bool kTwo>
+__global__ void __launch_bounds__(kStreamWarps * 32, stream_min_blocks<WQ, kTwo>())
 stream_gateup_kernel(FfnProblem p, int gpc) {
     pdl_enter();
-    stream_ffn_cta<TA, WQ, 1>(p, gpc);
+    stream_ffn_cta<TA, WQ, 1, kTwo>(p, gpc);
 }
 
-template <typename TA, int WQ>
-__global__ void __launch_bounds__(kStreamWarps * 32, stream_min_blocks<WQ>())
+template <typename TA, int WQ, bool kTwo>
+__global__ void __launch_bounds__(kStreamWarps * 32, stream_min_blocks<WQ, kTwo>())
 stream_down_kernel(FfnProblem p, int gpc) {
     pdl_enter();
-    stream_ffn_cta<TA, WQ, 2>(p, gpc);
+    stream_ffn_cta<TA, WQ, 2, kTwo>(p, gpc);
 }
 
 // Column groups per CTA: up to kMaxGroupsPerCta while the grid keeps at least
@@ -256,37 +257,53 @@ inline int passes_apart(int64_t n_rows, int max_active, int ctas) {
     return z;
 }
 
+// fp32: whether two CTAs share an SM: where the grid has a second one for it, and
+// where the rows of both leave the L1 cache room for the loads in flight (16 experts,
+// top 4, H 3584, 12 tokens: layer 337 us with both CTAs' 112 KB of rows, 263 with one
+// CTA and four chunks; H 3072, 96 KB each: 146 and 156).
+inline bool two_ctas(int64_t ctas, size_t smem) { return ctas > sm_count() && smem <= 96 * 1024; }
+
+template <typename TA, int WQ, bool kTwo>
+static cudaError_t launch_stream_gateup(const FfnProblem& p, dim3 grid, size_t smem, int gpc, cudaStream_t stream) {
+    static DeviceOnce smem_set;  // the most dynamic shared memory any problem may ask for, set once per device
+    const cudaError_t err = smem_set.run([] {
+        return cudaFuncSetAttribute(stream_gateup_kernel<TA, WQ, kTwo>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)stream_smem_budget());
+    });
+    if (err != cudaSuccess) return err;
+    return launch_k(stream_gateup_kernel<TA, WQ, kTwo>, grid, dim3(kStreamWarps * 32), smem, stream, p, gpc);
+}
+
+template <typename TA, int WQ, bool kTwo>
+static cudaError_t launch_stream_down(const FfnProblem& p, dim3 grid, size_t smem, int gpc, cudaStream_t stream) {
+    static DeviceOnce smem_set;
+    const cudaError_t err = smem_set.run([] {
+        return cudaFuncSetAttribute(stream_down_kernel<TA, WQ, kTwo>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)stream_smem_budget());
+    });
+    if (err != cudaSuccess) return err;
+    return launch_k(stream_down_kernel<TA, WQ, kTwo>, grid, dim3(kStreamWarps * 32), smem, stream, p, gpc);
+}
+
 template <typename TA, int WQ>
 static cudaError_t launch_stream_t(const FfnProblem& p, cudaStream_t stream) {
     const int max_active = (int)min64(p.E, p.n_rows);
     if (max_active == 0) return cudaSuccess;
     const size_t smem1 = (size_t)kNT * p.H * sizeof(TA);
     const size_t smem2 = (size_t)kNT * p.I * sizeof(TA);
-    cudaError_t err;
-    // the largest dynamic shared memory any problem may ask for, set once per device
-    static DeviceOnce smem_set;
-    err = smem_set.run([] {
-        const int most = (int)stream_smem_budget();
-        cudaError_t e = cudaFuncSetAttribute(stream_gateup_kernel<TA, WQ>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(stream_down_kernel<TA, WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    });
-    if (err != cudaSuccess) return err;
     const int groups1 = p.I / (2 * kStreamWarps), groups2 = p.H / (4 * kStreamWarps);
     const int gpc1 = groups_per_cta(max_active, groups1), gpc2 = groups_per_cta(max_active, groups2);
-    dim3 g1(max_active, groups1 / gpc1);
+    dim3 g1(max_active, groups1 / gpc1), g2(max_active, groups2 / gpc2);
     g1.z = passes_apart(p.n_rows, max_active, g1.x * g1.y);
-    if (const cudaError_t le = launch_k(stream_gateup_kernel<TA, WQ>, dim3(g1), dim3(kStreamWarps * 32), smem1,
-            stream, p, gpc1); le != cudaSuccess)
-        return le;
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    dim3 g2(max_active, groups2 / gpc2);
     g2.z = passes_apart(p.n_rows, max_active, g2.x * g2.y);
-    if (const cudaError_t le = launch_k(stream_down_kernel<TA, WQ>, dim3(g2), dim3(kStreamWarps * 32), smem2,
-            stream, p, gpc2); le != cudaSuccess)
-        return le;
-    return cudaGetLastError();
+    // (other formats have one variant)
+    constexpr bool kOne = WQ == GBMOE_F32;
+    auto two = [](const dim3& g, size_t smem) { return !kOne || two_ctas((int64_t)g.x * g.y * g.z, smem); };
+    const cudaError_t err = two(g1, smem1) ? launch_stream_gateup<TA, WQ, true>(p, g1, smem1, gpc1, stream)
+                                           : launch_stream_gateup<TA, WQ, !kOne>(p, g1, smem1, gpc1, stream);
+    if (err != cudaSuccess) return err;
+    return two(g2, smem2) ? launch_stream_down<TA, WQ, true>(p, g2, smem2, gpc2, stream)
+                          : launch_stream_down<TA, WQ, !kOne>(p, g2, smem2, gpc2, stream);
 }
 
 // launch_stream_t for one weight format, defined in ffn_stream_<format>.cu so
