@@ -74,10 +74,10 @@ int check_cfg(const gbmoe_config* c) {
 bool stream_fits(int act_dtype, int H, int I) { return stream_smem_bytes(act_dtype, H, I) <= stream_smem_budget(); }
 
 // most rows per expert of the feature-major GEMM
-int64_t fm_rows_per_expert(int w_dtype) {
-    return w_dtype == GBMOE_FP8_E4M3_B128 ? kFmFp8RowsPerExpert
-           : w_dtype == GBMOE_MXFP4       ? kFmMxfp4RowsPerExpert
-                                          : kFmRowsPerExpert;
+int64_t fm_rows_per_expert(const gbmoe_config* c) {
+    return c->w_dtype == GBMOE_FP8_E4M3_B128 ? fm_fp8_rows_per_expert(c->H)
+           : c->w_dtype == GBMOE_MXFP4       ? kFmMxfp4RowsPerExpert
+                                             : kFmRowsPerExpert;
 }
 
 // Whether a problem has so few rows that AUTO streams its weights whatever their
@@ -104,7 +104,7 @@ int pick_route(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     // int4 and MXFP4 weights with bf16 activations and few rows per expert: the
     // feature-major GEMM (use_fm), reported as TC
     const bool four_bit = c->w_dtype == GBMOE_INT4_G128 || c->w_dtype == GBMOE_MXFP4;
-    if (four_bit && c->combine_route != GBMOE_COMBINE_FUSED && n_rows <= fm_rows_per_expert(c->w_dtype) * E && ffn_fm_supported(probe))
+    if (four_bit && c->combine_route != GBMOE_COMBINE_FUSED && n_rows <= fm_rows_per_expert(c) * E && ffn_fm_supported(probe))
         return GBMOE_FFN_TC;
     if (n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I)) return GBMOE_FFN_STREAM;
     if (c->act_dtype == GBMOE_BF16) {
@@ -133,7 +133,7 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
     probe.w_dtype = c->w_dtype;
     probe.H = c->H;
     probe.I = I;
-    if (n_rows > fm_rows_per_expert(c->w_dtype) * E || !ffn_fm_supported(probe)) return false;
+    if (n_rows > fm_rows_per_expert(c) * E || !ffn_fm_supported(probe)) return false;
     if (c->w_dtype == GBMOE_BF16 && n_rows < kFmBf16MinRowsPerExpert * E) return false;
     if (c->ffn_route == GBMOE_FFN_AUTO && streams_few_rows(c, n_rows, E, I)) return false;
     return c->w_dtype == GBMOE_FP8_E4M3_B128 ? pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8

@@ -162,7 +162,11 @@ bool ffn_tc_fp8_supported(const FfnProblem& p);
 // unaligned weights, 3.46 at 64); int4, 64 experts, H 4096, I 2816: 0.59 against
 // 0.78 at 24, 0.78 against 0.78 at 48, 0.96 against 0.85 at 72; bf16, 128 experts, H 4096, I 1536: 0.775
 // against 0.800 at 21, 0.62 against 0.70 (streaming) at 2.
-constexpr int64_t kFmFp8RowsPerExpert = 52;
+// fp8 with narrow inputs leaves the gate/up items two or four k blocks, less than
+// their handover of sums costs: 128 experts, I 3072, H 256 1.07 times the speed of
+// the row-major GEMM (before its stacked tiles) at 28 rows, 0.97 at 36, 0.85 at 52; H
+// 512 1.00 at 44, 0.95 at 52; H 1024 1.02 at 52.
+inline int64_t fm_fp8_rows_per_expert(int H) { return H >= 1024 ? 52 : H >= 512 ? 40 : 28; }
 constexpr int64_t kFmMxfp4RowsPerExpert = 64;
 constexpr int64_t kFmRowsPerExpert = 40;
 // Factor 2^-kLowBits between the feature-major GEMM's second codes and its first (quant_act.cu).

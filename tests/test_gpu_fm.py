@@ -27,6 +27,8 @@ def few_rows(wq, H, I):
 
 def kernel_of(wl):
     most, beyond, _ = LIMITS[wl.wq]
+    if wl.wq == "fp8_b128" and wl.H < 1024:  # few k blocks
+        most = 40 if wl.H >= 512 else 28
     if wl.P <= min(few_rows(wl.wq, wl.H, wl.I), 16 * wl.E) or (wl.wq == "bf16" and wl.P < wl.E):
         return "stream"
     return "fm" if wl.P <= most * wl.E else beyond
@@ -61,6 +63,10 @@ def test_which_kernels_run(wq):
     cfg = lambda T, **kw: gb.make_config(T, 4096, 4096, 4, 1, act="bf16", w=wq, **kw)
     assert gb.ffn_kernel(cfg(4 * most)) == "fm"
     assert gb.ffn_kernel(cfg(4 * most + 1)) == other == gb.ffn_route(cfg(4 * most + 1))
+    if wq == "fp8_b128":
+        for H, last in ((256, 28), (512, 40), (768, 40), (1024, 52)):
+            narrow = lambda rows: gb.make_config(4 * rows, H, 4096, 4, 1, act="bf16", w=wq)
+            assert gb.ffn_kernel(narrow(last)) == "fm" and gb.ffn_kernel(narrow(last + 1)) == "tc_fp8"
     assert gb.ffn_kernel(cfg(40, ffn_route="simt")) == "simt"
     assert gb.ffn_kernel(cfg(40, ffn_route="tc")) == "tc"
     if wq == "bf16":
