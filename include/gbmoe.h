@@ -84,7 +84,8 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * with infinities contributes infinities or NaN to every output.
  * AUTO: with bf16 activations and so few rows that P - 1 <= c * (1/H + 1/I) (c:
  * 12000 for bf16 weights, 5000 fp8, 4800 int4, 1600 MXFP4) and P/E at most 16,
- * the weights are streamed. Else fp8 weights take GBMOE_FFN_TC_FP8, and
+ * the weights are streamed (not where the shared expert joins the routed ones on
+ * the route below, gbmoe_ffn_kernel). Else fp8 weights take GBMOE_FFN_TC_FP8, and
  * int4 (MXFP4) weights with at most 40 (64) rows per
  * expert (P/E) multiply the same activation codes on the fp8 tensor cores under
  * AUTO (as GBMOE_FFN_TC): every int4 and FP4 value is an e4m3 value; int4's group

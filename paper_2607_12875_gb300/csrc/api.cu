@@ -80,9 +80,28 @@ int64_t fm_rows_per_expert(const gbmoe_config* c) {
                                              : kFmRowsPerExpert;
 }
 
+// Whether the shared expert can be one more expert of the routed problem on the
+// feature-major GEMM: with coded activations, when the two have the same
+// intermediate size and few tokens (its own launches leave most SMs idle; many rows
+// are cheaper on the row-major GEMM). Joined against apart, ms:
+// fp8, 256 experts, H 7168, I 2048: 0.64 and 0.67 at 16 tokens, 1.36 and 1.42 at
+// 48, 1.78 and 1.79 at 256, 1.87 and 1.83 at 512, 2.18 and 2.14 at 1024; MXFP4, the
+// same layer: 0.52 and 0.57 at 16, 1.33 and 1.39 at 256, 1.52 and 1.78 at 512, 2.27
+// and 2.50 at 1024; int4, 64 experts, top 6, H 4096, I 2816: 0.29 and 0.34 at 16,
+// 0.62 and 0.66 at 256, 0.65 and 0.70 at 400 (512 is beyond its feature-major rows).
+constexpr int kJoinTokensFp8 = 256, kJoinTokens4Bit = 512;
+bool shared_may_join(const gbmoe_config* c) {
+    return c->has_shared && c->I_shared == c->I && c->w_dtype != GBMOE_BF16 &&
+           c->T <= (c->w_dtype == GBMOE_FP8_E4M3_B128 ? kJoinTokensFp8 : kJoinTokens4Bit);
+}
+
 // Whether a problem has so few rows that AUTO streams its weights whatever their
-// format (few_rows in kernels.h).
+// format (few_rows in kernels.h). Not the routed one that a shared expert can
+// join: streaming takes launches for both (fp8, 64 experts, top 8, H 2048, I 1024, 1
+// token: 51.5 us streamed apart, 39.5 joined; int4 55.9 and 43.8; with 2 rows of 8
+// experts the two are about even).
 bool streams_few_rows(const gbmoe_config* c, int64_t n_rows, int E, int I) {
+    if (shared_may_join(c) && E == c->E && n_rows == (int64_t)c->T * c->top_k) return false;
     return c->act_dtype == GBMOE_BF16 && n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I) &&
            (double)(n_rows - 1) <= few_rows(c->w_dtype) * (1.0 / c->H + 1.0 / I);
 }
@@ -141,19 +160,9 @@ bool use_fm(const gbmoe_config* c, int64_t n_rows, int E, int I) {
 }
 
 // Whether moe_forward runs the shared expert as one more expert of the routed
-// problem: on the feature-major GEMM with coded activations, when the two have
-// the same intermediate size and few tokens (its own launches leave most SMs
-// idle; many rows are cheaper on the row-major GEMM). Joined against apart, ms:
-// fp8, 256 experts, H 7168, I 2048: 0.64 and 0.67 at 16 tokens, 1.36 and 1.42 at
-// 48, 1.78 and 1.79 at 256, 1.87 and 1.83 at 512, 2.18 and 2.14 at 1024; MXFP4, the
-// same layer: 0.52 and 0.57 at 16, 1.33 and 1.39 at 256, 1.52 and 1.78 at 512, 2.27
-// and 2.50 at 1024; int4, 64 experts, top 6, H 4096, I 2816: 0.29 and 0.34 at 16,
-// 0.62 and 0.66 at 256, 0.65 and 0.70 at 400 (512 is beyond its feature-major rows).
-constexpr int kJoinTokensFp8 = 256, kJoinTokens4Bit = 512;
+// problem.
 bool shared_joins(const gbmoe_config* c) {
-    return c->has_shared && c->I_shared == c->I && c->w_dtype != GBMOE_BF16 &&
-           c->T <= (c->w_dtype == GBMOE_FP8_E4M3_B128 ? kJoinTokensFp8 : kJoinTokens4Bit) &&
-           use_fm(c, (int64_t)c->T * c->top_k, c->E, c->I);
+    return shared_may_join(c) && use_fm(c, (int64_t)c->T * c->top_k, c->E, c->I);
 }
 
 // Bytes of the bf16 weight copy the TC_DEQUANT route decodes into (0 when

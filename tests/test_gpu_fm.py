@@ -29,7 +29,9 @@ def kernel_of(wl):
     most, beyond, _ = LIMITS[wl.wq]
     if wl.wq == "fp8_b128" and wl.H < 1024:  # few k blocks
         most = 40 if wl.H >= 512 else 28
-    if wl.P <= min(few_rows(wl.wq, wl.H, wl.I), 16 * wl.E) or (wl.wq == "bf16" and wl.P < wl.E):
+    joins = wl.has_shared and wl.I_shared == wl.I and wl.wq != "bf16"
+    few = wl.P <= min(few_rows(wl.wq, wl.H, wl.I), 16 * wl.E) and not joins
+    if few or (wl.wq == "bf16" and wl.P < wl.E):
         return "stream"
     return "fm" if wl.P <= most * wl.E else beyond
 
@@ -78,7 +80,8 @@ def test_which_kernels_run(wq):
     same = dict(has_shared=True, I_shared=4096)
     assert gb.ffn_kernel(cfg(40, **same), shared=True) == ("fm" if wq == "bf16" else "joined")
     assert gb.ffn_kernel(cfg(40, has_shared=True, I_shared=2048), shared=True) == "fm"
-    assert gb.ffn_kernel(cfg(2, **same), shared=True) == {"mxfp4": "joined"}.get(wq, "stream")
+    assert gb.ffn_kernel(cfg(2, **same), shared=True) == ("stream" if wq == "bf16" else "joined")
+    assert gb.ffn_kernel(cfg(2, has_shared=True, I_shared=2048), shared=True) == "stream"
     assert gb.ffn_kernel(cfg(40, ffn_route="tc", **same), shared=True) == "tc"
     wide = gb.make_config(513, 4096, 4096, 64, 1, act="bf16", w=wq, **same)  # more tokens than join
     assert gb.ffn_kernel(wide) == "fm" and gb.ffn_kernel(wide, shared=True) == gb.ffn_route(wide, shared=True)
@@ -326,7 +329,7 @@ def test_shared_expert_with_the_routed_ones(T, I_shared, wq):
                       topk_group=2, has_shared=True, I_shared=I_shared, select_bias_sigma=0.01)
     inp = synth.make_inputs(wl)
     alone = kernel_of(wl) != "fm" or I_shared != wl.I
-    assert gb.ffn_kernel(config(wl), shared=True) == (kernel_of(wl.replace(E=1, top_k=1, I=I_shared)) if alone else "joined")
+    assert gb.ffn_kernel(config(wl), shared=True) == (kernel_of(wl.replace(E=1, top_k=1, I=I_shared, has_shared=False)) if alone else "joined")
     assert_close(act_np(forward(wl, to_device(wl, inp), kernel_of(wl))), oracle.forward(wl, inp)["out"], tol(wl, kernel_of(wl)))
 
 
