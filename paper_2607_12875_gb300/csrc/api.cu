@@ -99,9 +99,9 @@ bool shared_may_join(const gbmoe_config* c) {
 // format (few_rows in kernels.h). Not the routed one that a shared expert can
 // join: streaming takes launches for both (fp8, 64 experts, top 8, H 2048, I 1024, 1
 // token: 51.5 us streamed apart, 39.5 joined; int4 55.9 and 43.8; with 2 rows of 8
-// experts the two are about even).
+// experts the two are about even, with one row streaming is ahead).
 bool streams_few_rows(const gbmoe_config* c, int64_t n_rows, int E, int I) {
-    if (shared_may_join(c) && E == c->E && n_rows == (int64_t)c->T * c->top_k) return false;
+    if (shared_may_join(c) && n_rows > 1 && E == c->E && n_rows == (int64_t)c->T * c->top_k) return false;
     return c->act_dtype == GBMOE_BF16 && n_rows <= 16 * (int64_t)E && stream_fits(c->act_dtype, c->H, I) &&
            (double)(n_rows - 1) <= few_rows(c->w_dtype) * (1.0 / c->H + 1.0 / I);
 }

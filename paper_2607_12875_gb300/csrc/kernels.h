@@ -100,10 +100,10 @@ size_t ffn_sched_ints(int E, int64_t n_rows);
 // and 103 at 256 rows per expert; 24, 2048, 1024 (50 M) 222 and 221 at 260; 48, 3072,
 // 1024 (151 M) 478 and 498 at 260, 534 and 526 at 300; 40, 4096, 1408 (231 M) 724 and
 // 746 at 349, 910 and 842 at 399; 64, 4096, 2816 (738 M) 2018 and 2184 at 349, 2432 and
-// 2428 at 399.
+// 2428 at 399. (278, 5632, 128: layer 1570 and 1431 at 317.)
 inline int64_t dequant_rows_per_expert(int E, int H, int I) {
     const int64_t weights = (int64_t)E * H * I;
-    return weights < 90000000 ? 256 : weights < 200000000 ? 288 : weights < 400000000 ? 352 : 384;
+    return weights < 90000000 ? 256 : weights < 200000000 || I < 512 ? 288 : weights < 400000000 ? 352 : 384;
 }
 // AUTO: CTA pairs from this many rows per expert on. bf16, 128 experts, H 4096,
 // I 1536, pairs against single CTAs: 2.245 and 2.252 ms at 512 rows per expert,

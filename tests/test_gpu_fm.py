@@ -29,7 +29,7 @@ def kernel_of(wl):
     most, beyond, _ = LIMITS[wl.wq]
     if wl.wq == "fp8_b128" and wl.H < 1024:  # few k blocks
         most = 40 if wl.H >= 512 else 28
-    joins = wl.has_shared and wl.I_shared == wl.I and wl.wq != "bf16"
+    joins = wl.has_shared and wl.I_shared == wl.I and wl.wq != "bf16" and wl.P > 1
     few = wl.P <= min(few_rows(wl.wq, wl.H, wl.I), 16 * wl.E) and not joins
     if few or (wl.wq == "bf16" and wl.P < wl.E):
         return "stream"

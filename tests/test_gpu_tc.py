@@ -122,7 +122,7 @@ def test_auto_route_choice():
 
 
 @pytest.mark.parametrize("E,H,I,first,pairs_from", [(24, 1024, 512, 256, 1024), (48, 3072, 1024, 288, 1024),
-                                                    (40, 4096, 1408, 352, 400), (64, 4096, 2816, 384, 400),
+                                                    (278, 5632, 128, 288, 1024), (40, 4096, 1408, 352, 400), (64, 4096, 2816, 384, 400),
                                                     (1, 1536, 2688, 256, 1024)])
 def test_decode_once_and_pairs_by_size(E, H, I, first, pairs_from):
     """AUTO's lines for 4-bit weights: the rows per expert from which they are
