@@ -78,7 +78,9 @@ enum { GBMOE_SOFTMAX = 0, GBMOE_SIGMOID = 1 };
  * accumulated in fp32. With few rows per expert (the weights are the GEMM's M
  * operand) j = 5 and the block's largest |x / s| lies in [128, 256): a bf16 x is
  * held exactly where |x / s| >= 2^-7 and within 2^-15 * s below, 2^-22 of the
- * block's largest value. With many (the rows are the M operand) j = 0 and it lies
+ * block's largest value; where more than an eighth of a block's nonzero values
+ * are inexact, a second pair of codes holds the rest, to 2^-44, at the cost of a
+ * second walk of the GEMM over k. With many (the rows are the M operand) j = 0 and it lies
  * in [224, 448]: exactly where |x / s| >= 2^-2 and within 2^-10 * s below, 2^-17
  * of the block's largest value. A block that holds a NaN contributes NaN; one
  * with infinities contributes infinities or NaN to every output.

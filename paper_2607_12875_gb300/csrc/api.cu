@@ -203,13 +203,15 @@ struct Layout {
         wdq_sh, aq, as, hq, hs, total;
 };
 
-// true when the routed or the shared FFN problem of c multiplies e4m3 codes of
-// its activations (the fp8 route, the feature-major GEMM)
-bool uses_act_codes(const gbmoe_config* c) {
-    auto codes = [&](int64_t n_rows, int E, int I) {
-        return (c->w_dtype != GBMOE_BF16 && use_fm(c, n_rows, E, I)) || pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8;
+// e4m3 code planes of their activations that the routed and the shared FFN problem
+// of c need: four on the feature-major GEMM, two on the row-major fp8 GEMM, or none
+int act_code_planes(const gbmoe_config* c) {
+    auto planes = [&](int64_t n_rows, int E, int I) {
+        if (c->w_dtype != GBMOE_BF16 && use_fm(c, n_rows, E, I)) return 4;
+        return pick_route(c, n_rows, E, I) == GBMOE_FFN_TC_FP8 ? 2 : 0;
     };
-    return codes((int64_t)c->T * c->top_k, c->E, c->I) || (c->has_shared && codes(c->T, 1, c->I_shared));
+    const int routed = planes((int64_t)c->T * c->top_k, c->E, c->I);
+    return c->has_shared ? std::max(routed, planes(c->T, 1, c->I_shared)) : routed;
 }
 
 Layout layout(const gbmoe_config* c) {
@@ -242,10 +244,11 @@ Layout layout(const gbmoe_config* c) {
     L.xout = take((size_t)T * H * ab);
     L.wdq = take(dequant_bytes(c, P, (int)E, c->I));
     L.wdq_sh = take(c->has_shared ? dequant_bytes(c, T, 1, c->I_shared) : 0);
-    const bool codes = uses_act_codes(c);  // e4m3 copies of the GEMM inputs and their 1x128 scales
-    L.aq = take(codes ? (size_t)2 * rows_max * H : 0);  // two e4m3 code planes
+    const int planes = act_code_planes(c);  // e4m3 copies of the GEMM inputs and their 1x128 scales
+    const bool codes = planes > 0;
+    L.aq = take((size_t)planes * rows_max * H);
     L.as = take(codes ? (size_t)rows_max * (H / 128) * 4 : 0);
-    L.hq = take(codes ? (size_t)2 * rows_max * I_max : 0);
+    L.hq = take((size_t)planes * rows_max * I_max);
     L.hs = take(codes ? (size_t)rows_max * (I_max / 128) * 4 : 0);
     L.total = o;
     return L;

@@ -15,7 +15,8 @@
 // significant bits in full down to 2^-14 of the 128's largest value, and within
 // 2^-22 of that value below (quant_act.cu). q2's factor 2^-kLowBits is applied in
 // the promotion (short tiles) or by the MMAs, as a scale of their N operand (tall
-// ones, kind::mxf8f6f4 for every format).
+// ones, kind::mxf8f6f4 for every format). Rows whose values spread further have
+// a second pair of codes for the rest; every item then walks k twice.
 // Products of codes accumulate in fp32 in tensor memory over 128 k, then the
 // promotion warps add the partial sum times its scales to fp32 accumulators
 // in registers.
@@ -68,7 +69,8 @@ constexpr int BK = 128;                 // k per block: one swizzle row, one act
 constexpr int A_BYTES = 2 * MB * BK;    // the two 128-row halves of an item's weight tile
 constexpr int TMEM_COLS = 512;
 constexpr int GATHER_WARPS = 2;
-constexpr float kLowScale = 1.0f / (1 << kLowBits);  // of a second code
+constexpr float kLowScale = 1.0f / (1 << kLowBits);    // of a second code
+constexpr float kWideScale = 1.0f / (1 << kWideBits);  // of the second pair of planes
 constexpr int SMEM_BUDGET = 232448;
 // MXFP4 whose tiles TMA unpacks: 16 E2M1 codes of 8 bytes become 8 bytes and 8
 // bytes of padding in shared memory, which kind::mxf8f6f4 reads as they are
@@ -148,7 +150,8 @@ struct Params {
     int64_t n_shared;        // rows of the shared expert, after the routed ones (0: none)
     __nv_bfloat16* out;
     int32_t* err;
-    const uint8_t* q;        // code planes q1, q2: [2][plane_rows][K]
+    const uint8_t* q;        // code planes: [4][plane_rows][K], two pairs of q1, q2
+    const int32_t* wide;     // nonzero: the second pair counts, a second walk over k multiplies it
     int64_t plane_rows;
     const float* a_scale;    // [plane_rows][K/128]
     const int32_t* gather;   // row r of the sorted order is plane row gather[r] / gather_div; null: r itself
@@ -376,6 +379,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
     uint64_t* drain = xempty + 4;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* walk = abort_flag + 1;  // k blocks of an item, all walks over k
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -395,6 +399,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
         for (int b = 0; b < RING; ++b) mbar_init(&sfull[b], GATHER_WARPS + C::DECODE_WARPS);
         mbar_init(drain, 1);
         *abort_flag = 0;
+        *walk = (*p.wide ? 2 : 1) * (p.K / BK);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -425,6 +430,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
 
     const int total = p.sched[1] * p.n_tiles;
     const int nkb = p.K / BK;
+    const int passes = *p.wide ? 2 : 1;  // walks over k (the second: 2^-kWideBits of the first)
 
     // tall tiles: 16 warps start with 128 registers a thread; the promotion takes 168
     // (128 threads x (104 + 168 + 168 + 72) = 65536, what the block was launched with)
@@ -441,7 +447,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             const Work wk = decode_work(p, w);
             int a0, a1;
             w_rows<SWIGLU>(p, wk, a0, a1);
-            for (int kb = 0; kb < nkb; ++kb) {
+            for (int it = 0, kb = 0; it < passes * nkb; ++it) {
                 if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 inflight &= ~(1u << stage);
                 constexpr int BYTES = RAW ? RAW : A_BYTES;  // (int4: 64 bytes of a row are 128 weights)
@@ -453,6 +459,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 tma_load_2d(dst + BYTES / 2, wk.shared ? &tm_s1 : &tm_w1, x, a1, bar);
                 inflight |= 1u << stage;
                 inflight_par = (inflight_par & ~(1u << stage)) | (phase << stage);
+                if (++kb == nkb) kb = 0;
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
         }
@@ -473,7 +480,7 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             const int rp = __shfl_sync(0xffffffffu, rows_pad<C::JOINT>(wk.rows), 0);  // warp-uniform
             const int n = C::JOINT ? 2 * rp : rp;
             const uint32_t idesc = C::MX ? idesc_mxf8<C::UNPACKED>(n) : idesc_f8(n);
-            for (int kb = 0; kb < nkb; ++kb, ++kc) {
+            for (int it = 0; it < passes * nkb; ++it, ++kc) {
                 if (!warp_wait(&full[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                 // the row codes were written through the generic proxy (cp.async)
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -546,27 +553,35 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
             for (int i = 0; i < ROWS / 8; ++i) src[i] = p.q + (8 * i < rp ? src_row(r0 + 8 * i) : 0) * p.K + 16 * chunk;
             const float* s0 = p.a_scale + (t < rp ? src_row(t) : 0) * nkb;
             const float* s1 = p.a_scale + (t + 64 < rp ? src_row(t + 64) : 0) * nkb;
-            float n0 = s0[0], n1 = s1[0];
-            for (int kb = 0; kb < nkb; ++kb) {
-                if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
-                uint8_t* dst = sB + stage * B_BYTES;
+            for (int pass = 0; pass < passes && ok; ++pass) {
+                float n0 = s0[0], n1 = s1[0];
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
+                    uint8_t* dst = sB + stage * B_BYTES;
 #pragma unroll
-                for (int i = 0; i < ROWS / 8; ++i) {
-                    if (8 * i >= rp) break;
-                    const uint32_t off = sw128_off(r0 + 8 * i, chunk);
-                    cp_async_16(dst + off, src[i] + kb * BK);
-                    cp_async_16(dst + rp * BK + off, src[i] + plane + kb * BK);
+                    for (int i = 0; i < ROWS / 8; ++i) {
+                        if (8 * i >= rp) break;
+                        const uint32_t off = sw128_off(r0 + 8 * i, chunk);
+                        cp_async_16(dst + off, src[i] + kb * BK);
+                        cp_async_16(dst + rp * BK + off, src[i] + plane + kb * BK);
+                    }
+                    // one arrival of this thread once its copies above have landed
+                    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[stage])) : "memory");
+                    if (pass) {  // (a block that is not finite has no second codes, and 0 times its scale would be NaN)
+                        n0 = n0 < INFINITY ? n0 * kWideScale : 0.0f;
+                        n1 = n1 < INFINITY ? n1 * kWideScale : 0.0f;
+                    }
+                    float* sc = sS + ring * C::RING_FLOATS;
+                    if (t < rp) sc[t] = n0;
+                    if (t + 64 < rp) sc[t + 64] = n1;
+                    if (kb + 1 < nkb) { n0 = s0[kb + 1]; n1 = s1[kb + 1]; }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sfull[ring]);
+                    if (++ring == RING) ring = 0;
+                    if (++stage == STAGES) { stage = 0; phase ^= 1; }
                 }
-                // one arrival of this thread once its copies above have landed
-                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[stage])) : "memory");
-                float* sc = sS + ring * C::RING_FLOATS;
-                if (t < rp) sc[t] = n0;
-                if (t + 64 < rp) sc[t + 64] = n1;
-                if (kb + 1 < nkb) { n0 = s0[kb + 1]; n1 = s1[kb + 1]; }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sfull[ring]);
-                if (++ring == RING) ring = 0;
-                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+#pragma unroll
+                for (int i = 0; i < ROWS / 8; ++i) src[i] += 2 * plane;  // the second pair of planes
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");  // (after an abort too) copies land before the CTA leaves
@@ -598,12 +613,16 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 wn[h] = C::UNPACKED ? 1.0f : RAW ? 64.0f : ws[h][0];  // (MXFP4's decoded codes are the values times 2^-6, the MMAs scale)
             }
             bool ok = true;
-            for (int kb = 0; kb < nkb; ++kb, ++kc) {
+            // The count is read here: beside the accumulators there is no register to keep it in
+            // (held in one, the fp8 tall tiles spill: 8192 rows of 64 experts 2.03 -> 2.15 ms).
+            // MXFP4's tall tiles have one, and lose 5 % by the read (2048 tokens 2.52 -> 2.64 ms).
+            for (int left = C::UNPACKED && !C::JOINT ? passes * nkb : *walk, kb = 0; left > 0; --left, ++kc) {
+                if (++kb == nkb) kb = 0;  // the next block's
                 float wsc[C::HALVES_HELD];
 #pragma unroll
                 for (int h = 0; h < C::HALVES_HELD; ++h) {
                     wsc[h] = wn[h];
-                    if (!RAW && !C::UNPACKED && kb + 1 < nkb) wn[h] = ws[h][kb + 1];
+                    if (!RAW && !C::UNPACKED) wn[h] = ws[h][kb];
                 }
                 const float* sc = sS + ring * C::RING_FLOATS;
                 const uint32_t slot = C::JOINT ? kc % SLOTS : 2 * set + (kc & 1);
@@ -724,7 +743,8 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 w_rows<SWIGLU>(p, wk, a0, a1);
                 const uint8_t* s0 = static_cast<const uint8_t*>(wk.shared ? p.s_scale0 : p.w_scale0) + (int64_t)(a0 + r) * nkb * 4;
                 const uint8_t* s1 = static_cast<const uint8_t*>(wk.shared ? p.s_scale1 : p.w_scale1) + (int64_t)(a1 + r) * nkb * 4;
-                for (int kb = 0; kb < nkb; ++kb) {
+                for (int it = 0; it < passes * nkb; ++it) {
+                    const int kb = it < nkb ? it : it - nkb;
                     if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                     uint8_t* dst = sF + stage * C::SF_BYTES + 16 * (r & 31) + 4 * (r >> 5);
                     if (p.scale_words) {
@@ -775,12 +795,13 @@ fm_gemm_kernel(const __grid_constant__ CUtensorMap tm_w0, const __grid_constant_
                 uint32_t next[HALVES];
 #pragma unroll
                 for (int i = 0; i < HALVES; ++i) next[i] = scale_bits(i, 0);
-                for (int kb = 0; kb < nkb; ++kb) {
+                for (int it = 0, kb = 0; it < passes * nkb; ++it) {
+                    if (++kb == nkb) kb = 0;  // the next block's
                     uint32_t bits[HALVES];
 #pragma unroll
                     for (int i = 0; i < HALVES; ++i) {
                         bits[i] = next[i];
-                        if (kb + 1 < nkb) next[i] = scale_bits(i, kb + 1);
+                        next[i] = scale_bits(i, kb);
                     }
                     if (!warp_wait(&rfull[stage], phase, abort_flag, p.err, p.wait_limit_ns)) { ok = false; break; }
                     float* sc = sS + ring * C::RING_FLOATS + ROWS;  // (int4)
@@ -1111,7 +1132,8 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     // every row of x once (the shared expert's rows are x's own; a routed row is a token's)
     const int64_t x_rows = p.n_rows / p.pair_div;
     constexpr bool kFour = Cfg<WQ, ROWS>::RAW != 0;  // the order 4-bit weights are decoded in
-    if ((err = launch_quant_rows(p.x, nullptr, 1, x_rows, p.H, p.a_q, p.a_s, kFour, kLowBits, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_planes(p.x, x_rows, p.H, p.a_q, p.a_s, kFour, p.sched + kSchedWideX, nullptr, 0, stream)) != cudaSuccess)
+        return err;
     const int64_t max_m = sched_max_tiles(experts, rows, tile);
     CUtensorMap mg, mu, md, sg, su, sd;
     if (!map_weights(&mg, WQ, p.w_gate, (int64_t)p.E * p.I, p.H) ||
@@ -1127,18 +1149,21 @@ static cudaError_t launch_ffn(const FfnProblem& p, cudaStream_t stream) {
     g.counts = p.counts; g.offsets = p.offsets; g.sched = p.sched; g.E = experts; g.n_rows = p.n_rows;
     g.n_shared = p.n_shared;
     g.out = static_cast<__nv_bfloat16*>(p.h); g.err = p.err;
-    g.q = static_cast<const uint8_t*>(p.a_q); g.plane_rows = x_rows; g.a_scale = p.a_s;
+    g.q = static_cast<const uint8_t*>(p.a_q); g.plane_rows = x_rows; g.a_scale = p.a_s; g.wide = p.sched + kSchedWideX;
     g.gather = p.sorted_pair; g.gather_div = p.pair_div;
     g.w_scale0 = p.s_gate; g.w_scale1 = p.s_up; g.s_scale0 = p.ss_gate; g.s_scale1 = p.ss_up;
     auto words = [](const void* s) { return reinterpret_cast<uintptr_t>(s) % 4 == 0; };
     g.scale_words = words(p.s_gate) && words(p.s_up) && words(p.ss_gate) && words(p.ss_up);
     g.wait_limit_ns = tc_wait_limit_ns();
     if ((err = launch_gemm<WQ, ROWS, true>(mg, mu, sg, su, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
-    if ((err = launch_quant_rows(p.h, nullptr, 1, rows, p.I, p.h_q, p.h_s, kFour, kLowBits, stream)) != cudaSuccess) return err;
+    // (rows of h past the last kept pair were not written)
+    if ((err = launch_quant_planes(p.h, rows, p.I, p.h_q, p.h_s, kFour, p.sched + kSchedWideH, p.offsets ? p.offsets + p.E : nullptr,
+                                   p.offsets ? p.n_rows : 0, stream)) != cudaSuccess)
+        return err;
     Params d = g;
     d.K = p.I; d.n_tiles = p.H / (2 * MB); d.out_cols = p.H; d.w_rows_per_expert = p.H;
     d.out = static_cast<__nv_bfloat16*>(p.y);
-    d.q = static_cast<const uint8_t*>(p.h_q); d.plane_rows = rows; d.a_scale = p.h_s;
+    d.q = static_cast<const uint8_t*>(p.h_q); d.plane_rows = rows; d.a_scale = p.h_s; d.wide = p.sched + kSchedWideH;
     d.gather = nullptr; d.gather_div = 1;
     d.w_scale0 = d.w_scale1 = p.s_down; d.s_scale0 = d.s_scale1 = p.ss_down;
     d.scale_words = words(p.s_down) && words(p.ss_down);

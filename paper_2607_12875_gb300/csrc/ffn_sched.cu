@@ -46,6 +46,7 @@ ffn_schedule_kernel(const int32_t* __restrict__ counts, int E, int64_t n_rows, i
         }
         if (lane < nw) { s_warp_t[lane] = st - wt; s_warp_a[lane] = sa - wa; }
         if (lane == nw - 1) { sched[0] = sa; sched[1] = st; }
+        if (lane == 0) sched[kSchedWideX] = sched[kSchedWideH] = 0;
     }
     __syncthreads();
     const int tile0 = s_warp_t[warp] + it - nt;

@@ -6,7 +6,10 @@
 
 namespace gbmoe {
 
-constexpr int kSchedHeader = 8;  // [0] active experts, [1] tiles, rest reserved
+constexpr int kSchedHeader = 8;  // [0] active experts, [1] tiles, [2], [3] as below, rest reserved
+// Set when a block of x (h) needs its second pair of codes (quant_act.cu); the
+// schedule clears both.
+constexpr int kSchedWideX = 2, kSchedWideH = 3;
 constexpr int kSchedMinBM = 16;  // smallest tile height any FFN route uses
 
 inline int64_t sched_max_tiles(int E, int64_t n_rows, int BM) { return (n_rows + BM - 1) / BM + E; }

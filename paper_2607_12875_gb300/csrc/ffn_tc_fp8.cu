@@ -430,7 +430,7 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     if (err != cudaSuccess) return err;
     // x rows in sorted order (x itself for the shared expert), quantised per 1x128
     err = p.pair_pos ? launch_quant_scatter(p.x, p.pair_pos, p.pair_div, p.n_rows / p.pair_div, p.H, p.a_q, p.a_s, stream)
-                     : launch_quant_rows(p.x, p.sorted_pair, p.pair_div, p.n_rows, p.H, p.a_q, p.a_s, false, 0, stream);
+                     : launch_quant_rows(p.x, p.sorted_pair, p.pair_div, p.n_rows, p.H, p.a_q, p.a_s, stream);
     if (err != cudaSuccess) return err;
     const int64_t max_m = sched_max_tiles(p.E, p.n_rows, BM);
     const uint8_t* aq = static_cast<const uint8_t*>(p.a_q);
@@ -453,7 +453,7 @@ cudaError_t launch_ffn_tc_fp8(const FfnProblem& p, cudaStream_t stream) {
     g.wait_limit_ns = tc_wait_limit_ns();
     if ((err = launch_gemm<true>(ma1, ma2, ms1, ms2, mg, mu, g, max_m * g.n_tiles, stream)) != cudaSuccess) return err;
     // h quantised per 1x128 for the down GEMM
-    if ((err = launch_quant_rows(p.h, nullptr, 1, p.n_rows, p.I, p.h_q, p.h_s, false, 0, stream)) != cudaSuccess) return err;
+    if ((err = launch_quant_rows(p.h, nullptr, 1, p.n_rows, p.I, p.h_q, p.h_s, stream)) != cudaSuccess) return err;
     Params d = g;
     d.K = p.I; d.n_tiles = p.H / BN; d.out_cols = p.H; d.b_rows_per_expert = p.H;
     d.out = static_cast<__nv_bfloat16*>(p.y);

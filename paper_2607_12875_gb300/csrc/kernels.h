@@ -67,10 +67,10 @@ struct FfnProblem {
     void* w_dq;                 // bf16 [E, I, H] gate, [E, I, H] up, [E, H, I] down, or null:
                                 // quantised weights are then decoded once into it (TC_DEQUANT)
     void* a_q;                  // routes that multiply e4m3 codes: x as two e4m3 code planes (value and
-                                //   residual), [2, rows, H] in sorted order (row-major fp8 GEMM) or
-                                //   token order (feature-major GEMM)
+                                //   residual), [2, rows, H] in sorted order (row-major fp8 GEMM) or two
+                                //   pairs, [4, T, H] in token order (feature-major GEMM)
     float* a_s;                 //   and their 1x128 scales [rows, H/128]
-    void* h_q;                  //   h the same way, [2, n_rows, I]
+    void* h_q;                  //   h the same way, [2 or 4, n_rows, I]
     float* h_s;                 //   and its 1x128 scales [n_rows, I/128]
     // Feature-major GEMM: the shared expert (same I and weight format) as one more
     // expert of the problem, its n_shared rows (token order) after the routed
@@ -169,13 +169,18 @@ bool ffn_tc_fp8_supported(const FfnProblem& p);
 inline int64_t fm_fp8_rows_per_expert(int H) { return H >= 1024 ? 52 : H >= 512 ? 40 : 28; }
 constexpr int64_t kFmMxfp4RowsPerExpert = 64;
 constexpr int64_t kFmRowsPerExpert = 40;
-// Factor 2^-kLowBits between the feature-major GEMM's second codes and its first (quant_act.cu).
-constexpr int kLowBits = 5;
-// rows of src (bf16, gathered when gather is set) as two e4m3 code planes [2, n_rows, K] and 1x128 scales, the
-// second codes times 2^-low (low: kLowBits, or 0 without four_bit); four_bit: in the order 4-bit weights are decoded in
+// The feature-major GEMM's activation codes (quant_act.cu): factor 2^-kLowBits between the second codes and the
+// first, and 2^-kWideBits between the second pair of planes and the first.
+constexpr int kLowBits = 5, kWideBits = 22;
+// Rows of src (bf16) as four e4m3 code planes [4, n_rows, K] and 1x128 scales [n_rows, K / 128]; *wide is set when
+// the second pair counts. four_bit: in the order 4-bit weights are decoded in. With kept, rows *kept .. n_routed - 1
+// are left out (positions of dropped pairs).
+cudaError_t launch_quant_planes(const void* src, int64_t n_rows, int K, void* q, float* s, bool four_bit, int32_t* wide,
+                                const int32_t* kept, int64_t n_routed, cudaStream_t stream);
+// rows of src (gathered when gather is set) as the row-major GEMM's two code planes [2, n_rows, K], and scales
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, bool four_bit, int low, cudaStream_t stream);
-// the same (low 0) of every row of src once, row r's codes written to rows pair_pos[r * k ..] of [2, n_src * k, K]
+                              float* s, cudaStream_t stream);
+// the same of every row of src once, row r's codes written to rows pair_pos[r * k ..] of [2, n_src * k, K]
 cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
                                  cudaStream_t stream);
 cudaError_t launch_ffn_fm(const FfnProblem& p, cudaStream_t stream);

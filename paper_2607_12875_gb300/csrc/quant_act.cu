@@ -6,8 +6,16 @@
 //   kLow = 5 (feature-major GEMM, which scales the second codes' sums apart): s
 //     brings the block's largest magnitude into [128, 256), so that q2 just fits;
 //     x is exact for every |v| >= 2^-7 and within 2^-15 * s below that, 2^-22 of
-//     the block's largest value. Beside an outlier 10^4 times the rest of its
-//     block the rest keeps a relative accuracy of 2^-9, bf16's own.
+//     the block's largest value. What is left over there goes into a second pair
+//     of codes, 2^kWideBits further down, if it belongs to more than an eighth of
+//     the block's nonzero values: exact to 2^-44 of the largest. The GEMM walks k a
+//     second time, with those planes, when any block set the flag. (A block that
+//     leaves less has all its inexact values below the others, and they are few:
+//     2^-11 of the others' part of a sum at most. Normal rows leave one value in
+//     10^4. 16 experts, weights of 0 at one channel 2^16 times the rest: output
+//     within 2.9e-3 of 64 bits with the second pair, 1.4e-2 without; bf16 rounding
+//     alone gives 2.9e-3.) Blocks without one have zeros there, so that a row's
+//     outputs do not depend on other rows.
 //   kLow = 0 (row-major fp8 GEMM, which adds both codes' products up in the same
 //     columns): s brings it into [224, 448], as far up as e4m3 goes; x is exact
 //     for every |v| >= 2^-2 and within 2^-10 * s below that.
@@ -34,7 +42,7 @@ __device__ __forceinline__ uint32_t e4m3x2(float a, float b) {
 // kFourBit: the order that 4-bit weights are decoded in (ffn_fm.cu): within 8
 // consecutive values the even ones come before the odd ones.
 //
-// Rows of src [*, K] -> code planes q [2][n_rows][K] and scales s
+// Rows of src [*, K] -> code planes q [2 or (kLow > 0) 4][n_rows][K] and scales s
 // [n_rows][K/128]. Row r reads source row gather[r] / gather_div (r itself
 // without gather; a negative entry gives a zero row). With scatter, source row
 // r is quantised once and written to the n_copies rows scatter[r * n_copies ..]
@@ -46,15 +54,19 @@ template <bool kFourBit, bool kScatter, int kLow>
 __global__ void __launch_bounds__(QWARPS * 32)
 quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restrict__ gather, int gather_div,
                   const int32_t* __restrict__ scatter, int n_copies,
-                  int64_t n_rows, int K, uint8_t* __restrict__ q, float* __restrict__ s) {
+                  int64_t n_rows, int K, uint8_t* __restrict__ q, float* __restrict__ s, int32_t* __restrict__ wide,
+                  const int32_t* __restrict__ kept, int64_t n_routed) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int nblk = K / QB, parts = (nblk + QU - 1) / QU;
-    uint8_t* q2 = q + n_rows * (kScatter ? n_copies : 1) * K;
+    const int64_t plane = n_rows * (kScatter ? n_copies : 1) * K;
+    uint8_t* q2 = q + plane;
+    const int64_t first_left_out = kept ? *kept : n_routed;
     const int64_t units = n_rows * parts;
     for (int64_t w = (int64_t)blockIdx.x * QWARPS + (threadIdx.x >> 5); w < units; w += (int64_t)gridDim.x * QWARPS) {
         const int64_t r = w / parts;
         const int b0 = (int)(w - r * parts) * QU;
+        if (r >= first_left_out && r < n_routed) continue;
         int64_t from = r;
         if (gather) {
             const int32_t g = gather[r];
@@ -95,18 +107,43 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
             constexpr float kUp = 1 << kLow;
             const float rr[4] = {(t[0] - lo.x) * kUp, (t[1] - lo.y) * kUp, (t[2] - hi.x) * kUp, (t[3] - hi.y) * kUp};
             const uint32_t a2 = e4m3x2(rr[0], rr[1]) | (e4m3x2(rr[2], rr[3]) << 16);
+            uint32_t a3 = 0, a4 = 0;
+            if constexpr (kLow > 0) {
+                const float2 lo2 = e4m3x2_to_f32x2(a2 & 0xffffu), hi2 = e4m3x2_to_f32x2(a2 >> 16);
+                float left[4] = {rr[0] - lo2.x, rr[1] - lo2.y, rr[2] - hi2.x, rr[3] - hi2.y};
+                int n = 0;  // values that leave something over, and 2^16 times the nonzero ones
+#pragma unroll
+                for (int i = 0; i < 4; ++i) n += (left[i] != 0.0f) + ((t[i] != 0.0f) << 16);
+                n = __reduce_add_sync(0xffffffffu, n);
+                if (8 * (n & 0xffff) > n >> 16) {
+                    constexpr float kDown = 1 << (kWideBits - kLow);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) left[i] *= kDown;
+                    a3 = e4m3x2(left[0], left[1]) | (e4m3x2(left[2], left[3]) << 16);
+                    const float2 lo3 = e4m3x2_to_f32x2(a3 & 0xffffu), hi3 = e4m3x2_to_f32x2(a3 >> 16);
+                    a4 = e4m3x2((left[0] - lo3.x) * kUp, (left[1] - lo3.y) * kUp) |
+                         (e4m3x2((left[2] - hi3.x) * kUp, (left[3] - hi3.y) * kUp) << 16);
+                    if (lane == 0) *wide = 1;
+                }
+            }
             if constexpr (kFourBit) {
                 // this lane's values are 0..3 (even lane) or 4..7 of 8: the even two, then the odd two
                 const int64_t at = r * K + b * QB + 8 * (lane >> 1) + 2 * (lane & 1);
-                *reinterpret_cast<uint16_t*>(q + at) = (uint16_t)__byte_perm(a, 0, 0x4420);
-                *reinterpret_cast<uint16_t*>(q + at + 4) = (uint16_t)__byte_perm(a, 0, 0x4431);
-                *reinterpret_cast<uint16_t*>(q2 + at) = (uint16_t)__byte_perm(a2, 0, 0x4420);
-                *reinterpret_cast<uint16_t*>(q2 + at + 4) = (uint16_t)__byte_perm(a2, 0, 0x4431);
+                const uint32_t codes[4] = {a, a2, a3, a4};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    *reinterpret_cast<uint16_t*>(q + i * plane + at) = (uint16_t)__byte_perm(codes[i], 0, 0x4420);
+                    *reinterpret_cast<uint16_t*>(q + i * plane + at + 4) = (uint16_t)__byte_perm(codes[i], 0, 0x4431);
+                }
             } else {
                 auto put = [&](int64_t to) {
                     const int64_t at = to * K + b * QB + 4 * lane;
                     *reinterpret_cast<uint32_t*>(q + at) = a;
                     *reinterpret_cast<uint32_t*>(q2 + at) = a2;
+                    if constexpr (kLow > 0) {
+                        *reinterpret_cast<uint32_t*>(q2 + plane + at) = a3;
+                        *reinterpret_cast<uint32_t*>(q2 + 2 * plane + at) = a4;
+                    }
                     if (lane == 0) s[to * nblk + b] = sc;
                 };
                 if constexpr (kScatter) {
@@ -121,30 +158,34 @@ quant_rows_kernel(const __nv_bfloat16* __restrict__ src, const int32_t* __restri
     }
 }
 
+template <bool kFourBit, bool kScatter, int kLow>
 static cudaError_t launch_quant(const void* src, const int32_t* gather, int gather_div, const int32_t* scatter,
-                                int n_copies, int64_t n_rows, int K, void* q, float* s, bool four_bit, int low,
-                                cudaStream_t stream) {
+                                int n_copies, int64_t n_rows, int K, void* q, float* s, int32_t* wide,
+                                const int32_t* kept, int64_t n_routed, cudaStream_t stream) {
     const int64_t units = n_rows * ((K / QB + QU - 1) / QU);
     const int blocks = (int)min64((units + QWARPS - 1) / QWARPS, (int64_t)sm_count() * 16);
     if (blocks <= 0) return cudaSuccess;
-    auto kernel = scatter     ? quant_rows_kernel<false, true, 0>
-                  : four_bit  ? quant_rows_kernel<true, false, kLowBits>
-                  : low       ? quant_rows_kernel<false, false, kLowBits>
-                              : quant_rows_kernel<false, false, 0>;
-    return launch_k(kernel, dim3(blocks), dim3(QWARPS * 32), 0, stream, static_cast<const __nv_bfloat16*>(src), gather, gather_div, scatter, n_copies, n_rows, K,
-                    static_cast<uint8_t*>(q), s);
+    return launch_k(quant_rows_kernel<kFourBit, kScatter, kLow>, dim3(blocks), dim3(QWARPS * 32), 0, stream,
+                    static_cast<const __nv_bfloat16*>(src), gather, gather_div, scatter, n_copies, n_rows, K,
+                    static_cast<uint8_t*>(q), s, wide, kept, n_routed);
+}
+
+cudaError_t launch_quant_planes(const void* src, int64_t n_rows, int K, void* q, float* s, bool four_bit, int32_t* wide,
+                                const int32_t* kept, int64_t n_routed, cudaStream_t stream) {
+    auto launch = four_bit ? launch_quant<true, false, kLowBits> : launch_quant<false, false, kLowBits>;
+    return launch(src, nullptr, 1, nullptr, 1, n_rows, K, q, s, wide, kept, n_routed, stream);
 }
 
 cudaError_t launch_quant_rows(const void* src, const int32_t* gather, int gather_div, int64_t n_rows, int K, void* q,
-                              float* s, bool four_bit, int low, cudaStream_t stream) {
-    return launch_quant(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, four_bit, low, stream);
+                              float* s, cudaStream_t stream) {
+    return launch_quant<false, false, 0>(src, gather, gather_div, nullptr, 1, n_rows, K, q, s, nullptr, nullptr, 0, stream);
 }
 
 // 2048 tokens x 8 copies, H 7168: 45 us, against 86 quantising each of the
 // 16384 gathered rows (every one a full read and all the arithmetic again).
 cudaError_t launch_quant_scatter(const void* src, const int32_t* pair_pos, int k, int64_t n_src, int K, void* q, float* s,
                                  cudaStream_t stream) {
-    return launch_quant(src, nullptr, 1, pair_pos, k, n_src, K, q, s, false, 0, stream);
+    return launch_quant<false, true, 0>(src, nullptr, 1, pair_pos, k, n_src, K, q, s, nullptr, nullptr, 0, stream);
 }
 
 }  // namespace gbmoe

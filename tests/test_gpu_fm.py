@@ -236,16 +236,17 @@ def test_activation_codes_keep_every_value(wq, T, spread):
 
 
 @pytest.mark.parametrize("wq", CODED)
+@pytest.mark.parametrize("e", [13, 24, 30])
 @pytest.mark.parametrize("T", [8, 24, 60])
-def test_values_beside_an_outlier_keep_their_precision(T, wq):
-    """One channel in 128 of x, and (4-bit formats) of h, is 2^12 or more times the
-    others, and every weight is 0 there, so that the output is made of the others
-    alone: 16-, 32- and 80-row tiles. 1e-2: bf16 rounding of h and y (5e-3 at most
-    over rows of this length), and as much again for codes that end at 2^-22 of
-    the outlier."""
+def test_values_beside_an_outlier_keep_their_precision(T, e, wq):
+    """One channel in 128 of x is 2^e times the others, one of h (4-bit formats)
+    about as much, and every weight is 0 there, so that the output is made of the
+    others alone: 16-, 32- and 80-row tiles, with the first pair of codes (2^13) and
+    with the second. 1e-2: bf16 rounding of h and y (5e-3 at most over rows of this
+    length), and as much again for the codes."""
     wl = BASE.replace(T=T, E=4, top_k=2, H=1024, I=768, wq=wq, seed=T)
     inp = synth.make_inputs(wl)
-    inp["x"].reshape(-1, 128)[:, 5] = 0x4600  # bf16 8192
+    inp["x"].reshape(-1, 128)[:, 5] = (127 + e) << 7  # bf16 2^e
     inp["w_router"].reshape(-1, 128)[:, 5] = 0
     ex = inp["experts"]
     for k in ("w_gate", "w_up"):
@@ -254,10 +255,27 @@ def test_values_beside_an_outlier_keep_their_precision(T, wq):
         else:
             ex[k][..., 2::64] &= 0x0F  # (the high nibble of byte 2 is channel 5)
     if wq != "fp8_b128":
-        for k in ("s_gate", "s_up"):  # rows 9, 137, .. times 2^7: h there about 2^14 times the rest
-            ex[k][:, 9::128] += 7 if wq == "mxfp4" else 7 << 7
+        for k in ("s_gate", "s_up"):  # rows 9, 137, .. times 2^(e / 2): h there about 2^e times the rest
+            ex[k][:, 9::128] += e // 2 + 1 if wq == "mxfp4" else (e // 2 + 1) << 7
         ex["w_down"][..., 4::64] &= 0x0F
     assert_close(act_np(forward(wl, to_device(wl, inp))), oracle.forward(wl, inp)["out"], 1e-2)
+
+
+@pytest.mark.parametrize("wq", CODED)
+@pytest.mark.parametrize("T", [8, 24, 60])
+def test_second_codes_of_a_row_leave_the_others_alone(T, wq):
+    """Rows that need their second pair of codes make the GEMMs walk k twice; every
+    other token's output stays bit for bit as it was."""
+    wl = BASE.replace(T=T, E=4, top_k=2, H=1024, I=768, wq=wq, seed=T)
+    dev = to_device(wl, synth.make_inputs(wl))
+    dev["logit_bias"] = torch.arange(wl.E, device="cuda", dtype=torch.float32) * 1e9  # the routing stays
+    a = forward(wl, dev)
+    dev["x"][2, 5] = 2.0**30
+    dev["x"][5, 700] = -(2.0**24)
+    b = forward(wl, dev)
+    same = [t for t in range(T) if t not in (2, 5)]
+    assert torch.equal(a[same].view(torch.int16), b[same].view(torch.int16))
+    assert not torch.equal(a[2].view(torch.int16), b[2].view(torch.int16)) and torch.isfinite(b.float()).all()
 
 
 def test_mxfp4_scales_at_two_byte_alignment():
