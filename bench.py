@@ -48,17 +48,17 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # whenever the kernels changed since the counters were taken. Captures
 # (python bench.py --workload W --set ... --profile 1 under
 # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum):
-#   decode   T=8 E=32 (29 active):    feature-major gate/up + down     1.0962 GB
-#   prefill  T=2048 E=32 (32 active): gate/up GEMM (own row gather) + down GEMM  1.6488 GB
-#   fp8      T=512 E=64 (64 active):  quantise, gate/up, quantise, down  2.9961 GB
-#   MXFP4    T=512 E=64 (64 active):  quantise, feature-major gate/up, quantise, down  1.6966 GB
+#   decode   T=8 E=32 (29 active):    feature-major gate/up + down     1.0961 GB
+#   prefill  T=2048 E=32 (32 active): gate/up GEMM (own row gather) + down GEMM  1.6594 GB
+#   fp8      T=512 E=64 (64 active):  quantise, gate/up, quantise, down  2.9963 GB
+#   MXFP4    T=512 E=64 (64 active):  quantise, feature-major gate/up, quantise, down  1.6967 GB
 # (the skewed int4 workload's offsets exist for its full size only, so its
 # reduced case differs in I and is not scaled here)
 TRAFFIC_PER_ACTIVE_EXPERT: dict = {
-    ("decode_bf16_T32_H4096_E128_k8_I1536", "fm"): 1.0962e9 / 29,
-    ("prefill_bf16_T8192_H4096_E128_k8_I1536", "tc"): 1.6488e9 / 32,
-    ("dsv3_fp8_T2048_H7168_E256s1_k8_I2048", "tc_fp8"): 2.9961e9 / 64,
-    ("dsv4_mxfp4_T2048_H7168_E256s1_k8_I2048", "fm"): 1.6966e9 / 64,
+    ("decode_bf16_T32_H4096_E128_k8_I1536", "fm"): 1.0961e9 / 29,
+    ("prefill_bf16_T8192_H4096_E128_k8_I1536", "tc"): 1.6594e9 / 32,
+    ("dsv3_fp8_T2048_H7168_E256s1_k8_I2048", "tc_fp8"): 2.9963e9 / 64,
+    ("dsv4_mxfp4_T2048_H7168_E256s1_k8_I2048", "fm"): 1.6967e9 / 64,
 }
 
 

@@ -44,12 +44,12 @@
 // lane of two warps, which meet there once per item. Every mbarrier wait is bounded (tc_ptx.cuh).
 //
 // Measured, fp8, 48 tokens, top 8 of 256 experts, H 7168, I 2048 (about 2 rows
-// per expert, 8.8 GB of weights): gate/up 1826 -> 767 us and down 1052 -> 397
-// us against the streaming kernels, 7.5 TB/s; the layer 3121 -> 1347 us. What
-// held it back on the way, per 128-wide k block: waits as calls (2400 -> 1750
-// cycles once inlined) and MMAs issued under `lane == 0` (1750 -> 1500).
-// int4, 17 tokens, top 6 of 64 experts, H 4096, I 2816: layer 1397 -> 220 us.
-// MXFP4, 16 tokens of the fp8 layer: 2896 -> 495 us. Its E8M0 scales go to the
+// per expert, 8.8 GB of weights): the layer 3116 -> 1302 us against the streaming
+// kernels, the copy rate over its weights. What held it back on the way, per
+// 128-wide k block: waits as calls (2400 -> 1750 cycles once inlined) and MMAs
+// issued under `lane == 0` (1750 -> 1500).
+// int4, 17 tokens, top 6 of 64 experts, H 4096, I 2816: layer 1352 -> 241 us.
+// MXFP4, 16 tokens of the fp8 layer: 2893 -> 516 us. Its E8M0 scales go to the
 // MMAs (kind::mxf8f6f4) and its codes are an operand as TMA unpacks them, so no
 // warp touches a weight. Decoding them to e4m3 with shifts and masks was bound by
 // the decode (635 us; 2.15 ms in place of 1.35 at 256 tokens), and scaling the
@@ -119,7 +119,7 @@ struct Cfg {
     // UNPACKED: the ring leaves the L1 cache 60 KB. A k block reads 4 bytes of
     // scales in each of 256 lines, and eight k blocks share a sector, so the lines
     // (32 KB) have to outlive a k block: with all 228 KB as shared memory they
-    // were refetched each time (16-row tiles 597 us with 6 stages, 495 with 5 or
+    // were refetched each time (sweep: 16-row tiles 597 us with 6 stages, 495 with 5 or
     // 4; 32-row tiles at 8 rows per expert 1631 with 5, 1351 with 4, 1434 with 3).
     static constexpr int MAX_STAGES = !UNPACKED ? 6 : ROWS == 16 ? 5 : ROWS == 32 ? 4 : 3;
     static constexpr int MAX_RING = MAX_STAGES + 4;
